@@ -236,3 +236,86 @@ def tolerance(case):
     if case["dtype"] == F32:
         return {"rel": 5e-6, "max": 5e-5, "differ": 1e-3}
     return {"rel": 1e-2, "max": 8e-2, "differ": 1e-3}
+
+
+# ---------------------------------------------------------------- the same outputs in float64
+
+def _up_down(x, W1, W2, gate):
+    """sum over e of gate[:, e] * GeLU(x W1[e]) W2[e], only over the tokens with a gate."""
+    out = torch.zeros((x.shape[0], W2.shape[2]), dtype=torch.float64, device=x.device)
+    for e in range(W1.shape[0]):
+        t = gate[:, e].nonzero().flatten()
+        if t.numel():
+            h = torch.nn.functional.gelu(x[t] @ W1[e].double())
+            out.index_add_(0, t, gate[t, e:e + 1] * (h @ W2[e].double()))
+    return out
+
+
+def _attention(c, q, K, V, seq, pos):
+    """q [n, n_head, d_head] of tokens with sequences seq and last visible positions pos."""
+    o = torch.empty_like(q)
+    step = max(1, (1 << 27) // (c["n_head"] * c["cache"] * c["d_head"]))
+    at = torch.arange(c["cache"], device=q.device)
+    for i in range(0, q.shape[0], step):
+        k, v = K[seq[i:i + step]].double(), V[seq[i:i + step]].double()
+        a = torch.einsum("nhd,nhld->nhl", q[i:i + step], k) / math.sqrt(c["d_head"])
+        a = a.masked_fill(at[None, None, :] > pos[i:i + step, None, None], -math.inf).softmax(dim=-1)
+        o[i:i + step] = torch.einsum("nhl,nhld->nhd", a, v)
+    return o
+
+
+def exact(case, seed):
+    c, E = case, case["E"]
+    s = prepare(case, seed)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    # the weights again, as prepare() drew them before it packed them
+    dt = torch.float32 if c["dtype"] == F32 else torch.bfloat16
+    torch.randn((c["T"], c["d"]), generator=g, device="cuda", dtype=dt)
+    torch.randn((c["d"], E), generator=g, device="cuda", dtype=torch.float32)
+    if c["zipf"]:
+        torch.randperm(E, generator=g, device="cuda")
+    W1 = torch.randn((E, c["d"], c["H"]), generator=g, device="cuda", dtype=dt).mul_(0.02)
+    W2 = torch.randn((E, c["H"], c["d"]), generator=g, device="cuda", dtype=dt).mul_(0.02)
+    x = s["x"].double()
+    S = x @ s["Wr"].double()
+    if s["br"] is not None:
+        S = S + s["br"].double()
+    S = S.softmax(dim=1)
+    if c["kind"] == "training":
+        m = S.mean(dim=0)
+        logS, logm = S.log(), m.log()
+        H_cond, H_marg = -(S * logS).sum(dim=1).mean(), -(m * logm).sum()
+        # L = H(e|X) - H(e): the derivative by one score
+        dL = (logm[None, :] - logS) / c["T"]
+        dO = s["dO"].double()
+        dS = torch.empty_like(S)
+        dA = torch.empty((c["T"], E, c["H"]), dtype=torch.float64, device="cuda")
+        for e in range(E):
+            G = dO @ W2[e].double().T
+            dS[:, e] = (torch.nn.functional.gelu(x @ W1[e].double()) * G).sum(dim=1)
+            dA[:, e] = S[:, e:e + 1] * G
+        return {"loss": torch.stack([H_cond - H_marg, H_marg, H_cond]), "mi_grad": dL, "dS": dS, "dA": dA.view(c["T"], -1),
+                "scores": S}
+    if c["mode"] == "all":
+        sel = torch.ones_like(S, dtype=torch.bool)
+    elif c["mode"] == "threshold":
+        sel = S * E > c["eps"]
+    else:
+        k = c["K"]
+        if c["mode"] == "threshold_topk":
+            k = math.floor((S * E > c["eps"]).sum().item() / c["T"] + 0.5)
+        k = min(E, max(1, k))
+        sel = torch.zeros_like(S, dtype=torch.bool).scatter_(1, S.topk(k, dim=1).indices, True)
+    gate = S * sel
+    mask = None if E >= 64 else (sel.long() << torch.arange(E, device="cuda")).sum(dim=1)
+    counts = sel.sum(dim=0).int()
+    if c["kind"] == "moa":
+        out = torch.zeros((c["T"], c["d"]), dtype=torch.float64, device="cuda")
+        for e in range(E):
+            t = sel[:, e].nonzero().flatten()
+            if t.numel():
+                q = (x[t] @ W1[e].double()).view(-1, c["n_head"], c["d_head"])
+                o = _attention(c, q, s["K"], s["V"], s["seq"][t].long(), s["pos"][t].long())
+                out.index_add_(0, t, gate[t, e:e + 1] * (o.reshape(t.numel(), -1) @ W2[e].double()))
+        return {"out": out, "mask": mask, "counts": counts}
+    return {"out": _up_down(x, W1, W2, gate), "mask": mask, "counts": counts}
