@@ -261,8 +261,13 @@ __device__ __forceinline__ Tile decode_tile(const GemmParams& P, const Shared& s
     if (P.mode == GEMM_GROUPED) {
         const int splits = max(P.k_splits, 1), split = id % splits;
         id /= splits;
+        // The expert whose tiles `id` falls into (tile_prefix[e] <= id < tile_prefix[e + 1]), by bisection: every role
+        // decodes every tile, in series with its work, and walking up to 63 entries was a fair part of a narrow
+        // expert's tile (7001 tokens, 32 experts of 512, d 4096: layer 456 -> 449 us; 4096 tokens, 64 skewed experts: 717 -> 701).
         int e = 0;
-        while (e + 1 < P.E && id >= sh.tile_prefix[e + 1]) ++e;
+#pragma unroll
+        for (int step = kMaxExperts / 2; step > 0; step >>= 1)
+            if (e + step < P.E && id >= sh.tile_prefix[e + step]) e += step;
         const int local = id - sh.tile_prefix[e];
         const int cnt = sh.seg1[e] - sh.seg0[e];
         const int mtiles = (cnt + MT - 1) / MT;
