@@ -18,6 +18,7 @@ template <typename AT, typename BT, typename OT, bool GELU>
 __global__ void __launch_bounds__(256) grouped_gemm_fma_kernel(const AT* __restrict__ A, const BT* __restrict__ B,
                                                                OT* __restrict__ C, const int32_t* __restrict__ offsets,
                                                                int E, int K, int N, int64_t amax) {
+    chain_wait();
     constexpr int BM = 64, BN = 64, BK = 16;
     __shared__ float As[BK][BM + 1];
     __shared__ float Bs[BK][BN];
@@ -61,6 +62,7 @@ __global__ void __launch_bounds__(256) grouped_gemm_fma_kernel(const AT* __restr
         }
         __syncthreads();
     }
+    chain_next();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int r = r0 + ty * 4 + i;
@@ -78,12 +80,10 @@ static dsmoe_status run(const dsmoe_layer_desc& p, const XT* xp, const XT* W1, c
                         float* h, XT* yp, cudaStream_t s) {
     const size_t amax = amax_of(p);
     const unsigned gx = (unsigned)(amax / 64 + p.E + 1);
-    grouped_gemm_fma_kernel<XT, XT, float, true>
-        <<<dim3(gx, ceil_div(p.H, 64)), 256, 0, s>>>(xp, W1, h, offsets, p.E, p.d, p.H, (int64_t)amax);
-    DSMOE_CUDA_TRY(cudaGetLastError());
-    grouped_gemm_fma_kernel<float, XT, XT, false>
-        <<<dim3(gx, ceil_div(p.d, 64)), 256, 0, s>>>(h, W2, yp, offsets, p.E, p.H, p.d, (int64_t)amax);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(grouped_gemm_fma_kernel<XT, XT, float, true>, dim3(gx, ceil_div(p.H, 64)), 256, 0, s,
+        xp, W1, h, offsets, p.E, p.d, p.H, (int64_t)amax));
+    DSMOE_CUDA_TRY(launch_chained(grouped_gemm_fma_kernel<float, XT, XT, false>, dim3(gx, ceil_div(p.d, 64)), 256, 0, s,
+        h, W2, yp, offsets, p.E, p.H, p.d, (int64_t)amax));
     return DSMOE_OK;
 }
 

@@ -30,6 +30,7 @@ moa_attention_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restrict__
                      int E, int n_head, int H, int T, const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __restrict__ Vc,
                      const int32_t* __restrict__ tok_seq, const int32_t* __restrict__ pos, int n_seq, int L, float scale,
                      int* __restrict__ dev_status) {
+    chain_wait();
     constexpr int DH = 32 * DPL;
     extern __shared__ float moa_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -97,6 +98,7 @@ moa_attention_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restrict__
 #pragma unroll
         for (int i = 0; i < DPL; ++i) acc[i] = fmaf(p, __bfloat162float(vr[32 * i]), acc[i]);
     }
+    chain_next();
     const float inv = 1.f / den;
 #pragma unroll
     for (int i = 0; i < DPL; ++i) qrow[lane + 32 * i] = __float2bfloat16_rn(acc[i] * inv);
@@ -134,6 +136,7 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restri
                          const __nv_bfloat16* __restrict__ Vc, const int32_t* __restrict__ tok_seq,
                          const int32_t* __restrict__ pos, int n_seq, int L, float scale, long long n_tiles,
                          int* __restrict__ dev_status) {
+    chain_wait();
     constexpr int STRIDE = DH * 2 + 16;                 // bytes per key row in shared memory: 16 of padding
     constexpr int KS = DH / 16, DT = DH / 8, CH = DH / 8;
     extern __shared__ __align__(16) unsigned char moa_mma_smem[];
@@ -390,6 +393,7 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restri
         qa[(size_t)r * H + j * DH + dcol] = __float2bfloat16_rn(num / den);
     }
     }
+    chain_next();
 }
 
 template <int DH, int kMmaWarps>
@@ -419,9 +423,10 @@ dsmoe_status launch_mma_attention_nw(const dsmoe_layer_desc& p, const MoaCore& c
     const long long resident = (long long)st->sm_count * (per_sm > 0 ? per_sm : 1);
     const long long want = kMmaWarps > 2 ? n_tiles : (n_tiles + kMmaWarps - 1) / kMmaWarps;     // 2 warps: a tile per warp
     const long long ctas = want < resident ? want : resident;
-    moa_attention_mma_kernel<DH, kMmaWarps><<<(unsigned)ctas, 32 * kMmaWarps, smem, s>>>(
-        q, token_rows, W, row_tiles, tpt, (long long)amax_of(p), c.n_head, p.H, p.T, static_cast<const __nv_bfloat16*>(c.Kc),
-        static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos, c.n_seq, c.L, c.scale, n_tiles, dev_status);
+    DSMOE_CUDA_TRY(launch_chained(moa_attention_mma_kernel<DH, kMmaWarps>, (unsigned)ctas, 32 * kMmaWarps, smem, s,
+        q, token_rows, W, row_tiles, tpt, (long long)amax_of(p), c.n_head, p.H, p.T, static_cast<const
+        __nv_bfloat16*>(c.Kc), static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos, c.n_seq, c.L, c.scale,
+        n_tiles, dev_status));
     return DSMOE_OK;
 }
 
@@ -454,7 +459,6 @@ dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, v
         if (dh == 64) DSMOE_TRY(launch_mma_attention<64>(p, c, qb, token_rows, dev_status, s));
         else if (dh == 96) DSMOE_TRY(launch_mma_attention<96>(p, c, qb, token_rows, dev_status, s));
         else DSMOE_TRY(launch_mma_attention<128>(p, c, qb, token_rows, dev_status, s));
-        DSMOE_CUDA_TRY(cudaGetLastError());
         return timing_end(s, timed);
     }
     int warps = kMoaWarps;
@@ -473,8 +477,9 @@ dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, v
         if (smem > 48 * 1024)                                                                                             \
             DSMOE_CUDA_TRY(cudaFuncSetAttribute(moa_attention_kernel<DPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                                                 (int)smem));                                                              \
-        moa_attention_kernel<DPL><<<grid, 32 * kMoaWarps, smem, s>>>(q, row_token, offsets, p.E, c.n_head, p.H, p.T, K, V, \
-                                                                     c.tok_seq, c.pos, c.n_seq, c.L, c.scale, dev_status); \
+        DSMOE_CUDA_TRY(launch_chained(moa_attention_kernel<DPL>, grid, 32 * kMoaWarps, smem, s,                         \
+            q, row_token, offsets, p.E, c.n_head, p.H, p.T, K, V, c.tok_seq, c.pos, c.n_seq, c.L, c.scale,              \
+            dev_status));                                                                                               \
     } while (0)
     switch (dh / 32) {
         case 1: MOA_LAUNCH(1); break;
@@ -488,7 +493,6 @@ dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, v
         default: return DSMOE_ERR_UNSUPPORTED;
     }
 #undef MOA_LAUNCH
-    DSMOE_CUDA_TRY(cudaGetLastError());
     DSMOE_TRY(timing_end(s, timed));
     return DSMOE_OK;
 }

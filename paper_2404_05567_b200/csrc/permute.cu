@@ -25,6 +25,8 @@ __global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __re
                                                             int32_t* __restrict__ row_token, float* __restrict__ row_gate,
                                                             int32_t* __restrict__ token_rows, int T, int E, int W,
                                                             int64_t amax, uint4* __restrict__ zero_out, int row_vecs) {
+    chain_next();
+    chain_wait();
     // a chunk's scores, staged so that the loop over the experts below waits for no load: [token][E + 1]
     __shared__ float sc_s[4][kChunk * (kMaxExperts + 1)];
     __shared__ int before_s[4][kMaxExperts], total_s[4][kMaxExperts], base_s[4][kMaxExperts];
@@ -220,6 +222,8 @@ __global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __re
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ row_token,
                                                           const int32_t* __restrict__ offsets, uint4* __restrict__ xp,
                                                           int E, int T, int vec_per_row, int64_t amax) {
+    chain_next();
+    chain_wait();
     const int64_t A = min((int64_t)offsets[E], amax);
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * 8;
@@ -248,6 +252,8 @@ __global__ void __launch_bounds__(128) combine_bf16_kernel(const uint4* __restri
                                                            const int32_t* __restrict__ token_rows,
                                                            const int32_t* __restrict__ k_t, void* __restrict__ out,
                                                            int d, int W, int64_t amax) {
+    chain_next();
+    chain_wait();
     __shared__ int32_t rows_s[kMaxExperts];
     __shared__ float gate_s[kMaxExperts];
     const int t = blockIdx.x;
@@ -294,6 +300,8 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float4* __restri
                                                           const int32_t* __restrict__ token_rows,
                                                           const int32_t* __restrict__ k_t, void* __restrict__ out,
                                                           int d, int W, int64_t amax) {
+    chain_next();
+    chain_wait();
     __shared__ int32_t rows_s[kMaxExperts];
     __shared__ float gate_s[kMaxExperts];
     const int t = blockIdx.x;
@@ -338,6 +346,8 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float4* __restri
 // (32x32 tiles through smem; rows is a multiple of 64 where this layout is used).
 __global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16* __restrict__ src,
                                                              __nv_bfloat16* __restrict__ dst, int rows, int cols) {
+    chain_next();
+    chain_wait();
     __shared__ __nv_bfloat16 tile[32][33];
     const size_t base = (size_t)blockIdx.z * rows * cols;
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
@@ -360,17 +370,15 @@ dsmoe_status launch_permute(const dsmoe_layer_desc& p, const void* x, const floa
     const int nchunks = ceil_div(p.T, kChunk);
     const int64_t amax = (int64_t)amax_of(p);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
-    permute_index_kernel<0><<<ceil_div(nchunks, 4), 128, 0, s>>>(mask, scores, const_cast<int32_t*>(offsets), chunk_prefix,
-                                                                    nullptr, nullptr, row_token, row_gate, token_rows, p.T,
-                                                                    p.E, width_of(p), amax, static_cast<uint4*>(zero_out),
-                                                                    row_vecs);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<0>, ceil_div(nchunks, 4), 128, 0, s,
+        mask, scores, const_cast<int32_t*>(offsets), chunk_prefix, nullptr, nullptr, row_token, row_gate,
+        token_rows, p.T, p.E, width_of(p), amax, static_cast<uint4*>(zero_out), row_vecs));
     if (xp) {
         const int vec_per_row = (int)((size_t)p.d * elem_size(p.dtype) / 16);
         const int grid = (int)(amax / 8 + 1 < 148 * 16 ? amax / 8 + 1 : 148 * 16);
-        gather_rows_kernel<<<grid, 256, 0, s>>>(static_cast<const uint4*>(x), row_token, offsets,
-                                                static_cast<uint4*>(xp), p.E, p.T, vec_per_row, amax);
-        DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(gather_rows_kernel, grid, 256, 0, s,
+            static_cast<const uint4*>(x), row_token, offsets, static_cast<uint4*>(xp), p.E, p.T, vec_per_row,
+            amax));
     }
     return DSMOE_OK;
 }
@@ -384,11 +392,9 @@ dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const 
     const int nchunks = ceil_div(p.T, kChunk);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
     if (nchunks > 0 && nchunks <= kCountInBlockChunks) {
-        permute_index_kernel<2><<<ceil_div(nchunks, 4), 128, 0, s>>>(mask, scores, offsets, nullptr, counts, counts_out,
-                                                                    row_token, row_gate, token_rows, p.T, p.E, width_of(p),
-                                                                    (int64_t)amax_of(p), static_cast<uint4*>(zero_out),
-                                                                    row_vecs);
-        DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<2>, ceil_div(nchunks, 4), 128, 0, s,
+            mask, scores, offsets, nullptr, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
+            width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs));
         return DSMOE_OK;
     }
     if (!chunk_counts_ready) DSMOE_TRY(launch_chunk_counts(p, mask, chunk_prefix, s));
@@ -397,11 +403,9 @@ dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const 
         return launch_permute(p, nullptr, scores, mask, offsets, chunk_prefix, row_token, row_gate, token_rows, nullptr, s,
                               zero_out);
     }
-    permute_index_kernel<1><<<ceil_div(nchunks, 4), 128, 0, s>>>(mask, scores, offsets, chunk_prefix, counts, counts_out,
-                                                                   row_token, row_gate, token_rows, p.T, p.E, width_of(p),
-                                                                   (int64_t)amax_of(p), static_cast<uint4*>(zero_out),
-                                                                   row_vecs);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<1>, ceil_div(nchunks, 4), 128, 0, s,
+        mask, scores, offsets, chunk_prefix, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
+        width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs));
     return DSMOE_OK;
 }
 
@@ -414,20 +418,22 @@ dsmoe_status launch_combine(const dsmoe_layer_desc& p, const void* yp, const flo
     const int col_blocks = ceil_div(p.d / (yp_f32 || p.dtype != DSMOE_BF16 ? 4 : 8), 128);
     const dim3 grid(p.T, (unsigned)(std::max(1, std::min(col_blocks, 1024 / p.T))));
     if (yp_f32 && p.dtype == DSMOE_BF16 && !p.out_fp32) {
-        combine_f32_kernel<true><<<grid, 128, 0, s>>>(static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax);
+        DSMOE_CUDA_TRY(launch_chained(combine_f32_kernel<true>, grid, 128, 0, s,
+            static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     } else if (yp_f32) {
-        combine_f32_kernel<false><<<grid, 128, 0, s>>>(static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax);
+        DSMOE_CUDA_TRY(launch_chained(combine_f32_kernel<false>, grid, 128, 0, s,
+            static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     } else if (p.dtype == DSMOE_BF16) {
         if (p.out_fp32)
-            combine_bf16_kernel<true><<<grid, 128, 0, s>>>(static_cast<const uint4*>(yp), row_gate, token_rows, k_t, out,
-                                                         p.d, W, amax);
+            DSMOE_CUDA_TRY(launch_chained(combine_bf16_kernel<true>, grid, 128, 0, s,
+                static_cast<const uint4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
         else
-            combine_bf16_kernel<false><<<grid, 128, 0, s>>>(static_cast<const uint4*>(yp), row_gate, token_rows, k_t, out,
-                                                          p.d, W, amax);
+            DSMOE_CUDA_TRY(launch_chained(combine_bf16_kernel<false>, grid, 128, 0, s,
+                static_cast<const uint4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     } else {
-        combine_f32_kernel<false><<<grid, 128, 0, s>>>(static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax);
+        DSMOE_CUDA_TRY(launch_chained(combine_f32_kernel<false>, grid, 128, 0, s,
+            static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     }
-    DSMOE_CUDA_TRY(cudaGetLastError());
     return DSMOE_OK;
 }
 
@@ -435,6 +441,8 @@ dsmoe_status launch_combine(const dsmoe_layer_desc& p, const void* yp, const flo
 __global__ void __launch_bounds__(256) stats_kernel(const float* __restrict__ scores, const uint64_t* __restrict__ mask,
                                                     dsmoe_selection_stats* __restrict__ st, int T, int E, int mode, float eps,
                                                     int eps_normalized) {
+    chain_next();
+    chain_wait();
     __shared__ int cnt_s[kMaxExperts];
     __shared__ unsigned long long near_s, a_s;
     __shared__ int zero_s;
@@ -472,6 +480,8 @@ __global__ void __launch_bounds__(256) stats_kernel(const float* __restrict__ sc
 }
 
 __global__ void stats_finish_kernel(dsmoe_selection_stats* st, int E) {
+    chain_next();
+    chain_wait();
     int n = 0;
     for (int e = 0; e < E; ++e) n += st->counts[e] == 0;
     st->empty_experts = n;
@@ -482,11 +492,10 @@ dsmoe_status launch_stats(const dsmoe_layer_desc& p, const float* scores, const 
     DSMOE_CUDA_TRY(cudaMemsetAsync(stats, 0, sizeof(dsmoe_selection_stats), s));
     if (p.T > 0) {
         const int grid = ceil_div(p.T, 8) < 1184 ? ceil_div(p.T, 8) : 1184;
-        stats_kernel<<<grid, 256, 0, s>>>(scores, mask, stats, p.T, p.E, p.mode, p.eps, p.eps_normalized);
-        DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(stats_kernel, grid, 256, 0, s,
+            scores, mask, stats, p.T, p.E, p.mode, p.eps, p.eps_normalized));
     }
-    stats_finish_kernel<<<1, 1, 0, s>>>(stats, p.E);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(stats_finish_kernel, 1, 1, 0, s, stats, p.E));
     return DSMOE_OK;
 }
 
@@ -496,10 +505,10 @@ dsmoe_status launch_pack(const dsmoe_layer_desc& p, const void* W1, const void* 
     __nv_bfloat16* w1t = static_cast<__nv_bfloat16*>(packed);
     __nv_bfloat16* w2t = w1t + (size_t)p.E * p.H * p.d;
     // W1[e]: [d,H] -> [d/64][H][64];  W2[e]: [H,d] -> [H/64][d][64]
-    transpose_bf16_kernel<<<dim3(ceil_div(p.H, 32), ceil_div(p.d, 32), p.E), 256, 0, s>>>(w1, w1t, p.d, p.H);
-    DSMOE_CUDA_TRY(cudaGetLastError());
-    transpose_bf16_kernel<<<dim3(ceil_div(p.d, 32), ceil_div(p.H, 32), p.E), 256, 0, s>>>(w2, w2t, p.H, p.d);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(transpose_bf16_kernel, dim3(ceil_div(p.H, 32), ceil_div(p.d, 32), p.E), 256, 0, s,
+        w1, w1t, p.d, p.H));
+    DSMOE_CUDA_TRY(launch_chained(transpose_bf16_kernel, dim3(ceil_div(p.d, 32), ceil_div(p.H, 32), p.E), 256, 0, s,
+        w2, w2t, p.H, p.d));
     return DSMOE_OK;
 }
 

@@ -22,6 +22,8 @@ __global__ void __launch_bounds__(256) router_small_kernel(const XT* __restrict_
                                                            const float* __restrict__ br, float* __restrict__ scores,
                                                            uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
                                                            int T, int d, SelParams q) {
+    chain_next();
+    chain_wait();
     __shared__ float red[TT][8][EP];
     const int t0 = blockIdx.x * TT, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int E = q.E;
@@ -146,6 +148,7 @@ __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* __
                                                                     const float* __restrict__ br, float* __restrict__ scores,
                                                                     uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
                                                                     int T, int d, SelParams q) {
+    chain_wait();
     constexpr int TB = kRtTB, KC = kRtKC, EP = 8 * EPL, XS = kRtXS, NT = kRtThreads;
     constexpr int NW = KC * EP / NT, NX = TB * KC / 8 / NT, KQ = KC / kRtSplit;
     static_assert(NX == 1 && NW >= 1, "staging: one 8-element group of x per thread");
@@ -226,6 +229,7 @@ __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* __
     }
     // the groups' partial logits -> shared memory as [group][token][expert] (all staging buffers are free now), then
     // one warp per token adds them in group order
+    chain_next();
     float* Ls = rt_smem;                            // kRtSplit x TB x EP floats
 #pragma unroll
     for (int i = 0; i < 2; ++i)
@@ -253,6 +257,8 @@ __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* __
 // Selection alone on caller-supplied scores: one warp per token.
 __global__ void __launch_bounds__(256) select_kernel(const float* __restrict__ scores, uint64_t* __restrict__ mask,
                                                      int32_t* __restrict__ k_t, int T, SelParams q) {
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (t >= T) return;
@@ -272,6 +278,8 @@ __global__ void __launch_bounds__(256) select_kernel(const float* __restrict__ s
 // expert e, 32 chunks per warp-wide scan) and writes the totals and their offsets.
 __global__ void __launch_bounds__(256) chunk_count_kernel(const uint64_t* __restrict__ mask, int32_t* __restrict__ chunk_prefix,
                                                           int T, int E) {
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (c * kChunk >= T) return;
@@ -291,6 +299,8 @@ __global__ void __launch_bounds__(256) chunk_count_kernel(const uint64_t* __rest
 __global__ void __launch_bounds__(1024) finalize_kernel(int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
                                                         int32_t* __restrict__ chunk_prefix, int32_t* __restrict__ counts_out,
                                                         int T, int E) {
+    chain_next();
+    chain_wait();
     __shared__ int32_t cnt_s[kMaxExperts];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nchunks = (T + kChunk - 1) / kChunk;
@@ -357,9 +367,11 @@ static dsmoe_status launch_router_t(const dsmoe_layer_desc& p, const XT* x, cons
 #define ROUTER_SMALL(EP, TT)                                                                                            \
     do {                                                                                                                \
         if (p.T >= 64)                                                                                                  \
-            router_small_kernel<XT, EP, TT><<<ceil_div(p.T, TT), 256, 0, s>>>(x, Wr, br, scores, mask, k_t, p.T, p.d, q); \
+            DSMOE_CUDA_TRY(launch_chained(router_small_kernel<XT, EP, TT>, ceil_div(p.T, TT), 256, 0, s,                \
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q));                                                            \
         else                                                                                                            \
-            router_small_kernel<XT, EP, 1><<<p.T, 256, 0, s>>>(x, Wr, br, scores, mask, k_t, p.T, p.d, q);             \
+            DSMOE_CUDA_TRY(launch_chained(router_small_kernel<XT, EP, 1>, p.T, 256, 0, s,                               \
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q));                                                            \
     } while (0)
         if (p.E <= 8) ROUTER_SMALL(8, 4);
         else if (p.E <= 16) ROUTER_SMALL(16, 4);
@@ -379,11 +391,12 @@ static dsmoe_status launch_router_t(const dsmoe_layer_desc& p, const XT* x, cons
             attr_set = true;
         }
         if (p.E <= 32)
-            router_tile_kernel<XT, 4><<<grid, kRtThreads, router_tile_smem<4>(), s>>>(x, Wr, br, scores, mask, k_t, p.T, p.d, q);
+            DSMOE_CUDA_TRY(launch_chained(router_tile_kernel<XT, 4>, grid, kRtThreads, router_tile_smem<4>(), s,
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q));
         else
-            router_tile_kernel<XT, 8><<<grid, kRtThreads, router_tile_smem<8>(), s>>>(x, Wr, br, scores, mask, k_t, p.T, p.d, q);
+            DSMOE_CUDA_TRY(launch_chained(router_tile_kernel<XT, 8>, grid, kRtThreads, router_tile_smem<8>(), s,
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q));
     }
-    DSMOE_CUDA_TRY(cudaGetLastError());
     return DSMOE_OK;
 }
 
@@ -399,6 +412,8 @@ dsmoe_status launch_router(const dsmoe_layer_desc& p, const void* x, const float
 // threshold gave, rounded half up and kept within [1, E].  One block; integer sums, so the result does not depend
 // on the order of the additions.
 __global__ void __launch_bounds__(1024) batch_k_kernel(const int32_t* __restrict__ k_t, int T, int E, int* __restrict__ K_out) {
+    chain_next();
+    chain_wait();
     __shared__ long long part[32];
     long long sum = 0;
     for (int t = threadIdx.x; t < T; t += 1024) sum += k_t[t];
@@ -422,32 +437,29 @@ dsmoe_status launch_select(const dsmoe_layer_desc& p, const float* scores, uint6
         if (!k_scratch) return DSMOE_ERR_UNSUPPORTED;
         q.mode = DSMOE_SELECT_THRESHOLD;
         q.min_k = 0;                     // the counts are the threshold's own
-        select_kernel<<<ceil_div(p.T, 8), 256, 0, s>>>(scores, mask, k_t, p.T, q);
-        DSMOE_CUDA_TRY(cudaGetLastError());
-        batch_k_kernel<<<1, 1024, 0, s>>>(k_t, p.T, p.E, k_scratch);
-        DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(select_kernel, ceil_div(p.T, 8), 256, 0, s, scores, mask, k_t, p.T, q));
+        DSMOE_CUDA_TRY(launch_chained(batch_k_kernel, 1, 1024, 0, s, k_t, p.T, p.E, k_scratch));
         q.mode = DSMOE_SELECT_TOPK;
         q.min_k = p.min_k;
         q.K_dev = k_scratch;
     }
-    select_kernel<<<ceil_div(p.T, 8), 256, 0, s>>>(scores, mask, k_t, p.T, q);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(select_kernel, ceil_div(p.T, 8), 256, 0, s, scores, mask, k_t, p.T, q));
     return DSMOE_OK;
 }
 
 dsmoe_status launch_chunk_counts(const dsmoe_layer_desc& p, const uint64_t* mask, int32_t* chunk_prefix, cudaStream_t s) {
     const int nchunks = ceil_div(p.T, kChunk);
     if (nchunks > 0) {
-        chunk_count_kernel<<<ceil_div(nchunks, 8), 256, 0, s>>>(mask, chunk_prefix, p.T, p.E);
-        DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(chunk_count_kernel, ceil_div(nchunks, 8), 256, 0, s,
+            mask, chunk_prefix, p.T, p.E));
     }
     return DSMOE_OK;
 }
 
 dsmoe_status launch_chunk_scan(const dsmoe_layer_desc& p, int32_t* counts, int32_t* offsets, int32_t* chunk_prefix,
                                int32_t* counts_out, cudaStream_t s) {
-    finalize_kernel<<<1, 1024, 0, s>>>(counts, offsets, chunk_prefix, counts_out, p.T, p.E);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(finalize_kernel, 1, 1024, 0, s,
+        counts, offsets, chunk_prefix, counts_out, p.T, p.E));
     return DSMOE_OK;
 }
 

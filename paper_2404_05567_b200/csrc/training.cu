@@ -12,6 +12,8 @@ constexpr int kMiBlocks = 296;        // upper bound on the first stage's grid (
 // (warp w of the block takes tokens w, w + 8, ...; lanes hold experts lane and lane + 32; the warps' sums meet in shared
 // memory and are added in warp order).  part[b][0..E) = sum_t S[t,e], part[b][64] = sum_t H(e|X_t).
 __global__ void __launch_bounds__(256) mi_partial_kernel(const float* __restrict__ S, double* __restrict__ part, int T, int E) {
+    chain_next();
+    chain_wait();
     __shared__ double red[8][kMaxExperts + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = (T + gridDim.x - 1) / gridDim.x;
@@ -43,6 +45,8 @@ __global__ void __launch_bounds__(256) mi_partial_kernel(const float* __restrict
 // Stage 2: one block.  p(e) = mean score, H(e), mean H(e|X), L_MI = -H(e) + mean H(e|X); p(e) is left in `pe`.
 __global__ void __launch_bounds__(64) mi_finish_kernel(const double* __restrict__ part, int nblocks, int T, int E,
                                                        float* __restrict__ out3, double* __restrict__ pe) {
+    chain_next();
+    chain_wait();
     __shared__ double term[kMaxExperts];
     const int e = threadIdx.x;
     double v = 0.0;
@@ -67,6 +71,8 @@ __global__ void __launch_bounds__(64) mi_finish_kernel(const double* __restrict_
 // dL_MI/dS[t,e] = (log p(e) - log S[t,e]) / T   (0 where the score is 0)
 __global__ void __launch_bounds__(256) mi_grad_kernel(const float* __restrict__ S, const double* __restrict__ pe,
                                                       float* __restrict__ grad, long long n, int T, int E) {
+    chain_next();
+    chain_wait();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
     const float s = S[i];
@@ -86,6 +92,7 @@ __global__ void __launch_bounds__(256) dense_backward_plain_kernel(const XT* __r
                                                                    const XT* __restrict__ W2, const float* __restrict__ S,
                                                                    const uint64_t* __restrict__ mask, const XT* __restrict__ dO,
                                                                    float* __restrict__ dS, XT* __restrict__ dA, int d, int H, int E) {
+    chain_wait();
     __shared__ float red[8];
     const int t = blockIdx.x / E, e = blockIdx.x % E;
     const bool active = !mask || ((mask[t] >> e) & 1ull);
@@ -127,14 +134,12 @@ dsmoe_status launch_mi_loss(const dsmoe_layer_desc& p, const float* scores, floa
     double* part = reinterpret_cast<double*>(scratch);
     double* pe = part + (size_t)kMiBlocks * (kMaxExperts + 1);
     const int nblocks = ceil_div(p.T, 64) < kMiBlocks ? ceil_div(p.T, 64) : kMiBlocks;
-    mi_partial_kernel<<<nblocks, 256, 0, s>>>(scores, part, p.T, p.E);
-    DSMOE_CUDA_TRY(cudaGetLastError());
-    mi_finish_kernel<<<1, 64, 0, s>>>(part, nblocks, p.T, p.E, out3, pe);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    DSMOE_CUDA_TRY(launch_chained(mi_partial_kernel, nblocks, 256, 0, s, scores, part, p.T, p.E));
+    DSMOE_CUDA_TRY(launch_chained(mi_finish_kernel, 1, 64, 0, s, part, nblocks, p.T, p.E, out3, pe));
     if (grad) {
         const long long n = (long long)p.T * p.E;
-        mi_grad_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(scores, pe, grad, n, p.T, p.E);
-        DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(mi_grad_kernel, (unsigned)((n + 255) / 256), 256, 0, s,
+            scores, pe, grad, n, p.T, p.E));
     }
     return DSMOE_OK;
 }
@@ -145,15 +150,14 @@ dsmoe_status launch_dense_backward_plain(const dsmoe_layer_desc& p, const void* 
     if (p.T == 0) return DSMOE_OK;
     const unsigned grid = (unsigned)((size_t)p.T * p.E);
     if (p.dtype == DSMOE_BF16)
-        dense_backward_plain_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(
-            static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(W1), static_cast<const __nv_bfloat16*>(W2),
-            scores, mask, static_cast<const __nv_bfloat16*>(dO), dS, static_cast<__nv_bfloat16*>(dA), p.d, p.H, p.E);
+        DSMOE_CUDA_TRY(launch_chained(dense_backward_plain_kernel<__nv_bfloat16>, grid, 256, 0, s,
+            static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(W1), static_cast<const
+            __nv_bfloat16*>(W2), scores, mask, static_cast<const __nv_bfloat16*>(dO), dS,
+            static_cast<__nv_bfloat16*>(dA), p.d, p.H, p.E));
     else
-        dense_backward_plain_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float*>(x), static_cast<const float*>(W1),
-                                                                static_cast<const float*>(W2), scores, mask,
-                                                                static_cast<const float*>(dO), dS, static_cast<float*>(dA),
-                                                                p.d, p.H, p.E);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+        DSMOE_CUDA_TRY(launch_chained(dense_backward_plain_kernel<float>, grid, 256, 0, s,
+            static_cast<const float*>(x), static_cast<const float*>(W1), static_cast<const float*>(W2), scores,
+            mask, static_cast<const float*>(dO), dS, static_cast<float*>(dA), p.d, p.H, p.E));
     return DSMOE_OK;
 }
 
