@@ -263,7 +263,7 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
         if (done) return DSMOE_OK;
     }
 
-    // grouped path: duplicate tokens per selected expert, run the experts, aggregate
+    // grouped path: tokens by selected expert, run the experts, aggregate
     if (fast && fuses_combine(p)) {
         // no grouped copy of the tokens (the up-projection gathers rows of x by row_token), no buffer of expert
         // outputs and no aggregation pass: the down-projection's epilogue adds each expert's gate-weighted output
@@ -280,9 +280,9 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
         DSMOE_TRY(launch_mlp_umma(p, nullptr, packed, offsets, ws + L.h, ws + L.acc, dev_status, s, x, row_token, &gated));
         return launch_combine(p, ws + L.acc, nullptr, token_rows, k_t, out, s, true);
     }
-    DSMOE_TRY(launch_finalize(p, mask, counts, offsets, chunk_prefix, counts_out, s));
-    DSMOE_TRY(launch_permute(p, x, scores, mask, offsets, chunk_prefix, row_token, row_gate, token_rows, ws + L.xp, s));
-    DSMOE_TRY(launch_mlp_generic(p, ws + L.xp, W1, W2, offsets, reinterpret_cast<float*>(ws + L.h_plain), ws + L.yp, s));
+    // (the up-projection fetches its rows of x by row_token: no grouped copy)
+    DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr, false));
+    DSMOE_TRY(launch_mlp_generic(p, x, W1, W2, offsets, reinterpret_cast<float*>(ws + L.h_plain), ws + L.yp, s, row_token));
     return launch_combine(p, ws + L.yp, row_gate, token_rows, k_t, out, s);
 }
 

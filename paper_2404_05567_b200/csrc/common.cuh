@@ -141,8 +141,10 @@ dsmoe_status launch_pack(const dsmoe_layer_desc& p, const void* W1, const void* 
                          cudaStream_t s);
 
 // ---- mlp_generic.cu : plain fp32-FMA grouped GEMMs (any dtype, no packed weights needed)
-dsmoe_status launch_mlp_generic(const dsmoe_layer_desc& p, const void* xp, const void* W1, const void* W2,
-                                const int32_t* offsets, float* h, void* yp, cudaStream_t s);
+// x: the grouped rows; with row_token, the tokens, of which grouped row r is row_token[r]
+dsmoe_status launch_mlp_generic(const dsmoe_layer_desc& p, const void* x, const void* W1, const void* W2,
+                                const int32_t* offsets, float* h, void* yp, cudaStream_t s,
+                                const int32_t* row_token = nullptr);
 
 
 // ---- mlp_umma.cu : tcgen05 / TMEM / TMA kernels on packed bf16 weights
