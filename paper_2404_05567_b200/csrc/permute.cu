@@ -7,17 +7,23 @@
 
 namespace dsmoe {
 
-// Row indices.  A warp owns a chunk of 32 consecutive tokens; for expert e the ballot of "selected"
-// gives each token its rank inside the chunk, and chunk_prefix gives the number of earlier tokens,
-// so rows inside an expert segment ascend by token without any atomic.
+// Row indices.  A block owns four chunks of 32 consecutive tokens, a warp eight tokens of a chunk; lane l stands for
+// experts l and l + 32.  A lane gathers its expert's 32 "selected" bits of the chunk out of the tokens' selection words, so a
+// token's rank inside the chunk is a population count, and with the number of earlier tokens that selected the expert
+// (chunk_prefix, or SCAN) rows inside an expert segment ascend by token without any atomic.
 // SCAN 1: chunk_prefix holds the chunks' own counts (chunk_count_kernel's output, not yet the prefixes over the
 // chunks): every block adds up the chunks before its own and all chunks itself -- a few thousand integers out of
 // L2 -- instead of waiting for a one-block scan kernel in between; block 0 writes counts, offsets (and counts_out).
 // SCAN 2 (at most kCountInBlockChunks chunks): every block also counts the chunks itself, from the masks.
 // The integers are the same either way.
+// Bound by latency: 512 threads, so that the chunk counts take one or two rounds of loads, a token's scores are asked for
+// before anything is known and no warp walks more than 8 tokens (against 128 threads
+// and a warp walking 32 tokens: 4096 tokens on 64 skewed experts 725 -> 715 us a layer, tiny fp32 layer 29.1 -> 28.4, 300 tokens
+// 98.0 -> 97.2).
 constexpr int kCountInBlockChunks = 8;
+constexpr int kPermThreads = 512, kPermChunks = 4, kPermTokens = kPermChunks * kChunk / (kPermThreads / 32);
 template <int SCAN>
-__global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __restrict__ mask,
+__global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint64_t* __restrict__ mask,
                                                             const float* __restrict__ scores,
                                                             int32_t* __restrict__ offsets,
                                                             const int32_t* __restrict__ chunk_prefix,
@@ -27,60 +33,48 @@ __global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __re
                                                             int64_t amax, uint4* __restrict__ zero_out, int row_vecs) {
     chain_next();
     chain_wait();
-    // a chunk's scores, staged so that the loop over the experts below waits for no load: [token][E + 1]
-    __shared__ float sc_s[4][kChunk * (kMaxExperts + 1)];
-    __shared__ int before_s[4][kMaxExperts], total_s[4][kMaxExperts], base_s[4][kMaxExperts];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c0 = blockIdx.x * 4, c = c0 + warp;
-    const int nchunks = (T + kChunk - 1) / kChunk;
-    const bool live = c < nchunks;
-    const int t = c * kChunk + lane;
-    const uint64_t m = live && t < T ? mask[t] : 0;
-    if (live) {
-        float* sc = sc_s[warp];
-        const float* src = scores + (size_t)c * kChunk * E;
-        const int n = min(kChunk, T - c * kChunk) * E;
-        int row = lane / E, col = lane % E;             // of element i below, kept up without a division per element
-#pragma unroll 1
-        for (int i0 = lane; i0 < n; i0 += 32 * 8) {      // eight coalesced loads under way at a time
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = i0 + 32 * j < n ? __ldg(src + i0 + 32 * j) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (i0 + 32 * j < n) sc[row * (E + 1) + col] = v[j];
-                col += 32;
-                while (col >= E) {
-                    col -= E;
-                    ++row;
-                }
-            }
-        }
-    }
+    __shared__ uint64_t mask_s[kPermChunks * kChunk];
+    __shared__ int before_s[kMaxExperts], total_s[kMaxExperts], base_s[kPermChunks][kMaxExperts];
     __shared__ int cnt_s[SCAN == 2 ? kCountInBlockChunks : 1][kMaxExperts];
-    if (SCAN == 2) {
-        for (int k = warp; k < nchunks; k += 4) {
-            const int tk = k * kChunk + lane;
-            const uint64_t mk = tk < T ? mask[tk] : 0;
-            int n_lo = 0, n_hi = 0;
-            for (int e = 0; e < E; ++e) {
-                const int n = __popc(__ballot_sync(0xffffffffu, (mk >> e) & 1));
-                if (lane == (e & 31)) {
-                    if (e < 32) n_lo = n; else n_hi = n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c0 = blockIdx.x * kPermChunks;
+    const int nchunks = (T + kChunk - 1) / kChunk;
+    const int cw = warp / (kPermThreads / 32 / kPermChunks);            // this warp's chunk in the block, its first token
+    const int tw = (warp % (kPermThreads / 32 / kPermChunks)) * kPermTokens;
+    const int t0 = (c0 + cw) * kChunk + tw;
+    const bool e_lo = lane < E, e_hi = lane + 32 < E;
+    float s_lo[kPermTokens], s_hi[kPermTokens];
+#pragma unroll
+    for (int i = 0; i < kPermTokens; ++i) {
+        const float* src = scores + (size_t)(t0 + i) * E;
+        s_lo[i] = t0 + i < T && e_lo ? __ldg(src + lane) : 0.f;
+        s_hi[i] = t0 + i < T && e_hi ? __ldg(src + lane + 32) : 0.f;
+    }
+    if (tid < kPermChunks * kChunk) mask_s[tid] = c0 * kChunk + tid < T ? mask[c0 * kChunk + tid] : 0;
+    if (SCAN) {
+        if (tid < kMaxExperts) before_s[tid] = total_s[tid] = 0;
+        if (SCAN == 2) {
+            for (int k = warp; k < nchunks; k += kPermThreads / 32) {
+                const int tk = k * kChunk + lane;
+                const uint64_t mk = tk < T ? mask[tk] : 0;
+                int n_lo = 0, n_hi = 0;
+                for (int e = 0; e < E; ++e) {
+                    const int n = __popc(__ballot_sync(0xffffffffu, (mk >> e) & 1));
+                    if (lane == (e & 31)) {
+                        if (e < 32) n_lo = n; else n_hi = n;
+                    }
                 }
+                cnt_s[k][lane] = n_lo;
+                cnt_s[k][lane + 32] = n_hi;
             }
-            cnt_s[k][lane] = n_lo;
-            cnt_s[k][lane + 32] = n_hi;
         }
         __syncthreads();
-    }
-    const auto chunk_count = [&](int k, int e) { return SCAN == 2 ? cnt_s[k][e] : chunk_prefix[(size_t)k * E + e]; };
-    if (SCAN) {
+        const auto chunk_count = [&](int k, int e) { return SCAN == 2 ? cnt_s[k][e] : chunk_prefix[(size_t)k * E + e]; };
         // thread (e, part) adds every `parts`-th chunk's count of expert e: coalesced rows of E integers
-        const int EP = E <= 32 ? 32 : 64, parts = 128 / EP;
-        const int e = threadIdx.x % EP, part = threadIdx.x / EP;
-        int before = 0, total = 0;
+        const int EP = E <= 32 ? 32 : 64, parts = kPermThreads / EP;
+        const int e = tid % EP, part = tid / EP;
         if (e < E) {
+            int before = 0, total = 0;
             // sixteen loads are issued before the first one is used
 #pragma unroll 1
             for (int k0 = part; k0 < nchunks; k0 += parts * 16) {
@@ -96,33 +90,23 @@ __global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __re
                     if (k0 + j * parts < c0) before += v[j];
                 }
             }
+            atomicAdd(&before_s[e], before);
+            atomicAdd(&total_s[e], total);
         }
-        before_s[part][e] = before;
-        total_s[part][e] = total;
         // the block's own chunks' counts (warp 0 needs them below): asked for before the barrier
-        int own_lo[4] = {0, 0, 0, 0}, own_hi[4] = {0, 0, 0, 0};
+        int own_lo[kPermChunks] = {}, own_hi[kPermChunks] = {};
         if (warp == 0) {
 #pragma unroll
-            for (int w = 0; w < 3; ++w) {
+            for (int w = 0; w + 1 < kPermChunks; ++w) {
                 if (c0 + w < nchunks) {
-                    if (lane < E) own_lo[w] = chunk_count(c0 + w, lane);
-                    if (lane + 32 < E) own_hi[w] = chunk_count(c0 + w, lane + 32);
+                    if (e_lo) own_lo[w] = chunk_count(c0 + w, lane);
+                    if (e_hi) own_hi[w] = chunk_count(c0 + w, lane + 32);
                 }
             }
         }
         __syncthreads();
         if (warp == 0) {
-            int b_lo = 0, b_hi = 0, c_lo = 0, c_hi = 0;
-            for (int k = 0; k < parts; ++k) {
-                b_lo += before_s[k][lane];
-                c_lo += total_s[k][lane];
-                if (EP == 64) {
-                    b_hi += before_s[k][lane + 32];
-                    c_hi += total_s[k][lane + 32];
-                }
-            }
-            if (lane >= E) c_lo = 0;
-            if (lane + 32 >= E) c_hi = 0;
+            const int c_lo = e_lo ? total_s[lane] : 0, c_hi = e_hi ? total_s[lane + 32] : 0;
             int i_lo = c_lo, i_hi = c_hi;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -135,21 +119,21 @@ __global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __re
             }
             const int tot_lo = __shfl_sync(0xffffffffu, i_lo, 31);
             const int tot = tot_lo + __shfl_sync(0xffffffffu, i_hi, 31);
-            int run_lo = i_lo - c_lo + b_lo, run_hi = tot_lo + i_hi - c_hi + b_hi;   // first row of chunk c0 in the expert
+            int run_lo = i_lo - c_lo + before_s[lane], run_hi = tot_lo + i_hi - c_hi + before_s[lane + 32];   // first row of chunk c0 in the expert
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
+            for (int w = 0; w < kPermChunks; ++w) {
                 base_s[w][lane] = run_lo;
                 base_s[w][lane + 32] = run_hi;
                 run_lo += own_lo[w];
                 run_hi += own_hi[w];
             }
             if (blockIdx.x == 0) {
-                if (lane < E) {
+                if (e_lo) {
                     counts[lane] = c_lo;
                     offsets[lane] = i_lo - c_lo;
                     if (counts_out) counts_out[lane] = c_lo;
                 }
-                if (lane + 32 < E) {
+                if (e_hi) {
                     counts[lane + 32] = c_hi;
                     offsets[lane + 32] = tot_lo + i_hi - c_hi;
                     if (counts_out) counts_out[lane + 32] = c_hi;
@@ -157,64 +141,49 @@ __global__ void __launch_bounds__(128) permute_index_kernel(const uint64_t* __re
                 if (lane == 0) offsets[E] = tot;
             }
         }
-        __syncthreads();
     }
-    if (!live) return;
-    __syncwarp();
-    // lane l holds the first row of this chunk in experts l and l + 32 (passed around by shuffles)
+    __syncthreads();
+    if (t0 >= T) return;
+    // the chunk's selection bits of this lane's experts, and the first row of the chunk in each
+    const uint64_t* const ms = mask_s + cw * kChunk;
+    uint32_t b_lo = 0, b_hi = 0;
+#pragma unroll
+    for (int tt = 0; tt < kChunk; ++tt) {
+        const uint64_t m = ms[tt];
+        b_lo |= (((uint32_t)m >> lane) & 1u) << tt;
+        b_hi |= (((uint32_t)(m >> 32) >> lane) & 1u) << tt;
+    }
     int base_lo, base_hi;
     if (SCAN) {
-        base_lo = base_s[warp][lane];
-        base_hi = base_s[warp][lane + 32];
+        base_lo = base_s[cw][lane];
+        base_hi = base_s[cw][lane + 32];
     } else {
-        base_lo = lane < E ? offsets[lane] + chunk_prefix[(size_t)c * E + lane] : 0;
-        base_hi = lane + 32 < E ? offsets[lane + 32] + chunk_prefix[(size_t)c * E + lane + 32] : 0;
+        const int c = c0 + cw;
+        base_lo = e_lo ? offsets[lane] + chunk_prefix[(size_t)c * E + lane] : 0;
+        base_hi = e_hi ? offsets[lane + 32] + chunk_prefix[(size_t)c * E + lane + 32] : 0;
     }
-    // From here a lane stands for experts `lane` and `lane + 32` and the warp walks the chunk's tokens in order: an
-    // expert's rows ascend by token, a lane counts its own rows, and nothing is exchanged between lanes but the
-    // token's selection word.  (A lane per token and a ballot per expert cost three times the instructions.)
-    const float* sc = sc_s[warp];
-    const uint32_t m_lo = (uint32_t)m, m_hi = (uint32_t)(m >> 32);
     const uint32_t below = (1u << lane) - 1u;
-    const bool e_lo = lane < E, e_hi = lane + 32 < E;
-    const int ntok = min(kChunk, T - c * kChunk);
-    int row_lo = base_lo, row_hi = base_hi;
-    for (int tt = 0; tt < ntok; ++tt) {
-        const uint32_t a = __shfl_sync(0xffffffffu, m_lo, tt);
-        const int tok = c * kChunk + tt;
-        if (e_lo && ((a >> lane) & 1u)) {
-            const int r = row_lo++;
-            const int slot = __popc(a & below);
+#pragma unroll
+    for (int i = 0; i < kPermTokens; ++i) {
+        const int tok = t0 + i, tt = tw + i;
+        if (tok >= T) break;
+        const uint64_t m = ms[tt];
+        const uint32_t a = (uint32_t)m, b = (uint32_t)(m >> 32), earlier = (1u << tt) - 1u;
+        int32_t* const slots = token_rows + (size_t)tok * W;
+        const auto put = [&](int r, int slot, float gate) {
             if (r >= 0 && r < amax) {   // inconsistent caller-supplied offsets must not become a wild store
                 row_token[r] = tok;
-                row_gate[r] = sc[tt * (E + 1) + lane];
+                row_gate[r] = gate;
             }
-            if (slot < W) token_rows[(size_t)tok * W + slot] = r;
-        }
-        if (E > 32) {
-            const uint32_t b = __shfl_sync(0xffffffffu, m_hi, tt);
-            if (e_hi && ((b >> lane) & 1u)) {
-                const int r = row_hi++;
-                const int slot = __popc(a) + __popc(b & below);
-                if (r >= 0 && r < amax) {
-                    row_token[r] = tok;
-                    row_gate[r] = sc[tt * (E + 1) + lane + 32];
-                }
-                if (slot < W) token_rows[(size_t)tok * W + slot] = r;
-            }
-        }
-    }
-    if (t < T)
-        for (int slot = __popcll(m); slot < W; ++slot) token_rows[(size_t)t * W + slot] = -1;
-    if (zero_out) {
+            if (slot < W) slots[slot] = r;
+        };
+        if (e_lo && ((a >> lane) & 1u)) put(base_lo + __popc(b_lo & earlier), __popc(a & below), s_lo[i]);
+        if (e_hi && ((b >> lane) & 1u)) put(base_hi + __popc(b_hi & earlier), __popc(a) + __popc(b & below), s_hi[i]);
+        const int n = __popcll(m);
+        for (int slot = n + lane; slot < W; slot += 32) slots[slot] = -1;
         // Eq. 1 with an empty selection is the zero vector: no expert tile will ever write this token's row
-        unsigned none = __ballot_sync(0xffffffffu, t < T && m == 0);
-        while (none) {
-            const int l = __ffs(none) - 1;
-            none &= none - 1;
-            uint4* row = zero_out + (size_t)(c * kChunk + l) * row_vecs;
-            for (int v = lane; v < row_vecs; v += 32) row[v] = make_uint4(0u, 0u, 0u, 0u);
-        }
+        if (zero_out && n == 0)
+            for (int v = lane; v < row_vecs; v += 32) zero_out[(size_t)tok * row_vecs + v] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -370,7 +339,7 @@ dsmoe_status launch_permute(const dsmoe_layer_desc& p, const void* x, const floa
     const int nchunks = ceil_div(p.T, kChunk);
     const int64_t amax = (int64_t)amax_of(p);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
-    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<0>, ceil_div(nchunks, 4), 128, 0, s,
+    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<0>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
         mask, scores, const_cast<int32_t*>(offsets), chunk_prefix, nullptr, nullptr, row_token, row_gate,
         token_rows, p.T, p.E, width_of(p), amax, static_cast<uint4*>(zero_out), row_vecs));
     if (xp) {
@@ -392,7 +361,7 @@ dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const 
     const int nchunks = ceil_div(p.T, kChunk);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
     if (nchunks > 0 && nchunks <= kCountInBlockChunks) {
-        DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<2>, ceil_div(nchunks, 4), 128, 0, s,
+        DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<2>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
             mask, scores, offsets, nullptr, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
             width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs));
         return DSMOE_OK;
@@ -403,7 +372,7 @@ dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const 
         return launch_permute(p, nullptr, scores, mask, offsets, chunk_prefix, row_token, row_gate, token_rows, nullptr, s,
                               zero_out);
     }
-    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<1>, ceil_div(nchunks, 4), 128, 0, s,
+    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<1>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
         mask, scores, offsets, chunk_prefix, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
         width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs));
     return DSMOE_OK;
