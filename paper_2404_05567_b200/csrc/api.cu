@@ -375,7 +375,9 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
     int32_t* row_token = reinterpret_cast<int32_t*>(ws + L.row_token);
     float* row_gate = reinterpret_cast<float*>(ws + L.row_gate);
     int32_t* token_rows = reinterpret_cast<int32_t*>(ws + L.token_rows);
-    const MoaCore core{args->n_head, args->n_seq, args->L, args->scale, args->Kc, args->Vc, args->tok_seq, args->pos, token_rows};
+    const bool dense_down = moa_shares_keys(p, args->n_head, args->n_seq) && moa_dense_down(p, sm_count());
+    const MoaCore core{args->n_head, args->n_seq, args->L, args->scale, args->Kc, args->Vc, args->tok_seq, args->pos, token_rows,
+                       dense_down ? ws + L.acc : nullptr, mask, row_gate};
 
     // router, selection and grouping as in dsmoe_layer_forward's grouped path (also when every expert is selected)
     dsmoe_layer_desc pr = p;
@@ -389,7 +391,7 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
         DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s));
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK)
         DSMOE_TRY(launch_select(p, scores, mask, k_t, s, reinterpret_cast<int*>(ws + L.batch_k)));
-    if (fuses_combine(p)) {
+    if (fuses_combine(p) && !dense_down) {
         DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, out, counted));
         const CombineArgs cmb{row_token, row_gate, mask, reinterpret_cast<float*>(ws + L.acc),
                               reinterpret_cast<int*>(ws + L.tile_done), out};
@@ -398,6 +400,7 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
     DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr, counted));
     const CombineArgs gated{row_token, row_gate, nullptr, nullptr, nullptr, nullptr};
     DSMOE_TRY(launch_mlp_umma(p, nullptr, packed, offsets, ws + L.h, ws + L.acc, dev_status, s, x, row_token, &gated, &core));
+    if (dense_down) return launch_dense_down(p, ws + L.acc, packed, out, dev_status, s);
     return launch_combine(p, ws + L.acc, nullptr, token_rows, k_t, out, s, true);
 }
 

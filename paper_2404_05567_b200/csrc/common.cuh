@@ -181,7 +181,27 @@ struct MoaCore {
     const int32_t* tok_seq;  // [T] or NULL (one sequence)
     const int32_t* pos;      // [T]: token t sees keys 0..pos[t]
     const int32_t* token_rows;   // [T, W]: the grouped rows of each token (from the permute step)
+    // the dense form of the output projection (moa_dense_down): gate-weighted attention outputs go to dense[T][E*H]
+    void* dense;
+    const uint64_t* mask;
+    const float* row_gate;
 };
+// Whether launch_moa_attention takes the kernel whose tiles share their copies of the keys (the only one that serves `dense`)
+bool moa_shares_keys(const dsmoe_layer_desc& p, int n_head, int n_seq);
+// Output projection and the weighted sum of Eq. 8 as ONE dense GEMM over the experts side by side, out = dense . Wo[E*H, d], as
+// in the dense forward: E / K times the multiplications of the grouped form, but at the rate of a long reduction (E * H
+// instead of H) and without expert outputs written to and read back from memory as fp32 rows (8 bytes per row and column).
+// By the measured costs of both -- dense 1.43 fs per expert, hidden unit, token and column, grouped 1.6 ps plus 2 fs per hidden
+// unit for each selected expert -- the dense form wins while E * H < K * (H + 640) or so.  6B prompts (8 experts of 512, top-5,
+// 8192 tokens): 203 + 122 us grouped, 174 us dense.  Needs row tiles enough to cover the SMs, and the scratch of the
+// grouped form's fp32 rows for the [T, E*H] buffer.
+static inline bool moa_dense_down(const dsmoe_layer_desc& p, int sms) {
+    if (p.fuse_combine != 0 || (p.mode != DSMOE_SELECT_TOPK && p.mode != DSMOE_SELECT_ALL)) return false;
+    const long long K = width_of(p);
+    return (long long)p.E * p.H < K * (p.H + 640ll) && (long long)p.E * p.H <= (fuses_combine(p) ? 2ll : 2ll * K) * p.d &&
+           (long long)ceil_div(p.T, 128) * ceil_div(p.d, 256) >= sms;
+}
+
 dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const void* packed, const int32_t* offsets,
                              void* hbuf, void* yp, int32_t* dev_status, cudaStream_t s, const void* x = nullptr,
                              const int32_t* row_token = nullptr, const CombineArgs* cmb = nullptr,
@@ -210,6 +230,9 @@ dsmoe_status launch_mi_loss(const dsmoe_layer_desc& p, const float* scores, floa
 dsmoe_status launch_dense_backward_plain(const dsmoe_layer_desc& p, const void* x, const void* W1, const void* W2,
                                          const float* scores, const uint64_t* mask, const void* dO, float* dS, void* dA,
                                          cudaStream_t s);
+// out[T,d] = hg[T, E*H] . W2 over the experts side by side (the dense forward's down-projection)
+dsmoe_status launch_dense_down(const dsmoe_layer_desc& p, const void* hg, const void* packed, void* out, int32_t* dev_status,
+                               cudaStream_t s);
 dsmoe_status launch_dense_backward(const dsmoe_layer_desc& p, const void* x, const void* W2, const void* packed,
                                    const float* scores, const uint64_t* mask, const void* dO, float* dS, void* dA,
                                    void* act, float* dot_part, int32_t* dev_status, cudaStream_t s);

@@ -2192,7 +2192,7 @@ dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const vo
     // reduction blocks): the reduction is cut so that the launch covers the SMs; the partial sums (fp32, in the buffer
     // of the expert outputs, which is idle until the output projection) are added in order by split_sum_kernel
     int splits = 1;
-    if (moa && yp && cmb && !cmb->out) {
+    if (moa && !moa->dense && yp && cmb && !cmb->out) {
         const long long max_tiles = ((long long)(amax / BM) + p.E) * ceil_div(p.H, BN);
         while (splits < 8 && max_tiles * splits * 2 <= sm_count() && (p.d / BK) % (splits * 2) == 0 &&
                (p.d / BK) / (splits * 2) >= 4 && (long long)splits * 2 * p.H <= p.d)
@@ -2210,6 +2210,7 @@ dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const vo
         DSMOE_TRY(launch_gemm(*mA1, *mB1, up, sm_count(), s, true, moa ? 0 : pair_tiles));
     }
     if (moa) DSMOE_TRY(launch_moa_attention(p, *moa, hbuf, row_token, moa->token_rows, offsets, dev_status, s));
+    if (moa && moa->dense) return DSMOE_OK;      // the output projection is launch_dense_down's
     DSMOE_TRY(launch_gemm(*mA2, *mB2, down, sm_count(), s, true, pair_tiles));
     return DSMOE_OK;
 }
@@ -2277,6 +2278,20 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     return DSMOE_OK;
 }
 
+dsmoe_status launch_dense_down(const dsmoe_layer_desc& p, const void* hg, const void* packed, void* out, int32_t* dev_status,
+                               cudaStream_t s) {
+    const __nv_bfloat16* w2t = static_cast<const __nv_bfloat16*>(packed) + (size_t)p.E * p.H * p.d;
+    const CUtensorMap* mA;
+    const BMaps* mB;
+    DSMOE_TRY(cached_map_2d(&mA, hg, p.T, (uint64_t)p.E * p.H, BM));
+    DSMOE_TRY(cached_bmaps(&mB, w2t, p.E, p.d, p.H));
+    GemmParams down{};
+    down.mode = GEMM_DENSE_DOWN; down.epi = EPI_STORE; down.E = p.E; down.n_per_expert = p.d; down.k_per_expert = p.H;
+    down.rows = p.T; down.out = out; down.ld_out = p.d; down.out_f32 = p.out_fp32 ? 1 : 0; down.dev_status = dev_status;
+    const int tiles = ceil_div(p.T, BM) * ceil_div(p.d, BN);
+    return launch_gemm(*mA, *mB, down, tiles < sm_count() ? tiles : sm_count(), s, true, ceil_div(p.T, 2 * BM) * ceil_div(p.d, BN));
+}
+
 dsmoe_status launch_layer_umma(const dsmoe_layer_desc& p, const void* x, const void* packed, const float* scores,
                                const uint64_t* mask, const int32_t* k_t, int32_t* counts_out, void* out, char* ws,
                                const WsLayout& L, int32_t* dev_status, cudaStream_t s, bool* done) {
@@ -2285,25 +2300,18 @@ dsmoe_status launch_layer_umma(const dsmoe_layer_desc& p, const void* x, const v
     if (!umma_supported(p) || p.mode != DSMOE_SELECT_ALL) return DSMOE_OK;
     // Dense forward: gate folded into h, aggregation folded into the down-projection's reduction.
     const __nv_bfloat16* w1t = static_cast<const __nv_bfloat16*>(packed);
-    const __nv_bfloat16* w2t = w1t + (size_t)p.E * p.H * p.d;
     void* hg = ws + L.h;                                        // [T, E*H] bf16
-    const CUtensorMap *mA1, *mA2;
-    const BMaps *mB1, *mB2;
+    const CUtensorMap* mA1;
+    const BMaps* mB1;
     DSMOE_TRY(cached_map_2d(&mA1, x, p.T, p.d, BM));
     DSMOE_TRY(cached_bmaps(&mB1, w1t, p.E, p.H, p.d));
-    DSMOE_TRY(cached_map_2d(&mA2, hg, p.T, (uint64_t)p.E * p.H, BM));
-    DSMOE_TRY(cached_bmaps(&mB2, w2t, p.E, p.d, p.H));
     GemmParams up{};
     up.mode = GEMM_DENSE_UP; up.epi = EPI_GELU; up.E = p.E; up.n_per_expert = p.H; up.k_per_expert = p.d; up.rows = p.T;
     up.gate = scores; up.out = hg; up.ld_out = (long long)p.E * p.H; up.dev_status = dev_status;
-    GemmParams down{};
-    down.mode = GEMM_DENSE_DOWN; down.epi = EPI_STORE; down.E = p.E; down.n_per_expert = p.d; down.k_per_expert = p.H;
-    down.rows = p.T; down.out = out; down.ld_out = p.d; down.out_f32 = p.out_fp32 ? 1 : 0; down.dev_status = dev_status;
-    const int mt = ceil_div(p.T, BM);
-    const int tiles_up = mt * ceil_div(p.H, BN) * p.E, tiles_down = mt * ceil_div(p.d, BN);
-    const int mt2 = ceil_div(p.T, 2 * BM);
-    DSMOE_TRY(launch_gemm(*mA1, *mB1, up, tiles_up < sm_count() ? tiles_up : sm_count(), s, true, mt2 * ceil_div(p.H, BN) * p.E));
-    DSMOE_TRY(launch_gemm(*mA2, *mB2, down, tiles_down < sm_count() ? tiles_down : sm_count(), s, true, mt2 * ceil_div(p.d, BN)));
+    const int tiles_up = ceil_div(p.T, BM) * ceil_div(p.H, BN) * p.E;
+    DSMOE_TRY(launch_gemm(*mA1, *mB1, up, tiles_up < sm_count() ? tiles_up : sm_count(), s, true,
+                          ceil_div(p.T, 2 * BM) * ceil_div(p.H, BN) * p.E));
+    DSMOE_TRY(launch_dense_down(p, hg, packed, out, dev_status, s));
     if (counts_out) {
         int32_t* counts = reinterpret_cast<int32_t*>(ws + L.counts);
         int32_t* offsets = reinterpret_cast<int32_t*>(ws + L.offsets);

@@ -5,6 +5,7 @@
 // with the router-weighted sum of Eq. 8; in between every grouped row -- one (token, expert) pair, n_head query
 // vectors of d_head -- attends to the keys and values of its token's sequence, head j to key/value head j
 // (the keys and values are shared by all experts).  This file holds that middle step.
+#include <climits>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -396,6 +397,322 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restri
     chain_next();
 }
 
+// ---------------------------------------------------------------- prompts: neighbouring tokens share the copies of their keys
+//
+// One CTA per (head, four 16-row tiles of neighbouring tokens); a warp owns a tile (its rows, queries, sums), and all four walk
+// the same keys: blocks of 64 keys and values come by cp.async into two buffers, one under way while the other is worked on.
+// Tokens of a prompt see nearly the same keys, so a block is read once for 12 tokens (5 rows each) instead of once per tile,
+// and no warp waits behind its own copies.  Tokens of several sequences in one CTA are served sequence by sequence.  Both
+// operands' fragments come by ldmatrix.x4; exponents are base 2 with the scale folded in; a block that every row of the warp
+// sees in full is not masked, and sums are rescaled only where a maximum moved.  Three CTAs of 70 KB and 168 registers a
+// thread fill an SM.  Bound by the instruction issue of the warp-level tensor path and the exponentials.
+// 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 133 us with a tile per warp and its own copies, 83 with shared ones
+// (tensor pipe 31 % busy, 0.38 instructions a cycle and scheduler; the layer 702 -> 653 us).
+constexpr int kShWarps = 4, kShKeys = 64, kShTokens = kShWarps * 16;
+
+struct AttnArgs {
+    __nv_bfloat16* qa;
+    const int32_t* token_rows;
+    int W, row_tiles, tpt;
+    long long amax;
+    int n_head, H, T;
+    const __nv_bfloat16 *Kc, *Vc;
+    const int32_t *tok_seq, *pos;
+    int n_seq, L;
+    float scale;
+    int* dev_status;
+    // With `dense`, the outputs go to dense[T][E * H] instead: expert e's columns e * H .. of token t hold its gate times its
+    // attention output, zeros where the token did not select e
+    __nv_bfloat16* dense;
+    int E;
+    const uint64_t* mask;
+    const float* row_gate;
+};
+
+__device__ __forceinline__ float ex2(float v) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+template <int DH>
+constexpr size_t shared_attention_smem() { return (size_t)2 * 2 * kShKeys * (DH * 2 + 16); }
+
+template <int DH>
+__global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(const AttnArgs P) {
+    chain_wait();
+    constexpr int STRIDE = DH * 2 + 16;                 // bytes per key row in shared memory: 16 of padding, no bank conflicts
+    constexpr int KS = DH / 16, DT = DH / 8, CH = DH / 8;
+    extern __shared__ __align__(16) unsigned char moa_sh_smem[];
+    __shared__ int seq_s[kShTokens], last_s[kShTokens];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q4 = lane & 3;
+    const int j = (int)(blockIdx.x % P.n_head);
+    const int group = (int)(blockIdx.x / P.n_head);
+    // this CTA's tokens: their sequences and last visible keys, clamped into the cache (and reported)
+    const int tg0 = (group * kShWarps / P.row_tiles) * P.tpt;
+    const int tg1 = min(P.T, ((group * kShWarps + kShWarps - 1) / P.row_tiles) * P.tpt + P.tpt);
+    const int ng = tg1 - tg0;
+    if (threadIdx.x < ng) {
+        const int t = tg0 + threadIdx.x;
+        const int sq = P.tok_seq ? P.tok_seq[t] : 0, last = P.pos[t];
+        if (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L) *P.dev_status = DSMOE_ERR_INVALID_ARG;
+        seq_s[threadIdx.x] = min(max(sq, 0), P.n_seq - 1);
+        last_s[threadIdx.x] = min(max(last, 0), P.L - 1);
+    }
+    // this thread's two rows of the warp's tile (g and g + 8): grouped row (-1 = none), token
+    const int wt = group * kShWarps + warp, t0 = (wt / P.row_tiles) * P.tpt, rt = wt % P.row_tiles;
+    int r[2], tk[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = g + 8 * h;
+        int slot;
+        if (P.tpt == 1) {
+            tk[h] = t0;
+            slot = rt * 16 + i;
+        } else {
+            tk[h] = i < P.tpt * P.W ? t0 + i / P.W : P.T;
+            slot = i % P.W;
+        }
+        r[h] = tk[h] < P.T && slot < P.W ? P.token_rows[(size_t)tk[h] * P.W + slot] : -1;
+        if (r[h] >= P.amax) r[h] = -1;
+    }
+    __syncthreads();
+    int last[2], sq_of[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        last[h] = r[h] >= 0 ? last_s[tk[h] - tg0] : 0;
+        sq_of[h] = r[h] >= 0 ? seq_s[tk[h] - tg0] : -1;
+    }
+    // Q fragments (the A operand of S = Q.K^T)
+    uint32_t qf[KS][4];
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+        const int c = j * DH + ks * 16 + q4 * 2;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const __nv_bfloat16* q = P.qa + (size_t)max(r[h], 0) * P.H + c;
+            qf[ks][h] = r[h] >= 0 ? *reinterpret_cast<const uint32_t*>(q) : 0u;
+            qf[ks][2 + h] = r[h] >= 0 ? *reinterpret_cast<const uint32_t*>(q + 8) : 0u;
+        }
+    }
+    const float sl2 = P.scale * 1.4426950408889634f;
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+    float o[DT][4];
+#pragma unroll
+    for (int i = 0; i < DT; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+
+    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(moa_sh_smem);
+    // fragment addresses inside a block: K (rows = keys, two 8-key tiles x two 8-wide halves of k) and V (transposed)
+    const uint32_t kfrag = (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * STRIDE + ((lane >> 3) & 1) * 16);
+    const uint32_t vfrag = (uint32_t)((((lane >> 3) & 1) * 8 + (lane & 7)) * STRIDE + (lane >> 4) * 16);
+
+    for (int u = 0; u < ng; ++u) {
+        // one pass per sequence among the CTA's tokens (a prompt's tokens: one)
+        const int sq = seq_s[u];
+        bool again = false;
+        for (int v = 0; v < u && !again; ++v) again = seq_s[v] == sq;
+        if (again) continue;
+        int last_key = 0;
+        for (int v = u; v < ng; ++v)
+            if (seq_s[v] == sq) last_key = max(last_key, last_s[v]);
+        // this pass: which rows take part, the last key any of the warp's rows sees, the last one they all see
+        const bool act0 = sq_of[0] == sq, act1 = sq_of[1] == sq;
+        const int wlast = (int)__reduce_max_sync(0xffffffffu, max(act0 ? last[0] : -1, act1 ? last[1] : -1));
+        const int wfull = (int)__reduce_min_sync(0xffffffffu, min(act0 ? last[0] : r[0] >= 0 ? -1 : INT_MAX,
+                                                                  act1 ? last[1] : r[1] >= 0 ? -1 : INT_MAX));
+        const __nv_bfloat16* Kh = P.Kc + ((size_t)(sq * P.n_head + j) * P.L) * DH;
+        const __nv_bfloat16* Vh = P.Vc + ((size_t)(sq * P.n_head + j) * P.L) * DH;
+        const int nblocks = last_key / kShKeys + 1;
+        const auto fetch = [&](int b, int buf) {
+            const int key0 = b * kShKeys, nk = min(kShKeys, last_key + 1 - key0);
+            const uint32_t kd = smem0 + (uint32_t)(buf * 2 * kShKeys * STRIDE), vd = kd + kShKeys * STRIDE;
+#pragma unroll
+            for (int i = 0; i < CH * kShKeys / (32 * kShWarps); ++i) {
+                const int idx = threadIdx.x + 32 * kShWarps * i, row = idx / CH, ch = idx % CH;
+                // rows past the last visible key are filled with zeros
+                const size_t src = (size_t)(key0 + (row < nk ? row : 0)) * DH + ch * 8;
+                const uint32_t nbytes = row < nk ? 16u : 0u, dst = (uint32_t)(row * STRIDE + ch * 16);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(kd + dst), "l"(Kh + src), "r"(nbytes) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(vd + dst), "l"(Vh + src), "r"(nbytes) : "memory");
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        fetch(0, 0);
+        for (int b = 0; b < nblocks; ++b) {
+            const int buf = b & 1;
+            if (b + 1 < nblocks) {
+                fetch(b + 1, buf ^ 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                const int key0 = b * kShKeys + 32 * half;
+                if (key0 > wlast) break;                // (uniform in the warp) nothing more for this warp's rows
+                const uint32_t ka = smem0 + (uint32_t)(buf * 2 * kShKeys * STRIDE + 32 * half * STRIDE) + kfrag;
+                const uint32_t va = smem0 + (uint32_t)((buf * 2 + 1) * kShKeys * STRIDE + 32 * half * STRIDE) + vfrag;
+                float sc[4][4];
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
+#pragma unroll
+                for (int ks = 0; ks < KS; ++ks) {
+#pragma unroll
+                    for (int np = 0; np < 2; ++np) {
+                        uint32_t kb[4];
+                        ldsm4(kb, ka + (uint32_t)(np * 16 * STRIDE + ks * 32));
+                        mma_bf16_16816(sc[2 * np], qf[ks], kb[0], kb[1]);
+                        mma_bf16_16816(sc[2 * np + 1], qf[ks], kb[2], kb[3]);
+                    }
+                }
+                // scale (to base 2), hide the keys past each row's position and everything from rows not in this pass
+                float bm0 = -INFINITY, bm1 = -INFINITY;
+                if (key0 + 31 <= wfull) {
+#pragma unroll
+                    for (int nt = 0; nt < 4; ++nt) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) sc[nt][c] *= sl2;
+                        bm0 = fmaxf(bm0, fmaxf(sc[nt][0], sc[nt][1]));
+                        bm1 = fmaxf(bm1, fmaxf(sc[nt][2], sc[nt][3]));
+                    }
+                } else {
+                    const int e0 = act0 ? last[0] : -1, e1 = act1 ? last[1] : -1;
+#pragma unroll
+                    for (int nt = 0; nt < 4; ++nt) {
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const int key = key0 + nt * 8 + q4 * 2 + c;
+                            sc[nt][c] = key <= e0 ? sc[nt][c] * sl2 : -INFINITY;
+                            sc[nt][2 + c] = key <= e1 ? sc[nt][2 + c] * sl2 : -INFINITY;
+                        }
+                        bm0 = fmaxf(bm0, fmaxf(sc[nt][0], sc[nt][1]));
+                        bm1 = fmaxf(bm1, fmaxf(sc[nt][2], sc[nt][3]));
+                    }
+                }
+                bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 1));
+                bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 1));
+                bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 2));
+                bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 2));
+                if (__any_sync(0xffffffffu, bm0 > m[0] || bm1 > m[1])) {
+                    const float n0 = fmaxf(m[0], bm0), n1 = fmaxf(m[1], bm1);
+                    // a row that has seen no key yet (and sees none here) keeps m = -inf: nothing to rescale
+                    const float c0 = n0 == -INFINITY ? 1.f : ex2(m[0] - n0), c1 = n1 == -INFINITY ? 1.f : ex2(m[1] - n1);
+                    m[0] = n0;
+                    m[1] = n1;
+                    l[0] *= c0;
+                    l[1] *= c1;
+#pragma unroll
+                    for (int i = 0; i < DT; ++i) {
+                        o[i][0] *= c0;
+                        o[i][1] *= c0;
+                        o[i][2] *= c1;
+                        o[i][3] *= c1;
+                    }
+                }
+                const float z0 = m[0] == -INFINITY ? 0.f : m[0], z1 = m[1] == -INFINITY ? 0.f : m[1];
+                uint32_t pf[2][4];
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    const float p0 = ex2(sc[nt][0] - z0), p1 = ex2(sc[nt][1] - z0);
+                    const float p2 = ex2(sc[nt][2] - z1), p3 = ex2(sc[nt][3] - z1);
+                    l[0] += p0 + p1;
+                    l[1] += p2 + p3;
+                    pf[nt / 2][(nt & 1) * 2] = pack_bf16(p0, p1);
+                    pf[nt / 2][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
+                }
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk) {
+#pragma unroll
+                    for (int dp = 0; dp < DT / 2; ++dp) {
+                        uint32_t vb[4];
+                        ldsm4t(vb, va + (uint32_t)(kk * 16 * STRIDE + dp * 32));
+                        mma_bf16_16816(o[2 * dp], pf[kk], vb[0], vb[1]);
+                        mma_bf16_16816(o[2 * dp + 1], pf[kk], vb[2], vb[3]);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+    chain_next();
+    // normalise (and weigh); the rows go out through shared memory (the buffers are free), whole rows per store
+    float inv[2];
+    __nv_bfloat16* dst[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        l[h] += __shfl_xor_sync(0xffffffffu, l[h], 1);
+        l[h] += __shfl_xor_sync(0xffffffffu, l[h], 2);
+        inv[h] = 1.f / l[h];
+        dst[h] = r[h] >= 0 ? P.qa + (size_t)r[h] * P.H + j * DH : nullptr;
+        if (P.dense && r[h] >= 0) {
+            // the row is its token's slot-th selected expert, ascending
+            uint64_t sel = P.mask[tk[h]];
+            const int i = g + 8 * h;
+            for (int slot = P.tpt == 1 ? rt * 16 + i : i % P.W; slot > 0; --slot) sel &= sel - 1;
+            const int e = __ffsll((long long)sel) - 1;
+            dst[h] = e >= 0 ? P.dense + ((size_t)tk[h] * P.E + e) * P.H + j * DH : nullptr;
+            inv[h] *= P.row_gate[r[h]];
+        }
+    }
+    unsigned char* const st = moa_sh_smem + warp * 16 * STRIDE;
+#pragma unroll
+    for (int dt = 0; dt < DT; ++dt) {
+        *reinterpret_cast<uint32_t*>(st + g * STRIDE + (dt * 8 + q4 * 2) * 2) = pack_bf16(o[dt][0] * inv[0], o[dt][1] * inv[0]);
+        *reinterpret_cast<uint32_t*>(st + (g + 8) * STRIDE + (dt * 8 + q4 * 2) * 2) = pack_bf16(o[dt][2] * inv[1], o[dt][3] * inv[1]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16 * CH / 32; ++i) {
+        const int idx = lane + 32 * i, row = idx / CH, ch = idx % CH;
+        __nv_bfloat16* const da = reinterpret_cast<__nv_bfloat16*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst[0]), (row & 7) * 4));
+        __nv_bfloat16* const db = reinterpret_cast<__nv_bfloat16*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst[1]), (row & 7) * 4));
+        __nv_bfloat16* const to = row < 8 ? da : db;
+        if (to) *reinterpret_cast<uint4*>(to + ch * 8) = *reinterpret_cast<const uint4*>(st + row * STRIDE + ch * 16);
+    }
+    if (P.dense && rt == 0) {
+        for (int t = t0; t < min(P.T, t0 + P.tpt); ++t) {
+            const uint64_t sel = P.mask[t];
+            for (int idx = lane; idx < P.E * CH; idx += 32) {
+                const int e = idx / CH, ch = idx % CH;
+                if (!((sel >> e) & 1ull))
+                    *reinterpret_cast<uint4*>(P.dense + ((size_t)t * P.E + e) * P.H + j * DH + ch * 8) = make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+    }
+}
+
+template <int DH>
+dsmoe_status launch_shared_attention(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
+                                     int32_t* dev_status, cudaStream_t s) {
+    static bool attr[kMaxDeviceSlots] = {};
+    int dev = 0;
+    DeviceState* st = nullptr;
+    DSMOE_TRY(device_state(&st, &dev));
+    if (!attr[dev]) {
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(moa_attention_shared_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)shared_attention_smem<DH>()));
+        attr[dev] = true;
+    }
+    const int W = width_of(p), row_tiles = (W + 15) / 16, tpt = W <= 8 ? 16 / W : 1;
+    const AttnArgs a{q, token_rows, W, row_tiles, tpt, (long long)amax_of(p), c.n_head, p.H, p.T,
+                     static_cast<const __nv_bfloat16*>(c.Kc), static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos,
+                     c.n_seq, c.L, c.scale, dev_status, static_cast<__nv_bfloat16*>(c.dense), p.E, c.mask, c.row_gate};
+    const long long tiles = (long long)((p.T + tpt - 1) / tpt) * row_tiles;
+    const long long ctas = (tiles + kShWarps - 1) / kShWarps * c.n_head;
+    if (ctas > 0x7fffffffll) return DSMOE_ERR_UNSUPPORTED;
+    DSMOE_CUDA_TRY(launch_chained(moa_attention_shared_kernel<DH>, (unsigned)ctas, 32 * kShWarps, shared_attention_smem<DH>(), s, a));
+    return DSMOE_OK;
+}
+
 template <int DH, int kMmaWarps>
 dsmoe_status launch_mma_attention_nw(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
                                   int32_t* dev_status, cudaStream_t s) {
@@ -433,6 +750,7 @@ dsmoe_status launch_mma_attention_nw(const dsmoe_layer_desc& p, const MoaCore& c
 template <int DH>
 dsmoe_status launch_mma_attention(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
                                   int32_t* dev_status, cudaStream_t s) {
+    if (moa_shares_keys(p, c.n_head, c.n_seq)) return launch_shared_attention<DH>(p, c, q, token_rows, dev_status, s);
     if (c.L <= 512) return launch_mma_attention_nw<DH, 2>(p, c, q, token_rows, dev_status, s);
     return launch_mma_attention_nw<DH, 8>(p, c, q, token_rows, dev_status, s);
 }
@@ -445,6 +763,13 @@ bool moa_supported(const dsmoe_layer_desc& p, int n_head, int L) {
     if (L <= 0 || dh % 32 || dh > 256) return false;
     if (dh == 64 || dh == 96 || dh == 128) return true;                       // tensor-core kernel: any cache length
     return (size_t)(dh + L + 3) * 4 * kMoaWarps <= 200 * 1024;                // plain kernel: a warp's logits sit in shared memory
+}
+
+// Prompts: at least eight tokens per sequence on average, so that neighbouring tokens mostly share their keys.  (Decoding, one
+// token per sequence, would walk a CTA's sequences one after the other.)
+bool moa_shares_keys(const dsmoe_layer_desc& p, int n_head, int n_seq) {
+    const int dh = p.H / n_head;
+    return (dh == 64 || dh == 96 || dh == 128) && !getenv("DSMOE_MOA_PLAIN") && (long long)p.T >= 8ll * n_seq;
 }
 
 dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, void* qa, const int32_t* row_token,

@@ -147,3 +147,26 @@ def test_moa_plain_attention_kernel_on_a_common_head_width(monkeypatch):
     s, *rest = _moa_case("moa_plain", 200, 512, 8, 2, 64, 3, 77, "mixed", gi.MODE_TOPK, K=3)
     e, er = _run(s, *rest, 2, 0.125)
     assert er <= TOL_BF16, (e, er)
+
+
+# Many tokens per sequence: tiles that share their copies of the keys, grouped output projection (few row tiles) and the dense
+# one (row tiles enough to cover the SMs: 148 of 128 rows x 256 columns).  Ragged token counts, CTAs whose tokens belong to
+# several sequences, caches around the 64-key blocks, more than 16 rows per token, every head width.
+PROMPTS = [
+    ("prompt_grouped", 77, 512, 8, 2, 64, 3, 65, "mixed", gi.MODE_TOPK, dict(K=3)),
+    ("prompt_grouped_thr", 203, 512, 8, 2, 96, 7, 640, "mixed", gi.MODE_THRESHOLD, dict(eps=0.2)),       # some tokens select nothing
+    ("prompt_one_row", 130, 256, 4, 2, 128, 2, 129, "prefill", gi.MODE_TOPK, dict(K=1)),                 # 16 tokens a tile
+    ("prompt_two_row_tiles", 90, 256, 20, 2, 64, 4, 64, "mixed", gi.MODE_ALL, dict()),
+    ("prompt_dense", 4701, 1024, 8, 2, 64, 3, 300, "mixed", gi.MODE_TOPK, dict(K=4)),
+    ("prompt_dense_96", 4640, 1024, 8, 4, 96, 16, 290, "prefill", gi.MODE_TOPK, dict(K=5)),
+    ("prompt_dense_128", 2369, 2048, 8, 1, 128, 1, 2400, "prefill", gi.MODE_TOPK, dict(K=7)),
+    ("prompt_dense_all", 4609, 1024, 20, 2, 64, 11, 63, "mixed", gi.MODE_ALL, dict()),
+]
+
+
+@pytest.mark.parametrize("case", PROMPTS, ids=[c[0] for c in PROMPTS])
+def test_moa_prompts(case):
+    name, T, d, E, nh, dh, n_seq, L, layout, mode, sel = case
+    s, *rest = _moa_case(name, T, d, E, nh, dh, n_seq, L, layout, mode, **sel)
+    e, er = _run(s, *rest, nh, 1.0 / math.sqrt(dh), sample=200)
+    assert er <= TOL_BF16, (e, er)
