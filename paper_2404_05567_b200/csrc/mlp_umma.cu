@@ -2110,8 +2110,8 @@ dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const 
     __nv_bfloat16* wsplit = reinterpret_cast<__nv_bfloat16*>(scratch);
     float* sums = reinterpret_cast<float*>(scratch + split_bytes);
     DSMOE_CUDA_TRY(launch_chained(router_split_kernel, ceil_div(EP * p.d, 256), 256, 0, s, Wr, wsplit, p.d, p.E, EP));
-    const CUtensorMap* mA;
-    const BMaps* mB;
+    CUtensorMap mA;
+    BMaps mB;
     DSMOE_TRY(cached_map_2d(&mA, x, p.T, p.d, BM));
     const int row_tiles = ceil_div(p.T, BM);
     int pieces = kRouterMaxPieces;
@@ -2122,7 +2122,7 @@ dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const 
     g.a_expert_stride = p.d / pieces; g.rows = p.T;
     g.out = sums; g.ld_out = (long long)pieces * 3 * EP; g.out_f32 = 1; g.dev_status = dev_status;
     const int tiles = row_tiles * pieces;
-    DSMOE_TRY(launch_gemm(*mA, *mB, g, tiles < sm_count() ? tiles : sm_count(), s, false));
+    DSMOE_TRY(launch_gemm(mA, mB, g, tiles < sm_count() ? tiles : sm_count(), s, false));
     DSMOE_CUDA_TRY(launch_chained(router_finish_kernel, ceil_div(p.T, kChunk), 32 * kChunk, 0, s,
         sums, br, scores, mask, k_t, chunk_counts, p.T, EP, pieces, SelParams{p.E, p.mode, p.eps, p.eps_normalized,
         p.K, p.min_k, nullptr}));
@@ -2150,8 +2150,8 @@ dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const vo
     const size_t amax = amax_of(p);
     const __nv_bfloat16* w1t = static_cast<const __nv_bfloat16*>(packed);
     const __nv_bfloat16* w2t = w1t + (size_t)p.E * p.H * p.d;
-    const CUtensorMap *mA1, *mA2;
-    const BMaps *mB1, *mB2;
+    CUtensorMap mA1, mA2;
+    BMaps mB1, mB2;
     // with row_token, the up-projection fetches its rows straight from x (no grouped copy of the tokens); its A
     // tensor map is then unused, any valid one will do
     DSMOE_TRY(cached_map_2d(&mA1, row_token ? hbuf : xp, amax, row_token ? p.H : p.d, BM));
@@ -2201,17 +2201,17 @@ dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const vo
     if (splits > 1) {
         up.k_splits = splits; up.split_rows = (int)amax;
         up.out = yp; up.out_f32 = 1;
-        DSMOE_TRY(launch_gemm(*mA1, *mB1, up, sm_count(), s, true, 0));
+        DSMOE_TRY(launch_gemm(mA1, mB1, up, sm_count(), s, true, 0));
         const long long vecs = (long long)amax * p.H / 4;
         DSMOE_CUDA_TRY(launch_chained(split_sum_kernel, (int)std::min<long long>((vecs + 255) / 256, 8ll * sm_count()), 256, 0, s,
             static_cast<const float4*>(yp), splits, (int)amax, offsets, p.E, p.H,
             static_cast<__nv_bfloat16*>(hbuf)));
     } else {
-        DSMOE_TRY(launch_gemm(*mA1, *mB1, up, sm_count(), s, true, moa ? 0 : pair_tiles));
+        DSMOE_TRY(launch_gemm(mA1, mB1, up, sm_count(), s, true, moa ? 0 : pair_tiles));
     }
     if (moa) DSMOE_TRY(launch_moa_attention(p, *moa, hbuf, row_token, moa->token_rows, offsets, dev_status, s));
     if (moa && moa->dense) return DSMOE_OK;      // the output projection is launch_dense_down's
-    DSMOE_TRY(launch_gemm(*mA2, *mB2, down, sm_count(), s, true, pair_tiles));
+    DSMOE_TRY(launch_gemm(mA2, mB2, down, sm_count(), s, true, pair_tiles));
     return DSMOE_OK;
 }
 
@@ -2241,9 +2241,9 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     const int t_pad = (p.T + 7) / 8 * 8;
     int G = sm_count() < kSmallMaxCtas ? sm_count() : kSmallMaxCtas;
     void* hg = ws + L.h;
-    const CUtensorMap *mX, *mHg;
-    const BMaps16* mW1;
-    const BMaps* mW2;
+    CUtensorMap mX, mHg;
+    BMaps16 mW1;
+    BMaps mW2;
     DSMOE_TRY(cached_map_2d(&mX, x, p.T, p.d, t_pad));
     DSMOE_TRY(cached_bmaps16(&mW1, w1t, p.E, p.H, p.d));
     DSMOE_TRY(cached_map_2d(&mHg, hg, p.T, (uint64_t)p.E * p.H, t_pad));
@@ -2268,8 +2268,7 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     // up-projection under that assumption while its router is still running; it starts over if the router disagrees.
     P.spec = p.T >= kSpecMinT ? 1 : 0;
     DSMOE_CUDA_TRY(cudaMemsetAsync(P.sync, 0, 32, s));
-    void* args[] = {const_cast<CUtensorMap*>(mX), const_cast<BMaps16*>(mW1), const_cast<CUtensorMap*>(mHg),
-                    const_cast<BMaps*>(mW2), &P};
+    void* args[] = {&mX, &mW1, &mHg, &mW2, &P};
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));
     DSMOE_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(small_layer_kernel), dim3(G), dim3(SMALL_THREADS),
@@ -2281,15 +2280,15 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
 dsmoe_status launch_dense_down(const dsmoe_layer_desc& p, const void* hg, const void* packed, void* out, int32_t* dev_status,
                                cudaStream_t s) {
     const __nv_bfloat16* w2t = static_cast<const __nv_bfloat16*>(packed) + (size_t)p.E * p.H * p.d;
-    const CUtensorMap* mA;
-    const BMaps* mB;
+    CUtensorMap mA;
+    BMaps mB;
     DSMOE_TRY(cached_map_2d(&mA, hg, p.T, (uint64_t)p.E * p.H, BM));
     DSMOE_TRY(cached_bmaps(&mB, w2t, p.E, p.d, p.H));
     GemmParams down{};
     down.mode = GEMM_DENSE_DOWN; down.epi = EPI_STORE; down.E = p.E; down.n_per_expert = p.d; down.k_per_expert = p.H;
     down.rows = p.T; down.out = out; down.ld_out = p.d; down.out_f32 = p.out_fp32 ? 1 : 0; down.dev_status = dev_status;
     const int tiles = ceil_div(p.T, BM) * ceil_div(p.d, BN);
-    return launch_gemm(*mA, *mB, down, tiles < sm_count() ? tiles : sm_count(), s, true, ceil_div(p.T, 2 * BM) * ceil_div(p.d, BN));
+    return launch_gemm(mA, mB, down, tiles < sm_count() ? tiles : sm_count(), s, true, ceil_div(p.T, 2 * BM) * ceil_div(p.d, BN));
 }
 
 dsmoe_status launch_layer_umma(const dsmoe_layer_desc& p, const void* x, const void* packed, const float* scores,
@@ -2301,15 +2300,15 @@ dsmoe_status launch_layer_umma(const dsmoe_layer_desc& p, const void* x, const v
     // Dense forward: gate folded into h, aggregation folded into the down-projection's reduction.
     const __nv_bfloat16* w1t = static_cast<const __nv_bfloat16*>(packed);
     void* hg = ws + L.h;                                        // [T, E*H] bf16
-    const CUtensorMap* mA1;
-    const BMaps* mB1;
+    CUtensorMap mA1;
+    BMaps mB1;
     DSMOE_TRY(cached_map_2d(&mA1, x, p.T, p.d, BM));
     DSMOE_TRY(cached_bmaps(&mB1, w1t, p.E, p.H, p.d));
     GemmParams up{};
     up.mode = GEMM_DENSE_UP; up.epi = EPI_GELU; up.E = p.E; up.n_per_expert = p.H; up.k_per_expert = p.d; up.rows = p.T;
     up.gate = scores; up.out = hg; up.ld_out = (long long)p.E * p.H; up.dev_status = dev_status;
     const int tiles_up = ceil_div(p.T, BM) * ceil_div(p.H, BN) * p.E;
-    DSMOE_TRY(launch_gemm(*mA1, *mB1, up, tiles_up < sm_count() ? tiles_up : sm_count(), s, true,
+    DSMOE_TRY(launch_gemm(mA1, mB1, up, tiles_up < sm_count() ? tiles_up : sm_count(), s, true,
                           ceil_div(p.T, 2 * BM) * ceil_div(p.H, BN) * p.E));
     DSMOE_TRY(launch_dense_down(p, hg, packed, out, dev_status, s));
     if (counts_out) {
@@ -2343,8 +2342,8 @@ dsmoe_status launch_dense_backward(const dsmoe_layer_desc& p, const void* x, con
     if (p.T == 0) return DSMOE_OK;
     if (!umma_supported(p)) return DSMOE_ERR_UNSUPPORTED;
     const __nv_bfloat16* w1t = static_cast<const __nv_bfloat16*>(packed);
-    const CUtensorMap *mX, *mdO;
-    const BMaps *mB1, *mB2;
+    CUtensorMap mX, mdO;
+    BMaps mB1, mB2;
     DSMOE_TRY(cached_map_2d(&mX, x, p.T, p.d, BM));
     DSMOE_TRY(cached_bmaps(&mB1, w1t, p.E, p.H, p.d));
     DSMOE_TRY(cached_map_2d(&mdO, dO, p.T, p.d, BM));
@@ -2360,8 +2359,8 @@ dsmoe_status launch_dense_backward(const dsmoe_layer_desc& p, const void* x, con
     const int tiles = ceil_div(p.T, BM) * ntn * p.E;
     const int grid = tiles < sm_count() ? tiles : sm_count();
     const int pair_tiles = ceil_div(p.T, 2 * BM) * ntn * p.E;
-    DSMOE_TRY(launch_gemm(*mX, *mB1, up, grid, s, true, pair_tiles));
-    DSMOE_TRY(launch_gemm(*mdO, *mB2, bw, grid, s, true, pair_tiles));
+    DSMOE_TRY(launch_gemm(mX, mB1, up, grid, s, true, pair_tiles));
+    DSMOE_TRY(launch_gemm(mdO, mB2, bw, grid, s, true, pair_tiles));
     const long long n = (long long)p.T * p.E;
     DSMOE_CUDA_TRY(launch_chained(bwd_finish_kernel, (unsigned)((n + 255) / 256), 256, 0, s, dot_part, dS, n, ntn));
     return DSMOE_OK;

@@ -79,7 +79,8 @@ int sm_count() {
 
 // Tensor maps depend only on the buffer and the shape, and encoding one is a driver call of a few microseconds
 // (a layer call needs up to 23): they are encoded once and found again by (address, shape).  A decode loop or a
-// serving loop calls with the same buffers every step.  Not thread-safe, like the rest of the host side.
+// serving loop calls with the same buffers every step.  Maps are handed out by value: once the cache is full, the next map to be
+// encoded takes an older one's place, which may be one that the same call has just found.  Not thread-safe, like the rest of the host side.
 struct MapKey {
     const void* ptr;
     uint64_t a, b, c;
@@ -106,7 +107,7 @@ MapCache<CUtensorMap, 256> g_maps2d;
 MapCache<BMaps, 128> g_bmaps;
 MapCache<BMaps16, 64> g_bmaps16;
 
-dsmoe_status cached_map_2d(const CUtensorMap** out, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+dsmoe_status cached_map_2d(CUtensorMap* out, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
     const MapKey k{ptr, rows, cols, box_rows, 0};
     CUtensorMap* m = g_maps2d.find(k);
     if (!m) {
@@ -115,10 +116,10 @@ dsmoe_status cached_map_2d(const CUtensorMap** out, const void* ptr, uint64_t ro
         m = g_maps2d.slot(k);
         *m = tmp;
     }
-    *out = m;
+    *out = *m;
     return DSMOE_OK;
 }
-dsmoe_status cached_bmaps(const BMaps** out, const void* ptr, uint64_t E, uint64_t n, uint64_t kk) {
+dsmoe_status cached_bmaps(BMaps* out, const void* ptr, uint64_t E, uint64_t n, uint64_t kk) {
     const MapKey k{ptr, E, n, kk, 1};
     BMaps* m = g_bmaps.find(k);
     if (!m) {
@@ -127,10 +128,10 @@ dsmoe_status cached_bmaps(const BMaps** out, const void* ptr, uint64_t E, uint64
         m = g_bmaps.slot(k);
         *m = tmp;
     }
-    *out = m;
+    *out = *m;
     return DSMOE_OK;
 }
-dsmoe_status cached_bmaps_plain(const BMaps** out, const void* ptr, uint64_t E, uint64_t n, uint64_t kk) {
+dsmoe_status cached_bmaps_plain(BMaps* out, const void* ptr, uint64_t E, uint64_t n, uint64_t kk) {
     const MapKey k{ptr, E, n, kk, 3};
     BMaps* m = g_bmaps.find(k);
     if (!m) {
@@ -139,10 +140,10 @@ dsmoe_status cached_bmaps_plain(const BMaps** out, const void* ptr, uint64_t E, 
         m = g_bmaps.slot(k);
         *m = tmp;
     }
-    *out = m;
+    *out = *m;
     return DSMOE_OK;
 }
-dsmoe_status cached_bmaps16(const BMaps16** out, const void* ptr, uint64_t E, uint64_t n, uint64_t kk) {
+dsmoe_status cached_bmaps16(BMaps16* out, const void* ptr, uint64_t E, uint64_t n, uint64_t kk) {
     const MapKey k{ptr, E, n, kk, 2};
     BMaps16* m = g_bmaps16.find(k);
     if (!m) {
@@ -151,7 +152,7 @@ dsmoe_status cached_bmaps16(const BMaps16** out, const void* ptr, uint64_t E, ui
         m = g_bmaps16.slot(k);
         *m = tmp;
     }
-    *out = m;
+    *out = *m;
     return DSMOE_OK;
 }
 

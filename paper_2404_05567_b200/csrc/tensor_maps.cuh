@@ -32,12 +32,12 @@ EncodeTiledFn encode_fn();
 int sm_count();     // of the current device (148 when there is none: host-only sizing)
 
 // bf16 [rows, cols] row-major, box {64 cols, box_rows}, 128-byte swizzle
-dsmoe_status cached_map_2d(const CUtensorMap** out, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
+dsmoe_status cached_map_2d(CUtensorMap* out, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
 // packed weights [E][k / 64][n][64]
-dsmoe_status cached_bmaps(const BMaps** out, const void* ptr, uint64_t E, uint64_t n, uint64_t k);
-dsmoe_status cached_bmaps16(const BMaps16** out, const void* ptr, uint64_t E, uint64_t n, uint64_t k);
+dsmoe_status cached_bmaps(BMaps* out, const void* ptr, uint64_t E, uint64_t n, uint64_t k);
+dsmoe_status cached_bmaps16(BMaps16* out, const void* ptr, uint64_t E, uint64_t n, uint64_t k);
 // weights in their natural layout [E][n][k], k contiguous
-dsmoe_status cached_bmaps_plain(const BMaps** out, const void* ptr, uint64_t E, uint64_t n, uint64_t k);
+dsmoe_status cached_bmaps_plain(BMaps* out, const void* ptr, uint64_t E, uint64_t n, uint64_t k);
 
 // Event pair around a launch when the timing ring is on and has room: *slot = its index, or -1.
 dsmoe_status timing_begin(cudaStream_t s, int* slot);
