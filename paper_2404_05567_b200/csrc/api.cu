@@ -68,7 +68,6 @@ WsLayout ws_layout(const dsmoe_layer_desc& p) {
     L.acc = take(!umma_supported(p) ? 0 : fuses_combine(p) ? T * p.d * 4 : amax * p.d * 4);
     // fp32 partial sums of the small-T path: (CTA, 2 column ranges, T, 256)
     L.partial = take(umma_supported(p) && p.T <= kSmallMaxT ? (size_t)kSmallMaxCtas * 2 * T * 256 * 4 : 0);
-    L.router = take(router_umma_supported(p) ? router_umma_scratch(p) : 0);   // tensor-core router: split Wr, partial logits
     // dense backward: the experts' hidden activations go to `h` ([T,E*H]); per-column-tile partial dot products here
     L.bwd = take(umma_supported(p) ? T * E * ceil_div(p.H, 256) * 4 : 0);
     L.total_packed = off;
@@ -252,7 +251,7 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
     // selects again)
     const bool counted = fast && router_umma_supported(p) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
     if (fast && router_umma_supported(p))
-        DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, ws + L.router, dev_status, s, counted ? chunk_prefix : nullptr));
+        DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, dev_status, s, counted ? chunk_prefix : nullptr));
     else
         DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s));
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK)
@@ -386,7 +385,7 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
     // selects again)
     const bool counted = router_umma_supported(p) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
     if (router_umma_supported(p))
-        DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, ws + L.router, dev_status, s, counted ? chunk_prefix : nullptr));
+        DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, dev_status, s, counted ? chunk_prefix : nullptr));
     else
         DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s));
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK)

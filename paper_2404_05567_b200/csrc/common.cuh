@@ -50,21 +50,35 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 int sm_count();
 // Grids of more than one wave are launched the ordinary way: each of their blocks would pay for its chain_wait().
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                         Args... args) {
+static inline cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                                  int cluster, Args... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if ((size_t)grid.x * grid.y * grid.z * block.x <= (size_t)sm_count() * 2048) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = (size_t)grid.x * grid.y * grid.z * block.x <= (size_t)sm_count() * 2048 ? 1 : 0;
+    cfg.numAttrs = n;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
     if (err != cudaSuccess) cudaGetLastError();      // reported by the caller's status, not left behind for others
     return err;
+}
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                         Args... args) {
+    return launch_chained_clusters(kernel, grid, block, smem, s, 1, args...);
 }
 
 dsmoe_status check_desc(const dsmoe_layer_desc* desc);
@@ -75,13 +89,13 @@ static inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; 
 // activation buffers follow and overlap between the execution paths, of which a call takes exactly one:
 //   plain (fp32-FMA GEMMs)     xp, h (fp32), yp
 //   tensor-core paths          h (bf16: grouped [Amax,H]; dense and small-T [T,E*H]), acc (grouped: fp32 [T,d] running
-//                              sum of the expert outputs), partial (small-T), router (split Wr, partial logits)
+//                              sum of the expert outputs), partial (small-T)
 // total_packed = bytes a call with packed weights needs; total = the maximum over both kinds of call.
 struct WsLayout {
     size_t scores, mask, k_t, counts, offsets, chunk_prefix, batch_k, sync, tile_done, mi, row_token, row_gate, token_rows;
     size_t stage_total;
     size_t xp, h_plain, yp;                 // plain path
-    size_t h, acc, partial, router, bwd;    // tensor-core paths
+    size_t h, acc, partial, bwd;            // tensor-core paths
     size_t total_plain, total_packed, total;
 };
 WsLayout ws_layout(const dsmoe_layer_desc& p);
@@ -151,13 +165,12 @@ dsmoe_status launch_mlp_generic(const dsmoe_layer_desc& p, const void* x, const 
 dsmoe_status timing_enable(int n_pairs);
 dsmoe_status timing_read(float* ms, int n_max, int* n);
 bool umma_supported(const dsmoe_layer_desc& p);   // bf16, d and H multiples of 64
-// Router for many tokens with the logits on the tensor cores (bf16 x; Wr split exactly into three bf16 terms, fp32
-// accumulation), then softmax and selection.  `scratch` holds router_umma_scratch(p) bytes.
+// Router for many tokens (router_umma.cu): logits on the tensor cores (bf16 x; Wr split exactly into three bf16 terms, fp32
+// accumulation), softmax, selection; mask, k_t and chunk_counts (see launch_group) optional.
 bool router_umma_supported(const dsmoe_layer_desc& p);
-size_t router_umma_scratch(const dsmoe_layer_desc& p, size_t* split_bytes = nullptr);
 dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
-                                float* scores, uint64_t* mask, int32_t* k_t, char* scratch, int32_t* dev_status,
-                                cudaStream_t s, int32_t* chunk_counts = nullptr);   // chunk_counts: see launch_group
+                                float* scores, uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s,
+                                int32_t* chunk_counts = nullptr);
 // Grouped expert MLPs on expert-sorted rows: h = GeLU(xp.W1[e]) (bf16, in `hbuf`), yp = h.W2[e].
 // With row_token (and x), the up-projection gathers its rows from x by index and xp is not read.
 // With cmb->out, the down-projection's epilogue also aggregates (Eq. 1's weighted sum, ascending expert order per

@@ -125,9 +125,6 @@ struct GemmParams {
     // dot_part[(token * E + e) * column_tiles + column_tile] (Eq. 3's <e_j(X), dO>, see launch_dense_backward)
     const __nv_bfloat16* act;   // [rows, E * n_per_expert] hidden activations GeLU(x.W1[e])
     float* dot_part;
-    // GEMM_DENSE_UP: "expert" e reads A's columns from e * a_expert_stride on (0: every expert reads the same columns;
-    // the router's logits use it to cut their reduction into pieces with an output block each)
-    int a_expert_stride;
     // GEMM_GROUPED, EPI_STORE with out_f32, single CTAs: the reduction is cut into k_splits equal runs of 64-wide blocks
     // (0 or 1: not cut); split s of a tile stores its partial sums to rows split_rows * s + r of `out`
     int k_splits, split_rows;
@@ -184,10 +181,10 @@ static_assert(sizeof(Shared) <= SHARED_BYTES, "Shared must fit its slot");
 __device__ unsigned long long g_trace[192][32];
 #define TRACE(i) sh.trace[i] = ptx::globaltimer_ns()
 // ... and of umma_gemm_kernel: clock cycles its roles spent waiting, per CTA, for the last launch of each kind
-// (0 router logits, 1 up-projection, 2 down-projection or backward): [0] MMA issuer in all, [1] of these waiting for
+// (0 up-projection, 1 down-projection or backward): [0] MMA issuer in all, [1] of these waiting for
 // operands, [2] for a free accumulator; [3] producer in all, [4] of these waiting for a free slot; [5] first epilogue
 // warp in all, [6] of these waiting for an accumulator; [7] tiles
-__device__ long long g_gemm_trace[3][192][8];
+__device__ long long g_gemm_trace[2][192][8];
 #define GTRACE_T0(v) const long long v = clock64()
 #define GTRACE_ADD(slot, v) gtr[slot] += clock64() - (v)
 #else
@@ -456,7 +453,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     } else {
                         b_e = t.e;
                         b_k = (t.k0 + i) * BK;
-                        a_col = t.e * P.a_expert_stride + b_k;
+                        a_col = b_k;
                     }
                     if (!P.gather) {
                         if (PAIR) ptx::tma_load_2d_pair(smA + s * A_STAGE_BYTES, &tmA, bar, a_col, t.row0);
@@ -483,7 +480,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #ifdef DSMOE_TRACE
             GTRACE_ADD(3, t_all);
             if (blockIdx.x < 192) {
-                long long* g = g_gemm_trace[P.epi == EPI_GELU ? 1 : (P.n_per_expert <= 192 ? 0 : 2)][blockIdx.x];
+                long long* g = g_gemm_trace[P.epi == EPI_GELU ? 0 : 1][blockIdx.x];
                 g[3] = gtr[3];
                 g[4] = gtr[4];
             }
@@ -562,7 +559,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #ifdef DSMOE_TRACE
             GTRACE_ADD(0, t_all);
             if (blockIdx.x < 192) {
-                long long* g = g_gemm_trace[P.epi == EPI_GELU ? 1 : (P.n_per_expert <= 192 ? 0 : 2)][blockIdx.x];
+                long long* g = g_gemm_trace[P.epi == EPI_GELU ? 0 : 1][blockIdx.x];
                 g[0] = gtr[0];
                 g[1] = gtr[1];
                 g[2] = gtr[2];
@@ -897,7 +894,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #ifdef DSMOE_TRACE
         GTRACE_ADD(5, t_all);
         if (warp == 2 && lane == 0 && blockIdx.x < 192) {
-            long long* g = g_gemm_trace[P.epi == EPI_GELU ? 1 : (P.n_per_expert <= 192 ? 0 : 2)][blockIdx.x];
+            long long* g = g_gemm_trace[P.epi == EPI_GELU ? 0 : 1][blockIdx.x];
             g[5] = gtr[5];
             g[6] = gtr[6];
         }
@@ -1182,7 +1179,7 @@ __device__ __noinline__ void small_router_pass(const RouterArgs P, Shared& sh, i
         float s_lo, s_hi;
         softmax_warp(l_lo, l_hi, P.E, lane, s_lo, s_hi);
         if (mode == 0) {
-            const uint64_t m = select_warp(s_lo, s_hi, P.sel, lane);
+            const uint64_t m = select_warp<false>(s_lo, s_hi, P.sel, lane);
             if (lane == 0) {
                 sh.mask_s[tt] = m;
                 atomicOr(&sh.active_mask, (unsigned long long)m);
@@ -1669,7 +1666,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
             const bool v_lo = lane < P.E, v_hi = lane + 32 < P.E;
             const float l_lo = v_lo ? (P.br ? P.br[lane] : 0.f) + sh.gate_s[lane] : 0.f;
             const float l_hi = v_hi ? (P.br ? P.br[lane + 32] : 0.f) + sh.gate_s[lane + 32] : 0.f;
-            softmax_select_store(l_lo, l_hi, (int)blockIdx.x, P.sel, lane, P.scores, P.mask, P.k_t);
+            softmax_select_store<false>(l_lo, l_hi, (int)blockIdx.x, P.sel, lane, P.scores, P.mask, P.k_t);
         }
         EPI_SYNC();
         if (etid == 0) {
@@ -1983,7 +1980,7 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
     } else {
         // (the large dense launches are not chained: no gap to speak of, and 1 % slower with it, 3682 against 3732 us for the
         // dense layer at 16384 tokens)
-        if (P.mode == GEMM_GROUPED || P.rows <= kChainMaxRows || P.n_per_expert <= 3 * kMaxExperts)
+        if (P.mode == GEMM_GROUPED || P.rows <= kChainMaxRows)
             DSMOE_CUDA_TRY(launch_chained(umma_gemm_kernel<false>, grid, threads, smem, s, a, b, P));
         else {
             umma_gemm_kernel<false><<<grid, threads, smem, s>>>(a, b, P);
@@ -1992,73 +1989,6 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
     }
     DSMOE_TRY(timing_end(s, timed));
     return DSMOE_OK;
-}
-
-// ---------------------------------------------------------------- router logits on the tensor cores
-// Wr (fp32) is written as the exact sum of three bf16 terms, w = w1 + w2 + w3 (w1 = bf16(w), w2 = bf16(w - w1),
-// w3 = bf16(w - w1 - w2): 3 x 8 significant bits cover fp32's 24).  x is bf16, so every product x.w_i is exact in
-// fp32 and the three sums accumulate in fp32: the logits are as accurate as an fp32 dot product, at tensor-core
-// speed.  The three terms sit side by side along N: B = [3 * EP, d] bf16 in the packed weights' layout, EP = E rounded up to 32 or 64.
-__global__ void __launch_bounds__(256) router_split_kernel(const float* __restrict__ Wr, __nv_bfloat16* __restrict__ out,
-                                                           int d, int E, int EP) {
-    chain_next();
-    chain_wait();
-    const long long idx = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (idx >= (long long)EP * d) return;
-    const int e = (int)(idx / d), k = (int)(idx % d);
-    const float w = e < E ? Wr[(size_t)k * E + e] : 0.f;
-    const __nv_bfloat16 w1 = __float2bfloat16_rn(w);
-    const float r1 = w - __bfloat162float(w1);
-    const __nv_bfloat16 w2 = __float2bfloat16_rn(r1);
-    const float r2 = r1 - __bfloat162float(w2);
-    // block-major like the packed expert weights: [k / 64][3 * EP][64], term g in rows g * EP .. of every block
-    const long long o = ((long long)(k / BK) * (3 * EP) + e) * BK + k % BK;
-    out[o] = w1;
-    out[o + (long long)EP * BK] = w2;
-    out[o + 2ll * EP * BK] = __float2bfloat16_rn(r2);
-}
-
-// logits = (s1 + s2) + s3 + bias per expert, then softmax and selection: one warp per token
-// (the reduction over d may come in `pieces` blocks of 3 EP sums each, added in ascending order).  A block is one
-// chunk of 32 tokens; with chunk_counts its first warp then counts, per expert, the chunk's tokens that selected it
-// (what chunk_count_kernel would write to chunk_prefix[chunk,:]).
-__global__ void __launch_bounds__(32 * kChunk, 2) router_finish_kernel(const float* __restrict__ sums, const float* __restrict__ br,
-                                                                    float* __restrict__ scores, uint64_t* __restrict__ mask,
-                                                                    int32_t* __restrict__ k_t, int32_t* __restrict__ chunk_counts,
-                                                                    int T, int EP, int pieces, SelParams q) {
-    chain_next();
-    chain_wait();
-    __shared__ uint64_t mask_s[kChunk];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t = blockIdx.x * kChunk + warp;
-    uint64_t m = 0;
-    if (t < T) {
-        const float* row = sums + (size_t)t * 3 * EP * pieces;
-        const bool v_lo = lane < q.E, v_hi = lane + 32 < q.E;
-        float l_lo = 0.f, l_hi = 0.f;
-        for (int pc = 0; pc < pieces; ++pc, row += 3 * EP) {
-            if (v_lo) l_lo += (row[lane] + row[EP + lane]) + row[2 * EP + lane];
-            if (v_hi) l_hi += (row[lane + 32] + row[EP + lane + 32]) + row[2 * EP + lane + 32];
-        }
-        if (v_lo && br) l_lo += br[lane];
-        if (v_hi && br) l_hi += br[lane + 32];
-        m = softmax_select_store(l_lo, l_hi, t, q, lane, scores, mask, k_t);
-    }
-    if (!chunk_counts) return;
-    if (lane == 0) mask_s[warp] = m;
-    __syncthreads();
-    if (warp == 0) {
-        const uint64_t mt = mask_s[lane];
-        int c_lo = 0, c_hi = 0;
-        for (int e = 0; e < q.E; ++e) {
-            const int n = __popc(__ballot_sync(0xffffffffu, (mt >> e) & 1));
-            if (lane == (e & 31)) {
-                if (e < 32) c_lo = n; else c_hi = n;
-            }
-        }
-        if (lane < q.E) chunk_counts[(size_t)blockIdx.x * q.E + lane] = c_lo;
-        if (lane + 32 < q.E) chunk_counts[(size_t)blockIdx.x * q.E + lane + 32] = c_hi;
-    }
 }
 
 // out[r,:] (bf16) = the sum over the splits, in ascending order, of the fp32 partial rows part[s * split_rows + r,:]
@@ -2088,53 +2018,12 @@ __global__ void __launch_bounds__(256) split_sum_kernel(const float4* __restrict
 
 }  // namespace
 
-// With few row tiles the logits' reduction over d is cut into 2 or 4 pieces, each a tile with its own block of sums,
-// so that the launch covers most SMs instead of T / 128 of them.
-constexpr int kRouterMaxPieces = 4;
-
-size_t router_umma_scratch(const dsmoe_layer_desc& p, size_t* split_bytes) {
-    const size_t EP = p.E <= 32 ? 32 : 64;
-    const size_t a = align_up(3 * EP * (size_t)p.d * 2, 256);
-    if (split_bytes) *split_bytes = a;
-    return a + align_up((size_t)p.T * kRouterMaxPieces * 3 * EP * 4, 256);
-}
-
-bool router_umma_supported(const dsmoe_layer_desc& p) { return umma_supported(p) && p.T > 256; }
-
-dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
-                                float* scores, uint64_t* mask, int32_t* k_t, char* scratch, int32_t* dev_status,
-                                cudaStream_t s, int32_t* chunk_counts) {
-    const int EP = p.E <= 32 ? 32 : 64;
-    size_t split_bytes = 0;
-    router_umma_scratch(p, &split_bytes);
-    __nv_bfloat16* wsplit = reinterpret_cast<__nv_bfloat16*>(scratch);
-    float* sums = reinterpret_cast<float*>(scratch + split_bytes);
-    DSMOE_CUDA_TRY(launch_chained(router_split_kernel, ceil_div(EP * p.d, 256), 256, 0, s, Wr, wsplit, p.d, p.E, EP));
-    CUtensorMap mA;
-    BMaps mB;
-    DSMOE_TRY(cached_map_2d(&mA, x, p.T, p.d, BM));
-    const int row_tiles = ceil_div(p.T, BM);
-    int pieces = kRouterMaxPieces;
-    while (pieces > 1 && (row_tiles * pieces > sm_count() || (p.d / BK) % pieces)) pieces /= 2;
-    DSMOE_TRY(cached_bmaps(&mB, wsplit, pieces, 3 * EP, p.d / pieces));
-    GemmParams g{};
-    g.mode = GEMM_DENSE_UP; g.epi = EPI_STORE; g.E = pieces; g.n_per_expert = 3 * EP; g.k_per_expert = p.d / pieces;
-    g.a_expert_stride = p.d / pieces; g.rows = p.T;
-    g.out = sums; g.ld_out = (long long)pieces * 3 * EP; g.out_f32 = 1; g.dev_status = dev_status;
-    const int tiles = row_tiles * pieces;
-    DSMOE_TRY(launch_gemm(mA, mB, g, tiles < sm_count() ? tiles : sm_count(), s, false));
-    DSMOE_CUDA_TRY(launch_chained(router_finish_kernel, ceil_div(p.T, kChunk), 32 * kChunk, 0, s,
-        sums, br, scores, mask, k_t, chunk_counts, p.T, EP, pieces, SelParams{p.E, p.mode, p.eps, p.eps_normalized,
-        p.K, p.min_k, nullptr}));
-    return DSMOE_OK;
-}
-
 #ifdef DSMOE_TRACE
 extern "C" __attribute__((visibility("default"))) int dsmoe_trace_read(unsigned long long* out) {
     return (int)cudaMemcpyFromSymbol(out, g_trace, sizeof(unsigned long long) * 192 * 32);
 }
 extern "C" __attribute__((visibility("default"))) int dsmoe_gemm_trace_read(long long* out) {
-    return (int)cudaMemcpyFromSymbol(out, g_gemm_trace, sizeof(long long) * 3 * 192 * 8);
+    return (int)cudaMemcpyFromSymbol(out, g_gemm_trace, sizeof(long long) * 2 * 192 * 8);
 }
 #endif
 

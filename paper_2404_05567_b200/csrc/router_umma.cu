@@ -1,0 +1,305 @@
+// The router for many tokens (Eq. 1's S = softmax(x.Wr + b)) on the 5th-generation tensor cores, in one launch: logits,
+// softmax, selection and the per-chunk counts that the grouping step needs.
+//
+// Wr (fp32) enters as the exact sum of three bf16 terms, w = w1 + w2 + w3: the upper, middle and lower 8 of its 24
+// significant bits.  x is bf16, so every product x.w_i is exact in fp32 and
+// the three sums accumulate in fp32: the logits are as accurate as an fp32 dot product, at tensor-core speed.  The
+// terms sit side by side along the MMA's N: 3 * EP columns, EP = E rounded up to 32 or 64.
+//
+// A cluster of C CTAs (1, 2 or 4) owns 128 tokens and shares out the reduction over d, so that few row tiles still cover most
+// SMs.  Each CTA:
+//   warp 0      brings its 128 x 64 tiles of x by TMA                      (one lane)
+//   warp 1      issues the MMAs (M = 128, N = 3 EP); owns the TMEM columns (one lane)
+//   warps 2..17 split Wr: teams of four warps take every fourth 64-wide block of the reduction, an expert per lane, and write
+//               the three terms in the 128-byte-swizzle order the MMA reads; then they finish the tokens
+// The CTAs' partial logits meet through distributed shared memory: each CTA finishes 128 / C of the tokens, adding the
+// ranks' sums in ascending order.
+// At 7001 tokens of 4096 and 32 experts it takes 24.7 us (x once from HBM: 57 MB, 9 us); as three launches -- splitting Wr into a
+// global buffer, a GEMM, the finish over its sums -- 3.2 + 24.5 + 9.5 us and two gaps; 300 tokens of 2048: 10.6 against
+// 2.3 + 8.6 + 4.1 us and two gaps, the layer 97.2 -> 92.2 us.  What bounds it: shared memory (per 64-wide block 12 KB of terms
+// and 16 KB of x are written and read by the MMAs) and, below 1000 tokens, the chain of first loads, sums and softmax.
+#include "common.cuh"
+#include "router_device.cuh"
+#include "tensor_maps.cuh"
+#include "umma.cuh"
+
+namespace dsmoe {
+
+namespace {
+
+constexpr int kRuM = 128, kRuK = 64, kRuTeams = 4, kRuWarps = 16, kRuThreads = 64 + 32 * kRuWarps;
+
+template <int EP>
+struct RuGeo {
+    static constexpr int N = 3 * EP;
+    static constexpr int A_BYTES = kRuM * kRuK * 2, B_BYTES = N * kRuK * 2;
+    static constexpr int STA = 6, STB = EP == 32 ? 8 : 4;           // slots of x and of Wr's terms
+    static constexpr int RING = STA * A_BYTES + STB * B_BYTES;      // 192 KB
+    static constexpr int LD = EP + 1;                              // floats per token of the partial logits (in the idle ring)
+    static constexpr uint32_t TMEM = EP == 32 ? 128 : 256;
+    static_assert(kRuM * LD * 4 <= RING, "the partial logits take the ring's place");
+};
+
+struct RuShared {
+    uint64_t full_a[6], empty_a[6], full_b[8], empty_b[8], done;
+    uint32_t tmem_base;
+    volatile int abort_flag;
+    uint64_t mask_s[kRuM];
+};
+
+template <int EP>
+constexpr size_t router_umma_smem() { return 1024 + (size_t)RuGeo<EP>::RING + sizeof(RuShared); }
+
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+template <int EP, int C>
+__global__ void __launch_bounds__(kRuThreads, 1)
+router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restrict__ Wr, const float* __restrict__ br,
+                   float* __restrict__ scores, uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
+                   int32_t* __restrict__ chunk_counts, int T, int d, const SelParams q, int32_t* __restrict__ dev_status) {
+    using G = RuGeo<EP>;
+    extern __shared__ uint8_t ru_smem[];
+    const uint32_t raw = ptx::smem_u32(ru_smem), base = (raw + 1023u) & ~1023u;
+    RuShared& sh = *reinterpret_cast<RuShared*>(ru_smem + (base - raw) + G::RING);
+    const uint32_t smA = base, smB = base + G::STA * G::A_BYTES;
+    unsigned char* const pB = ru_smem + (base - raw) + G::STA * G::A_BYTES;
+    float* const part = reinterpret_cast<float*>(ru_smem + (base - raw));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)ptx::cluster_ctarank(), tile = (int)blockIdx.x / C;
+    const int nk = d / kRuK / C, kb0 = rank * nk;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < G::STA; ++s) {
+            ptx::mbar_init(ptx::smem_u32(&sh.full_a[s]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh.empty_a[s]), 1);
+        }
+        for (int s = 0; s < G::STB; ++s) {
+            ptx::mbar_init(ptx::smem_u32(&sh.full_b[s]), kRuWarps / kRuTeams);
+            ptx::mbar_init(ptx::smem_u32(&sh.empty_b[s]), 1);
+        }
+        ptx::mbar_init(ptx::smem_u32(&sh.done), 1);
+        sh.abort_flag = 0;
+        ptx::fence_barrier_init();
+        ptx::prefetch_tensormap(&tmX);
+    }
+    if (warp == 1) {
+        ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), G::TMEM);
+        ptx::tmem_relinquish();
+    }
+    chain_next();
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tmem = sh.tmem_base;
+    chain_wait();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            for (int n = 0; n < nk; ++n) {
+                const int s = n % G::STA;
+                if (!ptx::mbar_wait(ptx::smem_u32(&sh.empty_a[s]), ((uint32_t)(n / G::STA) & 1u) ^ 1u, &sh.abort_flag)) break;
+                const uint32_t bar = ptx::smem_u32(&sh.full_a[s]);
+                ptx::mbar_expect_tx(bar, G::A_BYTES);
+                ptx::tma_load_2d(smA + s * G::A_BYTES, &tmX, bar, (kb0 + n) * kRuK, tile * kRuM);
+            }
+            if (sh.abort_flag) {                      // copies already issued still land in this CTA's shared memory
+                const uint64_t t0 = ptx::globaltimer_ns();
+                while (ptx::globaltimer_ns() - t0 < 200000ull) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = ptx::make_idesc_bf16(kRuM, G::N);
+            bool alive = true;
+            for (int n = 0; n < nk; ++n) {
+                const int a = n % G::STA, b = n % G::STB;
+                if (!ptx::mbar_wait(ptx::smem_u32(&sh.full_b[b]), (uint32_t)(n / G::STB) & 1u, &sh.abort_flag) ||
+                    !ptx::mbar_wait(ptx::smem_u32(&sh.full_a[a]), (uint32_t)(n / G::STA) & 1u, &sh.abort_flag)) {
+                    alive = false;
+                    break;
+                }
+                ptx::tc_fence_after();
+#pragma unroll
+                for (int k = 0; k < kRuK / 16; ++k)
+                    ptx::umma_bf16(tmem, ptx::make_desc_k_sw128(smA + a * G::A_BYTES + k * 32),
+                                   ptx::make_desc_k_sw128(smB + b * G::B_BYTES + k * 32), idesc, (uint32_t)((n | k) != 0));
+                ptx::umma_commit(ptx::smem_u32(&sh.empty_a[a]));
+                ptx::umma_commit(ptx::smem_u32(&sh.empty_b[b]));
+            }
+            if (alive) ptx::umma_commit(ptx::smem_u32(&sh.done));
+        }
+    } else {
+        constexpr int PC = 8 / (kRuWarps / kRuTeams);                     // 16-byte pieces of a row per warp
+        const int w = warp - 2, team = w % kRuTeams, c0 = (w / kRuTeams) * PC;
+        for (int n = team; n < nk; n += kRuTeams) {
+            const int s = n % G::STB;
+            bool alive = true;
+#pragma unroll
+            for (int h = 0; h < EP / 32; ++h) {
+                const int e = lane + 32 * h;
+                const float* src = Wr + (size_t)((kb0 + n) * kRuK + c0 * 8) * q.E + e;
+                float v[8 * PC];
+#pragma unroll
+                for (int i = 0; i < 8 * PC; ++i) v[i] = e < q.E ? __ldg(src + (size_t)i * q.E) : 0.f;
+                if (h == 0 && !ptx::mbar_wait(ptx::smem_u32(&sh.empty_b[s]), ((uint32_t)(n / G::STB) & 1u) ^ 1u, &sh.abort_flag)) {
+                    alive = false;
+                    break;
+                }
+                unsigned char* const row0 = pB + s * G::B_BYTES + e * 128;
+#pragma unroll
+                for (int c = 0; c < PC; ++c) {
+                    // (cut off, not rounded: the terms are just as exact, and a mask and a subtraction each)
+                    uint32_t t1[4], t2[4], t3[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        uint32_t a[2], b[2], g[2];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            a[u] = __float_as_uint(v[8 * c + 2 * i + u]);
+                            const float r1 = v[8 * c + 2 * i + u] - __uint_as_float(a[u] & 0xffff0000u);
+                            b[u] = __float_as_uint(r1);
+                            g[u] = __float_as_uint(r1 - __uint_as_float(b[u] & 0xffff0000u));
+                        }
+                        t1[i] = __byte_perm(a[0], a[1], 0x7632);
+                        t2[i] = __byte_perm(b[0], b[1], 0x7632);
+                        t3[i] = __byte_perm(g[0], g[1], 0x7632);
+                    }
+                    const int at = ((c0 + c) ^ (e & 7)) * 16;           // EP is a multiple of 8: the same for all three terms
+                    *reinterpret_cast<uint4*>(row0 + at) = make_uint4(t1[0], t1[1], t1[2], t1[3]);
+                    *reinterpret_cast<uint4*>(row0 + EP * 128 + at) = make_uint4(t2[0], t2[1], t2[2], t2[3]);
+                    *reinterpret_cast<uint4*>(row0 + 2 * EP * 128 + at) = make_uint4(t3[0], t3[1], t3[2], t3[3]);
+                }
+            }
+            if (__any_sync(0xffffffffu, !alive)) break;
+            ptx::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.full_b[s]));
+        }
+        // this CTA's sums, (s1 + s2) + s3 per expert: eight of the warps, two per TMEM lane quarter, each half of the experts
+        const int qd = warp & 3, row = qd * 32 + lane;
+        const bool ok = !__any_sync(0xffffffffu, !ptx::mbar_wait(ptx::smem_u32(&sh.done), 0u, &sh.abort_flag));
+        if (ok && w < 8) {
+            ptx::tc_fence_after();
+#pragma unroll
+            for (int h = 0; h < EP / 32; ++h) {
+                const int e0 = (w >= 4 ? EP / 2 : 0) + 16 * h;
+                uint32_t a[16], b[16], g[16];
+                const uint32_t at = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)e0;
+                ptx::tmem_ld16(at, a);
+                ptx::tmem_ld16(at + EP, b);
+                ptx::tmem_ld16(at + 2 * EP, g);
+                ptx::tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    part[row * G::LD + e0 + i] = (__uint_as_float(a[i]) + __uint_as_float(b[i])) + __uint_as_float(g[i]);
+            }
+            ptx::tc_fence_before();
+        }
+    }
+    ptx::cluster_sync();                               // every rank's partial logits are in place
+    if (warp >= 2) {
+        const int w = warp - 2, per = kRuM / C, first = rank * per;
+        const bool v_lo = lane < q.E, v_hi = lane + 32 < q.E;
+        const float b_lo = br && v_lo ? br[lane] : 0.f, b_hi = br && v_hi ? br[lane + 32] : 0.f;
+        // a warp's 128 / 16 / C tokens: every rank's sums of all of them are asked for before the first is used
+        constexpr int NT = kRuM / kRuWarps;
+        float lo[NT], hi[NT];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {                 // j = token * C + rank
+            const int tl = first + w + (j / C) * kRuWarps, r = j % C;
+            const uint32_t at = ptx::map_to_cta(ptx::smem_u32(part + tl * G::LD + lane), (uint32_t)r);
+            lo[j] = v_lo ? ld_cluster(at) : 0.f;
+            hi[j] = EP > 32 && v_hi ? ld_cluster(at + 128) : 0.f;
+        }
+#pragma unroll 1
+        for (int i = 0; i < NT / C; ++i) {
+            const int t = tile * kRuM + first + w + i * kRuWarps;
+            float l_lo = 0.f, l_hi = 0.f;
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                if (j / C == i) {
+                    l_lo += lo[j];
+                    l_hi += hi[j];
+                }
+            }
+            if (br) {
+                l_lo += b_lo;
+                l_hi += b_hi;
+            }
+            uint64_t m = 0;
+            if (t < T && sh.abort_flag == 0) m = softmax_select_store(l_lo, l_hi, t, q, lane, scores, mask, k_t);
+            if (lane == 0) sh.mask_s[w + i * kRuWarps] = m;
+        }
+        if (chunk_counts) {
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kRuWarps) : "memory");
+            const int chunk = (tile * kRuM + first) / kChunk + w;
+            if (w < per / kChunk && chunk * kChunk < T) {
+                const uint64_t mt = sh.mask_s[w * kChunk + lane];
+                int c_lo = 0, c_hi = 0;
+                for (int e = 0; e < q.E; ++e) {
+                    const int n = __popc(__ballot_sync(0xffffffffu, (mt >> e) & 1));
+                    if (lane == (e & 31)) {
+                        if (e < 32) c_lo = n; else c_hi = n;
+                    }
+                }
+                if (v_lo) chunk_counts[(size_t)chunk * q.E + lane] = c_lo;
+                if (v_hi) chunk_counts[(size_t)chunk * q.E + lane + 32] = c_hi;
+            }
+        }
+    }
+    ptx::tc_fence_before();
+    ptx::cluster_sync();                               // nobody leaves while another rank may read its sums
+    if (warp == 1) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc(tmem, G::TMEM);
+    }
+    if (threadIdx.x == 0 && sh.abort_flag && dev_status) *dev_status = DSMOE_ERR_TIMEOUT;
+}
+
+template <int EP, int C>
+dsmoe_status launch_clusters(const dsmoe_layer_desc& p, const CUtensorMap& mX, const float* Wr, const float* br, float* scores,
+                             uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s) {
+    static bool attr[kMaxDeviceSlots] = {};
+    int dev = 0;
+    DeviceState* st = nullptr;
+    DSMOE_TRY(device_state(&st, &dev));
+    if (!attr[dev]) {
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(router_umma_kernel<EP, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)router_umma_smem<EP>()));
+        attr[dev] = true;
+    }
+    DSMOE_CUDA_TRY(launch_chained_clusters(router_umma_kernel<EP, C>, ceil_div(p.T, kRuM) * C, kRuThreads, router_umma_smem<EP>(), s, C,
+        mX, Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d, SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr},
+        dev_status));
+    return DSMOE_OK;
+}
+
+template <int EP>
+dsmoe_status launch_ep(const dsmoe_layer_desc& p, const CUtensorMap& mX, const float* Wr, const float* br, float* scores,
+                       uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s) {
+    // with few row tiles the reduction over d is cut into 2 or 4 pieces, a CTA each, so that the launch covers most SMs
+    const int row_tiles = ceil_div(p.T, kRuM), sms = sm_count(), blocks = p.d / kRuK;
+    if (row_tiles * 4 <= sms && blocks % 4 == 0)
+        return launch_clusters<EP, 4>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+    if (row_tiles * 2 <= sms && blocks % 2 == 0)
+        return launch_clusters<EP, 2>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+    return launch_clusters<EP, 1>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+}
+
+}  // namespace
+
+bool router_umma_supported(const dsmoe_layer_desc& p) { return umma_supported(p) && p.T > 256; }
+
+dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores,
+                                uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s, int32_t* chunk_counts) {
+    CUtensorMap mX;
+    DSMOE_TRY(cached_map_2d(&mX, x, p.T, p.d, kRuM));
+    return p.E <= 32 ? launch_ep<32>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s)
+                     : launch_ep<64>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+}
+
+}  // namespace dsmoe

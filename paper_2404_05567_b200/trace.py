@@ -74,13 +74,13 @@ def gemm_waits(a):
     for _ in range(a.reps):
         dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, pk, out, None, counts, ws, status)
     torch.cuda.synchronize()
-    buf = (ctypes.c_longlong * (3 * 192 * 8))()
+    buf = (ctypes.c_longlong * (2 * 192 * 8))()
     if dm.lib().dsmoe_gemm_trace_read(buf) != 0:
         raise RuntimeError("dsmoe_gemm_trace_read failed")
-    g = np.array(buf[:], dtype=np.float64).reshape(3, 192, 8)
+    g = np.array(buf[:], dtype=np.float64).reshape(2, 192, 8)
     print(f"{a.gemm}: T={T} d={d} H={H} E={E}, pairs {'library' if a.pairs is None else a.pairs}, device status {int(status.item())}")
     print("-- umma_gemm_kernel, last launch of each kind; medians over the CTAs that hold the role")
-    for k, name in enumerate(("router logits", "up-projection", "down-projection")):
+    for k, name in enumerate(("up-projection", "down-projection")):
         mm, pr, ep = g[k][g[k][:, 0] > 0], g[k][g[k][:, 3] > 0], g[k][g[k][:, 5] > 0]
         if not len(mm):
             continue
