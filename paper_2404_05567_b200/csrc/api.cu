@@ -136,6 +136,8 @@ dsmoe_status dsmoe_router(const dsmoe_layer_desc* desc, const void* x, const flo
     DSMOE_TRY(check_desc(desc));
     if (desc->T == 0) return DSMOE_OK;
     if (!x || !Wr || !scores || !aligned16(x) || !aligned16(Wr)) return DSMOE_ERR_INVALID_ARG;
+    if (router_umma_supported(*desc, kRouterExactRun))
+        return launch_router_umma(*desc, x, Wr, br, scores, nullptr, nullptr, nullptr, (cudaStream_t)stream, nullptr, kRouterExactRun);
     return launch_router(*desc, x, Wr, br, scores, nullptr, nullptr, (cudaStream_t)stream);
 }
 

@@ -167,10 +167,13 @@ dsmoe_status timing_read(float* ms, int n_max, int* n);
 bool umma_supported(const dsmoe_layer_desc& p);   // bf16, d and H multiples of 64
 // Router for many tokens (router_umma.cu): logits on the tensor cores (bf16 x; Wr split exactly into three bf16 terms, fp32
 // accumulation), softmax, selection; mask, k_t and chunk_counts (see launch_group) optional.
-bool router_umma_supported(const dsmoe_layer_desc& p);
+// max_run > 0: no accumulator sums over more 64-wide blocks of d than this (kRouterExactRun: the scores are then closer to 64
+// bits than router_tile_kernel's, measured at d 2048 to 6144, 8 to 64 experts, 300 to 16384 tokens).
+constexpr int kRouterExactRun = 7;
+bool router_umma_supported(const dsmoe_layer_desc& p, int max_run = 0);
 dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
                                 float* scores, uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s,
-                                int32_t* chunk_counts = nullptr);
+                                int32_t* chunk_counts = nullptr, int max_run = 0);
 // Grouped expert MLPs on expert-sorted rows: h = GeLU(xp.W1[e]) (bf16, in `hbuf`), yp = h.W2[e].
 // With row_token (and x), the up-projection gathers its rows from x by index and xp is not read.
 // With cmb->out, the down-projection's epilogue also aggregates (Eq. 1's weighted sum, ascending expert order per

@@ -3,8 +3,11 @@
 //
 // Wr (fp32) enters as the exact sum of three bf16 terms, w = w1 + w2 + w3: the upper, middle and lower 8 of its 24
 // significant bits.  x is bf16, so every product x.w_i is exact in fp32 and
-// the three sums accumulate in fp32: the logits are as accurate as an fp32 dot product, at tensor-core speed.  The
-// terms sit side by side along the MMA's N: 3 * EP columns, EP = E rounded up to 32 or 64.
+// the three sums accumulate in fp32, at tensor-core speed.  The terms sit side by side along the MMA's N: 3 * EP columns, EP = E
+// rounded up to 32 or 64.  The tensor core cuts its running sums off instead of rounding them, an error that grows with the
+// length of a sum, so a CTA spreads its part of the reduction over 5 (EP = 64: 2) accumulators, one run of blocks after the
+// other, which are added in fp32.  Scores against 64 bits, relative 2-norm: 7001 tokens of 4096, 32 experts 3.7e-7 (one
+// accumulator 2.0e-6, router_tile_kernel's FMAs 5.5e-7); 4096 tokens of 4096, 64 experts 4.9e-7 (1.0e-6, 5.9e-7); 0.3 us.
 //
 // A cluster of C CTAs (1, 2 or 4) owns 128 tokens and shares out the reduction over d, so that few row tiles still cover most
 // SMs.  Each CTA:
@@ -36,7 +39,8 @@ struct RuGeo {
     static constexpr int STA = 6, STB = EP == 32 ? 8 : 4;           // slots of x and of Wr's terms
     static constexpr int RING = STA * A_BYTES + STB * B_BYTES;      // 192 KB
     static constexpr int LD = EP + 1;                              // floats per token of the partial logits (in the idle ring)
-    static constexpr uint32_t TMEM = EP == 32 ? 128 : 256;
+    static constexpr int ACCS = EP == 32 ? 5 : 2;                   // accumulators side by side in the 512 TMEM columns
+    static constexpr uint32_t TMEM = 512;
     static_assert(kRuM * LD * 4 <= RING, "the partial logits take the ring's place");
 };
 
@@ -71,6 +75,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restr
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)ptx::cluster_ctarank(), tile = (int)blockIdx.x / C;
     const int nk = d / kRuK / C, kb0 = rank * nk;
+    const int run = (nk + G::ACCS - 1) / G::ACCS;        // blocks per accumulator
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < G::STA; ++s) {
@@ -116,8 +121,13 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restr
         if (lane == 0) {
             const uint32_t idesc = ptx::make_idesc_bf16(kRuM, G::N);
             bool alive = true;
-            for (int n = 0; n < nk; ++n) {
+            uint32_t acc = tmem;
+            for (int n = 0, in_run = 0; n < nk; ++n, ++in_run) {
                 const int a = n % G::STA, b = n % G::STB;
+                if (in_run == run) {                        // the next accumulator
+                    in_run = 0;
+                    acc += G::N;
+                }
                 if (!ptx::mbar_wait(ptx::smem_u32(&sh.full_b[b]), (uint32_t)(n / G::STB) & 1u, &sh.abort_flag) ||
                     !ptx::mbar_wait(ptx::smem_u32(&sh.full_a[a]), (uint32_t)(n / G::STA) & 1u, &sh.abort_flag)) {
                     alive = false;
@@ -126,8 +136,8 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restr
                 ptx::tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < kRuK / 16; ++k)
-                    ptx::umma_bf16(tmem, ptx::make_desc_k_sw128(smA + a * G::A_BYTES + k * 32),
-                                   ptx::make_desc_k_sw128(smB + b * G::B_BYTES + k * 32), idesc, (uint32_t)((n | k) != 0));
+                    ptx::umma_bf16(acc, ptx::make_desc_k_sw128(smA + a * G::A_BYTES + k * 32),
+                                   ptx::make_desc_k_sw128(smB + b * G::B_BYTES + k * 32), idesc, (uint32_t)((in_run | k) != 0));
                 ptx::umma_commit(ptx::smem_u32(&sh.empty_a[a]));
                 ptx::umma_commit(ptx::smem_u32(&sh.empty_b[b]));
             }
@@ -180,23 +190,36 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restr
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.full_b[s]));
         }
-        // this CTA's sums, (s1 + s2) + s3 per expert: eight of the warps, two per TMEM lane quarter, each half of the experts
+        // this CTA's sums, (s1 + s2) + s3 per expert and accumulator: four warps per TMEM lane quarter, a quarter of the experts each
+        constexpr int EW = EP / (kRuWarps / 4);
         const int qd = warp & 3, row = qd * 32 + lane;
         const bool ok = !__any_sync(0xffffffffu, !ptx::mbar_wait(ptx::smem_u32(&sh.done), 0u, &sh.abort_flag));
-        if (ok && w < 8) {
+        if (ok) {
             ptx::tc_fence_after();
 #pragma unroll
-            for (int h = 0; h < EP / 32; ++h) {
-                const int e0 = (w >= 4 ? EP / 2 : 0) + 16 * h;
-                uint32_t a[16], b[16], g[16];
-                const uint32_t at = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)e0;
-                ptx::tmem_ld16(at, a);
-                ptx::tmem_ld16(at + EP, b);
-                ptx::tmem_ld16(at + 2 * EP, g);
-                ptx::tmem_ld_wait();
+            for (int e0 = (w >> 2) * EW, h = 0; h < EW / 8; ++h, e0 += 8) {
+                float sum[8];
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    part[row * G::LD + e0 + i] = (__uint_as_float(a[i]) + __uint_as_float(b[i])) + __uint_as_float(g[i]);
+                for (int i = 0; i < 8; ++i) sum[i] = 0.f;
+#pragma unroll
+                for (int a0 = 0; a0 < G::ACCS; a0 += 3) {        // three accumulators' reads at a time
+                    uint32_t v[3][3][8];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int g = 0; g < 3; ++g)
+                            if (a0 + a < G::ACCS)
+                                ptx::tmem_ld8(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)((a0 + a) * G::N + g * EP + e0), v[a][g]);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        if (a0 + a < G::ACCS && (a0 + a) * run < nk)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                sum[i] += (__uint_as_float(v[a][0][i]) + __uint_as_float(v[a][1][i])) + __uint_as_float(v[a][2][i]);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) part[row * G::LD + e0 + i] = sum[i];
             }
             ptx::tc_fence_before();
         }
@@ -278,28 +301,44 @@ dsmoe_status launch_clusters(const dsmoe_layer_desc& p, const CUtensorMap& mX, c
     return DSMOE_OK;
 }
 
+// How many CTAs share out a row tile's reduction over d.  With few row tiles 2 or 4, so that the launch covers most SMs;
+// `max_run` > 0 also keeps an accumulator's run of 64-wide blocks that short.  0: no such number.
 template <int EP>
-dsmoe_status launch_ep(const dsmoe_layer_desc& p, const CUtensorMap& mX, const float* Wr, const float* br, float* scores,
+int clusters_of(const dsmoe_layer_desc& p, int max_run) {
+    const int row_tiles = ceil_div(p.T, kRuM), blocks = p.d / kRuK;
+    int C = 4;
+    while (C > 1 && (row_tiles * C > sm_count() || blocks % C)) C /= 2;
+    while (max_run > 0 && ceil_div(blocks / C, RuGeo<EP>::ACCS) > max_run) {
+        C *= 2;
+        if (C > 4 || blocks % C) return 0;
+    }
+    return C;
+}
+
+template <int EP>
+dsmoe_status launch_ep(const dsmoe_layer_desc& p, int max_run, const CUtensorMap& mX, const float* Wr, const float* br, float* scores,
                        uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s) {
-    // with few row tiles the reduction over d is cut into 2 or 4 pieces, a CTA each, so that the launch covers most SMs
-    const int row_tiles = ceil_div(p.T, kRuM), sms = sm_count(), blocks = p.d / kRuK;
-    if (row_tiles * 4 <= sms && blocks % 4 == 0)
-        return launch_clusters<EP, 4>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
-    if (row_tiles * 2 <= sms && blocks % 2 == 0)
-        return launch_clusters<EP, 2>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
-    return launch_clusters<EP, 1>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+    switch (clusters_of<EP>(p, max_run)) {
+        case 4: return launch_clusters<EP, 4>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+        case 2: return launch_clusters<EP, 2>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+        case 1: return launch_clusters<EP, 1>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+        default: return DSMOE_ERR_UNSUPPORTED;
+    }
 }
 
 }  // namespace
 
-bool router_umma_supported(const dsmoe_layer_desc& p) { return umma_supported(p) && p.T > 256; }
+bool router_umma_supported(const dsmoe_layer_desc& p, int max_run) {
+    return umma_supported(p) && p.T > 256 && (p.E <= 32 ? clusters_of<32>(p, max_run) : clusters_of<64>(p, max_run)) > 0;
+}
 
 dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores,
-                                uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s, int32_t* chunk_counts) {
+                                uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s, int32_t* chunk_counts,
+                                int max_run) {
     CUtensorMap mX;
     DSMOE_TRY(cached_map_2d(&mX, x, p.T, p.d, kRuM));
-    return p.E <= 32 ? launch_ep<32>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s)
-                     : launch_ep<64>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+    return p.E <= 32 ? launch_ep<32>(p, max_run, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s)
+                     : launch_ep<64>(p, max_run, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
 }
 
 }  // namespace dsmoe
