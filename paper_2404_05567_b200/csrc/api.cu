@@ -260,7 +260,7 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
         DSMOE_TRY(launch_select(p, scores, mask, k_t, s, reinterpret_cast<int*>(ws + L.batch_k)));
     if (fast) {
         bool done = false;
-        DSMOE_TRY(launch_layer_umma(p, x, packed, scores, mask, k_t, counts_out, out, ws, L, dev_status, s, &done));
+        DSMOE_TRY(launch_layer_umma(p, x, packed, scores, counts_out, out, ws, L, dev_status, s, &done));
         if (done) return DSMOE_OK;
     }
 

@@ -236,8 +236,8 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
                                 const void* packed, float* scores, uint64_t* mask, int32_t* k_t, int32_t* counts_out,
                                 void* out, char* ws, const WsLayout& L, int32_t* dev_status, cudaStream_t s);
 dsmoe_status launch_layer_umma(const dsmoe_layer_desc& p, const void* x, const void* packed, const float* scores,
-                               const uint64_t* mask, const int32_t* k_t, int32_t* counts_out, void* out, char* ws,
-                               const WsLayout& L, int32_t* dev_status, cudaStream_t s, bool* done);
+                               int32_t* counts_out, void* out, char* ws, const WsLayout& L, int32_t* dev_status, cudaStream_t s,
+                               bool* done);
 
 // ---- training.cu / mlp_umma.cu : the training side (Eq. 2-6)
 size_t mi_scratch_bytes();
