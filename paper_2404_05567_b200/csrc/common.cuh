@@ -48,6 +48,11 @@ static inline size_t amax_of(const dsmoe_layer_desc& p) { return (size_t)p.T * (
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Every entry point's dev_status is optional: the only place that stores to it.
+__device__ __forceinline__ void report_status(int32_t* dev_status, int32_t code) {
+    if (dev_status) *dev_status = code;
+}
+
 int sm_count();
 // Grids of more than one wave are launched the ordinary way: each of their blocks would pay for its chain_wait().
 template <typename... KArgs, typename... Args>

@@ -913,9 +913,9 @@ teardown:
         if (PAIR) ptx::tmem_dealloc_pair(tmem_base, TMEM_COLS);
         else ptx::tmem_dealloc(tmem_base, TMEM_COLS);
     }
-    if (threadIdx.x == 0 && P.dev_status) {
-        if (sh.abort_flag) *P.dev_status = DSMOE_ERR_TIMEOUT;
-        else if (sh.bad_offsets) *P.dev_status = DSMOE_ERR_INVALID_ARG;
+    if (threadIdx.x == 0) {
+        if (sh.abort_flag) report_status(P.dev_status, DSMOE_ERR_TIMEOUT);
+        else if (sh.bad_offsets) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
     }
 }
 
@@ -1965,7 +1965,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
     }
     if (threadIdx.x == 0 && sh.abort_flag) {
         atomicExch(&P.sync->aborted, 1);
-        if (P.dev_status) *P.dev_status = DSMOE_ERR_TIMEOUT;
+        report_status(P.dev_status, DSMOE_ERR_TIMEOUT);
     }
 }
 

@@ -48,7 +48,7 @@ moa_attention_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restrict__
     int sq = tok_seq ? tok_seq[t] : 0, last = pos[t];
     bad = bad || sq < 0 || sq >= n_seq || last < 0 || last >= L;
     if (bad) {                                        // report, and stay inside the cache
-        if (lane == 0) *dev_status = DSMOE_ERR_INVALID_ARG;
+        if (lane == 0) report_status(dev_status, DSMOE_ERR_INVALID_ARG);
         sq = min(max(sq, 0), n_seq - 1);
         last = min(max(last, 0), L - 1);
     }
@@ -337,7 +337,7 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restri
         }
     }
     }
-    if (bad && lane == 0) *dev_status = DSMOE_ERR_INVALID_ARG;             // clamped above: nothing left the cache
+    if (bad && lane == 0) report_status(dev_status, DSMOE_ERR_INVALID_ARG);             // clamped above: nothing left the cache
     l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
     l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
     l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
     if (threadIdx.x < ng) {
         const int t = tg0 + threadIdx.x;
         const int sq = P.tok_seq ? P.tok_seq[t] : 0, last = P.pos[t];
-        if (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L) *P.dev_status = DSMOE_ERR_INVALID_ARG;
+        if (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
         seq_s[threadIdx.x] = min(max(sq, 0), P.n_seq - 1);
         last_s[threadIdx.x] = min(max(last, 0), P.L - 1);
     }

@@ -281,7 +281,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restr
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, G::TMEM);
     }
-    if (threadIdx.x == 0 && sh.abort_flag && dev_status) *dev_status = DSMOE_ERR_TIMEOUT;
+    if (threadIdx.x == 0 && sh.abort_flag) report_status(dev_status, DSMOE_ERR_TIMEOUT);
 }
 
 template <int EP, int C>

@@ -170,3 +170,35 @@ def test_moa_prompts(case):
     s, *rest = _moa_case(name, T, d, E, nh, dh, n_seq, L, layout, mode, **sel)
     e, er = _run(s, *rest, nh, 1.0 / math.sqrt(dh), sample=200)
     assert er <= TOL_BF16, (e, er)
+
+
+# One case per attention kernel: tiles that share their keys, the key-splitting and the tile-per-warp form, the plain kernel
+CLAMPED = [("clamp_prompt", 40, 64, 3, 65), ("clamp_split", 12, 64, 4, 600), ("clamp_tiles", 12, 64, 4, 90), ("clamp_plain", 20, 32, 3, 33)]
+
+
+@pytest.mark.parametrize("case", CLAMPED, ids=[c[0] for c in CLAMPED])
+def test_moa_clamps_and_reports_entries_out_of_range_with_or_without_a_status_word(case):
+    """tok_seq and pos entries beyond the cache count as the nearest one inside; dev_status is optional."""
+    name, T, dh, n_seq, L = case
+    s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos = _moa_case(name, T, 256, 8, 2, dh, n_seq, L, "mixed", gi.MODE_TOPK, K=3)
+    desc = desc_of(s)
+    packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc, to_dev(Wq), to_dev(Wo), packed)
+    ws = torch.empty(dm.dsmoe_workspace_size_packed(desc), dtype=torch.uint8, device="cuda")
+    x_d, Wr_d, br_d, K_d, V_d = (to_dev(a) for a in (x, Wr, br, Kc, Vc))
+
+    def run(seq, pos, status):
+        out = torch.empty((T, 256), dtype=torch.bfloat16, device="cuda")
+        dm.dsmoe_moa_forward(desc, 2, 0.2, K_d, V_d, to_dev(seq), to_dev(pos), x_d, Wr_d, br_d, packed, out, None, None, ws, status)
+        torch.cuda.synchronize()
+        return out
+
+    wild_seq, wild_pos = seq.copy(), pos.copy()
+    wild_seq[[1, 5]], wild_pos[[2, 7]] = (-3, n_seq + 5), (-1, L + 7)
+    inside = np.clip(wild_seq, 0, n_seq - 1), np.clip(wild_pos, 0, L - 1)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    want = run(*inside, status)
+    assert int(status.item()) == 0
+    assert torch.equal(run(wild_seq, wild_pos, status), want)
+    assert int(status.item()) == 1                                   # DSMOE_ERR_INVALID_ARG
+    assert torch.equal(run(wild_seq, wild_pos, None), want)
