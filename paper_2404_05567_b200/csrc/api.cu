@@ -42,8 +42,9 @@ WsLayout ws_layout(const dsmoe_layer_desc& p) {
     L.offsets = take((kMaxExperts + 1) * 4);
     L.chunk_prefix = take((size_t)ceil_div(p.T, kChunk) * E * 4);
     L.batch_k = take(256);               // Threshold-TopK: the batch's K
+    L.sync = take(64);                   // grid-barrier counters of the small-T kernel
     L.tile_done = take((size_t)kMaxExperts * ceil_div(p.d, 256) * 4);   // grouped down-projection: finished tiles per (expert, column range)
-    L.mi = take(mi_scratch_bytes());     // mutual-information loss: per-block partial sums; small-T kernel: its grid barriers
+    L.mi = take(mi_scratch_bytes());     // mutual-information loss: per-block partial sums
     L.row_token = take(amax * 4);
     L.row_gate = take(amax * 4);
     L.token_rows = take(T * (size_t)width_of(p) * 4);

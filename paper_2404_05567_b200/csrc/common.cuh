@@ -15,7 +15,6 @@ constexpr int kMaxExperts = 64;
 constexpr int kChunk = 32;   // tokens per ballot chunk in the grouping kernels
 constexpr int kSmallMaxT = 128;      // the small-T (decode) path keeps all tokens in one 128-row MMA tile
 constexpr int kSmallMaxCtas = 192;   // upper bound on that path's grid (sizes its partial-sum buffer)
-constexpr int kSmallSyncBytes = 2048;   // its grid barriers, in the mutual-information loss's scratch
 
 #define DSMOE_CUDA_TRY(expr)                                  \
     do {                                                      \
@@ -98,7 +97,7 @@ static inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; 
 //                              sum of the expert outputs), partial (small-T)
 // total_packed = bytes a call with packed weights needs; total = the maximum over both kinds of call.
 struct WsLayout {
-    size_t scores, mask, k_t, counts, offsets, chunk_prefix, batch_k, tile_done, mi, row_token, row_gate, token_rows;
+    size_t scores, mask, k_t, counts, offsets, chunk_prefix, batch_k, sync, tile_done, mi, row_token, row_gate, token_rows;
     size_t stage_total;
     size_t xp, h_plain, yp;                 // plain path
     size_t h, acc, partial, bwd;            // tensor-core paths

@@ -15,8 +15,6 @@
 //               Eq. 1 folded into the reduction dimension, so no grouping and no aggregation pass
 // small_layer_kernel: the whole layer for a handful of tokens (decode) in one cooperative launch.
 #include <algorithm>
-#include <atomic>
-#include <chrono>
 #include <climits>
 #include <cstdlib>
 
@@ -955,85 +953,28 @@ struct SmallParams {
     float* partial;          // [grid][2][T][256]; doubles as the router's slice buffer
     void* out;
     int out_f32;
-    struct SmallSync* sync;      // grid barriers; any contents at launch
-    unsigned long long nonce;    // this call's
+    int* sync;               // 8 ints, zero at launch: barrier counters [0..2] and an abort flag [4]
     int spec;                // start streaming under "every expert selected" before the router has finished
     int32_t* dev_status;
 };
 
-// Grid barriers.  The second and third are counters that one thread per CTA adds to and waits for; CTA 0 zeroes them before it
-// arrives at the first.  The first needs nothing of the workspace's contents: a CTA arrives by writing the call's nonce -- a
-// 64-bit number that no other call of the process has -- to its own flag; a warp of the last CTA, which has the least to do in the
-// router, reads all the flags (at most 6 a lane) until they hold it and passes the nonce on in one word that the others wait
-// for.  So the call needs no memset before the kernel (1 us, and two launch gaps of 2 us instead
-// of one).  A call that is replayed from a graph comes back with the same nonce: flags and word are taken back behind the last
-// barrier, when every CTA has long seen them.
-struct SmallSync {
-    unsigned long long flag[kSmallMaxCtas];
-    unsigned long long all_here, pad[15];    // on a line of its own
-    int counter[2];                          // the second and third barrier's
-    int aborted;
-};
-static_assert(sizeof(SmallSync) <= kSmallSyncBytes, "its place in the workspace");
-
-__device__ __forceinline__ void first_arrive(const SmallParams& P) {              // one thread
-    if (blockIdx.x == 0) P.sync->counter[0] = P.sync->counter[1] = P.sync->aborted = 0;
+// One thread per CTA arrives at grid barrier `idx`; grid_wait spins (bounded) until all CTAs have.
+__device__ __forceinline__ void grid_arrive(int* sync, int idx) {
     __threadfence();
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(P.sync->flag + blockIdx.x), "l"(P.nonce) : "memory");
+    atomicAdd(sync + idx, 1);
 }
-// A whole warp; false = gave up
-__device__ __forceinline__ bool first_wait(const SmallParams& P, int lane, volatile int* abort_flag) {
-    const uint64_t t0 = ptx::globaltimer_ns();
-    const bool last = blockIdx.x == gridDim.x - 1;
-    for (uint32_t spin = 1;; ++spin) {
-        if (!last) {
-            unsigned long long w = 0;
-            if (lane == 0) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(&P.sync->all_here) : "memory");
-            if (__shfl_sync(0xffffffffu, w, 0) == P.nonce) return true;
-            if ((spin & 0x3f) == 0 && __any_sync(0xffffffffu, *abort_flag || ptx::globaltimer_ns() - t0 > ptx::kWaitLimitNs)) {
-                *abort_flag = 1;
-                return false;
-            }
-            continue;
-        }
-        unsigned long long v[kSmallMaxCtas / 32];         // relaxed loads, all under way together; one fence once they agree
-#pragma unroll
-        for (int i = 0; i < kSmallMaxCtas / 32; ++i) {
-            v[i] = P.nonce;
-            if (lane + 32 * i < (int)gridDim.x)
-                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[i]) : "l"(P.sync->flag + lane + 32 * i) : "memory");
-        }
-        bool all = true;
-#pragma unroll
-        for (int i = 0; i < kSmallMaxCtas / 32; ++i) all = all && v[i] == P.nonce;
-        if (__all_sync(0xffffffffu, all)) {
-            __threadfence();
-            if (lane == 0) asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&P.sync->all_here), "l"(P.nonce) : "memory");
-            return true;
-        }
-        if ((spin & 0x3f) == 0 && __any_sync(0xffffffffu, *abort_flag || ptx::globaltimer_ns() - t0 > ptx::kWaitLimitNs)) {
-            *abort_flag = 1;
-            return false;
-        }
-    }
-}
-// One thread per CTA arrives at barrier `idx` (0: the second, 1: the third); grid_wait spins (bounded) until all CTAs have.
-__device__ __forceinline__ void grid_arrive(SmallSync* sync, int idx) {
-    __threadfence();
-    atomicAdd(sync->counter + idx, 1);
-}
-__device__ __forceinline__ bool grid_wait(SmallSync* sync, int idx, int target, volatile int* abort_flag) {
+__device__ __forceinline__ bool grid_wait(int* sync, int idx, int target, volatile int* abort_flag) {
     const uint64_t t0 = ptx::globaltimer_ns();
     for (uint32_t spin = 0;; ++spin) {
         int v;
-        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(sync->counter + idx) : "memory");
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(sync + idx) : "memory");
         if (v >= target) return true;
         if ((spin & 0x3f) == 0x3f) {
             int ab;
-            asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(ab) : "l"(&sync->aborted) : "memory");
+            asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(ab) : "l"(sync + 4) : "memory");
             if (ab || *abort_flag || ptx::globaltimer_ns() - t0 > ptx::kWaitLimitNs) {
                 *abort_flag = 1;
-                atomicExch(&sync->aborted, 1);
+                atomicExch(sync + 4, 1);
                 return false;
             }
         }
@@ -1472,7 +1413,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
                 }
             }
             TRACE(5);
-            if (alive && !grid_wait(P.sync, 0, G, &sh.abort_flag)) alive = false;
+            if (alive && !grid_wait(P.sync, 1, G, &sh.abort_flag)) alive = false;
             TRACE(6);
             asm volatile("fence.proxy.async;" ::: "memory");   // hg was written through the generic proxy, TMA reads it
             for (int j = 0; alive && j < npend; ++j) {
@@ -1728,13 +1669,11 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
             softmax_select_store<false>(l_lo, l_hi, (int)blockIdx.x, P.sel, lane, P.scores, P.mask, P.k_t);
         }
         EPI_SYNC();
-        if (warp == 2) {
-            if (lane == 0) {
-                TRACE(1);
-                first_arrive(P);
-            }
-            first_wait(P, lane, &sh.abort_flag);
-            if (lane == 0) TRACE(14);
+        if (etid == 0) {
+            TRACE(1);
+            grid_arrive(P.sync, 0);
+            grid_wait(P.sync, 0, G, &sh.abort_flag);
+            TRACE(14);
         }
         EPI_SYNC();
         // ---- router, step 2: softmax and selection of every token, in every CTA (see small_router_pass)
@@ -1785,7 +1724,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
                 asm volatile("fence.proxy.async;" ::: "memory");
                 EPI_SYNC();
                 if (etid == 0) {
-                    grid_arrive(P.sync, 0);
+                    grid_arrive(P.sync, 1);
                     sh.up_arrived = 1;
                     TRACE(7);
                 }
@@ -1882,8 +1821,8 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         EPI_SYNC();
         if (etid == 0) {
             TRACE(9);
-            grid_arrive(P.sync, 1);
-            if (!grid_wait(P.sync, 1, G, &sh.abort_flag)) sh.abort_flag = 1;
+            grid_arrive(P.sync, 2);
+            if (!grid_wait(P.sync, 2, G, &sh.abort_flag)) sh.abort_flag = 1;
             TRACE(10);
         }
         EPI_SYNC();
@@ -1959,12 +1898,8 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         for (int i = 0; i < 32; ++i) g_trace[blockIdx.x][i] = sh.trace[i];
     }
 #endif
-    if (threadIdx.x == 0) {
-        P.sync->flag[blockIdx.x] = 0;      // taken back: see the barriers
-        if (blockIdx.x == 0) P.sync->all_here = 0;
-    }
     if (threadIdx.x == 0 && sh.abort_flag) {
-        atomicExch(&P.sync->aborted, 1);
+        atomicExch(P.sync + 4, 1);
         report_status(P.dev_status, DSMOE_ERR_TIMEOUT);
     }
 }
@@ -2181,17 +2116,6 @@ bool small_supported(const dsmoe_layer_desc& p) {
     return KS * ceil_div(p.T, kEpiThreads / 32) <= 16;
 }
 
-// A number that no other call of this process gets (a counter through a bijection, splitmix64's) and that a stale buffer
-// of another process will hardly hold (the counter starts at the clock)
-unsigned long long small_nonce() {
-    static std::atomic<unsigned long long> next{(unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count()};
-    unsigned long long z = next.fetch_add(1) * 0x9e3779b97f4a7c15ull;
-    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    z ^= z >> 31;
-    return z ? z : 1ull;
-}
-
 dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
                                 const void* packed, float* scores, uint64_t* mask, int32_t* k_t, int32_t* counts_out,
                                 void* out, char* ws, const WsLayout& L, int32_t* dev_status, cudaStream_t s) {
@@ -2227,12 +2151,12 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     P.partial = reinterpret_cast<float*>(ws + L.partial);
     P.out = out;
     P.out_f32 = p.out_fp32 ? 1 : 0;
-    P.sync = reinterpret_cast<SmallSync*>(ws + L.mi);      // (the loss's scratch: idle in a forward call)
-    P.nonce = small_nonce();
+    P.sync = reinterpret_cast<int*>(ws + L.sync);
     P.dev_status = dev_status;
     // From kSpecMinT tokens on it is rare that an expert is selected by none of them, so the kernel starts the
     // up-projection under that assumption while its router is still running; it starts over if the router disagrees.
     P.spec = p.T >= kSpecMinT ? 1 : 0;
+    DSMOE_CUDA_TRY(cudaMemsetAsync(P.sync, 0, 32, s));
     void* args[] = {&mX, &mW1, &mHg, &mW2, &P};
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));

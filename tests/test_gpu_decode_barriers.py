@@ -1,6 +1,6 @@
-"""The decode kernel's grid barriers need nothing of the workspace's contents and take part in graphs: calls on workspaces filled
-with any bytes, replays of one captured call (the same nonce again and again), and calls on two streams with a workspace each
-all give the bits of a plain call (GPU required)."""
+"""A decode call prepares its grid barriers itself: calls on workspaces filled with any bytes, replays of one captured call with
+plain calls on the same workspace in between, and calls on two streams with a workspace each all give the bits of a plain
+call (GPU required)."""
 import pytest
 import torch
 
@@ -37,7 +37,7 @@ def test_decode_calls_on_any_workspace_contents_and_replayed(T):
         x.copy_(L.x_d if i % 2 else other.x_d)
         graph.replay()
         if i % 5 == 0:
-            call(L.x_d, L.out, L.ws)                       # another nonce on the same workspace in between
+            call(L.x_d, L.out, L.ws)                       # a plain call on the same workspace in between
         assert torch.equal(out, want if i % 2 else want_other), i
     torch.cuda.synchronize()
     assert int(L.dev_status.item()) == 0
