@@ -44,6 +44,9 @@ static inline size_t amax_of(const dsmoe_layer_desc& p) { return (size_t)p.T * (
 // kernels before it have completed and their writes are visible -- and chain_next() to let its own successor be set up: short kernels at
 // once, long ones when their last loads are under way (blocks that wait beside a long kernel slow it down: with
 // chain_next() at its start the gradients of dense training took 2067 instead of 1989 us).
+// Such a kernel runs while its inputs are still being written, so it reads them with ordinary loads only: ld.global.nc (__ldg,
+// or what the compiler makes of a `const T* __restrict__` parameter) is for data that nothing writes during the whole kernel,
+// and as such may be served from a stale line or be moved above the wait.  No parameter that is only read is __restrict__.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -43,9 +43,9 @@ __device__ __forceinline__ void st_out4(__nv_bfloat16* p, float4 v) {
 }
 
 template <typename AT, typename BT, typename OT, bool GELU, int TM, int TN>
-__global__ void __launch_bounds__(256) grouped_gemm_fma_kernel(const AT* __restrict__ A, const int32_t* __restrict__ gather,
-                                                               int gather_rows, const BT* __restrict__ B, OT* __restrict__ C,
-                                                               const int32_t* __restrict__ offsets, int E, int K, int N,
+__global__ void __launch_bounds__(256) grouped_gemm_fma_kernel(const AT* A, const int32_t* gather,
+                                                               int gather_rows, const BT* B, OT* __restrict__ C,
+                                                               const int32_t* offsets, int E, int K, int N,
                                                                int64_t amax, int bufs) {
     chain_wait();
     using Geo = FmaGeo<TM, TN>;

@@ -772,7 +772,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const int rl = i * 8 + rr;
                         uint4 v = make_uint4(0, 0, 0, 0);
                         if (q * 32 + rl < t.rows_valid)
-                            v = __ldg(reinterpret_cast<const uint4*>(act + ((long long)t.row0 + q * 32 + rl) * P.ld_out + t.out_col0 + c + cc * 8));
+                            v = *reinterpret_cast<const uint4*>(act + ((long long)t.row0 + q * 32 + rl) * P.ld_out + t.out_col0 + c + cc * 8);
                         *reinterpret_cast<uint4*>(ta + rl * LDB + 16 * cc) = v;
                     }
                     uint32_t r[32];
@@ -1993,8 +1993,8 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
 
 // out[r,:] (bf16) = the sum over the splits, in ascending order, of the fp32 partial rows part[s * split_rows + r,:]
 // that a launch with k_splits left behind; rows from offsets[E] on do not exist
-__global__ void __launch_bounds__(256) split_sum_kernel(const float4* __restrict__ part, int splits, int split_rows,
-                                                        const int32_t* __restrict__ offsets, int E, int n,
+__global__ void __launch_bounds__(256) split_sum_kernel(const float4* part, int splits, int split_rows,
+                                                        const int32_t* offsets, int E, int n,
                                                         __nv_bfloat16* __restrict__ out) {
     chain_next();
     chain_wait();
@@ -2212,7 +2212,7 @@ dsmoe_status launch_layer_umma(const dsmoe_layer_desc& p, const void* x, const v
 }
 
 // dS[t,e] = the column tiles' partial sums added in ascending order
-__global__ void __launch_bounds__(256) bwd_finish_kernel(const float* __restrict__ part, float* __restrict__ dS, long long n,
+__global__ void __launch_bounds__(256) bwd_finish_kernel(const float* part, float* __restrict__ dS, long long n,
                                                          int ntn) {
     chain_next();
     chain_wait();

@@ -27,9 +27,9 @@ __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u 
 // query in place (the warp has read all of it before it writes).
 template <int DPL>   // d_head / 32
 __global__ void __launch_bounds__(32 * kMoaWarps)
-moa_attention_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restrict__ row_token, const int32_t* __restrict__ offsets,
-                     int E, int n_head, int H, int T, const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __restrict__ Vc,
-                     const int32_t* __restrict__ tok_seq, const int32_t* __restrict__ pos, int n_seq, int L, float scale,
+moa_attention_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* row_token, const int32_t* offsets,
+                     int E, int n_head, int H, int T, const __nv_bfloat16* Kc, const __nv_bfloat16* Vc,
+                     const int32_t* tok_seq, const int32_t* pos, int n_seq, int L, float scale,
                      int* __restrict__ dev_status) {
     chain_wait();
     constexpr int DH = 32 * DPL;
@@ -64,7 +64,7 @@ moa_attention_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restrict__
         float dot = 0.f;
 #pragma unroll
         for (int c = 0; c < DH / 8; ++c) {
-            const uint4 u = __ldg(kr + c);
+            const uint4 u = kr[c];
             const float4 q0 = *reinterpret_cast<const float4*>(qs + 8 * c), q1 = *reinterpret_cast<const float4*>(qs + 8 * c + 4);
             dot = fmaf(q0.x, bf16_lo(u.x), dot);
             dot = fmaf(q0.y, bf16_hi(u.x), dot);
@@ -132,10 +132,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 
 template <int DH, int kMmaWarps>      // long caches: 8 warps share out the keys; short ones: 2, and several CTAs fit an SM
 __global__ void __launch_bounds__(32 * kMmaWarps, kMmaWarps == 2 ? DSMOE_MOA_MINBLOCKS : 1)
-moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* __restrict__ token_rows, int W, int row_tiles,
-                         int tpt, long long amax, int n_head, int H, int T, const __nv_bfloat16* __restrict__ Kc,
-                         const __nv_bfloat16* __restrict__ Vc, const int32_t* __restrict__ tok_seq,
-                         const int32_t* __restrict__ pos, int n_seq, int L, float scale, long long n_tiles,
+moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* token_rows, int W, int row_tiles,
+                         int tpt, long long amax, int n_head, int H, int T, const __nv_bfloat16* Kc,
+                         const __nv_bfloat16* Vc, const int32_t* tok_seq,
+                         const int32_t* pos, int n_seq, int L, float scale, long long n_tiles,
                          int* __restrict__ dev_status) {
     chain_wait();
     constexpr int STRIDE = DH * 2 + 16;                 // bytes per key row in shared memory: 16 of padding

@@ -23,10 +23,10 @@ namespace dsmoe {
 constexpr int kCountInBlockChunks = 8;
 constexpr int kPermThreads = 512, kPermChunks = 4, kPermTokens = kPermChunks * kChunk / (kPermThreads / 32);
 template <int SCAN>
-__global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint64_t* __restrict__ mask,
-                                                            const float* __restrict__ scores,
-                                                            int32_t* __restrict__ offsets,
-                                                            const int32_t* __restrict__ chunk_prefix,
+__global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint64_t* mask,
+                                                            const float* scores,
+                                                            int32_t* offsets,
+                                                            const int32_t* chunk_prefix,
                                                             int32_t* __restrict__ counts, int32_t* __restrict__ counts_out,
                                                             int32_t* __restrict__ row_token, float* __restrict__ row_gate,
                                                             int32_t* __restrict__ token_rows, int T, int E, int W,
@@ -47,8 +47,8 @@ __global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint6
 #pragma unroll
     for (int i = 0; i < kPermTokens; ++i) {
         const float* src = scores + (size_t)(t0 + i) * E;
-        s_lo[i] = t0 + i < T && e_lo ? __ldg(src + lane) : 0.f;
-        s_hi[i] = t0 + i < T && e_hi ? __ldg(src + lane + 32) : 0.f;
+        s_lo[i] = t0 + i < T && e_lo ? src[lane] : 0.f;
+        s_hi[i] = t0 + i < T && e_hi ? src[lane + 32] : 0.f;
     }
     if (tid < kPermChunks * kChunk) mask_s[tid] = c0 * kChunk + tid < T ? mask[c0 * kChunk + tid] : 0;
     if (SCAN) {
@@ -188,8 +188,8 @@ __global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint6
 }
 
 // xp[r,:] = x[row_token[r],:] for r < A, 16 bytes per lane per step, one warp per row.
-__global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ row_token,
-                                                          const int32_t* __restrict__ offsets, uint4* __restrict__ xp,
+__global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* x, const int32_t* row_token,
+                                                          const int32_t* offsets, uint4* __restrict__ xp,
                                                           int E, int T, int vec_per_row, int64_t amax) {
     chain_next();
     chain_wait();
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restric
         if ((unsigned)t >= (unsigned)T) continue;   // never trust an index blindly
         const uint4* src = x + (size_t)t * vec_per_row;
         uint4* dst = xp + (size_t)r * vec_per_row;
-        for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
+        for (int v = lane; v < vec_per_row; v += 32) dst[v] = src[v];
     }
 }
 
@@ -217,9 +217,9 @@ __device__ __forceinline__ void fma8(float (&acc)[8], const uint4 v, float g) {
 
 // out[t,:] = sum_i gate[r_i] * yp[r_i,:] in ascending expert order, fp32, one rounding.  Block per token.
 template <bool OUT_F32>
-__global__ void __launch_bounds__(128) combine_bf16_kernel(const uint4* __restrict__ yp, const float* __restrict__ row_gate,
-                                                           const int32_t* __restrict__ token_rows,
-                                                           const int32_t* __restrict__ k_t, void* __restrict__ out,
+__global__ void __launch_bounds__(128) combine_bf16_kernel(const uint4* yp, const float* row_gate,
+                                                           const int32_t* token_rows,
+                                                           const int32_t* k_t, void* __restrict__ out,
                                                            int d, int W, int64_t amax) {
     chain_next();
     chain_wait();
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(128) combine_bf16_kernel(const uint4* __restri
         for (int i = 0; i < k; i += 4) {
             uint4 y[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) y[j] = __ldg(yp + (size_t)rows_s[i + j < k ? i + j : 0] * nvec + v);
+            for (int j = 0; j < 4; ++j) y[j] = yp[(size_t)rows_s[i + j < k ? i + j : 0] * nvec + v];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (i + j < k) fma8(acc, y[j], gate_s[i + j]);
@@ -265,9 +265,9 @@ __global__ void __launch_bounds__(128) combine_bf16_kernel(const uint4* __restri
 // fp32 rows: the plain path's fp32 layers (gates applied here) and the tensor-core path's gate-weighted fp32 expert
 // outputs (row_gate == NULL: only the sum is left to do; the output may be bf16)
 template <bool OUT_BF16>
-__global__ void __launch_bounds__(128) combine_f32_kernel(const float4* __restrict__ yp, const float* __restrict__ row_gate,
-                                                          const int32_t* __restrict__ token_rows,
-                                                          const int32_t* __restrict__ k_t, void* __restrict__ out,
+__global__ void __launch_bounds__(128) combine_f32_kernel(const float4* yp, const float* row_gate,
+                                                          const int32_t* token_rows,
+                                                          const int32_t* k_t, void* __restrict__ out,
                                                           int d, int W, int64_t amax) {
     chain_next();
     chain_wait();
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float4* __restri
         for (int i = 0; i < k; i += 4) {
             float4 y[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) y[j] = __ldg(yp + (size_t)rows_s[i + j < k ? i + j : 0] * nvec + v);
+            for (int j = 0; j < 4; ++j) y[j] = yp[(size_t)rows_s[i + j < k ? i + j : 0] * nvec + v];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if (i + j >= k) continue;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float4* __restri
 
 // Packing of a batch of [rows = reduction, cols = outputs] bf16 matrices: dst[b][r / 64][c][r % 64] = src[b][r][c]
 // (32x32 tiles through smem; rows is a multiple of 64 where this layout is used).
-__global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16* __restrict__ src,
+__global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16* src,
                                                              __nv_bfloat16* __restrict__ dst, int rows, int cols) {
     chain_next();
     chain_wait();
@@ -407,7 +407,7 @@ dsmoe_status launch_combine(const dsmoe_layer_desc& p, const void* yp, const flo
 }
 
 // Selection statistics.  One warp per token; integer atomics only, so the counts do not depend on the order.
-__global__ void __launch_bounds__(256) stats_kernel(const float* __restrict__ scores, const uint64_t* __restrict__ mask,
+__global__ void __launch_bounds__(256) stats_kernel(const float* scores, const uint64_t* mask,
                                                     dsmoe_selection_stats* __restrict__ st, int T, int E, int mode, float eps,
                                                     int eps_normalized) {
     chain_next();

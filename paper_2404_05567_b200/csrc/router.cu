@@ -18,8 +18,8 @@ static SelParams sel_params(const dsmoe_layer_desc& p) {
 // every block reads in full out of L2), the reduction over d split across all 256 threads.  A token's sums are formed
 // in the same order whatever TT is.
 template <typename XT, int EP, int TT>
-__global__ void __launch_bounds__(256) router_small_kernel(const XT* __restrict__ x, const float* __restrict__ Wr,
-                                                           const float* __restrict__ br, float* __restrict__ scores,
+__global__ void __launch_bounds__(256) router_small_kernel(const XT* x, const float* Wr,
+                                                           const float* br, float* __restrict__ scores,
                                                            uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
                                                            int T, int d, SelParams q) {
     chain_next();
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) router_small_kernel(const XT* __restrict_
 #pragma unroll
             for (int e4 = 0; e4 < EP / 4; ++e4) {
                 if (e4 * 4 < E) {
-                    const float4 wv = __ldg(w + e4);
+                    const float4 wv = w[e4];
 #pragma unroll
                     for (int u = 0; u < TT; ++u) {
                         acc[u][e4 * 4 + 0] = fmaf(xv[u], wv.x, acc[u][e4 * 4 + 0]);
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) router_small_kernel(const XT* __restrict_
 #pragma unroll
             for (int e = 0; e < EP; ++e) {
                 if (e < E) {
-                    const float wv = __ldg(w + e);
+                    const float wv = w[e];
 #pragma unroll
                     for (int u = 0; u < TT; ++u) acc[u][e] = fmaf(xv[u], wv, acc[u][e]);
                 }
@@ -109,7 +109,7 @@ __device__ __forceinline__ void load8_as_f32(const XT* p, bool vec, int nvalid, 
 template <>
 __device__ __forceinline__ void load8_as_f32<__nv_bfloat16>(const __nv_bfloat16* p, bool vec, int nvalid, float (&out)[8]) {
     if (vec && nvalid == 8) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+        const uint4 v = *reinterpret_cast<const uint4*>(p);
         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -125,7 +125,7 @@ __device__ __forceinline__ void load8_as_f32<__nv_bfloat16>(const __nv_bfloat16*
 template <>
 __device__ __forceinline__ void load8_as_f32<float>(const float* p, bool vec, int nvalid, float (&out)[8]) {
     if (vec && nvalid == 8) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+        const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
         out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
         out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
     } else {
@@ -144,8 +144,8 @@ constexpr size_t router_tile_smem() {
 // tile per thread in each group), so that every scheduler has 8 warps to hide the FMA and shared-memory latencies
 // behind.  The groups' partial sums meet in shared memory at the end and are added in group order.
 template <typename XT, int EPL>
-__global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* __restrict__ x, const float* __restrict__ Wr,
-                                                                    const float* __restrict__ br, float* __restrict__ scores,
+__global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* x, const float* Wr,
+                                                                    const float* br, float* __restrict__ scores,
                                                                     uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
                                                                     int T, int d, SelParams q) {
     chain_wait();
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* __
 #pragma unroll
         for (int i = 0; i < NW; ++i) {
             const int idx = tid + i * NT, kk = idx / EP, e = idx % EP;
-            wreg[i] = (e < E && k0 + kk < d) ? __ldg(Wr + (size_t)(k0 + kk) * E + e) : 0.f;
+            wreg[i] = (e < E && k0 + kk < d) ? Wr[(size_t)(k0 + kk) * E + e] : 0.f;
         }
     };
     auto stash = [&](int b) {
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* __
 }
 
 // Selection alone on caller-supplied scores: one warp per token.
-__global__ void __launch_bounds__(256) select_kernel(const float* __restrict__ scores, uint64_t* __restrict__ mask,
+__global__ void __launch_bounds__(256) select_kernel(const float* scores, uint64_t* __restrict__ mask,
                                                      int32_t* __restrict__ k_t, int T, SelParams q) {
     chain_next();
     chain_wait();
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(256) select_kernel(const float* __restrict__ s
 // chunk_count_kernel, one warp per chunk (lane = token, one ballot per expert), leaves the chunk's counts in
 // chunk_prefix[c,:]; finalize_kernel, one block, turns them into exclusive prefixes over the chunks (warp e scans
 // expert e, 32 chunks per warp-wide scan) and writes the totals and their offsets.
-__global__ void __launch_bounds__(256) chunk_count_kernel(const uint64_t* __restrict__ mask, int32_t* __restrict__ chunk_prefix,
+__global__ void __launch_bounds__(256) chunk_count_kernel(const uint64_t* mask, int32_t* __restrict__ chunk_prefix,
                                                           int T, int E) {
     chain_next();
     chain_wait();
@@ -411,7 +411,7 @@ dsmoe_status launch_router(const dsmoe_layer_desc& p, const void* x, const float
 // Threshold-TopK ("Expert Sampling Strategy" paragraph): K = the batch average of the per-token counts that the
 // threshold gave, rounded half up and kept within [1, E].  One block; integer sums, so the result does not depend
 // on the order of the additions.
-__global__ void __launch_bounds__(1024) batch_k_kernel(const int32_t* __restrict__ k_t, int T, int E, int* __restrict__ K_out) {
+__global__ void __launch_bounds__(1024) batch_k_kernel(const int32_t* k_t, int T, int E, int* __restrict__ K_out) {
     chain_next();
     chain_wait();
     __shared__ long long part[32];

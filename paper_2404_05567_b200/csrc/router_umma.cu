@@ -62,7 +62,7 @@ __device__ __forceinline__ float ld_cluster(uint32_t addr) {
 
 template <int EP, int C>
 __global__ void __launch_bounds__(kRuThreads, 1)
-router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restrict__ Wr, const float* __restrict__ br,
+router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, const float* br,
                    float* __restrict__ scores, uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
                    int32_t* __restrict__ chunk_counts, int T, int d, const SelParams q, int32_t* __restrict__ dev_status) {
     using G = RuGeo<EP>;
@@ -155,7 +155,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restr
                 const float* src = Wr + (size_t)((kb0 + n) * kRuK + c0 * 8) * q.E + e;
                 float v[8 * PC];
 #pragma unroll
-                for (int i = 0; i < 8 * PC; ++i) v[i] = e < q.E ? __ldg(src + (size_t)i * q.E) : 0.f;
+                for (int i = 0; i < 8 * PC; ++i) v[i] = e < q.E ? src[(size_t)i * q.E] : 0.f;
                 if (h == 0 && !ptx::mbar_wait(ptx::smem_u32(&sh.empty_b[s]), ((uint32_t)(n / G::STB) & 1u) ^ 1u, &sh.abort_flag)) {
                     alive = false;
                     break;

@@ -11,7 +11,7 @@ constexpr int kMiBlocks = 296;        // upper bound on the first stage's grid (
 // Stage 1: block b adds its tokens' scores per expert and their conditional entropies, in double, in a fixed order
 // (warp w of the block takes tokens w, w + 8, ...; lanes hold experts lane and lane + 32; the warps' sums meet in shared
 // memory and are added in warp order).  part[b][0..E) = sum_t S[t,e], part[b][64] = sum_t H(e|X_t).
-__global__ void __launch_bounds__(256) mi_partial_kernel(const float* __restrict__ S, double* __restrict__ part, int T, int E) {
+__global__ void __launch_bounds__(256) mi_partial_kernel(const float* S, double* __restrict__ part, int T, int E) {
     chain_next();
     chain_wait();
     __shared__ double red[8][kMaxExperts + 1];
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) mi_partial_kernel(const float* __restrict
 // more than 37 blocks' sums (one thread per expert and one for the entropies walked all 296: 11 of the loss's 22 us).  The parts
 // are added in order: the order is fixed.
 constexpr int kMiParts = 8;
-__global__ void __launch_bounds__(kMaxExperts * kMiParts + 32) mi_finish_kernel(const double* __restrict__ part, int nblocks, int T, int E,
+__global__ void __launch_bounds__(kMaxExperts * kMiParts + 32) mi_finish_kernel(const double* part, int nblocks, int T, int E,
                                                        float* __restrict__ out3, double* __restrict__ pe) {
     chain_next();
     chain_wait();
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kMaxExperts * kMiParts + 32) mi_finish_kernel(
 }
 
 // dL_MI/dS[t,e] = (log p(e) - log S[t,e]) / T   (0 where the score is 0)
-__global__ void __launch_bounds__(256) mi_grad_kernel(const float* __restrict__ S, const double* __restrict__ pe,
+__global__ void __launch_bounds__(256) mi_grad_kernel(const float* S, const double* pe,
                                                       float* __restrict__ grad, long long n, int T, int E) {
     chain_next();
     chain_wait();
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256) mi_grad_kernel(const float* __restrict__ 
     grad[i] = s > 0.f ? (float)((log(pe[i % E]) - log((double)s)) / (double)T) : 0.f;
 }
 
-__device__ __forceinline__ float ldv(const float* p) { return __ldg(p); }
+__device__ __forceinline__ float ldv(const float* p) { return *p; }
 __device__ __forceinline__ float ldv(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 __device__ __forceinline__ void stv(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stv(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
@@ -110,9 +110,9 @@ __device__ __forceinline__ void stv(__nv_bfloat16* p, float v) { *p = __float2bf
 // activation a_k = GeLU(x.W1[e][:,k]) and G_k = dO.W2[e][k,:], writes dA = S * G_k and adds a_k * G_k to the block's
 // dot product, which is <e_e(x), dO>.
 template <typename XT>
-__global__ void __launch_bounds__(256) dense_backward_plain_kernel(const XT* __restrict__ x, const XT* __restrict__ W1,
-                                                                   const XT* __restrict__ W2, const float* __restrict__ S,
-                                                                   const uint64_t* __restrict__ mask, const XT* __restrict__ dO,
+__global__ void __launch_bounds__(256) dense_backward_plain_kernel(const XT* x, const XT* W1,
+                                                                   const XT* W2, const float* S,
+                                                                   const uint64_t* mask, const XT* dO,
                                                                    float* __restrict__ dS, XT* __restrict__ dA, int d, int H, int E) {
     chain_wait();
     __shared__ float red[8];
