@@ -117,6 +117,8 @@ dsmoe_status dsmoe_workspace_size_stages(const dsmoe_layer_desc* desc, size_t* b
  * Router scores, Eq. 1 (first half): scores[t,:] = softmax(x[t,:].Wr + br) over all E
  * experts, fp32 with the row maximum subtracted.
  *   x [T,d] dtype; Wr [d,E] fp32; br [E] fp32 or NULL; scores [T,E] fp32 (written).
+ *   The tensor-core kernel (bf16, T > 256) has bounded waits.  Should one run out, the scores of the
+ *   tokens concerned are NaN: this call has no dev_status to report it through.
  */
 dsmoe_status dsmoe_router(const dsmoe_layer_desc* desc, const void* x, const float* Wr,
                           const float* br, float* scores, dsmoe_stream stream);

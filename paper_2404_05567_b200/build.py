@@ -73,5 +73,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_variant(name: str, source: str, flags) -> str:
+    """A second library for the tests: the built one with csrc/``source`` compiled with additional ``flags``."""
+    build()
+    lib, obj, src = (os.path.join(OBJ, f"libdsmoe_{name}.so"), os.path.join(OBJ, f"{name}.variant.o"), os.path.join(CSRC, source))
+    others = [os.path.join(OBJ, os.path.basename(p)[:-3] + ".o") for p in sorted(glob.glob(os.path.join(CSRC, "*.cu"))) if p != src]
+    if _stale(lib, [src, *others]):
+        subprocess.run([_nvcc(), *NVCC_FLAGS, *flags, "-c", src, "-o", obj], check=True)
+        subprocess.run([_nvcc(), "-shared", "-o", lib, obj, *others, "-Xcompiler", "-fPIC"], check=True)
+    return lib
+
+
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))

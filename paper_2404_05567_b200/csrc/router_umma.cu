@@ -87,7 +87,11 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
             ptx::mbar_init(ptx::smem_u32(&sh.empty_b[s]), 1);
         }
         ptx::mbar_init(ptx::smem_u32(&sh.done), 1);
+#ifdef DSMOE_TEST_GIVE_UP_RANK      // a build for the tests: this rank's CTAs behave as if a wait had run out
+        sh.abort_flag = rank == DSMOE_TEST_GIVE_UP_RANK;
+#else
         sh.abort_flag = 0;
+#endif
         ptx::fence_barrier_init();
         ptx::prefetch_tensormap(&tmX);
     }
@@ -110,11 +114,6 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
                 const uint32_t bar = ptx::smem_u32(&sh.full_a[s]);
                 ptx::mbar_expect_tx(bar, G::A_BYTES);
                 ptx::tma_load_2d(smA + s * G::A_BYTES, &tmX, bar, (kb0 + n) * kRuK, tile * kRuM);
-            }
-            if (sh.abort_flag) {                      // copies already issued still land in this CTA's shared memory
-                const uint64_t t0 = ptx::globaltimer_ns();
-                while (ptx::globaltimer_ns() - t0 < 200000ull) {
-                }
             }
         }
     } else if (warp == 1) {
@@ -225,6 +224,12 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
         }
     }
     ptx::cluster_sync();                               // every rank's partial logits are in place
+    // A rank whose wait ran out has no sums to add: the tokens of its cluster then have no scores.  They become NaN, which
+    // dsmoe_router's caller sees (it gets no status word), and select nothing.
+    bool gave_up = false;
+#pragma unroll
+    for (int r = 0; r < C; ++r)
+        gave_up |= __float_as_int(ld_cluster(ptx::map_to_cta(ptx::smem_u32(const_cast<int*>(&sh.abort_flag)), (uint32_t)r))) != 0;
     if (warp >= 2) {
         const int w = warp - 2, per = kRuM / C, first = rank * per;
         const bool v_lo = lane < q.E, v_hi = lane + 32 < q.E;
@@ -255,7 +260,13 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
                 l_hi += b_hi;
             }
             uint64_t m = 0;
-            if (t < T && sh.abort_flag == 0) m = softmax_select_store(l_lo, l_hi, t, q, lane, scores, mask, k_t);
+            if (t < T && !gave_up) m = softmax_select_store(l_lo, l_hi, t, q, lane, scores, mask, k_t);
+            if (t < T && gave_up) {
+                if (v_lo) scores[(size_t)t * q.E + lane] = __int_as_float(0x7fffffff);
+                if (v_hi) scores[(size_t)t * q.E + lane + 32] = __int_as_float(0x7fffffff);
+                if (lane == 0 && mask) mask[t] = 0;
+                if (lane == 0 && k_t) k_t[t] = 0;
+            }
             if (lane == 0) sh.mask_s[w + i * kRuWarps] = m;
         }
         if (chunk_counts) {
@@ -275,13 +286,18 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
             }
         }
     }
+    if (gave_up && threadIdx.x == 0) {                 // copies and MMAs already issued still land in this CTA's memory
+        const uint64_t t0 = ptx::globaltimer_ns();
+        while (ptx::globaltimer_ns() - t0 < 200000ull) {
+        }
+    }
     ptx::tc_fence_before();
     ptx::cluster_sync();                               // nobody leaves while another rank may read its sums
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, G::TMEM);
     }
-    if (threadIdx.x == 0 && sh.abort_flag) report_status(dev_status, DSMOE_ERR_TIMEOUT);
+    if (threadIdx.x == 0 && gave_up) report_status(dev_status, DSMOE_ERR_TIMEOUT);
 }
 
 template <int EP, int C>
