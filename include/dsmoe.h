@@ -50,7 +50,7 @@ typedef enum {
     DSMOE_OK = 0,
     DSMOE_ERR_INVALID_ARG = 1,   /* null pointer, bad shape, bad alignment, bad enum       */
     DSMOE_ERR_UNSUPPORTED = 2,   /* valid but outside the limits above (e.g. E > 64)       */
-    DSMOE_ERR_WORKSPACE = 3,     /* ws_bytes smaller than dsmoe_workspace_size reports     */
+    DSMOE_ERR_WORKSPACE = 3,     /* ws_bytes smaller than dsmoe_workspace_size reports, or a workspace that is not aligned */
     DSMOE_ERR_CUDA = 4,          /* a CUDA runtime/driver call failed                      */
     DSMOE_ERR_TIMEOUT = 5        /* written to *dev_status by a kernel whose bounded wait ran out */
 } dsmoe_status;

@@ -181,11 +181,12 @@ dsmoe_status dsmoe_expert_mlp(const dsmoe_layer_desc* desc, const void* xp, cons
     if (desc->T == 0) return DSMOE_OK;
     if (!xp || !offsets || !yp || !aligned16(xp) || !aligned16(yp)) return DSMOE_ERR_INVALID_ARG;
     if (packed && desc->dtype != DSMOE_BF16) return DSMOE_ERR_INVALID_ARG;
-    if (!packed && (!W1 || !W2 || !aligned16(W1) || !aligned16(W2))) return DSMOE_ERR_INVALID_ARG;
+    if (!packed && (!W1 || !W2)) return DSMOE_ERR_INVALID_ARG;
     const WsLayout L = ws_layout(*desc);
     const bool fast = packed && umma_supported(*desc);
     if (!fast && (!W1 || !W2)) return DSMOE_ERR_UNSUPPORTED;   // packed weights given, but this shape needs the plain path
-    if (!workspace || ws_bytes < (fast ? L.total_packed : L.total_plain)) return DSMOE_ERR_WORKSPACE;
+    if (!fast && (!aligned16(W1) || !aligned16(W2))) return DSMOE_ERR_INVALID_ARG;
+    if (!workspace || ws_bytes < (fast ? L.total_packed : L.total_plain) || !aligned16(workspace)) return DSMOE_ERR_WORKSPACE;
     char* ws = static_cast<char*>(workspace);
     cudaStream_t s = (cudaStream_t)stream;
     if (fast) return launch_mlp_umma(*desc, xp, packed, offsets, ws + L.h, yp, dev_status, s);
@@ -224,10 +225,11 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
     if (p.T == 0) return DSMOE_OK;
     if (!x || !Wr || !out || !aligned16(x) || !aligned16(Wr) || !aligned16(out)) return DSMOE_ERR_INVALID_ARG;
     if (packed && p.dtype != DSMOE_BF16) return DSMOE_ERR_INVALID_ARG;
-    if (!packed && (!W1 || !W2 || !aligned16(W1) || !aligned16(W2))) return DSMOE_ERR_INVALID_ARG;
+    if (!packed && (!W1 || !W2)) return DSMOE_ERR_INVALID_ARG;
     const WsLayout L = ws_layout(p);
     const bool fast = packed && umma_supported(p);
     if (!fast && (!W1 || !W2)) return DSMOE_ERR_UNSUPPORTED;   // this shape needs the unpacked weights
+    if (!fast && (!aligned16(W1) || !aligned16(W2))) return DSMOE_ERR_INVALID_ARG;
     if (!workspace || ws_bytes < (fast ? L.total_packed : L.total_plain) || !aligned16(workspace)) return DSMOE_ERR_WORKSPACE;
     char* ws = static_cast<char*>(workspace);
     cudaStream_t s = (cudaStream_t)stream;
@@ -327,7 +329,7 @@ dsmoe_status dsmoe_mi_loss(const dsmoe_layer_desc* desc, const float* scores, fl
     DSMOE_TRY(check_desc(desc));
     if (desc->T == 0 || !scores || !loss3) return DSMOE_ERR_INVALID_ARG;
     const WsLayout L = ws_layout(*desc);
-    if (!workspace || ws_bytes < L.stage_total) return DSMOE_ERR_WORKSPACE;
+    if (!workspace || ws_bytes < L.stage_total || ((uintptr_t)workspace & 7u)) return DSMOE_ERR_WORKSPACE;
     return launch_mi_loss(*desc, scores, loss3, grad, static_cast<char*>(workspace) + L.mi, (cudaStream_t)stream);
 }
 

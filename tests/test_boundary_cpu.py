@@ -92,3 +92,24 @@ def test_pack_rejects_shapes_that_are_not_multiples_of_64_and_the_new_selection_
     # ... a mode beyond it is not
     bad = dm.make_desc(128, 64, 64, 32, dm.BF16, mode=4)
     assert L.dsmoe_workspace_size(ctypes.byref(bad), ctypes.byref(ctypes.c_size_t(0))) == 1
+
+
+def test_misaligned_weights_and_workspaces_are_rejected_wherever_they_are_read():
+    """The plain path reads weights and hidden activations in pieces of 8 and 16 bytes, also when packed weights were given
+    but the shape has no tensor-core path."""
+    L = dm.lib()
+    fake, z, big = ctypes.c_void_p(4096), ctypes.c_void_p(0), ctypes.c_size_t(1 << 40)
+    plain_shape = dm.make_desc(16, 128, 72, 4, dm.BF16, dm.SELECT_TOPK, K=2)           # H = 72: no tensor-core path
+    for off in (2, 4, 8):
+        odd = ctypes.c_void_p(4096 + off)
+        for w1, w2 in ((odd, fake), (fake, odd)):
+            for packed in (z, fake):
+                assert L.dsmoe_layer_forward(ctypes.byref(plain_shape), fake, fake, z, w1, w2, packed, fake, z, z, fake, big, z, z) == 1
+                assert L.dsmoe_expert_mlp(ctypes.byref(plain_shape), fake, w1, w2, packed, fake, fake, fake, big, z, z) == 1
+        for desc, packed in ((plain_shape, z), (plain_shape, fake), (dm.make_desc(16, 128, 64, 4, dm.BF16), fake),
+                             (dm.make_desc(16, 128, 64, 4, dm.F32), z)):
+            assert L.dsmoe_expert_mlp(ctypes.byref(desc), fake, fake, fake, packed, fake, fake, odd, big, z, z) == 3
+            assert L.dsmoe_layer_forward(ctypes.byref(desc), fake, fake, z, fake, fake, packed, fake, z, z, odd, big, z, z) == 3
+    for off in (2, 4):                                                                  # sums in double precision
+        odd = ctypes.c_void_p(4096 + off)
+        assert L.dsmoe_mi_loss(ctypes.byref(plain_shape), fake, fake, z, odd, big, z) == 3
