@@ -378,9 +378,10 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
     int32_t* row_token = reinterpret_cast<int32_t*>(ws + L.row_token);
     float* row_gate = reinterpret_cast<float*>(ws + L.row_gate);
     int32_t* token_rows = reinterpret_cast<int32_t*>(ws + L.token_rows);
-    const bool dense_down = moa_shares_keys(p, args->n_head, args->n_seq) && moa_dense_down(p, sm_count());
-    const MoaCore core{args->n_head, args->n_seq, args->L, args->scale, args->Kc, args->Vc, args->tok_seq, args->pos, token_rows,
-                       dense_down ? ws + L.acc : nullptr, mask, row_gate};
+    MoaCore core{args->n_head, args->n_seq, args->L, args->scale, args->Kc, args->Vc, args->tok_seq, args->pos, token_rows,
+                 nullptr, mask, row_gate};
+    const bool dense_down = moa_shares_keys(p, core) && moa_dense_down(p, sm_count());
+    if (dense_down) core.dense = ws + L.acc;
 
     // router, selection and grouping as in dsmoe_layer_forward's grouped path (also when every expert is selected)
     dsmoe_layer_desc pr = p;

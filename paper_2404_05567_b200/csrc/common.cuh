@@ -210,8 +210,8 @@ struct MoaCore {
     const uint64_t* mask;
     const float* row_gate;
 };
-// Whether launch_moa_attention takes the kernel whose tiles share their copies of the keys (the only one that serves `dense`)
-bool moa_shares_keys(const dsmoe_layer_desc& p, int n_head, int n_seq);
+// Whether launch_moa_attention takes the kernel whose tiles share their copies of the keys (`dense` needs it)
+bool moa_shares_keys(const dsmoe_layer_desc& p, const MoaCore& c);
 // Output projection and the weighted sum of Eq. 8 as ONE dense GEMM over the experts side by side, out = dense . Wo[E*H, d], as
 // in the dense forward: E / K times the multiplications of the grouped form, but at the rate of a long reduction (E * H
 // instead of H) and without expert outputs written to and read back from memory as fp32 rows (8 bytes per row and column).

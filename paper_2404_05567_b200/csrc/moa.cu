@@ -130,13 +130,51 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-template <int DH, int kMmaWarps>      // long caches: 8 warps share out the keys; short ones: 2, and several CTAs fit an SM
+constexpr int kTileMaxKeys = 512;  // caches up to this many positions: a warp walks all keys of its tile; longer ones: 8 warps share them out
+constexpr int kShWarps = 4;        // tiles of a CTA that share their copies of the keys (moa_attention_shared_kernel)
+
+struct AttnArgs {
+    __nv_bfloat16* qa;
+    const int32_t* token_rows;
+    int W, row_tiles, tpt;      // rows of a token, 16-row tiles they take, tokens of a tile
+    int group_tpt;              // ... of the shared-key kernel's tiles, whatever this launch's are
+    long long amax;
+    int n_head, H, T;
+    const __nv_bfloat16 *Kc, *Vc;
+    const int32_t *tok_seq, *pos;
+    int n_seq, L;
+    float scale;
+    int* dev_status;
+    bool leave_mixed;           // mixed groups are another launch's
+    // With `dense`, the outputs go to dense[T][E * H] instead: expert e's columns e * H .. of token t hold its gate times its
+    // attention output, zeros where the token did not select e (these zeros are the shared-key kernel's)
+    __nv_bfloat16* dense;
+    int E;
+    const uint64_t* mask;
+    const float* row_gate;
+};
+
+// The expert of a token's slot-th grouped row (its selected experts ascend); -1: the token has fewer
+__device__ __forceinline__ int expert_of_slot(uint64_t selected, int slot) {
+    for (; slot > 0; --slot) selected &= selected - 1;
+    return __ffsll((long long)selected) - 1;
+}
+
+// Four neighbouring tiles are a mixed group if some token's sequence is neither the first token's nor the last one's: decoding
+// sequences side by side, or tokens in no order of sequences.  They share no keys.
+__device__ __forceinline__ void group_tokens(const AttnArgs& P, int group, int& t0, int& t1) {
+    t0 = (group * kShWarps / P.row_tiles) * P.group_tpt;
+    t1 = min(P.T, ((group * kShWarps + kShWarps - 1) / P.row_tiles) * P.group_tpt + P.group_tpt);
+}
+__device__ __forceinline__ int seq_of(const AttnArgs& P, int t) { return P.tok_seq ? min(max(P.tok_seq[t], 0), P.n_seq - 1) : 0; }
+
+template <int DH, int kMmaWarps, bool MIXED>      // long caches: 8 warps share out the keys; short ones: 2, and several CTAs fit an SM
 __global__ void __launch_bounds__(32 * kMmaWarps, kMmaWarps == 2 ? DSMOE_MOA_MINBLOCKS : 1)
 moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* token_rows, int W, int row_tiles,
                          int tpt, long long amax, int n_head, int H, int T, const __nv_bfloat16* Kc,
                          const __nv_bfloat16* Vc, const int32_t* tok_seq,
                          const int32_t* pos, int n_seq, int L, float scale, long long n_tiles,
-                         int* __restrict__ dev_status) {
+                         int* __restrict__ dev_status, const AttnArgs P /* MIXED only */) {
     chain_wait();
     constexpr int STRIDE = DH * 2 + 16;                 // bytes per key row in shared memory: 16 of padding
     constexpr int KS = DH / 16, DT = DH / 8, CH = DH / 8;
@@ -152,7 +190,36 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* token_ro
     // keys and writes its result straight from registers: no merge, no CTA-wide barrier.
     constexpr bool SPLIT = kMmaWarps > 2;
     constexpr int TW = SPLIT ? 1 : kMmaWarps;           // tiles a CTA works on at a time
-    for (long long tile = (long long)blockIdx.x * TW + (SPLIT ? 0 : warp); tile < n_tiles; tile += (long long)gridDim.x * TW) {
+    static_assert(SPLIT || !MIXED, "the tile loop must be the same for the whole CTA");
+    __shared__ int found_s;
+    // MIXED: the tiles of mixed groups alone; every thread looks at one of the CTA's next tiles
+    const auto next_tile = [&](long long from) {
+        if (!MIXED) return from;
+        for (; from < n_tiles; from += (long long)gridDim.x * blockDim.x) {
+            const long long mine = from + (long long)gridDim.x * threadIdx.x;
+            bool mixed = false;
+            if (mine < n_tiles) {
+                int a, b;
+                const int t = (int)(mine / ((long long)row_tiles * n_head)) * tpt;
+                group_tokens(P, (t / P.group_tpt * row_tiles + (int)(mine % row_tiles)) / kShWarps, a, b);
+                const int first = seq_of(P, a), last = seq_of(P, b - 1);
+                for (int u = a + 1; u + 1 < b; ++u) {
+                    const int sq = seq_of(P, u);
+                    mixed = mixed || (sq != first && sq != last);
+                }
+            }
+            if (threadIdx.x == 0) found_s = INT_MAX;
+            __syncthreads();
+            if (mixed) atomicMin(&found_s, (int)threadIdx.x);
+            __syncthreads();
+            const int found = found_s;
+            __syncthreads();
+            if (found != INT_MAX) return from + (long long)gridDim.x * found;
+        }
+        return from;
+    };
+    for (long long tile = next_tile((long long)blockIdx.x * TW + (SPLIT ? 0 : warp)); tile < n_tiles;
+         tile = next_tile(tile + (long long)gridDim.x * TW)) {
     if (SPLIT) __syncthreads();                         // the previous tile's merge has read shared memory
     const int rt = (int)(tile % row_tiles);
     const int j = (int)((tile / row_tiles) % n_head);
@@ -391,7 +458,11 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* token_ro
             num = fmaf(wgt, os[((size_t)w * 16 + row) * DH + dcol], num);
             den = fmaf(wgt, ls[w * 16 + row], den);
         }
-        qa[(size_t)r * H + j * DH + dcol] = __float2bfloat16_rn(num / den);
+        if (!MIXED || !P.dense) {
+            qa[(size_t)r * H + j * DH + dcol] = __float2bfloat16_rn(num / den);
+        } else if (const int e = expert_of_slot(P.mask[tok], slot); e >= 0) {
+            P.dense[((size_t)tok * P.E + e) * H + j * DH + dcol] = __float2bfloat16_rn(num / den * P.row_gate[r]);
+        }
     }
     }
     chain_next();
@@ -402,32 +473,16 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* token_ro
 // One CTA per (head, four 16-row tiles of neighbouring tokens); a warp owns a tile (its rows, queries, sums), and all four walk
 // the same keys: blocks of 64 keys and values come by cp.async into two buffers, one under way while the other is worked on.
 // Tokens of a prompt see nearly the same keys, so a block is read once for 12 tokens (5 rows each) instead of once per tile,
-// and no warp waits behind its own copies.  Tokens of several sequences in one CTA are served sequence by sequence.  Both
-// operands' fragments come by ldmatrix.x4; exponents are base 2 with the scale folded in; a block that every row of the warp
+// and no warp waits behind its own copies.  A group whose tokens belong to two sequences walks first the one's keys, then the
+// other's.  In a mixed group nothing is shared: with caches of up to kTileMaxKeys positions each warp walks its own tile's
+// sequences by itself, through its quarter of the buffers; with longer ones the group is left to moa_attention_mma_kernel, whose
+// CTAs share out a tile's keys (31 sequences decoding at 2048 positions beside a prompt of 512: the layer 693 us with shared
+// blocks of one active warp each, 157 so).  Both operands' fragments come by ldmatrix.x4; exponents are base 2 with the scale folded in; a block that every row of the warp
 // sees in full is not masked, and sums are rescaled only where a maximum moved.  Three CTAs of 70 KB and 168 registers a
 // thread fill an SM.  Bound by the instruction issue of the warp-level tensor path and the exponentials.
 // 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 133 us with a tile per warp and its own copies, 83 with shared ones
-// (tensor pipe 31 % busy, 0.38 instructions a cycle and scheduler; the layer 702 -> 653 us).
-constexpr int kShWarps = 4, kShKeys = 64, kShTokens = kShWarps * 16;
-
-struct AttnArgs {
-    __nv_bfloat16* qa;
-    const int32_t* token_rows;
-    int W, row_tiles, tpt;
-    long long amax;
-    int n_head, H, T;
-    const __nv_bfloat16 *Kc, *Vc;
-    const int32_t *tok_seq, *pos;
-    int n_seq, L;
-    float scale;
-    int* dev_status;
-    // With `dense`, the outputs go to dense[T][E * H] instead: expert e's columns e * H .. of token t hold its gate times its
-    // attention output, zeros where the token did not select e
-    __nv_bfloat16* dense;
-    int E;
-    const uint64_t* mask;
-    const float* row_gate;
-};
+// (tensor pipe 31 % busy, 0.38 instructions a cycle and scheduler; the layer 702 -> 653 us, before its dense output projection).
+constexpr int kShKeys = 64, kShTokens = kShWarps * 16;
 
 __device__ __forceinline__ float ex2(float v) {
     float r;
@@ -443,33 +498,17 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 
+int shared_tile_tokens(int W) { return W <= 8 ? 16 / W : 1; }
+long long shared_groups(const dsmoe_layer_desc& p) {
+    const int W = width_of(p), tpt = shared_tile_tokens(W);
+    return ((long long)((p.T + tpt - 1) / tpt) * ((W + 15) / 16) + kShWarps - 1) / kShWarps;
+}
+
 template <int DH>
 constexpr size_t shared_attention_smem() { return (size_t)2 * 2 * kShKeys * (DH * 2 + 16); }
 
-template <int DH>
-__global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(const AttnArgs P) {
-    chain_wait();
-    constexpr int STRIDE = DH * 2 + 16;                 // bytes per key row in shared memory: 16 of padding, no bank conflicts
-    constexpr int KS = DH / 16, DT = DH / 8, CH = DH / 8;
-    extern __shared__ __align__(16) unsigned char moa_sh_smem[];
-    __shared__ int seq_s[kShTokens], last_s[kShTokens];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q4 = lane & 3;
-    const int j = (int)(blockIdx.x % P.n_head);
-    const int group = (int)(blockIdx.x / P.n_head);
-    // this CTA's tokens: their sequences and last visible keys, clamped into the cache (and reported)
-    const int tg0 = (group * kShWarps / P.row_tiles) * P.tpt;
-    const int tg1 = min(P.T, ((group * kShWarps + kShWarps - 1) / P.row_tiles) * P.tpt + P.tpt);
-    const int ng = tg1 - tg0;
-    if (threadIdx.x < ng) {
-        const int t = tg0 + threadIdx.x;
-        const int sq = P.tok_seq ? P.tok_seq[t] : 0, last = P.pos[t];
-        if (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
-        seq_s[threadIdx.x] = min(max(sq, 0), P.n_seq - 1);
-        last_s[threadIdx.x] = min(max(last, 0), P.L - 1);
-    }
-    // this thread's two rows of the warp's tile (g and g + 8): grouped row (-1 = none), token
-    const int wt = group * kShWarps + warp, t0 = (wt / P.row_tiles) * P.tpt, rt = wt % P.row_tiles;
-    int r[2], tk[2];
+// This lane's two rows of tile (t0, rt), g and g + 8: grouped row (-1 = none), token
+__device__ __forceinline__ void tile_rows(const AttnArgs& P, int t0, int rt, int g, int (&r)[2], int (&tk)[2]) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int i = g + 8 * h;
@@ -484,7 +523,19 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
         r[h] = tk[h] < P.T && slot < P.W ? P.token_rows[(size_t)tk[h] * P.W + slot] : -1;
         if (r[h] >= P.amax) r[h] = -1;
     }
-    __syncthreads();
+}
+
+// Attends with this warp's tile (t0, rt) of head j and writes its rows.  The keys of tokens first_u .. end_u - 1 of the group (tokens
+// tg0 ..) are walked by the CTA together, or (ALONE) by the warp by itself.
+template <int DH, bool ALONE>
+__device__ __forceinline__ void attend(const AttnArgs& P, unsigned char* const smem, const int* const seq_s, const int* const last_s,
+                                       const int j, const int t0, const int rt, const int tg0, const int first_u, const int end_u,
+                                       int (&r)[2], int (&tk)[2]) {
+    constexpr int STRIDE = DH * 2 + 16;                 // bytes per key row in shared memory: 16 of padding, no bank conflicts
+    constexpr int KS = DH / 16, DT = DH / 8, CH = DH / 8;
+    constexpr int keys = ALONE ? kShKeys / 2 : kShKeys, workers = ALONE ? 32 : 32 * kShWarps;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q4 = lane & 3;
+    const int worker = ALONE ? lane : threadIdx.x;
     int last[2], sq_of[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -509,19 +560,20 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
 #pragma unroll
     for (int i = 0; i < DT; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
 
-    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(moa_sh_smem);
+    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem);
     // fragment addresses inside a block: K (rows = keys, two 8-key tiles x two 8-wide halves of k) and V (transposed)
     const uint32_t kfrag = (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * STRIDE + ((lane >> 3) & 1) * 16);
     const uint32_t vfrag = (uint32_t)((((lane >> 3) & 1) * 8 + (lane & 7)) * STRIDE + (lane >> 4) * 16);
 
-    for (int u = 0; u < ng; ++u) {
-        // one pass per sequence among the CTA's tokens (a prompt's tokens: one)
+    const uint32_t own = ALONE ? (uint32_t)(warp * kShKeys * STRIDE) : 0u;
+    for (int u = first_u; u < end_u; ++u) {
+        // one pass per sequence among them (a prompt's tokens: one)
         const int sq = seq_s[u];
         bool again = false;
-        for (int v = 0; v < u && !again; ++v) again = seq_s[v] == sq;
+        for (int v = first_u; v < u && !again; ++v) again = seq_s[v] == sq;
         if (again) continue;
         int last_key = 0;
-        for (int v = u; v < ng; ++v)
+        for (int v = u; v < end_u; ++v)
             if (seq_s[v] == sq) last_key = max(last_key, last_s[v]);
         // this pass: which rows take part, the last key any of the warp's rows sees, the last one they all see
         const bool act0 = sq_of[0] == sq, act1 = sq_of[1] == sq;
@@ -530,13 +582,13 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
                                                                   act1 ? last[1] : r[1] >= 0 ? -1 : INT_MAX));
         const __nv_bfloat16* Kh = P.Kc + ((size_t)(sq * P.n_head + j) * P.L) * DH;
         const __nv_bfloat16* Vh = P.Vc + ((size_t)(sq * P.n_head + j) * P.L) * DH;
-        const int nblocks = last_key / kShKeys + 1;
+        const int nblocks = last_key / keys + 1;
         const auto fetch = [&](int b, int buf) {
-            const int key0 = b * kShKeys, nk = min(kShKeys, last_key + 1 - key0);
-            const uint32_t kd = smem0 + (uint32_t)(buf * 2 * kShKeys * STRIDE), vd = kd + kShKeys * STRIDE;
-#pragma unroll
-            for (int i = 0; i < CH * kShKeys / (32 * kShWarps); ++i) {
-                const int idx = threadIdx.x + 32 * kShWarps * i, row = idx / CH, ch = idx % CH;
+            const int key0 = b * keys, nk = min(keys, last_key + 1 - key0);
+            const uint32_t kd = smem0 + own + (uint32_t)(buf * 2 * kShKeys * STRIDE), vd = kd + (uint32_t)(keys * STRIDE);
+#pragma unroll(ALONE ? 4 : CH * keys / workers)          // (ALONE in full: the kernel spills)
+            for (int i = 0; i < CH * keys / workers; ++i) {
+                const int idx = worker + workers * i, row = idx / CH, ch = idx % CH;
                 // rows past the last visible key are filled with zeros
                 const size_t src = (size_t)(key0 + (row < nk ? row : 0)) * DH + ch * 8;
                 const uint32_t nbytes = row < nk ? 16u : 0u, dst = (uint32_t)(row * STRIDE + ch * 16);
@@ -545,22 +597,25 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        fetch(0, 0);
+        if (!ALONE) fetch(0, 0);
         for (int b = 0; b < nblocks; ++b) {
-            const int buf = b & 1;
-            if (b + 1 < nblocks) {
+            const int buf = ALONE ? 0 : b & 1;
+            if (ALONE) fetch(b, 0);
+            if (!ALONE && b + 1 < nblocks) {
                 fetch(b + 1, buf ^ 1);
                 asm volatile("cp.async.wait_group 1;" ::: "memory");
             } else {
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
-            __syncthreads();
+            if (ALONE) __syncwarp();
+            else __syncthreads();
+            const uint32_t kblock = smem0 + own + (uint32_t)(buf * 2 * kShKeys * STRIDE), vblock = kblock + (uint32_t)(keys * STRIDE);
 #pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-                const int key0 = b * kShKeys + 32 * half;
+            for (int half = 0; half < keys / 32; ++half) {
+                const int key0 = b * keys + 32 * half;
                 if (key0 > wlast) break;                // (uniform in the warp) nothing more for this warp's rows
-                const uint32_t ka = smem0 + (uint32_t)(buf * 2 * kShKeys * STRIDE + 32 * half * STRIDE) + kfrag;
-                const uint32_t va = smem0 + (uint32_t)((buf * 2 + 1) * kShKeys * STRIDE + 32 * half * STRIDE) + vfrag;
+                const uint32_t ka = kblock + (uint32_t)(32 * half * STRIDE) + kfrag;
+                const uint32_t va = vblock + (uint32_t)(32 * half * STRIDE) + vfrag;
                 float sc[4][4];
 #pragma unroll
                 for (int nt = 0; nt < 4; ++nt) sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
@@ -640,7 +695,8 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
                     }
                 }
             }
-            __syncthreads();
+            if (ALONE) __syncwarp();
+            else __syncthreads();
         }
     }
     chain_next();
@@ -654,16 +710,12 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
         inv[h] = 1.f / l[h];
         dst[h] = r[h] >= 0 ? P.qa + (size_t)r[h] * P.H + j * DH : nullptr;
         if (P.dense && r[h] >= 0) {
-            // the row is its token's slot-th selected expert, ascending
-            uint64_t sel = P.mask[tk[h]];
-            const int i = g + 8 * h;
-            for (int slot = P.tpt == 1 ? rt * 16 + i : i % P.W; slot > 0; --slot) sel &= sel - 1;
-            const int e = __ffsll((long long)sel) - 1;
+            const int i = g + 8 * h, e = expert_of_slot(P.mask[tk[h]], P.tpt == 1 ? rt * 16 + i : i % P.W);
             dst[h] = e >= 0 ? P.dense + ((size_t)tk[h] * P.E + e) * P.H + j * DH : nullptr;
             inv[h] *= P.row_gate[r[h]];
         }
     }
-    unsigned char* const st = moa_sh_smem + warp * 16 * STRIDE;
+    unsigned char* const st = smem + warp * kShKeys * STRIDE;      // (where only this warp may still have been reading)
 #pragma unroll
     for (int dt = 0; dt < DT; ++dt) {
         *reinterpret_cast<uint32_t*>(st + g * STRIDE + (dt * 8 + q4 * 2) * 2) = pack_bf16(o[dt][0] * inv[0], o[dt][1] * inv[0]);
@@ -678,6 +730,35 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
         __nv_bfloat16* const to = row < 8 ? da : db;
         if (to) *reinterpret_cast<uint4*>(to + ch * 8) = *reinterpret_cast<const uint4*>(st + row * STRIDE + ch * 16);
     }
+}
+
+template <int DH>
+__global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(const __grid_constant__ AttnArgs P) {
+    chain_wait();
+    constexpr int CH = DH / 8;
+    extern __shared__ __align__(16) unsigned char moa_sh_smem[];
+    __shared__ int seq_s[kShTokens], last_s[kShTokens];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j = (int)(blockIdx.x % P.n_head);
+    const int group = (int)(blockIdx.x / P.n_head);
+    // this CTA's tokens: their sequences and last visible keys, clamped into the cache (and reported)
+    int tg0, tg1;
+    group_tokens(P, group, tg0, tg1);
+    const int ng = tg1 - tg0;
+    if (threadIdx.x < ng) {
+        const int t = tg0 + threadIdx.x;
+        const int sq = P.tok_seq ? P.tok_seq[t] : 0, last = P.pos[t];
+        if (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
+        seq_s[threadIdx.x] = min(max(sq, 0), P.n_seq - 1);
+        last_s[threadIdx.x] = min(max(last, 0), P.L - 1);
+    }
+    const int wt = group * kShWarps + warp, t0 = (wt / P.row_tiles) * P.tpt, rt = wt % P.row_tiles;
+    int r[2], tk[2];
+    tile_rows(P, t0, rt, lane >> 2, r, tk);
+    __syncthreads();
+    bool mixed = false;
+    for (int i = lane; i < ng; i += 32) mixed = mixed || (seq_s[i] != seq_s[0] && seq_s[i] != seq_s[ng - 1]);
+    mixed = __any_sync(0xffffffffu, mixed);
     if (P.dense && rt == 0) {
         for (int t = t0; t < min(P.T, t0 + P.tpt); ++t) {
             const uint64_t sel = P.mask[t];
@@ -688,6 +769,25 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
             }
         }
     }
+    if (!mixed) attend<DH, false>(P, moa_sh_smem, seq_s, last_s, j, t0, rt, tg0, 0, ng, r, tk);
+    else if (!P.leave_mixed) {
+        tile_rows(P, t0, rt, lane >> 2, r, tk);         // (again: kept over the branch, they cost registers that the common path lacks)
+        attend<DH, true>(P, moa_sh_smem, seq_s, last_s, j, t0, rt, tg0, t0 - tg0, min(t0 - tg0 + P.tpt, ng), r, tk);
+    }
+}
+
+// Whether the groups that share no keys go to the key-splitting kernel
+bool leaves_mixed(const dsmoe_layer_desc& p, const MoaCore& c) {
+    return c.tok_seq && c.n_seq > 1 && c.L > kTileMaxKeys;
+}
+
+// tpt: tokens of a tile in this launch
+AttnArgs attn_args(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows, int tpt,
+                   int32_t* dev_status) {
+    const int W = width_of(p);
+    return AttnArgs{q, token_rows, W, (W + 15) / 16, tpt, shared_tile_tokens(W), (long long)amax_of(p), c.n_head, p.H, p.T,
+                    static_cast<const __nv_bfloat16*>(c.Kc), static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos,
+                    c.n_seq, c.L, c.scale, dev_status, leaves_mixed(p, c), static_cast<__nv_bfloat16*>(c.dense), p.E, c.mask, c.row_gate};
 }
 
 template <int DH>
@@ -702,18 +802,15 @@ dsmoe_status launch_shared_attention(const dsmoe_layer_desc& p, const MoaCore& c
                                             (int)shared_attention_smem<DH>()));
         attr[dev] = true;
     }
-    const int W = width_of(p), row_tiles = (W + 15) / 16, tpt = W <= 8 ? 16 / W : 1;
-    const AttnArgs a{q, token_rows, W, row_tiles, tpt, (long long)amax_of(p), c.n_head, p.H, p.T,
-                     static_cast<const __nv_bfloat16*>(c.Kc), static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos,
-                     c.n_seq, c.L, c.scale, dev_status, static_cast<__nv_bfloat16*>(c.dense), p.E, c.mask, c.row_gate};
-    const long long tiles = (long long)((p.T + tpt - 1) / tpt) * row_tiles;
-    const long long ctas = (tiles + kShWarps - 1) / kShWarps * c.n_head;
+    const long long ctas = shared_groups(p) * c.n_head;
     if (ctas > 0x7fffffffll) return DSMOE_ERR_UNSUPPORTED;
-    DSMOE_CUDA_TRY(launch_chained(moa_attention_shared_kernel<DH>, (unsigned)ctas, 32 * kShWarps, shared_attention_smem<DH>(), s, a));
+    DSMOE_CUDA_TRY(launch_chained(moa_attention_shared_kernel<DH>, (unsigned)ctas, 32 * kShWarps, shared_attention_smem<DH>(), s,
+        attn_args(p, c, q, token_rows, shared_tile_tokens(width_of(p)), dev_status)));
     return DSMOE_OK;
 }
 
-template <int DH, int kMmaWarps>
+// MIXED: the groups that moa_attention_shared_kernel leaves, a token per tile (their tokens share no keys)
+template <int DH, int kMmaWarps, bool MIXED = false>
 dsmoe_status launch_mma_attention_nw(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
                                   int32_t* dev_status, cudaStream_t s) {
     constexpr size_t stride = DH * 2 + 16;
@@ -725,33 +822,36 @@ dsmoe_status launch_mma_attention_nw(const dsmoe_layer_desc& p, const MoaCore& c
     DeviceState* st = nullptr;
     DSMOE_TRY(device_state(&st, &dev));
     if (!attr[dev]) {
-        DSMOE_CUDA_TRY(cudaFuncSetAttribute(moa_attention_mma_kernel<DH, kMmaWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(moa_attention_mma_kernel<DH, kMmaWarps, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr[dev] = true;
     }
     const int W = width_of(p), row_tiles = (W + 15) / 16;
     // several tokens per tile where a token has few rows and there are tokens enough to fill the GPU without
-    const int tpt = (W <= 8 && (long long)p.T * c.n_head >= 8ll * st->sm_count) ? 16 / W : 1;
+    const int tpt = (W <= 8 && (long long)p.T * c.n_head >= (MIXED ? 64ll : 8ll) * st->sm_count) ? 16 / W : 1;
     const long long n_tiles = (long long)((p.T + tpt - 1) / tpt) * c.n_head * row_tiles;
     static int per_sm_of[kMaxDeviceSlots] = {};      // CTAs of this kernel that fit an SM, asked once per device
     if (!per_sm_of[dev])
-        DSMOE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_of[dev], moa_attention_mma_kernel<DH, kMmaWarps>,
+        DSMOE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_of[dev], moa_attention_mma_kernel<DH, kMmaWarps, MIXED>,
                                                                      32 * kMmaWarps, smem));
     const int per_sm = per_sm_of[dev];
     const long long resident = (long long)st->sm_count * (per_sm > 0 ? per_sm : 1);
     const long long want = kMmaWarps > 2 ? n_tiles : (n_tiles + kMmaWarps - 1) / kMmaWarps;     // 2 warps: a tile per warp
     const long long ctas = want < resident ? want : resident;
-    DSMOE_CUDA_TRY(launch_chained(moa_attention_mma_kernel<DH, kMmaWarps>, (unsigned)ctas, 32 * kMmaWarps, smem, s,
-        q, token_rows, W, row_tiles, tpt, (long long)amax_of(p), c.n_head, p.H, p.T, static_cast<const
-        __nv_bfloat16*>(c.Kc), static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos, c.n_seq, c.L, c.scale,
-        n_tiles, dev_status));
+    DSMOE_CUDA_TRY(launch_chained(moa_attention_mma_kernel<DH, kMmaWarps, MIXED>, (unsigned)ctas, 32 * kMmaWarps, smem, s,
+        q, token_rows, W, row_tiles, tpt, (long long)amax_of(p), c.n_head, p.H, p.T, static_cast<const __nv_bfloat16*>(c.Kc),
+        static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos, c.n_seq, c.L, c.scale, n_tiles, dev_status,
+        attn_args(p, c, q, token_rows, tpt, dev_status)));
     return DSMOE_OK;
 }
 
 template <int DH>
 dsmoe_status launch_mma_attention(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
                                   int32_t* dev_status, cudaStream_t s) {
-    if (moa_shares_keys(p, c.n_head, c.n_seq)) return launch_shared_attention<DH>(p, c, q, token_rows, dev_status, s);
-    if (c.L <= 512) return launch_mma_attention_nw<DH, 2>(p, c, q, token_rows, dev_status, s);
+    if (moa_shares_keys(p, c)) {
+        DSMOE_TRY(launch_shared_attention<DH>(p, c, q, token_rows, dev_status, s));
+        return leaves_mixed(p, c) ? launch_mma_attention_nw<DH, 8, true>(p, c, q, token_rows, dev_status, s) : DSMOE_OK;
+    }
+    if (c.L <= kTileMaxKeys) return launch_mma_attention_nw<DH, 2>(p, c, q, token_rows, dev_status, s);
     return launch_mma_attention_nw<DH, 8>(p, c, q, token_rows, dev_status, s);
 }
 
@@ -765,11 +865,26 @@ bool moa_supported(const dsmoe_layer_desc& p, int n_head, int L) {
     return (size_t)(dh + L + 3) * 4 * kMoaWarps <= 200 * 1024;                // plain kernel: a warp's logits sit in shared memory
 }
 
-// Prompts: at least eight tokens per sequence on average, so that neighbouring tokens mostly share their keys.  (Decoding, one
-// token per sequence, would walk a CTA's sequences one after the other.)
-bool moa_shares_keys(const dsmoe_layer_desc& p, int n_head, int n_seq) {
-    const int dh = p.H / n_head;
-    return (dh == 64 || dh == 96 || dh == 128) && !getenv("DSMOE_MOA_PLAIN") && (long long)p.T >= 8ll * n_seq;
+// Prompts and chunks of them.  The host knows neither how much of a cache is visible nor the tokens' order, so the rule sees to
+// it that no length and no order of sequences makes the shared-key kernel the much slower one (layer times key-splitting, shared
+// for 8 experts of 4 heads of 128, top-5; 16 of 2 heads of 64, top-6, are alike):
+//   long caches: its CTAs walk all keys by themselves, where the other kernel's warps share them out.  One sequence, 2048
+//   positions: 64 tokens (24 CTAs) 103, 155 us; 128 (44) 154, 156; 256 (88) 236, 169; 2048 534, 254; 16384 positions, 256
+//   tokens 1215, 842.  Of several sequences some CTAs walk two: 16384 positions, 12 sequences of 40 tokens (160 CTAs) 1083, 1294;
+//   44 of 18 (264) 1465, 1388; 11 of 72 (264) 1465, 888; 2048 positions, 32 prompts of 256 1280, 469; 31 sequences decoding
+//   beside a prompt of 768, their groups left to the other kernel, 271, 202.
+//   short caches: the other kernel walks a tile per warp as well, of one token while T * n_head < 8 SMs; mixed groups then have
+//   longer chains here, and groups of two sequences are walked twice.  4 sequences of 64 tokens, 256 positions: 96, 93; of 8
+//   tokens 73, 76; 31 sequences decoding beside a prompt of 512, 512 positions: 201, 188, with 2 heads of 64 98, 112; 32 prompts
+//   of 256: 633, 458; their tokens round-robin over the sequences 781, 619.
+bool moa_shares_keys(const dsmoe_layer_desc& p, const MoaCore& c) {
+    const int dh = p.H / c.n_head, n_seq = c.tok_seq ? c.n_seq : 1;
+    if ((dh != 64 && dh != 96 && dh != 128) || getenv("DSMOE_MOA_PLAIN")) return false;
+    const int W = width_of(p), group = kShWarps * shared_tile_tokens(W) / ((W + 15) / 16);       // tokens of a group
+    const bool longer = c.L > kTileMaxKeys;
+    const int least = longer ? 8 : (long long)p.T * c.n_head < 8ll * sm_count() ? 32 : group + group / 2;
+    if (p.T < 8 || (n_seq > 1 && p.T < (long long)(least > 8 ? least : 8) * n_seq)) return false;
+    return !longer || shared_groups(p) * c.n_head >= (n_seq > 1 ? 256 : 64);
 }
 
 dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, void* qa, const int32_t* row_token,

@@ -202,3 +202,36 @@ def test_moa_clamps_and_reports_entries_out_of_range_with_or_without_a_status_wo
     assert torch.equal(run(wild_seq, wild_pos, status), want)
     assert int(status.item()) == 1                                   # DSMOE_ERR_INVALID_ARG
     assert torch.equal(run(wild_seq, wild_pos, None), want)
+
+
+# Groups of four tiles whose tokens share no keys (a token whose sequence is neither the group's first nor its last): with short
+# caches each warp walks its own tile, with long ones the key-splitting kernel takes the group -- grouped and dense output
+# projection, prompts beside decoding sequences, tokens round-robin over the sequences, one and several row tiles per token.
+MIXED = [
+    # name, T, d, E, n_head, d_head, n_seq, L, order, mode, selection
+    ("round_robin_short", 200, 256, 8, 2, 64, 5, 90, "round", gi.MODE_TOPK, dict(K=5)),
+    ("round_robin_short_128", 333, 256, 4, 2, 128, 9, 65, "round", gi.MODE_TOPK, dict(K=3)),
+    ("round_robin_threshold", 300, 256, 16, 2, 96, 7, 512, "round", gi.MODE_THRESHOLD, dict(eps=0.15)),
+    ("round_robin_row_tiles", 90, 256, 20, 2, 64, 3, 70, "round", gi.MODE_ALL, dict()),
+    ("round_robin_long", 1600, 256, 8, 4, 64, 5, 530, "round", gi.MODE_TOPK, dict(K=5)),
+    ("decode_and_prompt_long", 1031, 256, 8, 4, 128, 32, 1100, "decode_prompt", gi.MODE_TOPK, dict(K=5)),
+    ("decode_and_prompt_short", 531, 256, 8, 4, 64, 20, 512, "decode_prompt", gi.MODE_TOPK, dict(K=5)),
+    ("long_row_tiles", 500, 256, 20, 2, 64, 4, 700, "round", gi.MODE_ALL, dict()),
+    ("round_robin_dense", 4701, 1024, 8, 2, 64, 7, 300, "round", gi.MODE_TOPK, dict(K=4)),
+    ("decode_and_prompt_dense_long", 4671, 1024, 8, 4, 96, 64, 4700, "decode_prompt", gi.MODE_TOPK, dict(K=5)),
+    ("round_robin_dense_long", 4640, 1024, 20, 2, 64, 11, 600, "round", gi.MODE_ALL, dict()),
+]
+
+
+@pytest.mark.parametrize("case", MIXED, ids=[c[0] for c in MIXED])
+def test_moa_mixed_groups(case):
+    name, T, d, E, nh, dh, n_seq, L, order, mode, sel = case
+    s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos = _moa_case(name, T, d, E, nh, dh, n_seq, L, "mixed", mode, **sel)
+    if order == "round":
+        seq = (np.arange(T) % n_seq).astype(np.int32)
+    else:                                          # one decoding token per sequence but the last, whose prompt is the rest
+        seq = np.minimum(np.arange(T), n_seq - 1).astype(np.int32)
+        pos[n_seq - 1:] = np.arange(T - n_seq + 1)
+        assert pos.max() < L
+    e, er = _run(s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos, nh, 1.0 / math.sqrt(dh), sample=200)
+    assert er <= TOL_BF16, (e, er)
