@@ -101,8 +101,8 @@ typedef void* dsmoe_stream;
 const char* dsmoe_status_string(dsmoe_status s);
 
 /* Bytes of scratch for this desc.  A call takes one of two kinds of path, and their buffers overlap:
- * the plain path (fp32 layers, or no packed weights: grouped copy of the tokens, fp32 hidden
- * activations, expert outputs) and the tensor-core paths (packed bf16 weights: bf16 hidden activations
+ * the plain path (fp32 layers, or no packed weights: fp32 hidden activations, expert outputs) and
+ * the tensor-core paths (packed bf16 weights: bf16 hidden activations
  * and an fp32 running sum of [T,d]).
  *   dsmoe_workspace_size         enough for any call with this desc (the larger of the two)
  *   dsmoe_workspace_size_packed  enough for dsmoe_expert_mlp / dsmoe_layer_forward when `packed` is

@@ -50,8 +50,7 @@ WsLayout ws_layout(const dsmoe_layer_desc& p) {
     L.token_rows = take(T * (size_t)width_of(p) * 4);
     L.stage_total = off;
     const size_t big0 = off;
-    // plain path: grouped copy of the tokens, fp32 hidden activations, expert outputs
-    L.xp = take(amax * p.d * es);
+    // plain path: fp32 hidden activations, expert outputs
     L.h_plain = take(amax * p.H * 4);
     L.yp = take(amax * p.d * es);
     L.total_plain = off;

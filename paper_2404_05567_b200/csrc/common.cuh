@@ -95,14 +95,14 @@ static inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; 
 // Byte offsets of every internal buffer inside the caller's workspace.  The small per-token and per-assignment
 // index buffers come first (`stage_total` bytes: all that dsmoe_select and dsmoe_permute touch); the large
 // activation buffers follow and overlap between the execution paths, of which a call takes exactly one:
-//   plain (fp32-FMA GEMMs)     xp, h (fp32), yp
+//   plain (fp32-FMA GEMMs)     h (fp32), yp
 //   tensor-core paths          h (bf16: grouped [Amax,H]; dense and small-T [T,E*H]), acc (grouped: fp32 [T,d] running
 //                              sum of the expert outputs), partial (small-T)
 // total_packed = bytes a call with packed weights needs; total = the maximum over both kinds of call.
 struct WsLayout {
     size_t scores, mask, k_t, counts, offsets, chunk_prefix, batch_k, sync, tile_done, mi, row_token, row_gate, token_rows;
     size_t stage_total;
-    size_t xp, h_plain, yp;                 // plain path
+    size_t h_plain, yp;                     // plain path
     size_t h, acc, partial, bwd;            // tensor-core paths
     size_t total_plain, total_packed, total;
 };

@@ -113,3 +113,12 @@ def test_misaligned_weights_and_workspaces_are_rejected_wherever_they_are_read()
     for off in (2, 4):                                                                  # sums in double precision
         odd = ctypes.c_void_p(4096 + off)
         assert L.dsmoe_mi_loss(ctypes.byref(plain_shape), fake, fake, z, odd, big, z) == 3
+
+
+def test_workspace_of_the_plain_path_holds_what_it_uses():
+    """Index buffers, fp32 hidden activations and expert outputs; the tokens are gathered from x itself, not copied."""
+    for T, d, H, E, dtype, es in ((512, 1024, 256, 8, dm.F32, 4), (300, 2048, 72, 16, dm.BF16, 2)):
+        desc = dm.make_desc(T, d, H, E, dtype, dm.SELECT_TOPK, K=2)
+        rows = dm.amax(desc)
+        used = dm.dsmoe_workspace_size_stages(desc) + rows * H * 4 + rows * d * es
+        assert used <= dm.dsmoe_workspace_size(desc) <= max(used, dm.dsmoe_workspace_size_packed(desc) if H % 64 == 0 and es == 2 else 0) + 2 * 256
