@@ -252,13 +252,14 @@ def kernels_per_step(s, decode):
     """Launches of this library's kernels in one dsmoe_layer_forward (memsets are not kernels)."""
     if decode:
         return 1                                   # small_layer_kernel
-    router = 3 if s.T > 256 else 1                 # split Wr, logits GEMM, softmax+select | one router kernel
     if s.mode == gi.MODE_ALL:
-        return router + 2                          # up, down
-    # chunk count, finalize, permute index, up, down, and the aggregation unless it runs inside the down-projection
+        return 3                                   # router, up, down
+    # router, row indices (counts and scan inside up to 16384 tokens), up, down, and the aggregation unless it runs inside the
+    # down-projection; Threshold-TopK selects again (batch K, selection) and counts the chunks itself
     fused = s.fuse_combine == 1 or (s.fuse_combine == 0 and s.mode == gi.MODE_TOPK and s.H >= 1024 and
                                     s.T * min(s.K, s.E) >= 1024 * s.E)        # the library's rule (dsmoe.h)
-    return router + 3 + 2 + (0 if fused else 1)
+    grouping = (2 if s.T > 16384 else 1) + (3 + (s.T > 256) if s.mode == gi.MODE_THRESHOLD_TOPK else 0)
+    return 1 + grouping + 2 + (0 if fused else 1)
 
 
 def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, sampler_index=0, graph=False):
@@ -613,13 +614,16 @@ def run_moa(name: str, steps: int, warmup: int, sampler_index=0):
         gbs = (weight_bytes + kv_bytes) / (float(durs.sum()) * 1e-3) / 1e9
         head = dict(bound="hbm", achieved=gbs, peak=P["hbm"], unit="GB/s", peak_source=P["source"] + " (copy bandwidth)",
                     frac=gbs / P["hbm"], frac_nominal=gbs / NOMINAL["hbm"])
-    roof = dict(head, kernel="umma_gemm_kernel (projections) + moa_attention_mma_kernel", roofline_ms=max(t_flop, t_byte) * 1e3,
+    roof = dict(head, kernel="umma_gemm_kernel (projections) + " + ("moa_attention_mma_kernel" if w["layout"] == "decode" else
+                                                                         "moa_attention_shared_kernel"), roofline_ms=max(t_flop, t_byte) * 1e3,
                 frac_of_roofline_time=max(t_flop, t_byte) / (float(durs.sum()) * 1e-3),
                 step_frac_of_roofline_time=max(t_flop, t_byte) / (ms * 1e-3), step_frac=max(t_flop, t_byte) / (ms * 1e-3),
                 algorithmic_per_launch=proj_flops / 2, attention_flops=att_flops, kv_bytes=kv_bytes, traffic=None,
                 kernel_ms_per_step=float(durs.sum()), ms_per_step_with_events=ms, launch_ms_each=[float(v) for v in durs],
                 launches_per_step=3)
-    return dict(workload=name, value=T / (ms * 1e-3), unit="tokens/s", ms_per_step=ms, steps=steps, roofline=roof, clocks=clocks,
+    # router, row indices, query projection, attention, output projection; few tokens also the sums of the projection's pieces and
+    # of a token's experts
+    return dict(workload=name, library_launches=7 if w["layout"] == "decode" else 5, value=T / (ms * 1e-3), unit="tokens/s", ms_per_step=ms, steps=steps, roofline=roof, clocks=clocks,
                 assignments=A, active_experts=E, config=dict(w))
 
 
@@ -782,7 +786,7 @@ def main():
         r = run_training_side(steps, warmup) if name == "c4_backward" else run_moa(name, steps, warmup)
         print(json.dumps(dict(metric="dense_backward_tokens_per_s" if name == "c4_backward" else "moa_layer_tokens_per_s",
                               n_gpus=1, warmup=max(warmup, 3), higher_is_better=True, dtype="bf16", data="synthetic",
-                              gpu_launches=(3 if name == "c4_backward" else 11) * steps, **r)))
+                              gpu_launches=(3 if name == "c4_backward" else r.pop("library_launches")) * steps, **r)))
         return
     if args.fuse_combine is not None:
         for k in WORKLOADS:

@@ -312,7 +312,11 @@ dsmoe_status dsmoe_dense_backward(const dsmoe_layer_desc* desc, const void* x, c
  * It is the feed-forward layer's pipeline with attention in place of GeLU: desc describes it with E = the number of
  * attention experts and H = n_head * d_head; router, selection (desc->mode ...), grouping and the router-weighted sum
  * are those of dsmoe_layer_forward.  Eq. 7 prints no scale under the softmax: `scale` is the caller's (1/sqrt(d_head)
- * in the usual form).  No biases.  Queries and attention outputs are rounded to bf16 between the steps.
+ * in the usual form).  No biases.  Queries and attention outputs are rounded to bf16 between the steps.  desc->fuse_combine as
+ * for dsmoe_layer_forward, with one more form that 0 may choose (top-K or all experts, many tokens, experts that overlap
+ * enough): the gate multiplies the attention output in fp32 before its one rounding, and projection and sum are one GEMM over
+ * the experts side by side.  Its distance from 64 bits was 0.8 to 3.2 % larger than with 1 or 2 (3.0e-3 of the output's norm),
+ * which keep the gate in the epilogue.
  *
  * args (host struct, read during the call): Kc, Vc  device, bf16 [n_seq][n_head][L][d_head]; tok_seq  device int32 [T],
  * the sequence of each token, or NULL (all 0); pos  device int32 [T], 0 <= pos[t] < L.

@@ -56,7 +56,9 @@ __device__ __forceinline__ void report_status(int32_t* dev_status, int32_t code)
 }
 
 int sm_count();
-// Grids of more than one wave are launched the ordinary way: each of their blocks would pay for its chain_wait().
+// Grids of more threads than the SMs hold are launched the ordinary way: most of their blocks would pay for a chain_wait() that
+// has nothing left to wait for.  (Threads are all that is looked at: kernels that fill an SM with shared memory or registers
+// stay chained over several waves.)
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                                   int cluster, Args... args) {

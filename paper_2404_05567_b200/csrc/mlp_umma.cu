@@ -1979,7 +1979,8 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
                                                    args, smem, s));
     } else {
         // (the large dense launches are not chained: no gap to speak of, and 1 % slower with it, 3682 against 3732 us for the
-        // dense layer at 16384 tokens)
+        // dense layer at 16384 tokens; grouped ones all are: 300 tokens of 2048 / 1024 93.7 against 98.7 us for the layer, 8192
+        // of 3072 / 1536 alike, 7001 of 4096 / 512 428 against 425)
         if (P.mode == GEMM_GROUPED || P.rows <= kChainMaxRows)
             DSMOE_CUDA_TRY(launch_chained(umma_gemm_kernel<false>, grid, threads, smem, s, a, b, P));
         else {
