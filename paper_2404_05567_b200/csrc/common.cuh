@@ -61,7 +61,7 @@ int sm_count();
 // stay chained over several waves.)
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                                  int cluster, Args... args) {
+                                                  int cluster, bool chain, Args... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -74,7 +74,7 @@ static inline cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3
         at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
         ++n;
     }
-    if ((size_t)grid.x * grid.y * grid.z * block.x <= (size_t)sm_count() * 2048) {
+    if (chain && (size_t)grid.x * grid.y * grid.z * block.x <= (size_t)sm_count() * 2048) {
         at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[n].val.programmaticStreamSerializationAllowed = 1;
         ++n;
@@ -88,7 +88,13 @@ static inline cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                          Args... args) {
-    return launch_chained_clusters(kernel, grid, block, smem, s, 1, args...);
+    return launch_chained_clusters(kernel, grid, block, smem, s, 1, true, args...);
+}
+// chain == false: the ordinary launch of a kernel that can be chained (its chain_wait() then returns at once)
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_chained_if(bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                            Args... args) {
+    return launch_chained_clusters(kernel, grid, block, smem, s, 1, chain, args...);
 }
 
 dsmoe_status check_desc(const dsmoe_layer_desc* desc);

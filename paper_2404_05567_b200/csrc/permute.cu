@@ -386,21 +386,27 @@ dsmoe_status launch_combine(const dsmoe_layer_desc& p, const void* yp, const flo
     // with few tokens a row's columns are shared out over several blocks (blockIdx.y), enough to cover the SMs
     const int col_blocks = ceil_div(p.d / (yp_f32 || p.dtype != DSMOE_BF16 ? 4 : 8), 128);
     const dim3 grid(p.T, (unsigned)(std::max(1, std::min(col_blocks, 1024 / p.T))));
+    // Set up while the down-projection's last tiles still run, all of these small blocks would land on the SMs that have finished,
+    // up to 16 on each, and the aggregation would run on that part of the chip: 1280 tokens of 3072, 1536 wide, top-12: the layer
+    // 439 us chained, 389 not (1600: 486, 451; 700 tokens of 2048, 1024 wide, by threshold 148, 131; 1024 of 3072, 384 wide, top-6
+    // 124, 105; 150 of 2048, 256 wide, top-6 65.1, 67.2, the most that any shape lost; beyond 2368 tokens the grid is too
+    // large to be chained in any case).  Decoding batches stay chained: few blocks, and the launch gap is a part of their time.
+    const bool chain = p.T <= kSmallMaxT;
     if (yp_f32 && p.dtype == DSMOE_BF16 && !p.out_fp32) {
-        DSMOE_CUDA_TRY(launch_chained(combine_f32_kernel<true>, grid, 128, 0, s,
+        DSMOE_CUDA_TRY(launch_chained_if(chain, combine_f32_kernel<true>, grid, 128, 0, s,
             static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     } else if (yp_f32) {
-        DSMOE_CUDA_TRY(launch_chained(combine_f32_kernel<false>, grid, 128, 0, s,
+        DSMOE_CUDA_TRY(launch_chained_if(chain, combine_f32_kernel<false>, grid, 128, 0, s,
             static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     } else if (p.dtype == DSMOE_BF16) {
         if (p.out_fp32)
-            DSMOE_CUDA_TRY(launch_chained(combine_bf16_kernel<true>, grid, 128, 0, s,
+            DSMOE_CUDA_TRY(launch_chained_if(chain, combine_bf16_kernel<true>, grid, 128, 0, s,
                 static_cast<const uint4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
         else
-            DSMOE_CUDA_TRY(launch_chained(combine_bf16_kernel<false>, grid, 128, 0, s,
+            DSMOE_CUDA_TRY(launch_chained_if(chain, combine_bf16_kernel<false>, grid, 128, 0, s,
                 static_cast<const uint4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     } else {
-        DSMOE_CUDA_TRY(launch_chained(combine_f32_kernel<false>, grid, 128, 0, s,
+        DSMOE_CUDA_TRY(launch_chained_if(chain, combine_f32_kernel<false>, grid, 128, 0, s,
             static_cast<const float4*>(yp), row_gate, token_rows, k_t, out, p.d, W, amax));
     }
     return DSMOE_OK;

@@ -311,7 +311,7 @@ dsmoe_status launch_clusters(const dsmoe_layer_desc& p, const CUtensorMap& mX, c
         DSMOE_CUDA_TRY(cudaFuncSetAttribute(router_umma_kernel<EP, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)router_umma_smem<EP>()));
         attr[dev] = true;
     }
-    DSMOE_CUDA_TRY(launch_chained_clusters(router_umma_kernel<EP, C>, ceil_div(p.T, kRuM) * C, kRuThreads, router_umma_smem<EP>(), s, C,
+    DSMOE_CUDA_TRY(launch_chained_clusters(router_umma_kernel<EP, C>, ceil_div(p.T, kRuM) * C, kRuThreads, router_umma_smem<EP>(), s, C, true,
         mX, Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d, SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr},
         dev_status));
     return DSMOE_OK;

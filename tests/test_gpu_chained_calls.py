@@ -95,6 +95,10 @@ CALLS = {
     "layer_fused_sum": lambda: _layer(T=700, d=512, H=256, E=4, dtype="bf16", mode=gi.MODE_TOPK, K=2, fuse_combine=1),
     "layer_threshold_topk": lambda: _layer(T=513, d=256, H=128, E=16, dtype="bf16", mode=gi.MODE_THRESHOLD_TOPK, eps=0.03),
     "layer_dense": lambda: _layer(T=700, d=256, H=128, E=8, dtype="bf16", mode=gi.MODE_ALL),
+    # either side of the number of tokens beyond which the aggregation is launched the ordinary way
+    "layer_plain_128": lambda: _layer(T=128, d=256, H=128, E=8, dtype="f32", mode=gi.MODE_TOPK, K=2),
+    "layer_plain_129": lambda: _layer(T=129, d=256, H=128, E=8, dtype="f32", mode=gi.MODE_TOPK, K=2),
+    "layer_grouped_129": lambda: _layer(T=129, d=512, H=256, E=32, dtype="bf16", mode=gi.MODE_TOPK, K=4, fuse_combine=0),
     "stages_f32": lambda: _stages(T=77, d=136, H=72, E=5, dtype="f32", mode=gi.MODE_TOPK, K=2),
     "stages_bf16": lambda: _stages(T=517, d=256, H=128, E=33, dtype="bf16", mode=gi.MODE_THRESHOLD, eps=0.02),
     "stages_threshold_topk": lambda: _stages(T=300, d=128, H=64, E=16, dtype="bf16", mode=gi.MODE_THRESHOLD_TOPK, eps=0.05),
