@@ -248,6 +248,17 @@ def drop_weights(torch, keep_shape=None):
     torch.cuda.empty_cache()
 
 
+def sums_inside(s):
+    """Whether the down-projection also aggregates (the library's rule, dsmoe.h)."""
+    return s.fuse_combine == 1 or (s.fuse_combine == 0 and s.mode == gi.MODE_TOPK and s.H >= 1024 and
+                                   s.T * min(s.K, s.E) >= 1024 * s.E)
+
+
+def mlp_launches(s):
+    """Launches of the expert MLPs: one (grouped_layer_kernel) where the library chooses and the aggregation is a kernel of its own."""
+    return 1 if s.mode != gi.MODE_ALL and s.fuse_combine == 0 and not sums_inside(s) else 2
+
+
 def kernels_per_step(s, decode):
     """Launches of this library's kernels in one dsmoe_layer_forward (memsets are not kernels)."""
     if decode:
@@ -256,10 +267,9 @@ def kernels_per_step(s, decode):
         return 3                                   # router, up, down
     # router, row indices (counts and scan inside up to 16384 tokens), up, down, and the aggregation unless it runs inside the
     # down-projection; Threshold-TopK selects again (batch K, selection) and counts the chunks itself
-    fused = s.fuse_combine == 1 or (s.fuse_combine == 0 and s.mode == gi.MODE_TOPK and s.H >= 1024 and
-                                    s.T * min(s.K, s.E) >= 1024 * s.E)        # the library's rule (dsmoe.h)
+    fused = sums_inside(s)
     grouping = (2 if s.T > 16384 else 1) + (3 + (s.T > 256) if s.mode == gi.MODE_THRESHOLD_TOPK else 0)
-    return 1 + grouping + 2 + (0 if fused else 1)
+    return 1 + grouping + mlp_launches(s) + (0 if fused else 1)
 
 
 def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, sampler_index=0, graph=False):
@@ -347,7 +357,7 @@ def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, s
         torch.cuda.synchronize()
 
     calls_per_step = n_layers if loop else 1
-    timed_per_call = 1 if decode else 2
+    timed_per_call = 1 if decode else mlp_launches(s)
     run_step = step
     if graph:
         # the whole step as one CUDA graph (launch overhead out of the way)
@@ -433,16 +443,16 @@ def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, s
             roof["step_frac"] = weight_bytes / step_s / 1e9 / roof["peak"]
             roof["algorithmic_per_launch"] = weight_bytes / calls_per_step      # loop workloads: the mean over the layers
         else:
-            # both projections: two launches of umma_gemm_kernel per step.  Peak: the burst figure unless the clock
+            # both projections: one launch of grouped_layer_kernel or two of umma_gemm_kernel per step.  Peak: the burst figure unless the clock
             # samples of this very region show the power cap (then the sustained one applies)
             kind = "sustained" if capped else "burst"
             peak = P["tf_sustained"] if capped else P["tf_burst"]
             ach = flops / (kernel_ms * 1e-3) / 1e12
             roof = dict(bound="tensor", achieved=ach, peak=peak, unit="TFLOP/s",
                         peak_source=f"{P['source']} ({kind} bf16: clocks of this region {'show' if capped else 'show no'} power cap)",
-                        kernel="umma_gemm_kernel", frac=ach / peak, frac_burst=ach / P["tf_burst"],
+                        kernel="umma_gemm_kernel" if timed_per_call == 2 else "grouped_layer_kernel", frac=ach / peak, frac_burst=ach / P["tf_burst"],
                         frac_sustained=ach / P["tf_sustained"], frac_nominal=ach / NOMINAL["tf"],
-                        step_frac=flops / step_s / 1e12 / peak, algorithmic_per_launch=flops / 2)
+                        step_frac=flops / step_s / 1e12 / peak, algorithmic_per_launch=flops / timed_per_call)
             # where few assignments are left the weights' bytes bound the step, not the flops: the roofline time is
             # the larger of the two
             t_flop, t_byte = flops / (peak * 1e12), weight_bytes / (P["hbm"] * 1e9)

@@ -92,7 +92,8 @@ typedef struct {
                                  2: the epilogue stores the gate-weighted outputs as fp32 rows and a
                                     second kernel adds a token's rows;
                                  0: the library chooses: 1 for a top-K selection with H >= 1024 and
-                                    T*K >= 1024*E (wide experts, many row tiles per expert), else 2. */
+                                    T*K >= 1024*E (wide experts, many row tiles per expert), else as 2
+                                    (bit for bit), with both projections in one launch. */
 } dsmoe_layer_desc;
 
 /* A void* stands for the caller's cudaStream_t so that this header needs no CUDA include. */

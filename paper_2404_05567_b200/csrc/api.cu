@@ -276,7 +276,14 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
         return launch_mlp_umma(p, nullptr, packed, offsets, ws + L.h, nullptr, dev_status, s, x, row_token, &cmb);
     }
     if (fast) {
-        // the down-projection's epilogue multiplies by the gate and stores fp32 rows; the aggregation only adds
+        // the down-projection's epilogue multiplies by the gate and stores fp32 rows; the aggregation only adds.  Both projections
+        // are one launch unless the caller asked for the separate ones (or a workspace of a few tokens has no room for its counters)
+        if (const GroupedScratch G = grouped_scratch(p, L); p.fuse_combine == 0 && G.fits) {
+            DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr,
+                                   counted, ZeroInts{reinterpret_cast<int*>(ws + G.sync), (long long)G.sync_ints}));
+            DSMOE_TRY(launch_grouped_layer(p, x, packed, offsets, row_token, row_gate, reinterpret_cast<float*>(ws + L.acc), ws, L, dev_status, s));
+            return launch_combine(p, ws + L.acc, nullptr, token_rows, k_t, out, s, true);
+        }
         DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr, counted));
         const CombineArgs gated{row_token, row_gate, nullptr, nullptr, nullptr, nullptr};
         DSMOE_TRY(launch_mlp_umma(p, nullptr, packed, offsets, ws + L.h, ws + L.acc, dev_status, s, x, row_token, &gated));

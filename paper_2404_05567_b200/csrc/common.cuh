@@ -29,7 +29,7 @@ constexpr int kSmallMaxCtas = 192;   // upper bound on that path's grid (sizes i
     } while (0)
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+__host__ __device__ static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 static inline size_t elem_size(int dtype) { return dtype == DSMOE_BF16 ? 2 : 4; }
 static inline int width_of(const dsmoe_layer_desc& p) {
@@ -121,7 +121,7 @@ WsLayout ws_layout(const dsmoe_layer_desc& p);
 constexpr int kMaxDeviceSlots = 64;
 struct DeviceState {
     int sm_count = 0;
-    bool attr_gemm = false, attr_small = false, attr_router_f32 = false, attr_router_bf16 = false;
+    bool attr_gemm = false, attr_small = false, attr_grouped = false, attr_router_f32 = false, attr_router_bf16 = false;
     int max_pairs = -1;   // CTA pairs of umma_gemm_kernel that can be resident at once; -1 not asked yet, 0 pairs unavailable
 };
 dsmoe_status device_state(DeviceState** out, int* device = nullptr);   // of the current device
@@ -141,16 +141,22 @@ dsmoe_status launch_finalize(const dsmoe_layer_desc& p, const uint64_t* mask, in
                              int32_t* offsets, int32_t* chunk_prefix, int32_t* counts_out, cudaStream_t s);
 
 // ---- permute.cu
+// Counters of a later launch that the row-index kernel sets to zero on its way
+struct ZeroInts {
+    int* at = nullptr;
+    long long n = 0;
+};
 // zero_out (optional): the layer output [T,d]; rows of tokens that selected no expert are set to zero
 dsmoe_status launch_permute(const dsmoe_layer_desc& p, const void* x, const float* scores,
                             const uint64_t* mask, const int32_t* offsets, const int32_t* chunk_prefix,
                             int32_t* row_token, float* row_gate, int32_t* token_rows, void* xp,
-                            cudaStream_t s, void* zero_out = nullptr);
+                            cudaStream_t s, void* zero_out = nullptr, const ZeroInts& zero = ZeroInts{});
 // Grouping for the fused layers: counts, offsets and the row indices of launch_finalize + launch_permute (without a
 // grouped copy of x).  chunk_counts_ready: chunk_prefix already holds the chunks' counts (the router wrote them).
 dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const uint64_t* mask, int32_t* counts,
                           int32_t* offsets, int32_t* chunk_prefix, int32_t* counts_out, int32_t* row_token,
-                          float* row_gate, int32_t* token_rows, cudaStream_t s, void* zero_out, bool chunk_counts_ready);
+                          float* row_gate, int32_t* token_rows, cudaStream_t s, void* zero_out, bool chunk_counts_ready,
+                          const ZeroInts& zero = ZeroInts{});
 // Selection statistics (see dsmoe_stats)
 dsmoe_status launch_stats(const dsmoe_layer_desc& p, const float* scores, const uint64_t* mask,
                           dsmoe_selection_stats* stats, cudaStream_t s);
@@ -238,6 +244,18 @@ dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const vo
                              void* hbuf, void* yp, int32_t* dev_status, cudaStream_t s, const void* x = nullptr,
                              const int32_t* row_token = nullptr, const CombineArgs* cmb = nullptr,
                              const MoaCore* moa = nullptr);
+
+// ---- mlp_grouped.cu : both projections of the sparse expert MLPs in one launch
+// Where its counters lie in the workspace (zeroed beforehand: ZeroInts); fits: there is room for them
+struct GroupedScratch {
+    size_t sync, sync_ints;
+    bool fits;
+};
+GroupedScratch grouped_scratch(const dsmoe_layer_desc& p, const WsLayout& L);
+// rows [Amax, d] fp32: the gate-weighted expert outputs
+dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, const void* packed, const int32_t* offsets,
+                                  const int32_t* row_token, const float* row_gate, float* rows, char* ws, const WsLayout& L,
+                                  int32_t* dev_status, cudaStream_t s);
 
 // ---- moa.cu : the attention step of the mixture-of-attention-heads layer
 bool moa_supported(const dsmoe_layer_desc& p, int n_head, int L);

@@ -30,9 +30,10 @@ __global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint6
                                                             int32_t* __restrict__ counts, int32_t* __restrict__ counts_out,
                                                             int32_t* __restrict__ row_token, float* __restrict__ row_gate,
                                                             int32_t* __restrict__ token_rows, int T, int E, int W,
-                                                            int64_t amax, uint4* __restrict__ zero_out, int row_vecs) {
+                                                            int64_t amax, uint4* __restrict__ zero_out, int row_vecs, const ZeroInts zero) {
     chain_next();
     chain_wait();
+    for (long long i = (long long)blockIdx.x * kPermThreads + threadIdx.x; i < zero.n; i += (long long)gridDim.x * kPermThreads) zero.at[i] = 0;
     __shared__ uint64_t mask_s[kPermChunks * kChunk];
     __shared__ int before_s[kMaxExperts], total_s[kMaxExperts], base_s[kPermChunks][kMaxExperts];
     __shared__ int cnt_s[SCAN == 2 ? kCountInBlockChunks : 1][kMaxExperts];
@@ -334,14 +335,14 @@ __global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16
 
 dsmoe_status launch_permute(const dsmoe_layer_desc& p, const void* x, const float* scores, const uint64_t* mask,
                             const int32_t* offsets, const int32_t* chunk_prefix, int32_t* row_token, float* row_gate,
-                            int32_t* token_rows, void* xp, cudaStream_t s, void* zero_out) {
+                            int32_t* token_rows, void* xp, cudaStream_t s, void* zero_out, const ZeroInts& zero) {
     if (p.T == 0) return DSMOE_OK;
     const int nchunks = ceil_div(p.T, kChunk);
     const int64_t amax = (int64_t)amax_of(p);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
     DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<0>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
         mask, scores, const_cast<int32_t*>(offsets), chunk_prefix, nullptr, nullptr, row_token, row_gate,
-        token_rows, p.T, p.E, width_of(p), amax, static_cast<uint4*>(zero_out), row_vecs));
+        token_rows, p.T, p.E, width_of(p), amax, static_cast<uint4*>(zero_out), row_vecs, zero));
     if (xp) {
         const int vec_per_row = (int)((size_t)p.d * elem_size(p.dtype) / 16);
         const int grid = (int)(amax / 8 + 1 < 148 * 16 ? amax / 8 + 1 : 148 * 16);
@@ -357,24 +358,25 @@ constexpr int kScanInBlockChunks = 512;
 
 dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const uint64_t* mask, int32_t* counts,
                           int32_t* offsets, int32_t* chunk_prefix, int32_t* counts_out, int32_t* row_token,
-                          float* row_gate, int32_t* token_rows, cudaStream_t s, void* zero_out, bool chunk_counts_ready) {
+                          float* row_gate, int32_t* token_rows, cudaStream_t s, void* zero_out, bool chunk_counts_ready,
+                          const ZeroInts& zero) {
     const int nchunks = ceil_div(p.T, kChunk);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
     if (nchunks > 0 && nchunks <= kCountInBlockChunks) {
         DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<2>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
             mask, scores, offsets, nullptr, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
-            width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs));
+            width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs, zero));
         return DSMOE_OK;
     }
     if (!chunk_counts_ready) DSMOE_TRY(launch_chunk_counts(p, mask, chunk_prefix, s));
     if (nchunks == 0 || nchunks > kScanInBlockChunks) {
         DSMOE_TRY(launch_chunk_scan(p, counts, offsets, chunk_prefix, counts_out, s));
         return launch_permute(p, nullptr, scores, mask, offsets, chunk_prefix, row_token, row_gate, token_rows, nullptr, s,
-                              zero_out);
+                              zero_out, zero);
     }
     DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<1>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
         mask, scores, offsets, chunk_prefix, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
-        width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs));
+        width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs, zero));
     return DSMOE_OK;
 }
 

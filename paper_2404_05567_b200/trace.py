@@ -74,6 +74,19 @@ def gemm_waits(a):
     for _ in range(a.reps):
         dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, pk, out, None, counts, ws, status)
     torch.cuda.synchronize()
+    if a.gemm == "paper6b" and a.fuse == 0:        # both projections in one launch
+        buf = (ctypes.c_longlong * (192 * 8))()
+        if dm.lib().dsmoe_grouped_trace_read(buf) != 0:
+            raise RuntimeError("dsmoe_grouped_trace_read failed")
+        g = np.array(buf[:], dtype=np.float64).reshape(192, 8)
+        g = g[g[:, 0] > 0]
+        at = (g[:, :4] - g[:, 0].min()) / 1e3
+        print(f"{a.gemm}: T={T} d={d} H={H} E={E}, device status {int(status.item())}\n-- grouped_layer_kernel, last launch, {len(g)} CTAs: median / min / max")
+        for k, name in enumerate(("MMA issuer starts", "last up tile issued", "last tile issued", "epilogue done")):
+            print(f"{name:28s} {np.median(at[:, k]):9.2f} {at[:, k].min():9.2f} {at[:, k].max():9.2f} us")
+        for k, name in enumerate(("issuer, operands of up tiles", "issuer, operands of down tiles", "issuer, accumulator", "producer, rows of h"), 4):
+            print(f"waits: {name:30s} {np.median(g[:, k]):9.0f} {g[:, k].min():9.0f} {g[:, k].max():9.0f} clk")
+        return
     buf = (ctypes.c_longlong * (2 * 192 * 8))()
     if dm.lib().dsmoe_gemm_trace_read(buf) != 0:
         raise RuntimeError("dsmoe_gemm_trace_read failed")

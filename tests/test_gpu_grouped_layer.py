@@ -1,0 +1,82 @@
+"""Both projections of the sparse expert MLPs in one launch (fuse_combine = 0) against the two separate launches (2), which the oracle
+tests cover: the same tiles, the same order of additions, so the same bits -- where the dealing out of tiles can go wrong:
+one and several rounds of up tiles, incomplete ones of every kind, experts of 0, 1, 128 and 129 rows, ragged column ranges, a
+reduction shorter than the ring, more tiles per CTA than one list holds (GPU required)."""
+import pytest
+import torch
+
+import paper_2404_05567_b200 as dm
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # T, d, H, E, mode, K, eps (normalised), out_fp32
+    (129, 64, 64, 3, dm.SELECT_TOPK, 1, 0.0, 0),              # fewer tiles than CTAs, one reduction block
+    (300, 320, 192, 8, dm.SELECT_TOPK, 3, 0.0, 1),            # ragged last column ranges of both projections
+    (1000, 2048, 256, 32, dm.SELECT_THRESHOLD, 0, 0.9, 0),    # one round of up tiles
+    (2000, 256, 1408, 64, dm.SELECT_THRESHOLD, 0, 2.5, 0),    # several rounds, few down tiles, empty experts
+    (4096, 1024, 512, 32, dm.SELECT_TOPK, 6, 0.0, 0),         # several rounds, the last incomplete
+    (5000, 6144, 64, 16, dm.SELECT_TOPK, 4, 0.0, 0),          # more than 32 down tiles per CTA
+    (6000, 128, 6144, 16, dm.SELECT_THRESHOLD, 0, 0.9, 1),    # more than 32 up tiles per CTA, one round or two of down tiles
+    (700, 512, 256, 5, dm.SELECT_THRESHOLD, 0, 1e9, 0),       # nothing selected
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"T{c[0]}-d{c[1]}-H{c[2]}-E{c[3]}")
+def test_one_launch_equals_two(case):
+    T, d, H, E, mode, K, eps, out_fp32 = case
+    g = torch.Generator(device="cuda").manual_seed(T)
+    randn = lambda *shape, dtype=torch.bfloat16: torch.randn(*shape, generator=g, device="cuda", dtype=dtype)
+    x, Wr = randn(T, d), randn(d, E, dtype=torch.float32) * (1.5 / d ** 0.5)
+    W1, W2 = randn(E, d, H) * 0.05, randn(E, H, d) * 0.05
+    outs = []
+    for fuse in (2, 0):
+        desc = dm.make_desc(T, d, H, E, dm.BF16, mode, eps, 1, max(K, 1), 0, out_fp32, fuse)
+        packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+        dm.dsmoe_pack_weights(desc, W1, W2, packed)
+        ws = torch.full((dm.dsmoe_workspace_size_packed(desc),), 0x5a, dtype=torch.uint8, device="cuda")     # counters are not zero by chance
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        out = torch.full((T, d), float("nan"), dtype=torch.float32 if out_fp32 else torch.bfloat16, device="cuda")
+        counts = torch.zeros(E, dtype=torch.int32, device="cuda")
+        for _ in range(2):                                                                                    # ... nor left over
+            dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, counts, ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        outs.append((out, counts))
+    assert torch.equal(outs[0][1], outs[1][1])
+    assert torch.equal(outs[0][0], outs[1][0])
+    if eps == 1e9:
+        assert not outs[1][0].any()
+
+
+def test_rows_around_a_tile():
+    """Experts of exactly 0, 1, 127, 128, 129 and 257 rows."""
+    rows = [0, 1, 127, 128, 129, 257]
+    E, d, H, T = len(rows), 128, 192, sum(rows)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    # the first E columns of x choose the expert (their weights are scaled out of the experts' way)
+    owner = torch.cat([torch.full((n,), e) for e, n in enumerate(rows)])[torch.randperm(T, generator=torch.Generator().manual_seed(3))].cuda()
+    x = torch.randn(T, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    x[:, :E] = torch.nn.functional.one_hot(owner, E).to(x.dtype) * 4
+    Wr = torch.zeros(d, E, device="cuda")
+    Wr[:E] = torch.eye(E, device="cuda") * 5
+    W1 = (torch.randn(E, d, H, generator=g, device="cuda") * 0.05).bfloat16()
+    W2 = (torch.randn(E, H, d, generator=g, device="cuda") * 0.05).bfloat16()
+    outs = []
+    for fuse in (2, 0):
+        desc = dm.make_desc(T, d, H, E, dm.BF16, dm.SELECT_TOPK, 0.0, 0, 1, 0, 1, fuse)
+        packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+        dm.dsmoe_pack_weights(desc, W1, W2, packed)
+        ws = torch.empty(dm.dsmoe_workspace_size_packed(desc), dtype=torch.uint8, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        out = torch.empty(T, d, device="cuda")
+        counts = torch.zeros(E, dtype=torch.int32, device="cuda")
+        dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, counts, ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and counts.tolist() == rows
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])
+    # ... and the value itself, in fp32 from the same bf16 operands: h is rounded to bf16 (2^-9) before the second product
+    want = torch.stack([torch.nn.functional.gelu(x[t].float() @ W1[e].float()) @ W2[e].float() for t, e in enumerate(owner.tolist())])
+    gate = torch.softmax(x.float() @ Wr, dim=1).gather(1, owner[:, None])
+    assert (outs[1] - gate * want).norm() <= 6e-3 * (gate * want).norm()
