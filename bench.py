@@ -262,7 +262,7 @@ def mlp_launches(s):
 def kernels_per_step(s, decode):
     """Launches of this library's kernels in one dsmoe_layer_forward (memsets are not kernels)."""
     if decode:
-        return 1                                   # small_layer_kernel
+        return 1                                   # few_tokens_kernel or small_layer_kernel
     if s.mode == gi.MODE_ALL:
         return 3                                   # router, up, down
     # router, row indices (counts and scan inside up to 16384 tokens), up, down, and the aggregation unless it runs inside the
@@ -437,7 +437,7 @@ def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, s
         if decode:
             # selected experts' weights (W1 and W2), each byte once, all inside one launch of small_layer_kernel
             roof = dict(bound="hbm", achieved=weight_bytes / (kernel_ms * 1e-3) / 1e9, peak=P["hbm"], unit="GB/s",
-                        peak_source=P["source"] + " (copy bandwidth)", kernel="small_layer_kernel")
+                        peak_source=P["source"] + " (copy bandwidth)", kernel="few_tokens_kernel" if s.T < 8 else "small_layer_kernel")
             roof["frac"] = roof["achieved"] / roof["peak"]
             roof["frac_nominal"] = roof["achieved"] / NOMINAL["hbm"]
             roof["step_frac"] = weight_bytes / step_s / 1e9 / roof["peak"]

@@ -243,6 +243,8 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
     float* row_gate = reinterpret_cast<float*>(ws + L.row_gate);
     int32_t* token_rows = reinterpret_cast<int32_t*>(ws + L.token_rows);
 
+    if (fast && few_supported(p, packed))
+        return launch_layer_few(p, x, Wr, br, packed, scores, mask, k_t, counts_out, out, ws, L, dev_status, s);
     if (fast && small_supported(p))
         return launch_layer_small(p, x, Wr, br, packed, scores, mask, k_t, counts_out, out, ws, L, dev_status, s);
 

@@ -121,7 +121,7 @@ WsLayout ws_layout(const dsmoe_layer_desc& p);
 constexpr int kMaxDeviceSlots = 64;
 struct DeviceState {
     int sm_count = 0;
-    bool attr_gemm = false, attr_small = false, attr_grouped = false, attr_router_f32 = false, attr_router_bf16 = false;
+    bool attr_gemm = false, attr_small = false, attr_grouped = false, attr_few = false, attr_router_f32 = false, attr_router_bf16 = false;
     int max_pairs = -1;   // CTA pairs of umma_gemm_kernel that can be resident at once; -1 not asked yet, 0 pairs unavailable
 };
 dsmoe_status device_state(DeviceState** out, int* device = nullptr);   // of the current device
@@ -262,6 +262,11 @@ bool moa_supported(const dsmoe_layer_desc& p, int n_head, int L);
 // qa [Amax, H] bf16: the grouped rows' queries on entry, their attention outputs on return
 dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, void* qa, const int32_t* row_token,
                                   const int32_t* token_rows, const int32_t* offsets, int32_t* dev_status, cudaStream_t s);
+// ---- few_tokens.cu : the whole layer for a handful of tokens, one cooperative launch
+bool few_supported(const dsmoe_layer_desc& p, const void* packed);
+dsmoe_status launch_layer_few(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, const void* packed,
+                              float* scores, uint64_t* mask, int32_t* k_t, int32_t* counts_out, void* out, char* ws, const WsLayout& L,
+                              int32_t* dev_status, cudaStream_t s);
 // Whole-layer paths that need no grouping (all experts selected, or few tokens).  *done = false
 // means "not taken": the caller continues with the grouped path.
 // Whole layer for few tokens (T <= 128) in one cooperative launch, router included.

@@ -32,6 +32,9 @@ SMALL_NAMES = {0: "CTA starts", 12: "router: first loads", 13: "router: slice su
                5: "producer: down-projection weights prefetched", 6: "producer: grid barrier passed", 8: "MMA issuer: first down-projection tile",
                9: "epilogue: partial sums written", 10: "last grid barrier passed", 11: "CTA ends"}
 
+FEW_NAMES = ("CTA starts", "router: at grid barrier", "router: grid barrier passed", "selected experts known", "up-projection multiplied (first warp)",
+             "hg written, at grid barrier", "grid barrier passed", "CTA ends")
+
 
 def build_trace_lib() -> str:
     out = os.path.join(PKG, "libdsmoe_trace.so")
@@ -144,6 +147,14 @@ def main():
     print(f"T={a.T} d={a.d} H={a.H} E={a.E}: {int((counts[:a.E] > 0).sum())} experts selected, device status {int(status.item())}")
     L = dm.lib()
     buf = (ctypes.c_ulonglong * (192 * 32))()
+    if a.T < 8 and L.dsmoe_few_trace_read(buf) == 0:          # few_tokens_kernel: [192][8] stamps
+        tr = np.frombuffer(buf, dtype=np.uint64)[:192 * 8].reshape(192, 8).astype(np.int64)
+        tr = tr[tr[:, 0] > 0]
+        print(f"-- few_tokens_kernel, last launch, {len(tr)} CTAs; microseconds after the first CTA's start: median / min / max")
+        for idx, name in enumerate(FEW_NAMES):
+            v = (tr[:, idx] - tr[:, 0].min()) / 1e3
+            print(f"{name:52s} {np.median(v):8.2f} {v.min():8.2f} {v.max():8.2f}")
+        return
     for reader, names in (("dsmoe_trace_read", SMALL_NAMES),):
         if not hasattr(L, reader) or getattr(L, reader)(buf) != 0:
             continue
