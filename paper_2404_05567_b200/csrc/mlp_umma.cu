@@ -79,7 +79,7 @@ constexpr int kFixBatch = 24;        // partial tiles a fix-up thread loads at o
 constexpr int kSmallInflightBytes = SMALL_RING_BYTES;
 static_assert(kSmallInflightBytes <= RING_BYTES, "in-flight bytes are ring bytes");
 #ifndef DSMOE_SMALL_L2_PREFETCH
-#define DSMOE_SMALL_L2_PREFETCH (384 * 1024)
+#define DSMOE_SMALL_L2_PREFETCH (192 * 1024)
 #endif
 constexpr int kSmallL2PrefetchBytes = DSMOE_SMALL_L2_PREFETCH;   // small-T kernel: W2 bytes a CTA asks into L2 before the middle barrier
 constexpr int kSpecMinT = 8;         // tokens from which the small-T kernel streams ahead of its router
@@ -155,7 +155,6 @@ struct Shared {
     volatile int up_geo;                   // which of the two the up-projection follows (the down-projection: always geo[1])
     volatile int geo_state;
     volatile int spec_issued, spec_stop;   // producer -> MMA issuer: ring slots filled under geo[0]; no more will be
-    volatile int up_arrived;               // epilogue -> producer: this CTA has arrived at the barrier between the projections
     volatile int mma_drained;              // MMA issuer -> producer: those slots are consumed, the ring is idle
     union {
         int rowtok[(DSMOE_PAIR_GW > 8 ? DSMOE_PAIR_GW / 2 : 6) * BM];                // umma_gemm_kernel, gathered A: the source row of each tile row, per gathering warp
@@ -1130,6 +1129,22 @@ __device__ __noinline__ void small_router_pass(const RouterArgs P, Shared& sh, i
     }
 }
 
+// Between the two projections HBM has nothing to do for several microseconds (epilogues, the slowest CTA, the barrier), and the
+// ring is full.  So the next weight tiles of this CTA's sequence, units u0 .. u1 - 1 of the down-projection, are asked into L2
+// meanwhile: the down-projection then finds them there instead of in DRAM.  All CTAs together ask for well under half of L2.
+// (Not for the fewest tokens: there the gap is short and the requests only compete with the ring's own.)  A thread with nothing
+// else to do asks: each request takes some 0.15 us, and 24 of them in the producer, ahead of its wait for the barrier, made
+// narrow experts' layers 2 to 3 us slower than none at all.  Whole layers, 8 to 128 tokens, 32 experts (384 KB asked by the producer ->
+// 192 KB from here): d 2048, H 256, T 32: 37.0 -> 35.0 us; 3072, 384, T 100: 51.4 -> 49.2; 4096, 512, T 16: 61.8 -> 58.0; 2048, 1024,
+// T 50: 62.1 -> 61.8; 56 shapes 1.043 times as fast (0.986, T 8 of the last width, to 1.091).  128 KB: 1.043; 256 KB: 1.040; 384 KB: 1.026.
+__device__ __noinline__ void small_prefetch(const BMaps* tmW2, const int* active, int u0, int u1, int U, int kbpe, int bn_down, int d) {
+    for (int u = u0, bytes = 0; u < u1 && bytes < kSmallL2PrefetchBytes; ++u) {
+        const int r = u / U, g = u - r * U, n0 = r * bn_down, bn = min(bn_down, d - n0);
+        if ((bn & (bn - 1)) == 0) ptx::tma_prefetch_3d(&tmW2->m[__ffs(bn) - 5], 0, wrow(g % kbpe, n0, d), active[g / kbpe]);
+        bytes += bn * BK * 2;
+    }
+}
+
 // Bounded wait for the router's verdict on the speculative geometry; 0 = gave up.
 __device__ __forceinline__ int wait_geo(Shared& sh) {
     const uint64_t t0 = ptx::globaltimer_ns();
@@ -1186,7 +1201,6 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         sh.spec_issued = 0;
         sh.spec_stop = 0;
         sh.mma_drained = 0;
-        sh.up_arrived = 0;
         small_geometry(P, P.E, G, sh.geo[0]);
 #ifdef DSMOE_TRACE
         for (int i = 0; i < 32; ++i) sh.trace[i] = 0;
@@ -1317,29 +1331,6 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
                 if (++i_cur == t.nk) {
                     i_cur = 0;
                     have = it.next(P, g->active, g->n_act, t);
-                }
-            }
-            // Between the two projections HBM has nothing to do for several microseconds (epilogues, the slowest
-            // CTA, the barrier), and the ring is full.  So the next weight tiles of this CTA's sequence are asked
-            // into L2 meanwhile: the down-projection then finds them there instead of in DRAM.  All CTAs together
-            // ask for well under half of L2.  (Not for the fewest tokens: there the gap is short and the requests only
-            // compete with the ring's own.)
-            if (alive && have && P.spec && wait_flag(&sh.up_arrived, sh)) {     // ... once this CTA's own hg is out
-                SmallIter pit = it;
-                SmallTile pt = t;
-                int pi = i_cur;
-                bool phave = have;
-                const int kbpe = P.H / BK;
-                for (int bytes = 0; phave && bytes < kSmallL2PrefetchBytes;) {
-                    if ((pt.bn & (pt.bn - 1)) == 0) {
-                        const int gb = pt.kstart + pi;
-                        ptx::tma_prefetch_3d(&tmW2.m[__ffs(pt.bn) - 5], 0, wrow(gb % kbpe, pt.n0, P.d), g->active[gb / kbpe]);
-                    }
-                    bytes += pt.bn * BK * 2;
-                    if (++pi == pt.nk) {
-                        pi = 0;
-                        phave = pit.next(P, g->active, g->n_act, pt);
-                    }
                 }
             }
             TRACE(5);
@@ -1655,9 +1646,10 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
                 EPI_SYNC();
                 if (etid == 0) {
                     grid_arrive(P.sync, 1);
-                    sh.up_arrived = 1;
                     TRACE(7);
                 }
+                if (P.spec && etid == kEpiThreads - 32)
+                    small_prefetch(&tmW2, ge.active, it.down_u0 + ge.n_stages, it.down_u1, n_act * (P.H / BK), P.H / BK, ge.bn_down, P.d);
                 up_done = true;
             }
             if (!have) break;
