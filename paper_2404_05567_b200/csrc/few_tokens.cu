@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) few_tokens_kernel(const FewPar
         const long long total = (long long)n_act * P.H;
         const int r_begin = (int)(total * blockIdx.x / G), rows = (int)(total * (blockIdx.x + 1) / G) - r_begin;
         const int nkb = P.d / BK, mine = warp < nkb ? (nkb - warp + kFewWarps - 1) / kFewWarps : 0;
-        // the run's rows lie in at most two experts (it is shorter than H): row r of it is at base + r * 64 of block 0
+        // the run's rows lie in at most two experts (it is no longer than H, few_fits): row r of it is at base + r * 64 of block 0
         const int i0 = r_begin / P.H, bound = (i0 + 1) * P.H - r_begin;
         const int ea = n_act ? active_s[min(i0, n_act - 1)] : 0, eb = n_act ? active_s[min(i0 + 1, n_act - 1)] : 0;
         const int j0 = r_begin - i0 * P.H;                    // the first row's hidden unit
@@ -417,10 +417,15 @@ extern "C" __attribute__((visibility("default"))) int dsmoe_few_trace_read(unsig
 }
 #endif
 
-// (weights are read 32 bytes at a time, 64 KB of partial sums hold 128 columns of a CTA)
+// What `ctas` CTAs can take: a run of hidden units touches no third expert, which takes a CTA for every expert that may be
+// selected (H * n_act / ctas <= H); 64 KB of partial sums hold 128 columns of a CTA; the tokens fit beside them.
+bool few_fits(const dsmoe_layer_desc& p, int ctas) {
+    return p.T <= kFewMaxT && p.E <= ctas && ceil_div(p.d, ctas) <= kFewChunk && few_smem_bytes(p) <= kFewMaxSmem;
+}
+
+// (weights are read 32 bytes at a time)
 bool few_supported(const dsmoe_layer_desc& p, const void* packed) {
-    return small_supported(p) && p.T <= kFewMaxT && ((uintptr_t)packed & 31u) == 0 && few_smem_bytes(p) <= kFewMaxSmem &&
-           ceil_div(p.d, std::min(sm_count(), kSmallMaxCtas)) <= kFewChunk;
+    return small_supported(p) && ((uintptr_t)packed & 31u) == 0 && few_fits(p, std::min(sm_count(), kSmallMaxCtas));
 }
 
 dsmoe_status launch_layer_few(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, const void* packed,
