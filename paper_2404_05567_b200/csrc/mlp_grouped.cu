@@ -41,6 +41,7 @@ struct GroupedParams {
     __nv_bfloat16* h;              // [amax, H]
     float* rows;                   // [amax, d]
     int* sync;                     // zero at launch: [0] row tiles of h that are complete; from kSyncH on, per row tile, its finished epilogue warps
+    int max_row_tiles;             // ... and so many of these there are
     int32_t* dev_status;
 };
 constexpr int kSyncH = 16;
@@ -56,8 +57,9 @@ struct GroupedShared {
     volatile int abort_flag;
     int row_tiles, up_tiles, down_tiles;   // totals
     int mine, skip;                // up tiles of this CTA; rounds of down tiles that CTAs with one more up tile sit out
-    int seg[kMaxExperts + 1];      // first row of each expert
-    int rt0[kMaxExperts + 1];      // ... and first row tile
+    int bad_offsets;
+    int seg0[kMaxExperts], seg1[kMaxExperts];      // rows of each expert
+    int rt0[kMaxExperts + 1];                      // its first row tile
     int rowtok[GATHER_WARPS * (BM / 2)];
 };
 constexpr size_t kGroupedShared = 4096;
@@ -109,8 +111,8 @@ __device__ __forceinline__ bool tile_at(const GroupedParams& P, const GroupedSha
     const int nt = local / mtiles, mt = local - nt * mtiles;
     t.e = e;
     t.rt = sh.rt0[e] + mt;
-    t.row0 = sh.seg[e] + mt * BM;
-    t.rows_valid = min(BM, sh.seg[e + 1] - t.row0);
+    t.row0 = sh.seg0[e] + mt * BM;
+    t.rows_valid = min(BM, sh.seg1[e] - t.row0);
     t.n0 = nt * BN;
     return true;
 }
@@ -192,6 +194,7 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
             ptx::mbar_init(ptx::smem_u32(&sh.tempty[a]), 4);
         }
         sh.abort_flag = 0;
+        sh.bad_offsets = 0;
         ptx::fence_barrier_init();
         ptx::prefetch_tensormap(&tmH);
         for (int i = 2; i < 5; ++i) ptx::prefetch_tensormap(&tmW1.m[i]);
@@ -203,20 +206,38 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
     }
     chain_wait();
     if (warp == 0) {
-        // segments (clamped: nothing here may send a tile out of range) and their row tiles
+        __syncwarp();
+        // Segments and their row tiles.  As in umma_gemm_kernel, one that is negative, decreasing or ends beyond the rows counts as
+        // empty and is reported: a corrupt array must not send a tile out of range.  Segments that overlap could still have more
+        // row tiles than there are counters; then all count as empty.
         int tiles[2];
+        bool bad = false;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int e = lane + 32 * j;
             int a = 0, b = 0;
             if (e < P.E) {
-                a = (int)min(max((long long)P.offsets[e], 0ll), P.amax);
-                b = (int)min(max((long long)P.offsets[e + 1], (long long)a), P.amax);
+                a = P.offsets[e];
+                b = P.offsets[e + 1];
             }
-            tiles[j] = (b - a + BM - 1) / BM;
-            if (e < P.E) sh.seg[e] = a;
-            if (e == P.E - 1) sh.seg[P.E] = b;
+            if (a < 0 || b < a || b > P.amax) {
+                bad = true;
+                a = b = 0;
+            }
+            tiles[j] = (int)(((long long)b - a + BM - 1) / BM);
+            if (e < P.E) {
+                sh.seg0[e] = a;
+                sh.seg1[e] = b;
+            }
         }
+        long long sum = (long long)tiles[0] + tiles[1];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (sum > P.max_row_tiles) {
+            bad = true;
+            tiles[0] = tiles[1] = 0;
+        }
+        if (__any_sync(0xffffffffu, bad) && lane == 0) sh.bad_offsets = 1;
         int lo = tiles[0], hi = tiles[1];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -532,7 +553,10 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, TMEM_COLS);
     }
-    if (threadIdx.x == 0 && sh.abort_flag) report_status(P.dev_status, DSMOE_ERR_TIMEOUT);
+    if (threadIdx.x == 0) {
+        if (sh.abort_flag) report_status(P.dev_status, DSMOE_ERR_TIMEOUT);
+        else if (sh.bad_offsets) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
+    }
 }
 
 }  // namespace
@@ -543,13 +567,15 @@ extern "C" __attribute__((visibility("default"))) int dsmoe_grouped_trace_read(l
 }
 #endif
 
+// (no more than E of the experts' last row tiles are incomplete)
+static size_t max_row_tiles(const dsmoe_layer_desc& p) { return amax_of(p) / BM + p.E; }
+
 // Counters of the grouped layer's launch: behind the hidden activations [Amax, H] if the workspace has room there (it keeps [T, E*H] for
 // other paths), else none
 GroupedScratch grouped_scratch(const dsmoe_layer_desc& p, const WsLayout& L) {
     GroupedScratch S{};
-    const size_t amax = amax_of(p);
     S.sync = L.bwd;
-    S.sync_ints = (size_t)kSyncH + amax / BM + p.E;
+    S.sync_ints = kSyncH + max_row_tiles(p);
     S.fits = umma_supported(p) && S.sync + S.sync_ints * 4 <= L.total_packed;
     return S;
 }
@@ -579,6 +605,7 @@ dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, cons
     P.h = reinterpret_cast<__nv_bfloat16*>(ws + L.h);
     P.rows = rows;
     P.sync = reinterpret_cast<int*>(ws + grouped_scratch(p, L).sync);
+    P.max_row_tiles = (int)max_row_tiles(p);
     P.dev_status = dev_status;
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));

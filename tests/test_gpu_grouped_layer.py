@@ -80,3 +80,33 @@ def test_rows_around_a_tile():
     want = torch.stack([torch.nn.functional.gelu(x[t].float() @ W1[e].float()) @ W2[e].float() for t, e in enumerate(owner.tolist())])
     gate = torch.softmax(x.float() @ Wr, dim=1).gather(1, owner[:, None])
     assert (outs[1] - gate * want).norm() <= 6e-3 * (gate * want).norm()
+
+
+def test_offsets_out_of_order_are_reported():
+    """A workspace whose expert offsets are overwritten during the call (here by counts_out, made to lie on them: counts that
+    descend somewhere are no offsets): no tile leaves its range, the call reports DSMOE_ERR_INVALID_ARG, and the next one is whole."""
+    T, d, H, E = 700, 128, 192, 8
+    g = torch.Generator(device="cuda").manual_seed(11)
+    x, Wr = torch.randn(T, d, generator=g, device="cuda").bfloat16(), torch.randn(d, E, generator=g, device="cuda") * 0.2
+    W1, W2 = (torch.randn(E, *s, generator=g, device="cuda").bfloat16() * 0.05 for s in ((d, H), (H, d)))
+    desc = dm.make_desc(T, d, H, E, dm.BF16, dm.SELECT_TOPK, 0.0, 0, 3, 0, 0, 0)
+    packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc, W1, W2, packed)
+    ws = torch.zeros(dm.dsmoe_workspace_size_packed(desc), dtype=torch.uint8, device="cuda")
+    status, out = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.empty(T, d, device="cuda", dtype=torch.bfloat16)
+    counts = torch.zeros(E, dtype=torch.int32, device="cuda")
+    dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, counts, ws, status)
+    want = out.clone()
+    assert int(status.item()) == 0 and any(a > b for a, b in zip(counts.tolist(), counts.tolist()[1:]))
+    up = lambda n: (n + 255) // 256 * 256
+    at = up(T * E * 4) + up(T * 8) + up(T * 4) + up(64 * 4)          # scores, mask, k_t, counts lie before the offsets
+    offsets = ws[at:at + 4 * (E + 1)].view(torch.int32)
+    ends = [0] + counts.cumsum(0).tolist()
+    assert offsets.tolist() == ends
+    dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, offsets, ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 1                                   # DSMOE_ERR_INVALID_ARG
+    status.zero_()
+    dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, counts, ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(out, want)
