@@ -110,3 +110,82 @@ def test_offsets_out_of_order_are_reported():
     dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, counts, ws, status)
     torch.cuda.synchronize()
     assert int(status.item()) == 0 and torch.equal(out, want)
+
+
+def _layer(T, d, H, E, K, seed):
+    """desc, call(x, out, ws, status), x and the workspace of a top-K layer"""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x, Wr = torch.randn(T, d, generator=g, device="cuda").bfloat16(), torch.randn(d, E, generator=g, device="cuda") * (1.5 / d ** 0.5)
+    W1, W2 = (torch.randn(E, *s, generator=g, device="cuda").bfloat16() * 0.05 for s in ((d, H), (H, d)))
+    desc = dm.make_desc(T, d, H, E, dm.BF16, dm.SELECT_TOPK, 0.0, 0, K, 0, 0, 0)
+    packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc, W1, W2, packed)
+
+    def call(x, out, ws, status):
+        dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, None, ws, status)
+    return call, x, torch.full((dm.dsmoe_workspace_size_packed(desc),), 0x5a, dtype=torch.uint8, device="cuda")
+
+
+# no up tile, and fewer of them than CTAs: the others begin with down tiles; several rounds
+PART = [(129, 64, 64, 3, 1), (300, 512, 256, 8, 3), (4096, 1024, 512, 32, 6)]
+
+
+@pytest.mark.parametrize("sms", [16, 72])
+def test_on_a_part_of_the_gpu(sms):
+    """A stream that owns some of the SMs: not every CTA of the launch runs at once, and the others' tiles are taken over."""
+    cu = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(r):
+        assert r[0] == cu.CUresult.CUDA_SUCCESS, r[0]
+        return r[1] if len(r) == 2 else r[1:]
+    torch.zeros(1, device="cuda")
+    dev = ok(cu.cuDeviceGet(torch.cuda.current_device()))
+    whole = ok(cu.cuDeviceGetDevResource(dev, cu.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM))
+    groups, n, _ = ok(cu.cuDevSmResourceSplitByCount(1, whole, 0, sms))
+    assert n == 1 and sms <= groups[0].sm.smCount < whole.sm.smCount
+    part = ok(cu.cuGreenCtxCreate(ok(cu.cuDevResourceGenerateDesc([groups[0]], 1)), dev, cu.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    raw = ok(cu.cuGreenCtxStreamCreate(part, cu.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))
+    stream = torch.cuda.ExternalStream(int(raw))
+    try:
+        for shape in PART:
+            call, x, ws = _layer(*shape, seed=sms)
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            xs = [x, x.flip(0).contiguous()]
+            want = [torch.empty_like(x) for _ in xs]
+            for a, b in zip(xs, want):
+                call(a, b, ws, status)
+            got = [torch.full_like(x, float("nan")) for _ in range(6)]
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                for i, out in enumerate(got):
+                    call(xs[i % 2], out, ws, status)
+            stream.synchronize()
+            assert int(status.item()) == 0
+            for i, out in enumerate(got):
+                assert torch.equal(out, want[i % 2]), (shape, i)
+    finally:
+        torch.cuda.synchronize()
+        ok(cu.cuStreamDestroy(raw) + (None,))
+        ok(cu.cuGreenCtxDestroy(part) + (None,))
+
+
+@pytest.mark.parametrize("shape", PART, ids=lambda s: f"T{s[0]}-d{s[1]}-H{s[2]}-E{s[3]}")
+def test_two_streams_with_a_workspace_each(shape):
+    call, x, ws = _layer(*shape, seed=3)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    xs = [x, x.flip(0).contiguous()]
+    want = [torch.empty_like(x) for _ in xs]
+    for a, b in zip(xs, want):
+        call(a, b, ws, status)
+    streams, wss = [torch.cuda.Stream(), torch.cuda.Stream()], [ws, torch.full_like(ws, 0x5a)]
+    got = [[torch.full_like(x, float("nan")) for _ in range(20)] for _ in streams]
+    torch.cuda.synchronize()
+    for i in range(20):
+        for k, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                call(xs[(i + k) % 2], got[k][i], wss[k], status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    for k in range(2):
+        for i in range(20):
+            assert torch.equal(got[k][i], want[(i + k) % 2]), (k, i)
