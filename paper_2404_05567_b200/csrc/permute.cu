@@ -22,7 +22,7 @@ namespace dsmoe {
 // 98.0 -> 97.2).
 constexpr int kCountInBlockChunks = 8;
 constexpr int kPermThreads = 512, kPermChunks = 4, kPermTokens = kPermChunks * kChunk / (kPermThreads / 32);
-template <int SCAN>
+template <int SCAN, bool ZERO>
 __global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint64_t* mask,
                                                             const float* scores,
                                                             int32_t* offsets,
@@ -33,7 +33,8 @@ __global__ void __launch_bounds__(kPermThreads) permute_index_kernel(const uint6
                                                             int64_t amax, uint4* __restrict__ zero_out, int row_vecs, const ZeroInts zero) {
     chain_next();
     chain_wait();
-    for (long long i = (long long)blockIdx.x * kPermThreads + threadIdx.x; i < zero.n; i += (long long)gridDim.x * kPermThreads) zero.at[i] = 0;
+    if (ZERO)      // (compiled in for the callers that ask for it only: the others' code is as without it)
+        for (long long i = (long long)blockIdx.x * kPermThreads + threadIdx.x; i < zero.n; i += (long long)gridDim.x * kPermThreads) zero.at[i] = 0;
     __shared__ uint64_t mask_s[kPermChunks * kChunk];
     __shared__ int before_s[kMaxExperts], total_s[kMaxExperts], base_s[kPermChunks][kMaxExperts];
     __shared__ int cnt_s[SCAN == 2 ? kCountInBlockChunks : 1][kMaxExperts];
@@ -340,7 +341,7 @@ dsmoe_status launch_permute(const dsmoe_layer_desc& p, const void* x, const floa
     const int nchunks = ceil_div(p.T, kChunk);
     const int64_t amax = (int64_t)amax_of(p);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
-    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<0>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
+    DSMOE_CUDA_TRY(launch_chained(zero.n > 0 ? permute_index_kernel<0, true> : permute_index_kernel<0, false>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
         mask, scores, const_cast<int32_t*>(offsets), chunk_prefix, nullptr, nullptr, row_token, row_gate,
         token_rows, p.T, p.E, width_of(p), amax, static_cast<uint4*>(zero_out), row_vecs, zero));
     if (xp) {
@@ -363,7 +364,7 @@ dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const 
     const int nchunks = ceil_div(p.T, kChunk);
     const int row_vecs = (int)((size_t)p.d * (p.out_fp32 ? 4 : elem_size(p.dtype)) / 16);
     if (nchunks > 0 && nchunks <= kCountInBlockChunks) {
-        DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<2>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
+        DSMOE_CUDA_TRY(launch_chained(zero.n > 0 ? permute_index_kernel<2, true> : permute_index_kernel<2, false>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
             mask, scores, offsets, nullptr, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
             width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs, zero));
         return DSMOE_OK;
@@ -374,7 +375,7 @@ dsmoe_status launch_group(const dsmoe_layer_desc& p, const float* scores, const 
         return launch_permute(p, nullptr, scores, mask, offsets, chunk_prefix, row_token, row_gate, token_rows, nullptr, s,
                               zero_out, zero);
     }
-    DSMOE_CUDA_TRY(launch_chained(permute_index_kernel<1>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
+    DSMOE_CUDA_TRY(launch_chained(zero.n > 0 ? permute_index_kernel<1, true> : permute_index_kernel<1, false>, ceil_div(nchunks, kPermChunks), kPermThreads, 0, s,
         mask, scores, offsets, chunk_prefix, counts, counts_out, row_token, row_gate, token_rows, p.T, p.E,
         width_of(p), (int64_t)amax_of(p), static_cast<uint4*>(zero_out), row_vecs, zero));
     return DSMOE_OK;
