@@ -61,7 +61,8 @@ def torch_dtype(s: gi.LayerSpec):
 class Layer:
     """One synthetic layer resident on the GPU plus the numpy originals for the oracle."""
 
-    def __init__(self, s: gi.LayerSpec, pack: bool = True, layer: int = 0, batch: str = "x"):
+    def __init__(self, s: gi.LayerSpec, pack: bool = True, layer: int = 0, batch: str = "x", packed_at: int = 0):
+        """packed_at: the packed weights' address modulo 32, a multiple of 16."""
         self.s = s
         self.desc = desc_of(s)
         self.x = gi.tokens(s, batch)
@@ -71,7 +72,10 @@ class Layer:
         self.W1_d, self.W2_d = to_dev(self.W1), to_dev(self.W2)
         self.packed = None
         if pack and s.dtype == "bf16" and s.d % 64 == 0 and s.H % 64 == 0:      # the packed layout is in blocks of 64
-            self.packed = torch.empty(dm.dsmoe_packed_size(self.desc), dtype=torch.uint8, device="cuda")
+            n = dm.dsmoe_packed_size(self.desc)
+            buf = torch.empty(n + 32, dtype=torch.uint8, device="cuda")
+            at = (packed_at - buf.data_ptr()) % 32
+            self.packed = buf[at:at + n]
             dm.dsmoe_pack_weights(self.desc, self.W1_d, self.W2_d, self.packed)
         # a call with packed weights needs only the tensor-core paths' (smaller) workspace
         nbytes = dm.dsmoe_workspace_size_packed(self.desc) if self.packed is not None else dm.dsmoe_workspace_size(self.desc)
@@ -154,11 +158,11 @@ def rel_err_rows(gpu: np.ndarray, ref: np.ndarray) -> float:
     return float(e.max())
 
 
-def layer_parity(s: gi.LayerSpec, pack: bool = True, sample: int | None = None):
+def layer_parity(s: gi.LayerSpec, pack: bool = True, sample: int | None = None, packed_at: int = 0):
     """Runs dsmoe_layer_forward and the oracle on the same inputs; returns a dict of measurements.
 
     ``sample`` = number of seeded tokens the oracle evaluates (None: all tokens)."""
-    L = Layer(s, pack=pack)
+    L = Layer(s, pack=pack, packed_at=packed_at)
     # The tolerance is applied to the value the layer computes, i.e. its fp32 output.  Storing that
     # value as bf16 is one more rounding (<= 2^-8 relative, by itself more than 2e-2 * RMS for any
     # element beyond 5.1 sigma), so the bf16 output is checked separately: it must be exactly the

@@ -1,6 +1,7 @@
 """One to seven tokens (few_tokens_kernel) against the oracle where its work is cut: fewer reduction blocks than warps, experts not a
 multiple of four, runs of hidden units that cross an expert's end, more of them than one chunk holds, several passes over a CTA's
-columns, fewer columns than CTAs, nothing selected; and weights that are aligned to 16 bytes only (GPU required)."""
+columns, fewer columns than CTAs, nothing selected; the same calls with weights that are aligned to 16 bytes only, which small_layer_kernel
+takes; and tokens that are not numbers (GPU required)."""
 import pytest
 import torch
 
@@ -22,9 +23,11 @@ CASES = [
 ]
 
 
+@pytest.mark.parametrize("packed_at", [0, 16])
 @pytest.mark.parametrize("case", CASES, ids=lambda c: f"T{c['T']}-d{c['d']}-H{c['H']}-E{c['E']}")
-def test_a_handful_of_tokens(case):
-    r = layer_parity(gi.LayerSpec(f"few{CASES.index(case)}", dtype="bf16", router_gain=4.0, **case))
+def test_a_handful_of_tokens(case, packed_at):
+    r = layer_parity(gi.LayerSpec(f"few{CASES.index(case)}", dtype="bf16", router_gain=4.0, **case), packed_at=packed_at)
+    assert r["layer"].packed.data_ptr() % 32 == packed_at
     assert r["err_rows"] <= TOL_BF16        # the tolerance of every bf16 layer test
     assert r["zero_tokens"] == (case["T"] if case.get("eps") == 0.999 else 0)
 
@@ -39,3 +42,17 @@ def test_weights_aligned_to_16_bytes_only():
     dm.dsmoe_pack_weights(L.desc, L.W1_d, L.W2_d, L.packed)
     b = L.forward(out_fp32=True)                   # another kernel: sums in another order, hidden activations rounded to bf16 (2^-9) alike
     assert (a - b).norm() <= 2e-3 * a.norm()
+
+
+def test_a_token_that_is_not_a_number():
+    """Its scores are no numbers and exceed no threshold: it selects nothing and its row is zeros (Eq. 1 with an empty selection, as
+    with more than 128 tokens).  The other tokens do not see it."""
+    L = Layer(gi.LayerSpec("few_nan", T=5, d=512, H=256, E=8, dtype="bf16", mode=gi.MODE_THRESHOLD, eps=0.5, eps_normalized=1))
+    plain = L.forward(out_fp32=True).clone()
+    L.x_d = L.x_d.clone()
+    L.x_d[2] = float("nan")
+    out = L.forward(out_fp32=True)
+    others = [0, 1, 3, 4]
+    assert int(L.mask[2]) == 0 and not out[2].any()
+    # (fewer experts may be selected: the sums over them then run in another order)
+    assert (out[others] - plain[others]).norm() <= 1e-5 * plain[others].norm()

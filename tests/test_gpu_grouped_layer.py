@@ -19,6 +19,9 @@ CASES = [
     (5000, 6144, 64, 16, dm.SELECT_TOPK, 4, 0.0, 0),          # more than 32 down tiles per CTA
     (6000, 128, 6144, 16, dm.SELECT_THRESHOLD, 0, 0.9, 1),    # more than 32 up tiles per CTA, one round or two of down tiles
     (700, 512, 256, 5, dm.SELECT_THRESHOLD, 0, 1e9, 0),       # nothing selected
+    (16384 + 70, 64, 64, 8, dm.SELECT_TOPK, 2, 0.0, 0),       # the counters are zeroed behind the one-block scan kernel
+    (2, 64, 64, 64, dm.SELECT_THRESHOLD_TOPK, 0, 0.9, 0),     # few tokens; of one token the workspace has no room for the counters: two launches
+    (1, 64, 64, 64, dm.SELECT_THRESHOLD_TOPK, 0, 0.9, 0),
 ]
 
 
@@ -29,24 +32,29 @@ def test_one_launch_equals_two(case):
     randn = lambda *shape, dtype=torch.bfloat16: torch.randn(*shape, generator=g, device="cuda", dtype=dtype)
     x, Wr = randn(T, d), randn(d, E, dtype=torch.float32) * (1.5 / d ** 0.5)
     W1, W2 = randn(E, d, H) * 0.05, randn(E, H, d) * 0.05
-    outs = []
+    xs = [x, x.flip(0).contiguous(), randn(T, d)]
+    want = {}
     for fuse in (2, 0):
         desc = dm.make_desc(T, d, H, E, dm.BF16, mode, eps, 1, max(K, 1), 0, out_fp32, fuse)
         packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
         dm.dsmoe_pack_weights(desc, W1, W2, packed)
         ws = torch.full((dm.dsmoe_workspace_size_packed(desc),), 0x5a, dtype=torch.uint8, device="cuda")     # counters are not zero by chance
         status = torch.zeros(1, dtype=torch.int32, device="cuda")
-        out = torch.full((T, d), float("nan"), dtype=torch.float32 if out_fp32 else torch.bfloat16, device="cuda")
-        counts = torch.zeros(E, dtype=torch.int32, device="cuda")
-        for _ in range(2):                                                                                    # ... nor left over
-            dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, counts, ws, status)
+        got = []
+        # the first call finds the fill, every later one another input's hidden activations and counters; no waits in between
+        for i in (0, 1, 2, 0, 2, 1) if fuse == 0 else (0, 1, 2):
+            out = torch.full((T, d), float("nan"), dtype=torch.float32 if out_fp32 else torch.bfloat16, device="cuda")
+            counts = torch.zeros(E, dtype=torch.int32, device="cuda")
+            dm.dsmoe_layer_forward(desc, xs[i], Wr, None, None, None, packed, out, None, counts, ws, status)
+            got.append((i, out, counts))
         torch.cuda.synchronize()
         assert int(status.item()) == 0
-        outs.append((out, counts))
-    assert torch.equal(outs[0][1], outs[1][1])
-    assert torch.equal(outs[0][0], outs[1][0])
-    if eps == 1e9:
-        assert not outs[1][0].any()
+        for i, out, counts in got:
+            if fuse == 2:
+                want[i] = (out, counts)
+            assert torch.equal(out, want[i][0]) and torch.equal(counts, want[i][1]), i
+            if eps == 1e9:
+                assert not out.any()
 
 
 def test_rows_around_a_tile():
