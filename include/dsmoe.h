@@ -203,7 +203,9 @@ dsmoe_status dsmoe_combine(const dsmoe_layer_desc* desc, const void* yp, const f
  * [E][d/64][H][64] followed by W2 as [E][H/64][d][64] (block-major along the reduction), so
  * that every tensor-core operand is contiguous along the reduction and every tile a kernel
  * fetches is one contiguous piece of memory.  dtype must be DSMOE_BF16; d and H multiples of 64.
- * dsmoe_packed_size reports the bytes `packed` must hold.
+ * dsmoe_packed_size reports the bytes `packed` must hold; its address is a multiple of 16.  With one that is
+ * a multiple of 32 (cudaMalloc's all are), dsmoe_layer_forward on one to seven tokens takes a kernel that reads the
+ * weights 32 bytes at a time; otherwise the one for up to 128 tokens, slower and with its sums in another order.
  */
 dsmoe_status dsmoe_packed_size(const dsmoe_layer_desc* desc, size_t* bytes);
 dsmoe_status dsmoe_pack_weights(const dsmoe_layer_desc* desc, const void* W1, const void* W2,
@@ -342,9 +344,11 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
 /*
  * Measurement aid (no counterpart in the paper): a ring of CUDA event pairs on the caller's stream.
  * After dsmoe_timing_enable(n_pairs) (n_pairs > 0; events are created here, so call it outside any
- * timed region), every launch of an expert-MLP tensor-core kernel (the two grouped or dense GEMMs of
- * a prefill call, the one kernel of a decode call) is bracketed by the next pair until n_pairs are
- * used.  dsmoe_timing_read waits for the recorded pairs, writes their durations in milliseconds, in
+ * timed region), every launch of an expert-MLP tensor-core kernel is bracketed by the next pair until
+ * n_pairs are used: one pair for a call of up to 128 tokens (Threshold-TopK excepted) and for a sparse call whose
+ * projections are one launch (fuse_combine 0 unless it means 1, see above; with so few tokens and experts that the
+ * workspace has no room for that launch's counters, two); two, up and down, for the dense forward, the
+ * gradients and fuse_combine 1 or 2; for dsmoe_moa_forward three: query projection, attention, output projection.  dsmoe_timing_read waits for the recorded pairs, writes their durations in milliseconds, in
  * launch order, to the HOST array ms (at most n_max), sets *n and empties the ring.
  * dsmoe_timing_enable(0) switches it off.  Off by default.
  */
