@@ -6,7 +6,8 @@ the dominant kernel, with the CPU oracle timed beside it.
 A step is one dsmoe_layer_forward over one batch of synthetic tokens.  The decode-shaped workloads
 cycle through many distinct sets of expert weights (far more than L2 in total) so that every step reads
 its weights from HBM, as consecutive layers of a real model do; the prefill-shaped and dense workloads
-touch far more than L2 per step by themselves.  One JSON line goes to stdout.
+touch far more than L2 per step by themselves.  One JSON line goes to stdout; the other workloads that a run
+without --no-extra measures go to stderr, a JSON line each, so that the one line stays short.
 
 --gpus N > 1 without a torchrun environment starts N ranks itself (one process per GPU); under
 torchrun the ranks are already there.  The layer shards by token with no exchange, so the ranks are
@@ -435,7 +436,8 @@ def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, s
         weight_bytes = 2.0 * sum(n_act_layers) * s.d * s.H * 2.0 * (1 if loop else calls_per_step)
         flops = 4.0 * A * s.d * s.H * calls_per_step
         if decode:
-            # selected experts' weights (W1 and W2), each byte once, all inside one launch of small_layer_kernel
+            # selected experts' weights (W1 and W2), each byte once, all inside one launch of few_tokens_kernel
+            # (up to 7 tokens) or small_layer_kernel
             roof = dict(bound="hbm", achieved=weight_bytes / (kernel_ms * 1e-3) / 1e9, peak=P["hbm"], unit="GB/s",
                         peak_source=P["source"] + " (copy bandwidth)", kernel="few_tokens_kernel" if s.T < 8 else "small_layer_kernel")
             roof["frac"] = roof["achieved"] / roof["peak"]
@@ -857,7 +859,8 @@ def main():
         line["cpu_baseline"] = {"value": cb["value"], "unit": "tokens/s", "cores": cb["cores"], "kind": "oracle",
                                 "sample": cb["sample"]}
         if not args.no_extra:
-            also = []
+            def also(entry):
+                print(json.dumps(entry), file=sys.stderr, flush=True)
             shape = None
             for other, k in ALSO:
                 if other == name:
@@ -867,18 +870,17 @@ def main():
                     drop_weights(torch, keep_shape=(so.d, so.H, so.E))   # keep the device's memory use bounded
                 shape = (so.d, so.H, so.E)
                 r = run_workload(other, k, 5, with_e2e=False, sampler_index=physical_gpu_index(local_rank))
-                also.append({"workload": other, "value": r["value"], "unit": "tokens/s", "ms_per_step": r["ms_per_step"],
-                             "steps": k, "roofline": r.get("roofline"), "clocks": r["clocks"], "assignments": r["A"],
-                             "active_experts": r["active_experts"],
-                             "active_experts_per_layer": r["active_experts_per_layer"],
-                             "activation_rms_per_layer": r["activation_rms_per_layer"],
-                             "near_threshold_1e-6": r["stats"]["near_threshold"]})
+                also({"workload": other, "value": r["value"], "unit": "tokens/s", "ms_per_step": r["ms_per_step"],
+                      "steps": k, "roofline": r.get("roofline"), "clocks": r["clocks"], "assignments": r["A"],
+                      "active_experts": r["active_experts"],
+                      "active_experts_per_layer": r["active_experts_per_layer"],
+                      "activation_rms_per_layer": r["activation_rms_per_layer"],
+                      "near_threshold_1e-6": r["stats"]["near_threshold"]})
             drop_weights(torch)
-            also.append(run_training_side(10, 3, sampler_index=physical_gpu_index(local_rank)))
+            also(run_training_side(10, 3, sampler_index=physical_gpu_index(local_rank)))
             for other, k in (("moa6b_prefill", 20), ("moa6b_decode", 200)):
                 drop_weights(torch)
-                also.append(run_moa(other, k, 5, sampler_index=physical_gpu_index(local_rank)))
-            line["also"] = also
+                also(run_moa(other, k, 5, sampler_index=physical_gpu_index(local_rank)))
     print(json.dumps(line))
     if dist is not None:
         dist.destroy_process_group()
