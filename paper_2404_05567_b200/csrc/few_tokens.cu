@@ -17,10 +17,11 @@
 // A load covers 8 weight rows x 128 bytes; neighbouring rows of a packed block are neighbours in memory.  A register that has been
 // used is loaded again at once, with its place in the next block: 8 KB are under way per warp, 128 KB per SM.
 //
-// Against small_layer_kernel (us a layer of 32 experts, by threshold / top-4): 1 token of 2048, 1024 wide 39.2 -> 25.8 / 34.8 -> 17.1;
-// 2 of 4096, 512 wide 51.4 -> 41.1 / 47.1 -> 24.5; 4 of 3072, 384 wide 45.1 -> 40.6 / 43.2 -> 28.2; 7 tokens 1.03 to 1.57 times as fast.  One
-// token of 2048, 1024 wide with 13 selected experts (109 MB): experts known at 4.9 us, the two streams 19 us (5.7 TB/s), the barrier
-// and reductions between them 3, and some 4 us between two launches.
+// Against small_layer_kernel (us a layer call of 32 experts, by threshold / top-4; in brackets the experts that the threshold selected):
+// 1 token of 2048, 1024 wide 39.1 -> 26.1 (9) / 34.7 -> 16.8; 2 of 4096, 512 wide 51.3 -> 41.0 (20) / 47.1 -> 24.2; 4 of 3072, 384 wide
+// 45.1 -> 40.7 (30) / 43.1 -> 27.9; 7 tokens 1.03 to 1.58 times as fast.  One token of 2048, 1024 wide with 13 selected experts (109 MB)
+// takes 31 us: experts known at 4.9, the two streams 19 (5.7 TB/s), the barrier and reductions between them 3, and some 4 between two
+// launches.
 #include <algorithm>
 
 #include "common.cuh"

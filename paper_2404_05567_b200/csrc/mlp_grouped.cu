@@ -24,8 +24,9 @@
 // Against two launches of umma_gemm_kernel (dealt out, cooperative), layers of 32 experts (us): 300 tokens of 2048, 1024 wide, by
 // threshold 91 -> 86; 1500 of 3072, 384 wide, by threshold 214 -> 180; 3333 of 3072, 384 wide, top-6 237 -> 205; 7001 of 4096, 512 wide,
 // top-4 441 -> 422; 8192 of 6144, 768 wide, top-4 904 -> 882 (76 shapes of 150 to 8192 tokens: 1.06 times on average, 0.98 to 1.22).
-// Bound by the operands' way out of L2 (up) and, with narrow experts, the fp32 rows' way to memory (down: 158 us of which 108
-// without its stores, at the first shape).
+// Bound by the latency of the operands' way out of L2 (2048 tokens of 4096, 512 wide, top-4: tensor pipe 42 % busy, L2 at 37 % of its
+// throughput, DRAM at 47 %; the issuer waits while four ring slots are under way) and, with narrow experts, the fp32 rows' way to memory
+// (7001 tokens of that shape: the down tiles 158 us, 108 without their stores).
 // The weighted sum of Eq. 1 inside this launch, over groups of columns whose rows were to stay in L2, was slower than its own launch
 // in every form (355 us and more against 248 + 78): beside a 200 KB ring an SM has too few bytes of rows under way, and handing
 // small groups from stores to sums and back costs more than the rows' way to memory and back.

@@ -865,7 +865,7 @@ teardown:
 //
 // From 8 tokens on the up-projection starts before the router has finished, under "every expert selected"
 // (see the kernel).  The operand ring keeps running across the up/down barrier: the producer prefetches the
-// first W2 tiles (which do not depend on hg) while other CTAs finish, asks the next ones into L2, and adds
+// first W2 tiles (which do not depend on hg) while other CTAs finish (an epilogue thread asks the next ones into L2), and adds
 // the hg tiles once the barrier has passed.  Every wait, on an mbarrier or on a grid barrier, is bounded.
 
 struct SmallParams {

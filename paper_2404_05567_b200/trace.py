@@ -29,7 +29,7 @@ from .build import CSRC, NVCC_FLAGS, PKG, ROOT, _nvcc
 SMALL_NAMES = {0: "CTA starts", 12: "router: first loads", 13: "router: slice sums done", 1: "router: at grid barrier",
                14: "router: grid barrier passed", 2: "router: partition known", 4: "MMA issuer: first tile in shared memory",
                3: "producer: up-projection issued", 28: "epilogue: first accumulator complete", 7: "epilogue: hg written, at grid barrier",
-               5: "producer: down-projection weights prefetched", 6: "producer: grid barrier passed", 8: "MMA issuer: first down-projection tile",
+               5: "producer: ring filled with W2", 6: "producer: grid barrier passed", 8: "MMA issuer: first down-projection tile",
                9: "epilogue: partial sums written", 10: "last grid barrier passed", 11: "CTA ends"}
 
 FEW_NAMES = ("CTA starts", "router: at grid barrier", "router: grid barrier passed", "selected experts known", "up-projection multiplied (first warp)",
