@@ -16,7 +16,7 @@
 // Every up tile that a down tile may wait for is in the hands of a CTA that runs, and no CTA has a down tile before its last up
 // tile.  So the waits end with any number of resident CTAs: in a context that owns a part of the SMs, and beside other streams'
 // kernels, whose SMs join in as they become free.  (Dealt out by CTA index, as it was first, the list needed every SM at once, a
-// cooperative launch.)  Claimed against dealt out: 32 shapes of 150 to 1500 tokens 1.01 times as fast (0.99 to 1.07), 48 of 1024 to
+// cooperative launch.)  Claimed against dealt out: 32 shapes of 150 to 1500 tokens 1.01 times as fast (0.98 to 1.09), 48 of 1024 to
 // 8192 1.02 (0.97 to 1.09): a CTA that is done early takes more.
 // The first round alone is not first come, first served: tile b is CTA b's, and goes to another only if CTA b has not begun.  CTAs of
 // neighbouring indices sit on SMs far apart, so that 64 up tiles do not share the 74 SM pairs' ways to L2 by chance (150 tokens
@@ -682,7 +682,8 @@ dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, cons
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));
     // Not chained to the row-index kernel: its CTAs would be set up beside that kernel's blocks, which leave no room for one on their
-    // SMs, and come in another order (8 shapes of 150 to 700 tokens: 0.3 to 1 % slower on average than this, 3 % at 300 of 2048, 1024 wide).
+    // SMs, and come in another order (8 shapes of 150 to 700 tokens, two boxes: 0.3 and 1 % slower on average than this,
+    // 4 % faster to 2.3 % slower).
     grouped_layer_kernel<<<std::min(sm_count(), kGroupedMaxCtas), kGroupedThreads, kGroupedSmem, s>>>(mW1, mH, mW2, P);
     DSMOE_CUDA_TRY(cudaGetLastError());
     DSMOE_TRY(timing_end(s, timed));
