@@ -388,6 +388,8 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
     int32_t* token_rows = reinterpret_cast<int32_t*>(ws + L.token_rows);
     MoaCore core{args->n_head, args->n_seq, args->L, args->scale, args->Kc, args->Vc, args->tok_seq, args->pos, token_rows,
                  nullptr, mask, row_gate};
+    if (moa_decode_supported(p, core))
+        return launch_moa_decode(p, core, x, Wr, br, packed, scores, mask, k_t, counts_out, out, ws, L, dev_status, s);
     const bool dense_down = moa_shares_keys(p, core) && moa_dense_down(p, sm_count());
     if (dense_down) core.dense = ws + L.acc;
 

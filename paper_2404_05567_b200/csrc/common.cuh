@@ -262,6 +262,11 @@ bool moa_supported(const dsmoe_layer_desc& p, int n_head, int L);
 // qa [Amax, H] bf16: the grouped rows' queries on entry, their attention outputs on return
 dsmoe_status launch_moa_attention(const dsmoe_layer_desc& p, const MoaCore& c, void* qa, const int32_t* row_token,
                                   const int32_t* token_rows, const int32_t* offsets, int32_t* dev_status, cudaStream_t s);
+// ---- moa_decode.cu : the whole layer of attention heads for a few decoding tokens, three launches
+bool moa_decode_supported(const dsmoe_layer_desc& p, const MoaCore& c);
+dsmoe_status launch_moa_decode(const dsmoe_layer_desc& p, const MoaCore& c, const void* x, const float* Wr, const float* br, const void* packed,
+                               float* scores, uint64_t* mask, int32_t* k_t, int32_t* counts_out, void* out, char* ws, const WsLayout& L,
+                               int32_t* dev_status, cudaStream_t s);
 // ---- few_tokens.cu : the whole layer for a handful of tokens, one cooperative launch
 bool few_fits(const dsmoe_layer_desc& p, int ctas);
 bool few_supported(const dsmoe_layer_desc& p, const void* packed);
