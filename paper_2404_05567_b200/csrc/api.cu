@@ -247,6 +247,8 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
         return launch_layer_few(p, x, Wr, br, packed, scores, mask, k_t, counts_out, out, ws, L, dev_status, s);
     if (fast && small_supported(p))
         return launch_layer_small(p, x, Wr, br, packed, scores, mask, k_t, counts_out, out, ws, L, dev_status, s);
+    if (layer_f32_supported(p))
+        return launch_layer_f32(p, x, Wr, br, W1, W2, scores, mask, k_t, counts_out, out, ws, L, s);
 
     // Threshold-TopK needs the whole batch's threshold counts before any token can be selected: the router runs
     // with the threshold rule, then the selection is redone with the batch's K

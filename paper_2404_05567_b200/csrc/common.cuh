@@ -183,6 +183,12 @@ dsmoe_status launch_mlp_generic(const dsmoe_layer_desc& p, const void* x, const 
                                 const int32_t* row_token = nullptr);
 
 
+// ---- layer_f32.cu : the whole layer for small fp32 layers, three launches
+bool layer_f32_supported(const dsmoe_layer_desc& p);
+dsmoe_status launch_layer_f32(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, const void* W1, const void* W2,
+                              float* scores, uint64_t* mask, int32_t* k_t, int32_t* counts_out, void* out, char* ws, const WsLayout& L,
+                              cudaStream_t s);
+
 // ---- mlp_umma.cu : tcgen05 / TMEM / TMA kernels on packed bf16 weights
 dsmoe_status timing_enable(int n_pairs);
 dsmoe_status timing_read(float* ms, int n_max, int* n);
