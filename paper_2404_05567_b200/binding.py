@@ -46,6 +46,19 @@ class DsmoeError(RuntimeError):
         super().__init__(f"{where}: {status_string(code)} (status {code})")
 
 
+# Arguments of the entry points by letter: d(escriptor), p(ointer), n (size_t), i(nt).  Declared once, so that a call passes plain numbers:
+# building a ctypes object for each of a call's dozen arguments cost as much host time as the call's launches.
+_ARGTYPES = {"d": ctypes.POINTER(LayerDesc), "p": ctypes.c_void_p, "n": ctypes.c_size_t, "i": ctypes.c_int}
+_SIGNATURES = {
+    "dsmoe_workspace_size": "dp", "dsmoe_workspace_size_packed": "dp", "dsmoe_workspace_size_stages": "dp", "dsmoe_packed_size": "dp",
+    "dsmoe_router": "dppppp", "dsmoe_select": "dppppppnp", "dsmoe_select_static": "dpppppp", "dsmoe_permute": "dpppppppppnp",
+    "dsmoe_expert_mlp": "dpppppppnpp", "dsmoe_combine": "dpppppp", "dsmoe_pack_weights": "dpppp",
+    "dsmoe_layer_forward": "dppppppppppnpp", "dsmoe_layer_forward_host": "dppppppppppnpp",
+    "dsmoe_layer_forward_host_async": "dppppppppppnpp", "dsmoe_stats": "dpppp", "dsmoe_mi_loss": "dppppnp",
+    "dsmoe_dense_backward": "dppppppppppnpp", "dsmoe_moa_forward": "dpppppppppnpp",
+    "dsmoe_timing_enable": "i", "dsmoe_timing_read": "pip",
+}
+
 _lib = None
 
 
@@ -60,6 +73,7 @@ def lib() -> ctypes.CDLL:
         L.dsmoe_status_string.argtypes = [ctypes.c_int]
         for name in EXPORTS[1:]:
             getattr(L, name).restype = ctypes.c_int
+            getattr(L, name).argtypes = [_ARGTYPES[c] for c in _SIGNATURES[name]]
         _lib = L
     return _lib
 
@@ -74,17 +88,20 @@ def _check(code: int, where: str):
 
 
 def _ptr(t):
-    if t is None:
-        return ctypes.c_void_p(0)
-    if isinstance(t, int):
-        return ctypes.c_void_p(t)
+    if t is None or isinstance(t, int):
+        return t
     assert t.is_contiguous(), "dsmoe takes contiguous tensors"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# The current stream's handle.  torch.cuda.current_stream() makes a Stream object for it, 3.3 of the 15 us that a call took on the host.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch.cuda.current_stream().cuda_stream if _raw_stream is None else _raw_stream(torch.cuda.current_device())
 
 
 def make_desc(T, d, H, E, dtype=BF16, mode=SELECT_THRESHOLD, eps=0.0, eps_normalized=0, K=0, min_k=0,
@@ -150,21 +167,21 @@ def dsmoe_router(desc, x, Wr, br, scores, stream=None):
 
 def dsmoe_select(desc, scores, mask, k_t, counts, offsets, workspace, stream=None):
     _check(lib().dsmoe_select(ctypes.byref(desc), _ptr(scores), _ptr(mask), _ptr(k_t), _ptr(counts), _ptr(offsets),
-                              _ptr(workspace), ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                              _ptr(workspace), workspace.numel() if workspace is not None else 0,
                               _stream(stream)), "dsmoe_select")
 
 
 def dsmoe_permute(desc, x, scores, mask, offsets, row_token, row_gate, token_rows, xp, workspace, stream=None):
     _check(lib().dsmoe_permute(ctypes.byref(desc), _ptr(x), _ptr(scores), _ptr(mask), _ptr(offsets), _ptr(row_token),
                                _ptr(row_gate), _ptr(token_rows), _ptr(xp), _ptr(workspace),
-                               ctypes.c_size_t(workspace.numel() if workspace is not None else 0), _stream(stream)),
+                               workspace.numel() if workspace is not None else 0, _stream(stream)),
            "dsmoe_permute")
 
 
 def dsmoe_expert_mlp(desc, xp, W1, W2, packed, offsets, yp, workspace, dev_status=None, stream=None):
     _check(lib().dsmoe_expert_mlp(ctypes.byref(desc), _ptr(xp), _ptr(W1), _ptr(W2), _ptr(packed), _ptr(offsets),
                                   _ptr(yp), _ptr(workspace),
-                                  ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                                  workspace.numel() if workspace is not None else 0,
                                   _ptr(dev_status), _stream(stream)), "dsmoe_expert_mlp")
 
 
@@ -182,7 +199,7 @@ def dsmoe_layer_forward(desc, x, Wr, br, W1, W2, packed, out, mask_out, counts_o
                         stream=None):
     _check(lib().dsmoe_layer_forward(ctypes.byref(desc), _ptr(x), _ptr(Wr), _ptr(br), _ptr(W1), _ptr(W2),
                                      _ptr(packed), _ptr(out), _ptr(mask_out), _ptr(counts_out), _ptr(workspace),
-                                     ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                                     workspace.numel() if workspace is not None else 0,
                                      _ptr(dev_status), _stream(stream)), "dsmoe_layer_forward")
 
 
@@ -193,7 +210,7 @@ def dsmoe_layer_forward_host(desc, x_host, x_dev, Wr, br, W1, W2, packed, out_de
     _check(lib().dsmoe_layer_forward_host(ctypes.byref(desc), _ptr(x_host), _ptr(x_dev), _ptr(Wr), _ptr(br),
                                           _ptr(W1), _ptr(W2), _ptr(packed), _ptr(out_dev), _ptr(out_host),
                                           _ptr(workspace),
-                                          ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                                          workspace.numel() if workspace is not None else 0,
                                           _ptr(dev_status), _stream(stream)), "dsmoe_layer_forward_host")
 
 
@@ -204,20 +221,20 @@ def dsmoe_layer_forward_host_async(desc, x_host, x_dev, Wr, br, W1, W2, packed, 
     _check(lib().dsmoe_layer_forward_host_async(ctypes.byref(desc), _ptr(x_host), _ptr(x_dev), _ptr(Wr), _ptr(br),
                                                 _ptr(W1), _ptr(W2), _ptr(packed), _ptr(out_dev), _ptr(out_host),
                                                 _ptr(workspace),
-                                                ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                                                workspace.numel() if workspace is not None else 0,
                                                 _ptr(dev_status), _stream(stream)), "dsmoe_layer_forward_host_async")
 
 
 def dsmoe_mi_loss(desc, scores, loss3, grad, workspace, stream=None):
     _check(lib().dsmoe_mi_loss(ctypes.byref(desc), _ptr(scores), _ptr(loss3), _ptr(grad), _ptr(workspace),
-                               ctypes.c_size_t(workspace.numel() if workspace is not None else 0), _stream(stream)),
+                               workspace.numel() if workspace is not None else 0, _stream(stream)),
            "dsmoe_mi_loss")
 
 
 def dsmoe_dense_backward(desc, x, W1, W2, packed, scores, mask, dO, dS, dA, workspace, dev_status=None, stream=None):
     _check(lib().dsmoe_dense_backward(ctypes.byref(desc), _ptr(x), _ptr(W1), _ptr(W2), _ptr(packed), _ptr(scores),
                                       _ptr(mask), _ptr(dO), _ptr(dS), _ptr(dA), _ptr(workspace),
-                                      ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                                      workspace.numel() if workspace is not None else 0,
                                       _ptr(dev_status), _stream(stream)), "dsmoe_dense_backward")
 
 
@@ -229,19 +246,19 @@ def dsmoe_moa_forward(desc, n_head, scale, Kc, Vc, tok_seq, pos, x, Wr, br, pack
     args = MoaArgs(int(n_head), int(n_seq), int(L), float(scale), _ptr(Kc), _ptr(Vc), _ptr(tok_seq), _ptr(pos))
     _check(lib().dsmoe_moa_forward(ctypes.byref(desc), ctypes.byref(args), _ptr(x), _ptr(Wr), _ptr(br), _ptr(packed),
                                    _ptr(out), _ptr(mask_out), _ptr(counts_out), _ptr(workspace),
-                                   ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                                   workspace.numel() if workspace is not None else 0,
                                    _ptr(dev_status), _stream(stream)), "dsmoe_moa_forward")
 
 
 def dsmoe_timing_enable(n_pairs: int):
-    _check(lib().dsmoe_timing_enable(ctypes.c_int(int(n_pairs))), "dsmoe_timing_enable")
+    _check(lib().dsmoe_timing_enable(int(n_pairs)), "dsmoe_timing_enable")
 
 
 def dsmoe_timing_read(n_max: int):
     """Durations (ms) of the timed launches since the ring was enabled or last read, in launch order."""
     buf = (ctypes.c_float * max(n_max, 1))()
     n = ctypes.c_int(0)
-    _check(lib().dsmoe_timing_read(buf, ctypes.c_int(n_max), ctypes.byref(n)), "dsmoe_timing_read")
+    _check(lib().dsmoe_timing_read(buf, n_max, ctypes.byref(n)), "dsmoe_timing_read")
     return [float(buf[i]) for i in range(n.value)]
 
 
