@@ -324,7 +324,8 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
         const auto want_next = [&]() { ptx::mbar_arrive(ptx::smem_u32(&sh.want)); };
         while (alive && tiles.next(sh, lane, t)) {
             const int claim_at = max(t.nk - kClaimAhead, 0);
-            if (lane == 0 && t.up) {
+            const bool elected = ptx::elect_one();
+            if (elected && t.up) {
                 for (int i = 0; i < t.nk; ++i) {
                     if (i == claim_at) want_next();
                     if (!ptx::mbar_wait(ptx::smem_u32(&sh.empty[s]), ((phb >> s) & 1u) ^ 1u, &sh.abort_flag)) {
@@ -335,7 +336,7 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
                     load_b(&tmW1, i, P.H);
                     next_slot();
                 }
-            } else if (lane == 0) {
+            } else if (elected) {
                 // the weights do not wait for h: while its rows are being finished elsewhere, a ring of them is on its way
                 int ahead = 0, s0 = s;
                 if (!h_complete) {
@@ -377,7 +378,7 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
                     next_slot();
                 }
             }
-            alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
+            alive = __all_sync(0xffffffffu, alive);
         }
         chain_next();
         if (lane == 0) GT_PUT(7, gt_h);
@@ -402,7 +403,7 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
             if (!t.up && !gt_seen && lane == 0) GT_SET(1);
             gt_seen = gt_seen || !t.up;
 #endif
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 GT_T0(t_acc);
                 alive = ptx::mbar_wait(ptx::smem_u32(&sh.tempty[acc]), aph ^ 1u, &sh.abort_flag);
                 GT_ADD(gt_acc, t_acc);
@@ -431,7 +432,7 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
                 }
                 if (alive) ptx::umma_commit(ptx::smem_u32(&sh.tfull[acc]));       // accumulator complete
             }
-            alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
+            alive = __all_sync(0xffffffffu, alive);
             if (++acc == 2) {
                 acc = 0;
                 aph ^= 1u;

@@ -352,7 +352,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             int s = 0;
             uint32_t ph = 0;
             bool alive = true;
@@ -362,6 +362,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             GTRACE_T0(t_all);
             for (int id = first_tile; id < ntiles && alive; id += tile_step) {
                 const Tile t = decode_tile<PAIR>(P, sh, id, half);
+                int down_e = 0, down_kb = 0;       // dense down: the block's expert, and which of its blocks it is
                 for (int i = 0; i < t.nk; ++i) {
                     GTRACE_T0(t_w);
                     if (!bar_wait<PAIR>(ptx::smem_u32(&sh.empty[s]), ph ^ 1u, &sh.abort_flag)) {
@@ -376,9 +377,13 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     else if (half == 0) ptx::mbar_expect_tx(ptx::smem_u32(&sh.full[s]), bytes + (P.gather ? 0u : (uint32_t)A_STAGE_BYTES));
                     int a_col, b_e, b_k;
                     if (P.mode == GEMM_DENSE_DOWN) {
-                        b_e = i / kbpe;
-                        b_k = (i % kbpe) * BK;
-                        a_col = b_e * P.k_per_expert + b_k;
+                        b_e = down_e;
+                        b_k = down_kb * BK;
+                        a_col = i * BK;
+                        if (++down_kb == kbpe) {
+                            down_kb = 0;
+                            ++down_e;
+                        }
                     } else {
                         b_e = t.e;
                         b_k = (t.k0 + i) * BK;
@@ -423,7 +428,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && half == 0) {
+        if (half == 0 && ptx::elect_one()) {
             int s = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
             bool alive = true;
@@ -1232,7 +1237,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
     // at that point without touching the barriers.
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             int s = 0;
             uint32_t phb = 0;
             bool alive = true, spec = P.spec != 0;
@@ -1366,7 +1371,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             int s = 0, acc = 0;
             uint32_t phb = 0, aph = 0;
             bool alive = true, spec = P.spec != 0;

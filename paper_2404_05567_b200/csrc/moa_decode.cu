@@ -232,12 +232,12 @@ moa_decode_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
         ptx::tma_load_2d(ring + (uint32_t)(s * G::STAGE + G::W_BYTES), &tmX, ptx::smem_u32(&sh.full[warp][s]), (b0 + i) * 64, 0);
     };
     // the output projection's first weights do not wait for the attention step: nothing that the call writes
-    if (!QUERY && lane == 0)
+    if (!QUERY && ptx::elect_one())
         for (int s = 0; s < S; ++s)
             if (warp + s * kDgWarps < n) load_w(warp + s * kDgWarps, s);
     chain_wait();
     chain_next();
-    if (lane == 0)
+    if (ptx::elect_one())
         for (int s = 0; s < S; ++s)
             if (warp + s * kDgWarps < n) {
                 if (QUERY) load_w(warp + s * kDgWarps, s);
@@ -314,7 +314,7 @@ moa_decode_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
                 }
             }
             __syncwarp();
-            if (lane == 0 && i + S * kDgWarps < n) {
+            if (i + S * kDgWarps < n && ptx::elect_one()) {
                 load_w(i + S * kDgWarps, (int)s);
                 load_x(i + S * kDgWarps, (int)s);
             }

@@ -107,7 +107,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
     chain_wait();
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             for (int n = 0; n < nk; ++n) {
                 const int s = n % G::STA;
                 if (!ptx::mbar_wait(ptx::smem_u32(&sh.empty_a[s]), ((uint32_t)(n / G::STA) & 1u) ^ 1u, &sh.abort_flag)) break;
@@ -117,7 +117,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t idesc = ptx::make_idesc_bf16(kRuM, G::N);
             bool alive = true;
             uint32_t acc = tmem;
