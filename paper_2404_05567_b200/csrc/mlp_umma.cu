@@ -1872,13 +1872,19 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
         }
         st->max_pairs = n < st->sm_count / 2 ? n : st->sm_count / 2;
     }
-    // Measured (C3, C4 and the paper's shapes): pairs gain 3 to 8 % where a long mainloop runs against a light
-    // epilogue (plain stores after a reduction of 1024 or more), lose up to 9 % under the GeLU and gathering
-    // up-projections and on short reductions, and change nothing under the aggregating epilogue.
+    // Dense launches of more rows than one CTA's tile always pair (us, single CTAs and pairs): the forward of 16384 tokens of d 2048, H 1024
+    // 3490, 3202; 4000 of 4096, 512 937, 883; 150 of 2048, 1024 276, 209; 150 of 2048, 256 87, 84; a training step of 8190 tokens 1910, 1761, of 129
+    // 73, 72.  Grouped launches do where a long mainloop runs against a light epilogue (plain stores after a reduction of 1024 or more): half
+    // of a pair's tile is empty more often, and under the gathering up-projection, on short reductions and with the aggregation
+    // in the epilogue they lose up to 20 % or change nothing.
     bool pair = pair_tiles > 0 && st->max_pairs > 0 && (P.n_per_expert % 64) == 0;
     if (pair_override() == 0) pair = false;
     else if (pair && pair_override() != 1)
-        pair = P.epi == EPI_STORE && pair_tiles >= st->max_pairs && (P.mode == GEMM_DENSE_DOWN || P.k_per_expert >= 1024);
+        pair = P.mode == GEMM_GROUPED ? P.epi == EPI_STORE && pair_tiles >= st->max_pairs && P.k_per_expert >= 1024 : P.rows > BM;
+    // (the large dense launches are not chained: no gap to speak of, and 1 % slower with it, 3682 against 3732 us for the
+    // dense layer at 16384 tokens; grouped ones all are: 300 tokens of 2048 / 1024 93.7 against 98.7 us for the layer, 8192
+    // of 3072 / 1536 alike, 7001 of 4096 / 512 428 against 425)
+    const bool chain = P.mode == GEMM_GROUPED || P.rows <= kChainMaxRows;
     int timed = -1;
     if (may_time) DSMOE_TRY(timing_begin(s, &timed));
     if (pair) {
@@ -1896,6 +1902,10 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
             at[na].id = cudaLaunchAttributeCooperative;
             at[na].val.cooperative = 1;
             ++na;
+        } else if (chain) {
+            at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[na].val.programmaticStreamSerializationAllowed = 1;
+            ++na;
         }
         cfg.attrs = at; cfg.numAttrs = na;
         DSMOE_CUDA_TRY(cudaLaunchKernelEx(&cfg, umma_gemm_kernel<true>, a, b, P));
@@ -1905,10 +1915,7 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
         DSMOE_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(umma_gemm_kernel<false>), dim3(grid), dim3(threads),
                                                    args, smem, s));
     } else {
-        // (the large dense launches are not chained: no gap to speak of, and 1 % slower with it, 3682 against 3732 us for the
-        // dense layer at 16384 tokens; grouped ones all are: 300 tokens of 2048 / 1024 93.7 against 98.7 us for the layer, 8192
-        // of 3072 / 1536 alike, 7001 of 4096 / 512 428 against 425)
-        if (P.mode == GEMM_GROUPED || P.rows <= kChainMaxRows)
+        if (chain)
             DSMOE_CUDA_TRY(launch_chained(umma_gemm_kernel<false>, grid, threads, smem, s, a, b, P));
         else {
             umma_gemm_kernel<false><<<grid, threads, smem, s>>>(a, b, P);
