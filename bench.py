@@ -250,9 +250,9 @@ def drop_weights(torch, keep_shape=None):
 
 
 def sums_inside(s):
-    """Whether the down-projection also aggregates (the library's rule, dsmoe.h)."""
-    return s.fuse_combine == 1 or (s.fuse_combine == 0 and s.mode == gi.MODE_TOPK and s.H >= 1024 and
-                                   s.T * min(s.K, s.E) >= 1024 * s.E)
+    """Whether the down-projection also aggregates (the library's rule with a workspace of the size that it reports, dsmoe.h)."""
+    return s.fuse_combine == 1 or (s.fuse_combine == 0 and s.mode == gi.MODE_TOPK and s.H >= 1536 and
+                                   s.T * min(s.K, s.E) >= 2560 * s.E)
 
 
 def mlp_launches(s):

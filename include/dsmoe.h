@@ -91,9 +91,10 @@ typedef struct {
                                     through L2 and is hidden only when the experts are wide);
                                  2: the epilogue stores the gate-weighted outputs as fp32 rows and a
                                     second kernel adds a token's rows;
-                                 0: the library chooses: 1 for a top-K selection with H >= 1024 and
-                                    T*K >= 1024*E (wide experts, many row tiles per expert), else as 2
-                                    (bit for bit), with both projections in one launch. */
+                                 0: the library chooses: 1 for a top-K selection with H >= 1536 and
+                                    T*K >= 2560*E (wide experts, very many rows), else as 2 (bit for
+                                    bit), with both projections in one launch; with H >= 1024,
+                                    T*K >= 1024*E and a workspace that holds only what 1 needs, 1. */
 } dsmoe_layer_desc;
 
 /* A void* stands for the caller's cudaStream_t so that this header needs no CUDA include. */

@@ -74,6 +74,19 @@ WsLayout ws_layout(const dsmoe_layer_desc& p) {
     return L;
 }
 
+WsLayout ws_layout_within(dsmoe_layer_desc* p, size_t ws_bytes) {
+    const WsLayout L = ws_layout(*p);
+    if (ws_bytes >= L.total_packed || p->fuse_combine != 0 || p->mode != DSMOE_SELECT_TOPK || p->H < 1024 ||
+        (long long)p->T * width_of(*p) < 1024ll * p->E)
+        return L;
+    dsmoe_layer_desc inside = *p;
+    inside.fuse_combine = 1;
+    const WsLayout I = ws_layout(inside);
+    if (ws_bytes < I.total_packed) return L;
+    *p = inside;
+    return I;
+}
+
 namespace {
 DeviceState g_dev_state[kMaxDeviceSlots];
 }
@@ -181,8 +194,9 @@ dsmoe_status dsmoe_expert_mlp(const dsmoe_layer_desc* desc, const void* xp, cons
     if (!xp || !offsets || !yp || !aligned16(xp) || !aligned16(yp)) return DSMOE_ERR_INVALID_ARG;
     if (packed && desc->dtype != DSMOE_BF16) return DSMOE_ERR_INVALID_ARG;
     if (!packed && (!W1 || !W2)) return DSMOE_ERR_INVALID_ARG;
-    const WsLayout L = ws_layout(*desc);
     const bool fast = packed && umma_supported(*desc);
+    dsmoe_layer_desc p = *desc;
+    const WsLayout L = fast ? ws_layout_within(&p, ws_bytes) : ws_layout(p);
     if (!fast && (!W1 || !W2)) return DSMOE_ERR_UNSUPPORTED;   // packed weights given, but this shape needs the plain path
     if (!fast && (!aligned16(W1) || !aligned16(W2))) return DSMOE_ERR_INVALID_ARG;
     if (!workspace || ws_bytes < (fast ? L.total_packed : L.total_plain) || !aligned16(workspace)) return DSMOE_ERR_WORKSPACE;
@@ -220,13 +234,13 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
                                  uint64_t* mask_out, int32_t* counts_out, void* workspace, size_t ws_bytes,
                                  int32_t* dev_status, dsmoe_stream stream) {
     DSMOE_TRY(check_desc(desc));
-    const dsmoe_layer_desc& p = *desc;
+    dsmoe_layer_desc p = *desc;
     if (p.T == 0) return DSMOE_OK;
     if (!x || !Wr || !out || !aligned16(x) || !aligned16(Wr) || !aligned16(out)) return DSMOE_ERR_INVALID_ARG;
     if (packed && p.dtype != DSMOE_BF16) return DSMOE_ERR_INVALID_ARG;
     if (!packed && (!W1 || !W2)) return DSMOE_ERR_INVALID_ARG;
-    const WsLayout L = ws_layout(p);
     const bool fast = packed && umma_supported(p);
+    const WsLayout L = fast ? ws_layout_within(&p, ws_bytes) : ws_layout(p);
     if (!fast && (!W1 || !W2)) return DSMOE_ERR_UNSUPPORTED;   // this shape needs the unpacked weights
     if (!fast && (!aligned16(W1) || !aligned16(W2))) return DSMOE_ERR_INVALID_ARG;
     if (!workspace || ws_bytes < (fast ? L.total_packed : L.total_plain) || !aligned16(workspace)) return DSMOE_ERR_WORKSPACE;
@@ -354,7 +368,8 @@ dsmoe_status dsmoe_dense_backward(const dsmoe_layer_desc* desc, const void* x, c
     if (packed && desc->dtype != DSMOE_BF16) return DSMOE_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if (packed && umma_supported(*desc)) {
-        const WsLayout L = ws_layout(*desc);
+        dsmoe_layer_desc p = *desc;
+        const WsLayout L = ws_layout_within(&p, ws_bytes);
         if (!workspace || ws_bytes < L.total_packed || !aligned16(workspace)) return DSMOE_ERR_WORKSPACE;
         char* ws = static_cast<char*>(workspace);
         return launch_dense_backward(*desc, x, W2, packed, scores, mask, dO, dS, dA, ws + L.h,
@@ -368,14 +383,14 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
                                const float* br, const void* packed, void* out, uint64_t* mask_out, int32_t* counts_out,
                                void* workspace, size_t ws_bytes, int32_t* dev_status, dsmoe_stream stream) {
     DSMOE_TRY(check_desc(desc));
-    const dsmoe_layer_desc& p = *desc;
+    dsmoe_layer_desc p = *desc;
     if (p.T == 0) return DSMOE_OK;
     if (!args || !x || !Wr || !out || !packed || !args->Kc || !args->Vc || !args->pos) return DSMOE_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(Wr) || !aligned16(out) || !aligned16(packed) || !aligned16(args->Kc) || !aligned16(args->Vc))
         return DSMOE_ERR_INVALID_ARG;
     if (args->n_seq <= 0 || args->L <= 0) return DSMOE_ERR_INVALID_ARG;
     if (p.dtype != DSMOE_BF16 || !moa_supported(p, args->n_head, args->L)) return DSMOE_ERR_UNSUPPORTED;
-    const WsLayout L = ws_layout(p);
+    const WsLayout L = ws_layout_within(&p, ws_bytes);
     if (!workspace || ws_bytes < L.total_packed || !aligned16(workspace)) return DSMOE_ERR_WORKSPACE;
     char* ws = static_cast<char*>(workspace);
     cudaStream_t s = (cudaStream_t)stream;

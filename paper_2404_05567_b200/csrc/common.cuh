@@ -115,6 +115,9 @@ struct WsLayout {
     size_t total_plain, total_packed, total;
 };
 WsLayout ws_layout(const dsmoe_layer_desc& p);
+// The layout of a call with packed weights and ws_bytes of workspace.  A workspace too small for the outputs' rows that the second
+// kernel adds up, but large enough for the tokens' running sums, has the sum taken inside the down-projection (*p changes).
+WsLayout ws_layout_within(dsmoe_layer_desc* p, size_t ws_bytes);
 
 // What the library keeps per device (attributes that must be set once per device, the SM count).  Entry points
 // are not thread-safe: one host thread at a time may call into the library.
@@ -164,14 +167,13 @@ dsmoe_status launch_stats(const dsmoe_layer_desc& p, const float* scores, const 
 dsmoe_status launch_combine(const dsmoe_layer_desc& p, const void* yp, const float* row_gate,
                             const int32_t* token_rows, const int32_t* k_t, void* out, cudaStream_t s,
                             bool yp_f32 = false);
-// Whether dsmoe_layer_forward's tensor-core grouped path aggregates inside the down-projection (see dsmoe.h)
-// The library's own choice (fuse_combine == 0): inside only where it was measured to be as fast as the second
-// kernel -- wide experts (a long enough mainloop to hide the read-modify-write of the sums) and a top-K selection
-// with at least eight row tiles per expert on average (few tiles per expert make consecutive experts' tiles, which
-// must take turns on the same sums, run at the same time).
+// Whether dsmoe_layer_forward's tensor-core grouped path aggregates inside the down-projection (see dsmoe.h).  The library's own choice
+// (fuse_combine == 0) is the second kernel, both projections then being one launch, except for wide experts of very many rows.  us a layer of
+// 32 experts, inside and beside: 8192 tokens of d 2048, H 1024 top-4 610, 333, top-12 (3072 rows an expert) 1018, 925; of d 3072, H 1536 top-4
+// 910, 673, top-6 1105, 988, top-12 1906, 1962; 5000 tokens top-12 (1875 rows) 1230, 1210; 3333 tokens 959, 774.
 static inline bool fuses_combine(const dsmoe_layer_desc& p) {
     if (p.fuse_combine != 0) return p.fuse_combine == 1;
-    return p.mode == DSMOE_SELECT_TOPK && p.H >= 1024 && (long long)p.T * width_of(p) >= 1024ll * p.E;
+    return p.mode == DSMOE_SELECT_TOPK && p.H >= 1536 && (long long)p.T * width_of(p) >= 2560ll * p.E;
 }
 dsmoe_status launch_pack(const dsmoe_layer_desc& p, const void* W1, const void* W2, void* packed,
                          cudaStream_t s);

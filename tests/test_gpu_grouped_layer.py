@@ -197,3 +197,36 @@ def test_two_streams_with_a_workspace_each(shape):
     for k in range(2):
         for i in range(20):
             assert torch.equal(got[k][i], want[(i + k) % 2]), (k, i)
+
+
+def test_a_workspace_for_the_running_sums_alone_is_still_enough():
+    """Wide experts with many rows under top-K: with room for the tokens' sums but not for the expert outputs' rows the sum is taken inside
+    the down-projection, as with fuse_combine = 1; with less the call is refused, and so is a narrower layer with as little."""
+    T, d, E, K = 2048, 128, 4, 2
+    g = torch.Generator(device="cuda").manual_seed(5)
+    for H in (1024, 512):
+        W1, W2 = (torch.randn(s, generator=g, device="cuda").bfloat16() * 0.05 for s in ((E, d, H), (E, H, d)))
+        x, Wr = torch.randn((T, d), generator=g, device="cuda").bfloat16(), torch.randn((d, E), generator=g, device="cuda") * 0.1
+        desc = {f: dm.make_desc(T, d, H, E, dm.BF16, dm.SELECT_TOPK, K=K, fuse_combine=f) for f in (0, 1)}
+        packed = torch.empty(dm.dsmoe_packed_size(desc[0]), dtype=torch.uint8, device="cuda")
+        dm.dsmoe_pack_weights(desc[0], W1, W2, packed)
+        small, full = dm.dsmoe_workspace_size_packed(desc[1]), dm.dsmoe_workspace_size_packed(desc[0])
+        assert small < full
+
+        def run(f, nbytes):
+            ws, out = torch.empty(nbytes, dtype=torch.uint8, device="cuda"), torch.empty((T, d), dtype=torch.bfloat16, device="cuda")
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            dm.dsmoe_layer_forward(desc[f], x, Wr, None, None, None, packed, out, None, None, ws, status)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0
+            return out
+
+        if H == 1024:
+            assert torch.equal(run(0, small), run(1, small))
+            with pytest.raises(dm.DsmoeError):
+                run(0, small - 1)
+        else:
+            with pytest.raises(dm.DsmoeError):
+                run(0, small)
+        err = (run(0, full).float() - run(1, small).float()).norm() / run(1, small).float().norm()
+        assert err <= 2 ** -8                                     # one rounding to bf16 of sums that differ by rounding in fp32
