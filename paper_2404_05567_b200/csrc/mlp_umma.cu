@@ -71,7 +71,8 @@ enum { GEMM_GROUPED = 0, GEMM_DENSE_UP = 1, GEMM_DENSE_DOWN = 2 };
 enum { EPI_GELU = 0, EPI_STORE = 1, EPI_COMBINE = 2, EPI_BWD = 3 };
 constexpr int kUpUnit = 16;          // small-T up-projection: weight rows per work unit
 constexpr int kUpTileUnits = 16;     // ... and units per tile (256 rows)
-constexpr int kRouterBatch = 12;     // rows of Wr a router thread loads at once
+constexpr int kRouterBatch = 12;     // rows of Wr a router thread loads at once (for one token; fewer for several)
+constexpr int kRouterSlices = 16;    // most slices of the router's reduction
 constexpr int kFixBatch = 24;        // partial tiles a fix-up thread loads at once
 // small-T kernel: bytes of loads a CTA keeps in flight (<= RING_BYTES).  Four 36 KB slots per SM already cover the
 // bandwidth-delay product; a deeper ring only lengthens the queues that the router's loads, the grid barriers and
@@ -156,6 +157,7 @@ struct Shared {
     volatile int geo_state;
     volatile int spec_issued, spec_stop;   // producer -> MMA issuer: ring slots filled under geo[0]; no more will be
     volatile int mma_drained;              // MMA issuer -> producer: those slots are consumed, the ring is idle
+    int router_last;                       // small_layer_kernel: this CTA's slice was its token group's last
     union {
         int rowtok[(DSMOE_PAIR_GW > 8 ? DSMOE_PAIR_GW / 2 : 6) * BM];                // umma_gemm_kernel, gathered A: the source row of each tile row, per gathering warp
         struct {                           // small_layer_kernel: router gates and every token's selection word
@@ -888,6 +890,7 @@ struct SmallParams {
     void* out;
     int out_f32;
     int* sync;               // 8 ints, zero at launch: barrier counters [0..2] and an abort flag [4]
+    int* group_done;         // zero at launch: the router's finished slices of each group of tokens
     int spec;                // start streaming under "every expert selected" before the router has finished
     int32_t* dev_status;
 };
@@ -1063,11 +1066,13 @@ struct RouterArgs {
     int32_t* k_t;
     SelParams sel;
 };
+// READ: compiled for KS == 0 alone.
+template <bool READ>
 __device__ __noinline__ void small_router_pass(const RouterArgs P, Shared& sh, int KS, int w, int lane, int mode, int e,
                                                int e2) {
     constexpr int NW = kEpiThreads / 32;
-    if (KS == 0) {
-        // One CTA per token held the whole reduction (KS = 1 in the kernel) and has written that token's scores and
+    if (READ || KS == 0) {
+        // The token's CTA (KS = 1 in the kernel), or the last of its group's, has written its scores and
         // selection itself before the grid barrier: here they are only read (a thread per token)
         const int tt = w * 32 + lane;
         if (mode == 0) {
@@ -1134,6 +1139,91 @@ __device__ __noinline__ void small_router_pass(const RouterArgs P, Shared& sh, i
     }
 }
 
+// Router, one slice of the reduction over d for TT neighbouring tokens (nt of them exist), by the 12 epilogue warps.  A row of Wr (E
+// floats) is covered by E/4 neighbouring threads with one 16-byte load each, so a warp reads whole rows, coalesced, and a thread keeps
+// only its four experts' sums over every rpp-th row, BATCH rows' loads at a time.  The threads' sums meet inside the warp (where its
+// lanes hold whole rows) and in shared memory.
+template <int TT, int BATCH>
+__device__ __forceinline__ void small_router_slice(const SmallParams& P, float* stg, int t0, int nt, int sl, int KS, int etid) {
+    const int E = P.E, lane = etid & 31;
+    const int klen = (P.d + KS - 1) / KS, kbeg = sl * klen, kend = min(P.d, kbeg + klen);
+    const int quads = (E + 3) / 4;                  // threads per row
+    const int rpp = kEpiThreads / quads;            // rows per pass
+    const int qd = etid % quads, r0 = etid / quads;
+    const __nv_bfloat16* xr[TT];
+#pragma unroll
+    for (int u = 0; u < TT; ++u) xr[u] = P.x + (size_t)(t0 + min(u, nt - 1)) * P.d;      // past the last token: it again, unused
+    float4 acc[TT];
+#pragma unroll
+    for (int u = 0; u < TT; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r0 < rpp) {
+        if ((E & 3) == 0) {
+#pragma unroll 1
+            for (int kb = kbeg + r0; kb < kend; kb += BATCH * rpp) {
+                float4 w[BATCH];
+                float xs[TT][BATCH];
+#pragma unroll
+                for (int j = 0; j < BATCH; ++j) {
+                    const int k = kb + j * rpp;
+                    const bool ok = k < kend;
+                    w[j] = ok ? reinterpret_cast<const float4*>(P.Wr + (size_t)k * E)[qd] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int u = 0; u < TT; ++u) xs[u][j] = ok ? __bfloat162float(xr[u][k]) : 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < BATCH; ++j) {
+#pragma unroll
+                    for (int u = 0; u < TT; ++u) {
+                        acc[u].x = fmaf(xs[u][j], w[j].x, acc[u].x);
+                        acc[u].y = fmaf(xs[u][j], w[j].y, acc[u].y);
+                        acc[u].z = fmaf(xs[u][j], w[j].z, acc[u].z);
+                        acc[u].w = fmaf(xs[u][j], w[j].w, acc[u].w);
+                    }
+                }
+            }
+        } else {
+            const int e0 = qd * 4;
+            for (int k = kbeg + r0; k < kend; k += rpp) {
+                const float* const w = P.Wr + (size_t)k * E + e0;
+#pragma unroll
+                for (int u = 0; u < TT; ++u) {
+                    const float xv = __bfloat162float(xr[u][k]);
+                    acc[u].x = fmaf(xv, w[0], acc[u].x);
+                    if (e0 + 1 < E) acc[u].y = fmaf(xv, w[1], acc[u].y);
+                    if (e0 + 2 < E) acc[u].z = fmaf(xv, w[2], acc[u].z);
+                    if (e0 + 3 < E) acc[u].w = fmaf(xv, w[3], acc[u].w);
+                }
+            }
+        }
+    }
+    int rows = rpp, slot = r0;
+    bool writes = r0 < rpp;
+    if ((32 % quads) == 0) {
+#pragma unroll
+        for (int u = 0; u < TT; ++u)
+            for (int o = 16; o >= quads; o >>= 1) {
+                acc[u].x += __shfl_xor_sync(0xffffffffu, acc[u].x, o);
+                acc[u].y += __shfl_xor_sync(0xffffffffu, acc[u].y, o);
+                acc[u].z += __shfl_xor_sync(0xffffffffu, acc[u].z, o);
+                acc[u].w += __shfl_xor_sync(0xffffffffu, acc[u].w, o);
+            }
+        rows = kEpiThreads / 32;
+        slot = etid >> 5;
+        writes = lane < quads;
+    }
+    float4* const st = reinterpret_cast<float4*>(stg);               // [token][row][quad]
+    if (writes)
+#pragma unroll
+        for (int u = 0; u < TT; ++u) st[(u * rows + slot) * quads + qd] = acc[u];
+    asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+    for (int i = etid; i < nt * E; i += kEpiThreads) {
+        const int u = i / E, e = i % E;
+        float v = 0.f;
+        for (int r = 0; r < rows; ++r) v += stg[((u * rows + r) * quads + (e >> 2)) * 4 + (e & 3)];
+        P.partial[((size_t)(t0 + u) * KS + sl) * kMaxExperts + e] = v;       // the partial-sum buffer is free until the down-projection
+    }
+}
+
 // Between the two projections HBM has nothing to do for several microseconds (epilogues, the slowest CTA, the barrier), and the
 // ring is full.  So the next weight tiles of this CTA's sequence, units u0 .. u1 - 1 of the down-projection, are asked into L2
 // meanwhile: the down-projection then finds them there instead of in DRAM.  All CTAs together ask for well under half of L2.
@@ -1179,6 +1269,9 @@ __device__ __forceinline__ bool wait_flag(volatile int* flag, Shared& sh) {
     }
 }
 
+// GROUPS: the router by groups of tokens (small_groups).  The two forms are kernels of their own: with both in one, calls that take the
+// other ran 2 to 5 % slower on the same bits.
+template <bool GROUPS>
 __global__ void __launch_bounds__(SMALL_THREADS, 1)
 small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ BMaps16 tmW1,
                    const __grid_constant__ CUtensorMap tmHg, const __grid_constant__ BMaps tmW2, const SmallParams P) {
@@ -1522,73 +1615,110 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         const int etid = (int)threadIdx.x - 64;         // 0 .. kEpiThreads-1
 #define EPI_SYNC() asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory")
         // ---- router, step 1
-        // The reduction over d of every token is cut into KS slices, one CTA per (token, slice).  A row of Wr
-        // (E floats) is covered by E/4 neighbouring threads with one 16-byte load each, so a warp reads whole
-        // rows, coalesced, and a thread keeps only its four experts' sums over every rpp-th row; all its loads are
-        // independent.  The threads' sums meet in shared memory.
-        int KS = 1;                                   // 1, 2, 4, 8 or 16 slices
-        while (KS < 16 && KS * 2 * P.T <= G) KS *= 2;
-        if ((int)blockIdx.x < P.T * KS) {
-            const int t = blockIdx.x / KS, sl = blockIdx.x % KS, E = P.E;
-            const int klen = (P.d + KS - 1) / KS, kbeg = sl * klen, kend = min(P.d, kbeg + klen);
-            const __nv_bfloat16* __restrict__ xr = P.x + (size_t)t * P.d;
-            const float* __restrict__ Wr = P.Wr;
-            const int quads = (E + 3) / 4;                  // threads per row
-            const int rpp = kEpiThreads / quads;            // rows per pass
-            const int qd = etid % quads, r0 = etid / quads;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (etid == 0) TRACE(12);
-            if (r0 < rpp) {
-                if ((E & 3) == 0) {
-                    // batches of kRouterBatch rows: every load of a batch is issued before its first use
-                    for (int kb = kbeg + r0; kb < kend; kb += kRouterBatch * rpp) {
-                        float4 w[kRouterBatch];
-                        float xs[kRouterBatch];
+        // The reduction over d is cut into KS slices, one CTA each, and every CTA adds every token's slices itself after the grid barrier
+        // (small_router_pass; a single slice's CTA finishes the token before it); or groups of 2 or 4 tokens share a CTA's loads of Wr, the CTA of a group that comes last adds the
+        // slices in order, takes softmax and selection and writes them out, and after the barrier they are only read.
+        int KS = 1;                                   // without groups 1, 4, 8 or 16 slices
+        while (!GROUPS && KS < kRouterSlices && KS * 2 * P.T <= G) KS *= 2;
+        if (!GROUPS) {
+            if ((int)blockIdx.x < P.T * KS) {
+                // A row of Wr (E floats) is covered by E/4 neighbouring threads with one 16-byte load each, so a warp reads whole
+                // rows, coalesced, and a thread keeps only its four experts' sums over every rpp-th row; all its loads are
+                // independent.  The threads' sums meet in shared memory.
+                const int t = blockIdx.x / KS, sl = blockIdx.x % KS, E = P.E;
+                const int klen = (P.d + KS - 1) / KS, kbeg = sl * klen, kend = min(P.d, kbeg + klen);
+                const __nv_bfloat16* __restrict__ xr = P.x + (size_t)t * P.d;
+                const float* __restrict__ Wr = P.Wr;
+                const int quads = (E + 3) / 4;                  // threads per row
+                const int rpp = kEpiThreads / quads;            // rows per pass
+                const int qd = etid % quads, r0 = etid / quads;
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (etid == 0) TRACE(12);
+                if (r0 < rpp) {
+                    if ((E & 3) == 0) {
+                        // batches of kRouterBatch rows: every load of a batch is issued before its first use
+                        for (int kb = kbeg + r0; kb < kend; kb += kRouterBatch * rpp) {
+                            float4 w[kRouterBatch];
+                            float xs[kRouterBatch];
 #pragma unroll
-                        for (int j = 0; j < kRouterBatch; ++j) {
-                            const int k = kb + j * rpp;
-                            const bool ok = k < kend;
-                            w[j] = ok ? __ldg(reinterpret_cast<const float4*>(Wr + (size_t)k * E) + qd) : make_float4(0.f, 0.f, 0.f, 0.f);
-                            xs[j] = ok ? __bfloat162float(xr[k]) : 0.f;
-                        }
+                            for (int j = 0; j < kRouterBatch; ++j) {
+                                const int k = kb + j * rpp;
+                                const bool ok = k < kend;
+                                w[j] = ok ? __ldg(reinterpret_cast<const float4*>(Wr + (size_t)k * E) + qd) : make_float4(0.f, 0.f, 0.f, 0.f);
+                                xs[j] = ok ? __bfloat162float(xr[k]) : 0.f;
+                            }
 #pragma unroll
-                        for (int j = 0; j < kRouterBatch; ++j) {
-                            acc.x = fmaf(xs[j], w[j].x, acc.x);
-                            acc.y = fmaf(xs[j], w[j].y, acc.y);
-                            acc.z = fmaf(xs[j], w[j].z, acc.z);
-                            acc.w = fmaf(xs[j], w[j].w, acc.w);
+                            for (int j = 0; j < kRouterBatch; ++j) {
+                                acc.x = fmaf(xs[j], w[j].x, acc.x);
+                                acc.y = fmaf(xs[j], w[j].y, acc.y);
+                                acc.z = fmaf(xs[j], w[j].z, acc.z);
+                                acc.w = fmaf(xs[j], w[j].w, acc.w);
+                            }
                         }
-                    }
-                } else {
-                    const int e0 = qd * 4;
-                    for (int k = kbeg + r0; k < kend; k += rpp) {
-                        const float xv = __bfloat162float(xr[k]);
-                        const float* w = Wr + (size_t)k * E + e0;
-                        acc.x = fmaf(xv, __ldg(w), acc.x);
-                        if (e0 + 1 < E) acc.y = fmaf(xv, __ldg(w + 1), acc.y);
-                        if (e0 + 2 < E) acc.z = fmaf(xv, __ldg(w + 2), acc.z);
-                        if (e0 + 3 < E) acc.w = fmaf(xv, __ldg(w + 3), acc.w);
+                    } else {
+                        const int e0 = qd * 4;
+                        for (int k = kbeg + r0; k < kend; k += rpp) {
+                            const float xv = __bfloat162float(xr[k]);
+                            const float* w = Wr + (size_t)k * E + e0;
+                            acc.x = fmaf(xv, __ldg(w), acc.x);
+                            if (e0 + 1 < E) acc.y = fmaf(xv, __ldg(w + 1), acc.y);
+                            if (e0 + 2 < E) acc.z = fmaf(xv, __ldg(w + 2), acc.z);
+                            if (e0 + 3 < E) acc.w = fmaf(xv, __ldg(w + 3), acc.w);
+                        }
                     }
                 }
+                if (etid == 0) TRACE(13);
+                reinterpret_cast<float4*>(stg)[etid] = acc;      // stg[(r0 * quads + qd) * 4 + j]
+                EPI_SYNC();
+                if (etid < E) {
+                    const int e = etid;
+                    float v = 0.f;
+                    for (int r = 0; r < rpp; ++r) v += stg[(r * quads + (e >> 2)) * 4 + (e & 3)];
+                    P.partial[((size_t)t * KS + sl) * kMaxExperts + e] = v;   // the partial-sum buffer is free until the down-projection
+                    if (KS == 1) sh.gate_s[e] = v;          // the whole reduction: this CTA finishes its token below
+                }
             }
-            if (etid == 0) TRACE(13);
-            reinterpret_cast<float4*>(stg)[etid] = acc;      // stg[(r0 * quads + qd) * 4 + j]
-            EPI_SYNC();
-            if (etid < E) {
-                const int e = etid;
-                float v = 0.f;
-                for (int r = 0; r < rpp; ++r) v += stg[(r * quads + (e >> 2)) * 4 + (e & 3)];
-                P.partial[((size_t)t * KS + sl) * kMaxExperts + e] = v;   // the partial-sum buffer is free until the down-projection
-                if (KS == 1) sh.gate_s[e] = v;          // the whole reduction: this CTA finishes its token below
+        } else {
+            const int TT = 4 * ceil_div(P.T, 2) > G ? 4 : 2, groups = ceil_div(P.T, TT);
+            KS = min(kRouterSlices, G / groups);      // (T <= G: at least one)
+            const int group = blockIdx.x / KS, sl = blockIdx.x % KS, t0 = group * TT, nt = min(TT, P.T - t0);
+            if (group < groups) {
+                if (etid == 0) TRACE(12);
+                if (TT == 2) small_router_slice<2, kRouterBatch / 2>(P, stg, t0, nt, sl, KS, etid);
+                else small_router_slice<4, kRouterBatch / 3>(P, stg, t0, nt, sl, KS, etid);
+                if (etid == 0) TRACE(13);
+                __threadfence();
+                EPI_SYNC();
+                if (etid == 0) sh.router_last = atomicAdd(P.group_done + group, 1) == KS - 1;
+                EPI_SYNC();
+                if (sh.router_last && warp - 2 < nt) {
+                    __threadfence();
+                    const int t = t0 + warp - 2;
+                    const bool v_lo = lane < P.E, v_hi = lane + 32 < P.E;
+                    float lo[kRouterSlices], hi[kRouterSlices];
+#pragma unroll
+                    for (int j = 0; j < kRouterSlices; ++j) {
+                        const float* const pl = P.partial + ((size_t)t * KS + j) * kMaxExperts;
+                        lo[j] = j < KS && v_lo ? __ldcg(pl + lane) : 0.f;
+                        hi[j] = j < KS && v_hi ? __ldcg(pl + lane + 32) : 0.f;
+                    }
+                    float l_lo = P.br && v_lo ? P.br[lane] : 0.f, l_hi = P.br && v_hi ? P.br[lane + 32] : 0.f;
+#pragma unroll
+                    for (int j = 0; j < kRouterSlices; ++j) {
+                        l_lo += lo[j];
+                        l_hi += hi[j];
+                    }
+                    softmax_select_store<false>(l_lo, l_hi, t, P.sel, lane, P.scores, P.mask, P.k_t);
+                }
             }
         }
         EPI_SYNC();
-        // With one CTA per token (KS = 1: 37 tokens or more) the CTA holds its token's logits: it takes softmax and
+        // With one CTA per token (KS = 1: 75 tokens or more) the CTA holds its token's logits: it takes softmax and
         // selection itself and writes them out, and after the barrier every CTA reads all tokens' results instead of
         // repeating every token's softmax (at 128 tokens that repetition, once for the selection and once for the
         // gates, took 18 of the kernel's 76 us).  Same arithmetic as small_router_pass: bias + sum, softmax, selection.
-        const bool direct = KS == 1;
-        if (direct && (int)blockIdx.x < P.T && warp == 2) {
+        const bool direct = GROUPS || KS == 1;
+        if (!GROUPS && direct && (int)blockIdx.x < P.T && warp == 2) {
             const bool v_lo = lane < P.E, v_hi = lane + 32 < P.E;
             const float l_lo = v_lo ? (P.br ? P.br[lane] : 0.f) + sh.gate_s[lane] : 0.f;
             const float l_hi = v_hi ? (P.br ? P.br[lane + 32] : 0.f) + sh.gate_s[lane + 32] : 0.f;
@@ -1604,7 +1734,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         EPI_SYNC();
         // ---- router, step 2: softmax and selection of every token, in every CTA (see small_router_pass)
         const RouterArgs RA{P.T, P.E, P.br, P.partial, P.scores, P.mask, P.k_t, P.sel};
-        if (!sh.abort_flag) small_router_pass(RA, sh, direct ? 0 : KS, warp - 2, lane, 0, 0, 0);
+        if (!sh.abort_flag) small_router_pass<GROUPS>(RA, sh, direct ? 0 : KS, warp - 2, lane, 0, 0, 0);
         EPI_SYNC();
         if (etid == 0) {
             unsigned long long m = sh.active_mask;
@@ -1660,7 +1790,7 @@ small_layer_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
             if (!have) break;
             // router gate of every token for this tile's expert(s), recomputed from the slice sums (other CTAs' copies
             // of the scores are not visible yet) while the mainloop is still running
-            if (t.phase == 0 && !dead) small_router_pass(RA, sh, direct ? 0 : KS, warp - 2, lane, 1, t.e, t.e2);
+            if (t.phase == 0 && !dead) small_router_pass<GROUPS>(RA, sh, direct ? 0 : KS, warp - 2, lane, 1, t.e, t.e2);
             if (tmem_warp && !dead && !ptx::mbar_wait(ptx::smem_u32(&sh.tfull[acc]), aph, &sh.abort_flag)) dead = true;
             dead = __any_sync(0xffffffffu, dead);     // the TMEM reads below are warp-collective
 #ifdef DSMOE_TRACE
@@ -2039,6 +2169,14 @@ dsmoe_status launch_mlp_umma(const dsmoe_layer_desc& p, const void* xp, const vo
     return DSMOE_OK;
 }
 
+// The router by groups of tokens: where a token would have two slices or one (38 tokens or more).  Adding every token's slices in every CTA
+// takes longer with every token (64 tokens: 10.7 us before the partition was known, and as long again for the gates), and with one CTA
+// per token, the other form from 75 tokens on, each reads all of Wr.  For fewer tokens groups cost more than they save: under the weights'
+// stream a round trip through L2 takes 2 us, and they need three more of them (8 tokens of d 2048, H 1024 top-6 57.4 -> 60.5 us), as they do
+// for 75 tokens and more of a short reduction (100 of d 2048, H 256 37.1 -> 38.6).  us a layer, top-6 of 32, 64 tokens of d 2048, H 256 43.7 -> 35.8,
+// of d 3072, H 384 53.4 -> 43.0, of d 4096, H 512 70.1 -> 59.5, of d 2048, H 1024 67.1 -> 61.5; 75 tokens of d 3072, H 384 47.7 -> 45.2; 100 51.3 -> 50.6.
+bool small_groups(const dsmoe_layer_desc& p, int G) { return 4 * p.T > G && (2 * p.T <= G || p.d > 2048); }
+
 // Few tokens (decode): one cooperative launch of small_layer_kernel runs router, both projections and the
 // fix-up.
 bool small_supported(const dsmoe_layer_desc& p) {
@@ -2057,7 +2195,8 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     DeviceState* st = nullptr;
     DSMOE_TRY(device_state(&st));
     if (!st->attr_small) {
-        DSMOE_CUDA_TRY(cudaFuncSetAttribute(small_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(small_layer_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(small_layer_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
         st->attr_small = true;
     }
     const __nv_bfloat16* w1t = static_cast<const __nv_bfloat16*>(packed);
@@ -2091,11 +2230,15 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     // From kSpecMinT tokens on it is rare that an expert is selected by none of them, so the kernel starts the
     // up-projection under that assumption while its router is still running; it starts over if the router disagrees.
     P.spec = p.T >= kSpecMinT ? 1 : 0;
-    DSMOE_CUDA_TRY(cudaMemsetAsync(P.sync, 0, 32, s));
+    P.group_done = reinterpret_cast<int*>(ws + L.tile_done);
+    // (tile_done follows sync in the workspace)
+    const bool by_groups = small_groups(p, G);
+    DSMOE_CUDA_TRY(cudaMemsetAsync(P.sync, 0, by_groups ? L.tile_done - L.sync + (size_t)p.T * sizeof(int) : 32, s));
     void* args[] = {&mX, &mW1, &mHg, &mW2, &P};
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));
-    DSMOE_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(small_layer_kernel), dim3(G), dim3(SMALL_THREADS),
+    DSMOE_CUDA_TRY(cudaLaunchCooperativeKernel(by_groups ? reinterpret_cast<const void*>(small_layer_kernel<true>)
+                                                         : reinterpret_cast<const void*>(small_layer_kernel<false>), dim3(G), dim3(SMALL_THREADS),
                                                args, SMEM_BYTES, s));
     DSMOE_TRY(timing_end(s, timed));
     return DSMOE_OK;

@@ -1,0 +1,20 @@
+"""The decode kernel's router by groups of tokens against the oracle where the groups change: the first and last token counts of groups of
+2 and of 4, a last group that is not full, expert counts whose rows of the router's weights do and do not fill a warp (GPU required)."""
+import pytest
+
+import dsmoe_inputs as gi
+from harness import TOL_BF16, layer_parity
+
+pytestmark = pytest.mark.gpu
+
+CASES = [(37, 2112, 32), (38, 2112, 32), (39, 256, 64), (73, 192, 5), (74, 2112, 48), (75, 2112, 33), (77, 3072, 8), (128, 2112, 64)]
+
+
+@pytest.mark.parametrize("T,d,E", CASES, ids=[f"T{T}-d{d}-E{E}" for T, d, E in CASES])
+def test_router_by_groups(T, d, E):
+    r = layer_parity(gi.LayerSpec(f"groups{T}x{d}x{E}", T=T, d=d, H=128, E=E, dtype="bf16", mode=gi.MODE_TOPK, K=3, router_gain=4.0))
+    assert r["err_rows"] <= TOL_BF16, (r["err_rows"], r["err"])
+    L = r["layer"]
+    first = L.forward().clone()
+    for _ in range(3):                                     # the counters are zeroed by every call, the slices' order is fixed
+        assert (L.forward() == first).all()
