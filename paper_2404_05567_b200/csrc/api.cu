@@ -270,8 +270,11 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK) pr.mode = DSMOE_SELECT_THRESHOLD;
     // the tensor-core router leaves the per-chunk counts of its own selection behind (not Threshold-TopK's: that one
     // selects again)
-    const bool counted = fast && router_umma_supported(p) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
-    if (fast && router_umma_supported(p))
+    const bool by_cluster = fast && router_cluster_supported(p);
+    const bool counted = (by_cluster || (fast && router_umma_supported(p))) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
+    if (by_cluster)
+        DSMOE_TRY(launch_router_cluster(pr, x, Wr, br, scores, mask, k_t, s, counted ? chunk_prefix : nullptr));
+    else if (fast && router_umma_supported(p))
         DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, dev_status, s, counted ? chunk_prefix : nullptr));
     else
         DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s));
@@ -415,8 +418,11 @@ dsmoe_status dsmoe_moa_forward(const dsmoe_layer_desc* desc, const dsmoe_moa_arg
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK) pr.mode = DSMOE_SELECT_THRESHOLD;
     // the tensor-core router leaves the per-chunk counts of its own selection behind (not Threshold-TopK's: that one
     // selects again)
-    const bool counted = router_umma_supported(p) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
-    if (router_umma_supported(p))
+    const bool by_cluster = router_cluster_supported(p);
+    const bool counted = (by_cluster || router_umma_supported(p)) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
+    if (by_cluster)
+        DSMOE_TRY(launch_router_cluster(pr, x, Wr, br, scores, mask, k_t, s, counted ? chunk_prefix : nullptr));
+    else if (router_umma_supported(p))
         DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, dev_status, s, counted ? chunk_prefix : nullptr));
     else
         DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s));

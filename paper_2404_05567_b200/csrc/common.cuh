@@ -204,6 +204,10 @@ bool router_umma_supported(const dsmoe_layer_desc& p, int max_run = 0);
 dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
                                 float* scores, uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s,
                                 int32_t* chunk_counts = nullptr, int max_run = 0);
+// Router for some hundred tokens (router_cluster.cu), as launch_router_umma otherwise.
+bool router_cluster_supported(const dsmoe_layer_desc& p);
+dsmoe_status launch_router_cluster(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores, uint64_t* mask,
+                                   int32_t* k_t, cudaStream_t s, int32_t* chunk_counts);
 // Grouped expert MLPs on expert-sorted rows: h = GeLU(xp.W1[e]) (bf16, in `hbuf`), yp = h.W2[e].
 // With row_token (and x), the up-projection gathers its rows from x by index and xp is not read.
 // With cmb->out, the down-projection's epilogue also aggregates (Eq. 1's weighted sum, ascending expert order per
