@@ -269,7 +269,10 @@ def kernels_per_step(s, decode):
     # router, row indices (counts and scan inside up to 16384 tokens), up, down, and the aggregation unless it runs inside the
     # down-projection; Threshold-TopK selects again (batch K, selection) and counts the chunks itself
     fused = sums_inside(s)
-    grouping = (2 if s.T > 16384 else 1) + (3 + (s.T > 256) if s.mode == gi.MODE_THRESHOLD_TOPK else 0)
+    # (the one-launch expert MLPs find the rows of few tokens themselves)
+    grouping = 0 if mlp_launches(s) == 1 and s.T <= (2048 if s.E <= 32 else 1024) else 2 if s.T > 16384 else 1
+    if s.mode == gi.MODE_THRESHOLD_TOPK:
+        grouping += 3 + (grouping > 0 and s.T > 256)
     return 1 + grouping + mlp_launches(s) + (0 if fused else 1)
 
 

@@ -272,12 +272,20 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
     // selects again)
     const bool by_cluster = fast && router_cluster_supported(p);
     const bool counted = (by_cluster || (fast && router_umma_supported(p))) && p.mode != DSMOE_SELECT_THRESHOLD_TOPK;
+    // both projections in one launch, which for few tokens also finds its rows itself
+    const GroupedScratch G = grouped_scratch(p, L);
+    const bool one_launch = fast && p.fuse_combine == 0 && G.fits && !fuses_combine(p);
+    // (not with counts_out in the workspace, where it may lie on the offsets: the other form finds what it reads there out of order)
+    const bool fold = one_launch && grouped_folds(p) &&
+                      !(reinterpret_cast<char*>(counts_out) >= ws && reinterpret_cast<char*>(counts_out) < ws + ws_bytes);
+    const ZeroInts zero = one_launch ? ZeroInts{reinterpret_cast<int*>(ws + G.sync), (long long)G.sync_ints} : ZeroInts{};
+    const ZeroInts early = fold ? zero : ZeroInts{};
     if (by_cluster)
-        DSMOE_TRY(launch_router_cluster(pr, x, Wr, br, scores, mask, k_t, s, counted ? chunk_prefix : nullptr));
+        DSMOE_TRY(launch_router_cluster(pr, x, Wr, br, scores, mask, k_t, s, counted && !fold ? chunk_prefix : nullptr, early));
     else if (fast && router_umma_supported(p))
-        DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, dev_status, s, counted ? chunk_prefix : nullptr));
+        DSMOE_TRY(launch_router_umma(pr, x, Wr, br, scores, mask, k_t, dev_status, s, counted && !fold ? chunk_prefix : nullptr, 0, early));
     else
-        DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s));
+        DSMOE_TRY(launch_router(pr, x, Wr, br, scores, mask, k_t, s, early));
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK)
         DSMOE_TRY(launch_select(p, scores, mask, k_t, s, reinterpret_cast<int*>(ws + L.batch_k)));
     if (fast) {
@@ -299,10 +307,13 @@ dsmoe_status dsmoe_layer_forward(const dsmoe_layer_desc* desc, const void* x, co
     if (fast) {
         // the down-projection's epilogue multiplies by the gate and stores fp32 rows; the aggregation only adds.  Both projections
         // are one launch unless the caller asked for the separate ones (or a workspace of a few tokens has no room for its counters)
-        if (const GroupedScratch G = grouped_scratch(p, L); p.fuse_combine == 0 && G.fits) {
-            DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr,
-                                   counted, ZeroInts{reinterpret_cast<int*>(ws + G.sync), (long long)G.sync_ints}));
-            DSMOE_TRY(launch_grouped_layer(p, x, packed, offsets, row_token, row_gate, reinterpret_cast<float*>(ws + L.acc), ws, L, dev_status, s));
+        if (one_launch) {
+            const GroupedFold f{mask, scores, token_rows, counts, offsets, counts_out};
+            if (!fold)
+                DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr,
+                                       counted, zero));
+            DSMOE_TRY(launch_grouped_layer(p, x, packed, offsets, row_token, row_gate, fold ? &f : nullptr, reinterpret_cast<float*>(ws + L.acc),
+                                           ws, L, dev_status, s));
             return launch_combine(p, ws + L.acc, nullptr, token_rows, k_t, out, s, true);
         }
         DSMOE_TRY(launch_group(p, scores, mask, counts, offsets, chunk_prefix, counts_out, row_token, row_gate, token_rows, s, nullptr, counted));

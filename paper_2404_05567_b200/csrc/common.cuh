@@ -129,9 +129,15 @@ struct DeviceState {
 };
 dsmoe_status device_state(DeviceState** out, int* device = nullptr);   // of the current device
 
+// Counters of a later launch that an earlier kernel of the call sets to zero on its way
+struct ZeroInts {
+    int* at = nullptr;
+    long long n = 0;
+};
+
 // ---- router.cu
 dsmoe_status launch_router(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
-                           float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s);
+                           float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s, const ZeroInts& zero = ZeroInts{});
 // k_scratch: one int of device memory, needed by DSMOE_SELECT_THRESHOLD_TOPK only (the batch's K)
 dsmoe_status launch_select(const dsmoe_layer_desc& p, const float* scores, uint64_t* mask, int32_t* k_t,
                            cudaStream_t s, int* k_scratch = nullptr);
@@ -144,11 +150,6 @@ dsmoe_status launch_finalize(const dsmoe_layer_desc& p, const uint64_t* mask, in
                              int32_t* offsets, int32_t* chunk_prefix, int32_t* counts_out, cudaStream_t s);
 
 // ---- permute.cu
-// Counters of a later launch that the row-index kernel sets to zero on its way
-struct ZeroInts {
-    int* at = nullptr;
-    long long n = 0;
-};
 // zero_out (optional): the layer output [T,d]; rows of tokens that selected no expert are set to zero
 dsmoe_status launch_permute(const dsmoe_layer_desc& p, const void* x, const float* scores,
                             const uint64_t* mask, const int32_t* offsets, const int32_t* chunk_prefix,
@@ -203,11 +204,11 @@ constexpr int kRouterExactRun = 7;
 bool router_umma_supported(const dsmoe_layer_desc& p, int max_run = 0);
 dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
                                 float* scores, uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s,
-                                int32_t* chunk_counts = nullptr, int max_run = 0);
+                                int32_t* chunk_counts = nullptr, int max_run = 0, const ZeroInts& zero = ZeroInts{});
 // Router for some hundred tokens (router_cluster.cu), as launch_router_umma otherwise.
 bool router_cluster_supported(const dsmoe_layer_desc& p);
 dsmoe_status launch_router_cluster(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores, uint64_t* mask,
-                                   int32_t* k_t, cudaStream_t s, int32_t* chunk_counts);
+                                   int32_t* k_t, cudaStream_t s, int32_t* chunk_counts, const ZeroInts& zero = ZeroInts{});
 // Grouped expert MLPs on expert-sorted rows: h = GeLU(xp.W1[e]) (bf16, in `hbuf`), yp = h.W2[e].
 // With row_token (and x), the up-projection gathers its rows from x by index and xp is not read.
 // With cmb->out, the down-projection's epilogue also aggregates (Eq. 1's weighted sum, ascending expert order per
@@ -264,10 +265,19 @@ struct GroupedScratch {
     bool fits;
 };
 GroupedScratch grouped_scratch(const dsmoe_layer_desc& p, const WsLayout& L);
-// rows [Amax, d] fp32: the gate-weighted expert outputs
+// Whether the launch finds its rows in the selection words itself, without a row-index kernel before it
+constexpr int kGroupedFoldWords = 64 * 33;
+static inline bool grouped_folds(const dsmoe_layer_desc& p) { return p.T <= (p.E <= 32 ? 2048 : 1024); }
+struct GroupedFold {
+    const uint64_t* mask;
+    const float* scores;
+    int32_t *token_rows, *counts, *offsets;      // written: what the row-index kernel would have
+    int32_t* counts_out;                         // nullable, written
+};
+// rows [Amax, d] fp32: the gate-weighted expert outputs.  With `fold`, offsets, row_token and row_gate are not read
 dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, const void* packed, const int32_t* offsets,
-                                  const int32_t* row_token, const float* row_gate, float* rows, char* ws, const WsLayout& L,
-                                  int32_t* dev_status, cudaStream_t s);
+                                  const int32_t* row_token, const float* row_gate, const GroupedFold* fold, float* rows, char* ws,
+                                  const WsLayout& L, int32_t* dev_status, cudaStream_t s);
 
 // ---- moa.cu : the attention step of the mixture-of-attention-heads layer
 bool moa_supported(const dsmoe_layer_desc& p, int n_head, int L);

@@ -27,6 +27,11 @@
 // Bound by the latency of the operands' way out of L2 (2048 tokens of 4096, 512 wide, top-4: tensor pipe 42 % busy, L2 at 37 % of its
 // throughput, DRAM at 47 %; the issuer waits while four ring slots are under way) and, with narrow experts, the fp32 rows' way to memory
 // (7001 tokens of that shape: the down tiles 158 us, 108 without their stores).
+// Up to 2048 tokens (1024 of more than 32 experts: what the selection words' table may take of the shared memory) there is no row-index
+// kernel before this one: every CTA turns the selection words into a bit per expert, chunk and token and finds its tiles' rows there.
+// Without that kernel, its launch and the one that cannot be chained to it, whole calls (us): 300 tokens of 2048, 256 wide, 32 experts,
+// top-4 53.1 -> 45.1; 1500 of 4096, 512 wide 132.8 -> 121.9; 700 of 128, 192 wide, 8 experts 35.0 -> 28.8 (130 shapes of 130 to
+// 2048 tokens: 1.02 to 1.30 times).  Beyond that the 8 us are a per cent or two.
 // The weighted sum of Eq. 1 inside this launch, over groups of columns whose rows were to stay in L2, was slower than its own launch
 // in every form (355 us and more against 248 + 78): beside a 200 KB ring an SM has too few bytes of rows under way, and handing
 // small groups from stores to sums and back costs more than the rows' way to memory and back.
@@ -42,8 +47,9 @@ namespace {
 constexpr int kStageRow = 144;                   // bytes of a row of the tiles through which the epilogue's rows leave
 
 struct GroupedParams {
-    int E, d, H, T;
+    int E, d, H, T, W;
     long long amax;
+    GroupedFold fold;              // FOLD: in place of offsets, row_token and row_gate
     const int32_t* offsets;
     const int32_t* row_token;
     const float* row_gate;
@@ -83,8 +89,15 @@ struct GroupedShared {
 };
 constexpr size_t kGroupedShared = 4096;
 static_assert(sizeof(GroupedShared) <= kGroupedShared, "barriers and tables");
+// FOLD (1: up to 1024 tokens, 2: up to 2048 of at most 32 experts): which of a chunk's tokens selected an expert, [chunk][expert]
+constexpr size_t kFoldBytes = kGroupedFoldWords * sizeof(uint32_t);
+template <int FOLD>
+struct FoldTable {
+    static constexpr int CHUNKS = 32 * FOLD, LD = FOLD == 2 ? 33 : 65;      // (odd: a column's words lie in different banks)
+    static_assert(CHUNKS * LD <= kGroupedFoldWords, "");
+};
 constexpr size_t kGroupedSmem = 1024 + (size_t)RING_BYTES + kGroupedShared + 4 * 32 * kStageRow;
-static_assert(kGroupedSmem <= 227 * 1024, "shared memory of one CTA");
+static_assert(kGroupedSmem + kFoldBytes <= 227 * 1024, "shared memory of one CTA");
 
 #ifdef DSMOE_TRACE
 // Diagnostic build only, per CTA.  Time stamps (globaltimer): [0] start, [1] last up tile multiplied, [2] last tile multiplied, [3] epilogue
@@ -203,6 +216,66 @@ __device__ __forceinline__ int left_over(int* sync, int n, int lane, uint64_t& t
     }
 }
 
+// 32 words of 32 bits, one a lane, transposed: bit i of lane e's result is bit e of lane i's word
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane) {
+    uint32_t low = 0xffffu;                          // the low half of every 2 j bits
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+        x = lane & j ? (x & ~low) | ((y >> j) & low) : (x & low) | ((y << j) & ~low);
+        low ^= low << (j >> 1);
+    }
+    return x;
+}
+
+// The tokens of an expert's rows min(first + lane + 32 j, last), counted within the expert, whose rows ascend by token (the whole warp asks).
+template <int FOLD, int N>
+__device__ __forceinline__ void find_tokens(const uint32_t* bits, int e, int first, int last, int lane, int (&tok)[N]) {
+    uint32_t w[FOLD];
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < FOLD; ++i) {
+        w[i] = bits[(lane * FOLD + i) * FoldTable<FOLD>::LD + e];
+        n += __popc(w[i]);
+    }
+    int before = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += v;
+    }
+    before -= n;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const int r = min(first + lane + 32 * j, last);
+        int c = 0;                                   // the last lane whose chunks begin at or before r: the one that has it
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, before, c + o) <= r) c += o;
+        int k = r - __shfl_sync(0xffffffffu, before, c), at = c * FOLD * kChunk;
+        uint32_t b = __shfl_sync(0xffffffffu, w[0], c);
+        if (FOLD == 2) {
+            const uint32_t b1 = __shfl_sync(0xffffffffu, w[FOLD - 1], c);
+            if (const int n0 = __popc(b); k >= n0) {
+                k -= n0;
+                b = b1;
+                at += kChunk;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {           // its k-th bit
+            const int low = __popc(b & ((1u << o) - 1u));
+            if (k >= low) {
+                k -= low;
+                b >>= o;
+                at += o;
+            }
+        }
+        tok[j] = at;
+    }
+}
+
+template <int FOLD>
 __global__ void __launch_bounds__(kGroupedThreads, 1)
 grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__ CUtensorMap tmH,
                      const __grid_constant__ BMaps tmW2, const GroupedParams P) {
@@ -212,6 +285,8 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
     const uint32_t smA = base, smB = base + STAGES * A_STAGE_BYTES;
     GroupedShared& sh = *reinterpret_cast<GroupedShared*>(smem_raw + (base - raw) + RING_BYTES);
     uint8_t* const stage = smem_raw + (base - raw) + RING_BYTES + kGroupedShared;
+    uint32_t* const bits = reinterpret_cast<uint32_t*>(stage + 4 * 32 * kStageRow);       // (FOLD only)
+    using Table = FoldTable<FOLD ? FOLD : 1>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -239,11 +314,50 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
         ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), TMEM_COLS);
         ptx::tmem_relinquish();
     }
+    if (FOLD) chain_wait();
     // (the dealer's; asked before the tables below are there)
     bool first_is_mine = false;
     if (warp == kGroupedThreads / 32 - 1 && lane == 0) first_is_mine = take_first_round(P.sync, blockIdx.x);
+    if (FOLD) {
+#pragma unroll 4
+        for (int c = warp; c < Table::CHUNKS; c += kGroupedThreads / 32) {
+            const uint64_t m = c * kChunk + lane < P.T ? P.fold.mask[c * kChunk + lane] : 0ull;
+            bits[c * Table::LD + lane] = transpose_bits((uint32_t)m, lane);
+            if (FOLD == 1) bits[c * Table::LD + lane + 32] = transpose_bits((uint32_t)(m >> 32), lane);
+        }
+        __syncthreads();
+    }
     if (warp == 0) {
         __syncwarp();
+        int first[2], count[2] = {0, 0};             // FOLD: experts lane, lane + 32
+        if (FOLD) {
+#pragma unroll
+            for (int c = 0; c < Table::CHUNKS; ++c) {
+                count[0] += __popc(bits[c * Table::LD + lane]);
+                if (FOLD == 1) count[1] += __popc(bits[c * Table::LD + lane + 32]);
+            }
+            first[0] = count[0];
+            first[1] = count[1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int a = __shfl_up_sync(0xffffffffu, first[0], o), b = __shfl_up_sync(0xffffffffu, first[1], o);
+                if (lane >= o) {
+                    first[0] += a;
+                    first[1] += b;
+                }
+            }
+            first[1] += __shfl_sync(0xffffffffu, first[0], 31);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                first[j] -= count[j];
+                if (blockIdx.x == 0 && lane + 32 * j < P.E) {
+                    P.fold.counts[lane + 32 * j] = count[j];
+                    P.fold.offsets[lane + 32 * j + 1] = first[j] + count[j];
+                    if (P.fold.counts_out) P.fold.counts_out[lane + 32 * j] = count[j];
+                }
+            }
+            if (blockIdx.x == 0 && lane == 0) P.fold.offsets[0] = 0;
+        }
         // Segments and their row tiles.  As in umma_gemm_kernel, one that is negative, decreasing or ends beyond the rows counts as
         // empty and is reported: a corrupt array must not send a tile out of range.  Segments that overlap could still have more
         // row tiles than there are counters; then all count as empty.
@@ -254,8 +368,8 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
             const int e = lane + 32 * j;
             int a = 0, b = 0;
             if (e < P.E) {
-                a = P.offsets[e];
-                b = P.offsets[e + 1];
+                a = FOLD ? first[j] : P.offsets[e];
+                b = FOLD ? first[j] + count[j] : P.offsets[e + 1];
             }
             if (a < 0 || b < a || b > P.amax) {
                 bad = true;
@@ -456,7 +570,19 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
             const int row = q * 32 + lane;
             const bool valid = row < t.rows_valid;
             const int nrows = min(32, max(0, t.rows_valid - q * 32));       // rows of this warp
-            const float g = !t.up && valid ? P.row_gate[t.row0 + row] : 1.f;
+            float g = 1.f;
+            if (FOLD && !t.up) {
+                int tok[1];
+                const int first = t.row0 - sh.seg0[t.e];
+                find_tokens<FOLD ? FOLD : 1>(bits, t.e, first + q * 32, first + t.rows_valid - 1, lane, tok);
+                if (valid) {
+                    g = P.fold.scores[(size_t)tok[0] * P.E + t.e];
+                    if (t.n0 == 0)       // once a row: where the aggregation finds it
+                        P.fold.token_rows[(size_t)tok[0] * P.W + __popcll(P.fold.mask[tok[0]] & ((1ull << t.e) - 1ull))] = t.row0 + row;
+                }
+            } else if (!t.up && valid) {
+                g = P.row_gate[t.row0 + row];
+            }
             // the TMEM reads below are warp-collective: the warp leaves as one
             if (__any_sync(0xffffffffu, !ptx::mbar_wait(ptx::smem_u32(&sh.tfull[acc]), aph, &sh.abort_flag))) break;
             ptx::tc_fence_after();
@@ -549,12 +675,17 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
             int n = 0;                       // stages of the sequence seen so far
             while (alive && tiles.next(sh, lane, t)) {
                 if (!t.up) continue;
+                // rows past the segment, which nobody reads: its last one again (all tiles' the same token: up to 1.4 times as long)
+                int tok[ROWS / 32];
+                if (FOLD) {
+                    const int first = t.row0 - sh.seg0[t.e];
+                    find_tokens<FOLD ? FOLD : 1>(bits, t.e, first + part * ROWS, first + t.rows_valid - 1, lane, tok);
+                } else {
 #pragma unroll
-                for (int j = 0; j < ROWS / 32; ++j) {
-                    const int r = part * ROWS + lane + 32 * j;
-                    const int tok = P.row_token[t.row0 + min(r, t.rows_valid - 1)];   // rows past the segment: nobody reads them
-                    rowtok[lane + 32 * j] = min(max(tok, 0), P.T - 1);
+                    for (int j = 0; j < ROWS / 32; ++j) tok[j] = P.row_token[t.row0 + min(part * ROWS + lane + 32 * j, t.rows_valid - 1)];
                 }
+#pragma unroll
+                for (int j = 0; j < ROWS / 32; ++j) rowtok[lane + 32 * j] = min(max(tok[j], 0), P.T - 1);
                 __syncwarp();
                 // this lane's rows (4 jj + lane / 8 of the warp's share): where they start in x, in 16-byte units
                 uint32_t src_off[ROWS / 4];
@@ -654,12 +785,14 @@ GroupedScratch grouped_scratch(const dsmoe_layer_desc& p, const WsLayout& L) {
 }
 
 dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, const void* packed, const int32_t* offsets,
-                                  const int32_t* row_token, const float* row_gate, float* rows, char* ws, const WsLayout& L,
-                                  int32_t* dev_status, cudaStream_t s) {
+                                  const int32_t* row_token, const float* row_gate, const GroupedFold* fold, float* rows, char* ws,
+                                  const WsLayout& L, int32_t* dev_status, cudaStream_t s) {
     DeviceState* st = nullptr;
     DSMOE_TRY(device_state(&st));
     if (!st->attr_grouped) {
-        DSMOE_CUDA_TRY(cudaFuncSetAttribute(grouped_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGroupedSmem));
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(grouped_layer_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGroupedSmem));
+        for (auto* k : {grouped_layer_kernel<1>, grouped_layer_kernel<2>})
+            DSMOE_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kGroupedSmem + kFoldBytes)));
         st->attr_grouped = true;
     }
     const size_t amax = amax_of(p);
@@ -671,7 +804,8 @@ dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, cons
     DSMOE_TRY(cached_map_2d(&mH, ws + L.h, amax, p.H, BM));
     DSMOE_TRY(cached_bmaps(&mW2, w2t, p.E, p.d, p.H));
     GroupedParams P{};
-    P.E = p.E; P.d = p.d; P.H = p.H; P.T = p.T;
+    P.E = p.E; P.d = p.d; P.H = p.H; P.T = p.T; P.W = width_of(p);
+    if (fold) P.fold = *fold;
     P.amax = (long long)amax;
     P.offsets = offsets; P.row_token = row_token; P.row_gate = row_gate;
     P.x = static_cast<const __nv_bfloat16*>(x);
@@ -682,11 +816,17 @@ dsmoe_status launch_grouped_layer(const dsmoe_layer_desc& p, const void* x, cons
     P.dev_status = dev_status;
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));
-    // Not chained to the row-index kernel: its CTAs would be set up beside that kernel's blocks, which leave no room for one on their
+    // Chained to the router, whose CTAs leave SMs free (fold, unchained: 1.06 to 1.07 times as fast as with the row-index kernel; chained:
+    // 1.08 to 1.13).  Not chained to the row-index kernel: its CTAs would be set up beside that kernel's blocks, which leave no room for one on their
     // SMs, and come in another order (8 shapes of 150 to 700 tokens, two boxes: 0.3 and 1 % slower on average than this,
     // 4 % faster to 2.3 % slower).
-    grouped_layer_kernel<<<std::min(sm_count(), kGroupedMaxCtas), kGroupedThreads, kGroupedSmem, s>>>(mW1, mH, mW2, P);
-    DSMOE_CUDA_TRY(cudaGetLastError());
+    const int grid = std::min(sm_count(), kGroupedMaxCtas);
+    if (fold) {
+        DSMOE_CUDA_TRY(launch_chained(p.T <= 1024 ? grouped_layer_kernel<1> : grouped_layer_kernel<2>, grid, kGroupedThreads, kGroupedSmem + kFoldBytes, s, mW1, mH, mW2, P));
+    } else {
+        grouped_layer_kernel<0><<<grid, kGroupedThreads, kGroupedSmem, s>>>(mW1, mH, mW2, P);
+        DSMOE_CUDA_TRY(cudaGetLastError());
+    }
     DSMOE_TRY(timing_end(s, timed));
     return DSMOE_OK;
 }

@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(256) router_small_kernel(const XT* x, const fl
                                                            int T, int d, SelParams q) {
     chain_next();
     chain_wait();
+    zero_ints(q.zero);
     __shared__ float red[TT][8][EP];
     const int t0 = blockIdx.x * TT, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int E = q.E;
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* x,
                                                                     uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
                                                                     int T, int d, SelParams q) {
     chain_wait();
+    zero_ints(q.zero);
     constexpr int TB = kRtTB, KC = kRtKC, EP = 8 * EPL, XS = kRtXS, NT = kRtThreads;
     constexpr int NW = KC * EP / NT, NX = TB * KC / 8 / NT, KQ = KC / kRtSplit;
     static_assert(NX == 1 && NW >= 1, "staging: one 8-element group of x per thread");
@@ -361,8 +363,9 @@ __global__ void __launch_bounds__(1024) finalize_kernel(int32_t* __restrict__ co
 
 template <typename XT>
 static dsmoe_status launch_router_t(const dsmoe_layer_desc& p, const XT* x, const float* Wr, const float* br,
-                                    float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s) {
-    const SelParams q = sel_params(p);
+                                    float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s, const ZeroInts& zero) {
+    SelParams q = sel_params(p);
+    q.zero = zero;
     if (p.T <= 256) {
 #define ROUTER_SMALL(EP, TT)                                                                                            \
     do {                                                                                                                \
@@ -401,11 +404,11 @@ static dsmoe_status launch_router_t(const dsmoe_layer_desc& p, const XT* x, cons
 }
 
 dsmoe_status launch_router(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br,
-                           float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s) {
+                           float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s, const ZeroInts& zero) {
     if (p.T == 0) return DSMOE_OK;
     if (p.dtype == DSMOE_BF16)
-        return launch_router_t(p, static_cast<const __nv_bfloat16*>(x), Wr, br, scores, mask, k_t, s);
-    return launch_router_t(p, static_cast<const float*>(x), Wr, br, scores, mask, k_t, s);
+        return launch_router_t(p, static_cast<const __nv_bfloat16*>(x), Wr, br, scores, mask, k_t, s, zero);
+    return launch_router_t(p, static_cast<const float*>(x), Wr, br, scores, mask, k_t, s, zero);
 }
 
 // Threshold-TopK ("Expert Sampling Strategy" paragraph): K = the batch average of the per-token counts that the

@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(kRcThreads, PER_SM) router_cluster_kernel(cons
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q4 = lane & 3, E = q.E;
     const int group = blockIdx.x / kRcCtas, rank = blockIdx.x % kRcCtas;
     chain_wait();
+    zero_ints(q.zero);
     const int t0 = group * kRcTokens, steps = d / kRcStep;
     float acc[2][NT][4];
 #pragma unroll
@@ -158,7 +159,7 @@ static_assert(kRcTokens == kChunk, "a cluster's tokens are a chunk");
 
 template <int EP, int PER_SM = 1>
 dsmoe_status launch_ep(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores, uint64_t* mask, int32_t* k_t,
-                       cudaStream_t s, int32_t* chunk_counts) {
+                       cudaStream_t s, int32_t* chunk_counts, const ZeroInts& zero) {
     constexpr size_t smem = (size_t)kRcWarps * kRcTokens * (EP + 8) * sizeof(float);
     static bool attr[kMaxDeviceSlots] = {};
     int dev = 0;
@@ -170,7 +171,7 @@ dsmoe_status launch_ep(const dsmoe_layer_desc& p, const void* x, const float* Wr
     }
     DSMOE_CUDA_TRY(launch_chained_clusters(router_cluster_kernel<EP, PER_SM>, (unsigned)(ceil_div(p.T, kRcTokens) * kRcCtas), kRcThreads,
         smem, s, kRcCtas, true, static_cast<const __nv_bfloat16*>(x), Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d,
-        SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr}));
+        SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr, zero}));
     return DSMOE_OK;
 }
 
@@ -188,12 +189,12 @@ bool router_cluster_supported(const dsmoe_layer_desc& p) {
 }
 
 dsmoe_status launch_router_cluster(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores, uint64_t* mask,
-                                   int32_t* k_t, cudaStream_t s, int32_t* chunk_counts) {
-    return p.E <= 8 ? launch_ep<8>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts)
-           : p.E <= 16 ? launch_ep<16>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts)
-           : p.E <= 32 && p.T <= 384 ? launch_ep<32>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts)
-           : p.E <= 32 ? launch_ep<32, 2>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts)
-                       : launch_ep<64>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts);
+                                   int32_t* k_t, cudaStream_t s, int32_t* chunk_counts, const ZeroInts& zero) {
+    return p.E <= 8 ? launch_ep<8>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts, zero)
+           : p.E <= 16 ? launch_ep<16>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts, zero)
+           : p.E <= 32 && p.T <= 384 ? launch_ep<32>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts, zero)
+           : p.E <= 32 ? launch_ep<32, 2>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts, zero)
+                       : launch_ep<64>(p, x, Wr, br, scores, mask, k_t, s, chunk_counts, zero);
 }
 
 }  // namespace dsmoe

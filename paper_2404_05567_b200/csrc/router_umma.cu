@@ -105,6 +105,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
     ptx::tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
     chain_wait();
+    zero_ints(q.zero);
 
     if (warp == 0) {
         if (ptx::elect_one()) {
@@ -302,7 +303,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
 
 template <int EP, int C>
 dsmoe_status launch_clusters(const dsmoe_layer_desc& p, const CUtensorMap& mX, const float* Wr, const float* br, float* scores,
-                             uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s) {
+                             uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s, const ZeroInts& zero) {
     static bool attr[kMaxDeviceSlots] = {};
     int dev = 0;
     DeviceState* st = nullptr;
@@ -312,7 +313,7 @@ dsmoe_status launch_clusters(const dsmoe_layer_desc& p, const CUtensorMap& mX, c
         attr[dev] = true;
     }
     DSMOE_CUDA_TRY(launch_chained_clusters(router_umma_kernel<EP, C>, ceil_div(p.T, kRuM) * C, kRuThreads, router_umma_smem<EP>(), s, C, true,
-        mX, Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d, SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr},
+        mX, Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d, SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr, zero},
         dev_status));
     return DSMOE_OK;
 }
@@ -333,11 +334,11 @@ int clusters_of(const dsmoe_layer_desc& p, int max_run) {
 
 template <int EP>
 dsmoe_status launch_ep(const dsmoe_layer_desc& p, int max_run, const CUtensorMap& mX, const float* Wr, const float* br, float* scores,
-                       uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s) {
+                       uint64_t* mask, int32_t* k_t, int32_t* chunk_counts, int32_t* dev_status, cudaStream_t s, const ZeroInts& zero) {
     switch (clusters_of<EP>(p, max_run)) {
-        case 4: return launch_clusters<EP, 4>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
-        case 2: return launch_clusters<EP, 2>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
-        case 1: return launch_clusters<EP, 1>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+        case 4: return launch_clusters<EP, 4>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s, zero);
+        case 2: return launch_clusters<EP, 2>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s, zero);
+        case 1: return launch_clusters<EP, 1>(p, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s, zero);
         default: return DSMOE_ERR_UNSUPPORTED;
     }
 }
@@ -350,11 +351,11 @@ bool router_umma_supported(const dsmoe_layer_desc& p, int max_run) {
 
 dsmoe_status launch_router_umma(const dsmoe_layer_desc& p, const void* x, const float* Wr, const float* br, float* scores,
                                 uint64_t* mask, int32_t* k_t, int32_t* dev_status, cudaStream_t s, int32_t* chunk_counts,
-                                int max_run) {
+                                int max_run, const ZeroInts& zero) {
     CUtensorMap mX;
     DSMOE_TRY(cached_map_2d(&mX, x, p.T, p.d, kRuM));
-    return p.E <= 32 ? launch_ep<32>(p, max_run, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s)
-                     : launch_ep<64>(p, max_run, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s);
+    return p.E <= 32 ? launch_ep<32>(p, max_run, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s, zero)
+                     : launch_ep<64>(p, max_run, mX, Wr, br, scores, mask, k_t, chunk_counts, dev_status, s, zero);
 }
 
 }  // namespace dsmoe
