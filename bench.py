@@ -260,9 +260,15 @@ def mlp_launches(s):
     return 1 if s.mode != gi.MODE_ALL and s.fuse_combine == 0 and not sums_inside(s) else 2
 
 
+def grouped_decode(s):
+    """Up to 128 tokens that the library groups by expert all the same (many wide experts; csrc/mlp_umma.cu, small_grouped)."""
+    return (s.T > (80 if s.d <= 1536 else 96) and s.d <= 2048 and s.E >= 32 and s.H <= 2048 and s.E * s.H >= 32768 and
+            s.mode != gi.MODE_ALL and s.fuse_combine == 0)
+
+
 def kernels_per_step(s, decode):
     """Launches of this library's kernels in one dsmoe_layer_forward (memsets are not kernels)."""
-    if decode:
+    if decode and not grouped_decode(s):
         return 1                                   # few_tokens_kernel or small_layer_kernel
     if s.mode == gi.MODE_ALL:
         return 3                                   # router, up, down
@@ -440,9 +446,9 @@ def run_workload(name: str, steps: int, warmup: int, dist=None, with_e2e=True, s
         flops = 4.0 * A * s.d * s.H * calls_per_step
         if decode:
             # selected experts' weights (W1 and W2), each byte once, all inside one launch of few_tokens_kernel
-            # (up to 7 tokens) or small_layer_kernel
+            # (up to 7 tokens), small_layer_kernel or grouped_layer_kernel
             roof = dict(bound="hbm", achieved=weight_bytes / (kernel_ms * 1e-3) / 1e9, peak=P["hbm"], unit="GB/s",
-                        peak_source=P["source"] + " (copy bandwidth)", kernel="few_tokens_kernel" if s.T < 8 else "small_layer_kernel")
+                        peak_source=P["source"] + " (copy bandwidth)", kernel="few_tokens_kernel" if s.T < 8 else "grouped_layer_kernel" if grouped_decode(s) else "small_layer_kernel")
             roof["frac"] = roof["achieved"] / roof["peak"]
             roof["frac_nominal"] = roof["achieved"] / NOMINAL["hbm"]
             roof["step_frac"] = weight_bytes / step_s / 1e9 / roof["peak"]

@@ -2179,10 +2179,21 @@ bool small_groups(const dsmoe_layer_desc& p, int G) { return 4 * p.T > G && (2 *
 
 // Few tokens (decode): one cooperative launch of small_layer_kernel runs router, both projections and the
 // fix-up.
+// It multiplies every token by every selected expert, which with many wide experts and short rows takes longer than the weights' way:
+// those layers are grouped from here on.  us a layer in one launch and grouped, by threshold, top-4 and top-6: 97 tokens of d 2048, H 1024,
+// 32 experts 69, 68; 69, 63; 69, 64 (128: 74, 68; 75, 64; 75, 65; 84: 66, 67; 66, 62; 66, 64); of 64 such experts 123, 116; 126, 106; 126, 111;
+// 90 tokens of d 1024, H 512, 64 experts 52, 48; 54, 44; 54, 44 (73: 48, 48; 49, 43; 49, 43).  Less work beside the weights, and it is the
+// other way round: 100 tokens of d 3072, H 384, 32 experts 51, 65 by threshold, of d 1024, H 512, 32 experts 35, 38, of d 1024, H 2048, 16
+// experts 48, 53, of d 128, H 4096, 32 experts 61, 69.
+static bool small_grouped(const dsmoe_layer_desc& p) {
+    return p.T > (p.d <= 1536 ? 80 : 96) && p.d <= 2048 && p.E >= 32 && p.H <= 2048 && p.E * p.H >= 32768 && p.mode != DSMOE_SELECT_ALL &&
+           p.fuse_combine == 0;
+}
 bool small_supported(const dsmoe_layer_desc& p) {
     const int G = sm_count() < kSmallMaxCtas ? sm_count() : kSmallMaxCtas;
     if (!(umma_supported(p) && p.T >= 1 && p.T <= kSmallMaxT && p.T <= G && ceil_div(p.d, 64) <= G)) return false;
     if (p.mode == DSMOE_SELECT_THRESHOLD_TOPK) return false;   // its K needs a pass over the batch first: grouped path
+    if (small_grouped(p)) return false;
     // the router's second half fetches all slice sums of a warp's tokens in one batch of 16 (small_router_pass)
     int KS = 1;
     while (KS < 16 && KS * 2 * p.T <= G) KS *= 2;

@@ -18,3 +18,18 @@ def test_router_by_groups(T, d, E):
     first = L.forward().clone()
     for _ in range(3):                                     # the counters are zeroed by every call, the slices' order is fixed
         assert (L.forward() == first).all()
+
+
+# many wide experts are grouped by expert beyond 80 (d up to 1536) and 96 tokens: both sides of each line
+WIDE = [(80, 1536, 1024, 32), (81, 1536, 1024, 32), (96, 2048, 512, 64), (97, 2048, 512, 64), (128, 64, 2048, 33)]
+
+
+@pytest.mark.parametrize("mode", [gi.MODE_TOPK, gi.MODE_THRESHOLD], ids=["topk", "threshold"])
+@pytest.mark.parametrize("T,d,H,E", WIDE, ids=[f"T{T}-d{d}-H{H}-E{E}" for T, d, H, E in WIDE])
+def test_many_wide_experts(T, d, H, E, mode):
+    sel = dict(K=3) if mode == gi.MODE_TOPK else dict(eps=1.0, eps_normalized=1)
+    r = layer_parity(gi.LayerSpec(f"wide{T}x{d}x{H}x{E}-{mode}", T=T, d=d, H=H, E=E, dtype="bf16", mode=mode, router_gain=4.0, **sel), sample=24)
+    assert r["err_rows"] <= TOL_BF16, (r["err_rows"], r["err"])
+    L = r["layer"]
+    first = L.forward().clone()
+    assert (L.forward() == first).all()
