@@ -636,7 +636,7 @@ def run_moa(name: str, steps: int, warmup: int, sampler_index=0):
         head = dict(bound="hbm", achieved=gbs, peak=P["hbm"], unit="GB/s", peak_source=P["source"] + " (copy bandwidth)",
                     frac=gbs / P["hbm"], frac_nominal=gbs / NOMINAL["hbm"])
     roof = dict(head, kernel="umma_gemm_kernel (projections) + " + ("moa_attention_mma_kernel" if w["layout"] == "decode" else
-                                                                         "moa_attention_shared_kernel"), roofline_ms=max(t_flop, t_byte) * 1e3,
+                                                                         "moa_attention_umma_kernel"), roofline_ms=max(t_flop, t_byte) * 1e3,
                 frac_of_roofline_time=max(t_flop, t_byte) / (float(durs.sum()) * 1e-3),
                 step_frac_of_roofline_time=max(t_flop, t_byte) / (ms * 1e-3), step_frac=max(t_flop, t_byte) / (ms * 1e-3),
                 algorithmic_per_launch=proj_flops / 2, attention_flops=att_flops, kv_bytes=kv_bytes, traffic=None,

@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "tensor_maps.cuh"
+#include "umma.cuh"
 
 namespace dsmoe {
 
@@ -733,15 +734,12 @@ __device__ __forceinline__ void attend(const AttnArgs& P, unsigned char* const s
     }
 }
 
+// Four tiles of neighbouring tokens, by the whole CTA: its smem of shared_attention_smem<DH>() bytes, room for kShTokens tokens
 template <int DH>
-__global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(const __grid_constant__ AttnArgs P) {
-    chain_wait();
+__device__ __forceinline__ void attend_group(const AttnArgs& P, unsigned char* const smem, int* const seq_s, int* const last_s, const int j,
+                                             const int group) {
     constexpr int CH = DH / 8;
-    extern __shared__ __align__(16) unsigned char moa_sh_smem[];
-    __shared__ int seq_s[kShTokens], last_s[kShTokens];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j = (int)(blockIdx.x % P.n_head);
-    const int group = (int)(blockIdx.x / P.n_head);
     // this CTA's tokens: their sequences and last visible keys, clamped into the cache (and reported)
     int tg0, tg1;
     group_tokens(P, group, tg0, tg1);
@@ -770,10 +768,309 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
             }
         }
     }
-    if (!mixed) attend<DH, false>(P, moa_sh_smem, seq_s, last_s, j, t0, rt, tg0, 0, ng, r, tk);
+    if (!mixed) attend<DH, false>(P, smem, seq_s, last_s, j, t0, rt, tg0, 0, ng, r, tk);
     else if (!P.leave_mixed) {
         tile_rows(P, t0, rt, lane >> 2, r, tk);         // (again: kept over the branch, they cost registers that the common path lacks)
-        attend<DH, true>(P, moa_sh_smem, seq_s, last_s, j, t0, rt, tg0, t0 - tg0, min(t0 - tg0 + P.tpt, ng), r, tk);
+        attend<DH, true>(P, smem, seq_s, last_s, j, t0, rt, tg0, t0 - tg0, min(t0 - tg0 + P.tpt, ng), r, tk);
+    }
+}
+
+template <int DH>
+__global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(const __grid_constant__ AttnArgs P) {
+    chain_wait();
+    extern __shared__ __align__(16) unsigned char moa_sh_smem[];
+    __shared__ int seq_s[kShTokens], last_s[kShTokens];
+    attend_group<DH>(P, moa_sh_smem, seq_s, last_s, (int)(blockIdx.x % P.n_head), (int)(blockIdx.x / P.n_head));
+}
+
+// ---------------------------------------------------------------- the same for a tile of up to 128 rows on the 5th-generation tensor cores
+// One CTA per (head, tile of neighbouring tokens: 24 of 5 rows each); a thread owns a row.  Per 64 keys: S = Q.K^T into TMEM, each thread its
+// row's maximum, weights and sum without a word from its neighbours, P (bf16) into the 128-byte swizzle where the keys lay, P.V into TMEM,
+// and the running values in the thread's registers (fp32; nothing is rescaled in TMEM).  Keys and values lie as in memory; V is an N-major
+// operand.  A block of both is copied while the one before is worked on, two CTAs fill an SM (113 KB, 255 registers a thread).
+// 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 102 us with the warp-level path, 81 so (cold caches; the layer 470 -> 445, 482 -> 452 by another
+// day's clocks).  Bound by the instruction issue of the weights and of the copies' addresses (0.34 a cycle and scheduler with two warps each; the
+// tensor pipe 9 % busy).  Asking for the next block's S before this one's weights, and adding P.V a block later: 85 us (registers).
+// The sums are of the rounded weights, which P.V is made of: whole layers of 4 heads of 128 and of 96 and 2 of 64 are 1.970e-3, 2.017e-3 and
+// 2.030e-3 from 64 bits (1.988e-3, 2.031e-3, 2.041e-3 before; 1.995e-3, 2.040e-3, 2.044e-3 with sums of the unrounded ones).
+// What it does not take -- tiles of tokens of three sequences and more, keys or values that are not finite -- it does in the other form.
+constexpr int kUaRows = 128, kUaKeys = 64;
+
+// Groups of four 16-row tiles that one 128-row tile takes (0: not this kernel's)
+int umma_attention_groups(int W) { return W <= 16 ? kUaRows / (W * kShWarps * shared_tile_tokens(W)) : 0; }
+
+// Where it is the faster one: with an SM's worth of CTAs each, which are half as many as the shared-key kernel's (8 experts of 4 heads of 128,
+// top-5, us a layer, that kernel and this one: 400 tokens, 68 CTAs, 83, 86; 1024, 172 CTAs, 119, 117; 8192 482, 452; one prompt of 2048
+// 243, 215; 16 of 2 heads of 64, top-6: 800 tokens, 100 CTAs, 63, 65; 2048, 256 CTAs, 101, 98), and with prompts long enough that few tiles walk two
+// (16 of 2 heads of 64: 30 prompts of 100 tokens 86, 88, of 128 159, 156; 8 of 4 heads of 128: 60 of 64 234, 237, 30 of 100 192, 181).
+bool umma_attention_fits(const dsmoe_layer_desc& p, const MoaCore& c) {
+    const int W = width_of(p);
+    const long long span = (long long)umma_attention_groups(W) * kShWarps * shared_tile_tokens(W), n_seq = c.tok_seq ? c.n_seq : 1;
+    return span > 0 && (p.T + span - 1) / span * c.n_head >= sm_count() && p.T >= n_seq * (p.H / c.n_head == 64 ? 128 : 96);
+}
+
+template <int DH>
+struct UaShape {
+    static constexpr int HALVES = (DH + 63) / 64;                 // a row's 128-byte pieces
+    static constexpr uint32_t QB = HALVES * kUaRows * 128, KB = HALVES * kUaKeys * 128;
+    static constexpr uint32_t TMEM = DH <= 64 ? 128 : 256;        // 64 columns of logits, DH of weighted values
+    // the weights lie where the block's keys did, if they fit there: two CTAs on an SM
+    static constexpr bool P_ON_K = KB >= kUaRows * 128;
+    static constexpr size_t smem = 1024 + QB + 4 * KB + (P_ON_K ? 0 : kUaRows * 128);
+    static_assert(smem - 1024 >= (size_t)2 * 2 * kShKeys * (DH * 2 + 16), "room for attend_group");
+};
+
+// Operand B = V as it lies in memory, [keys][64 columns] in the 128-byte swizzle: N-major.  Eight keys are 1024 bytes, the next 64 columns
+// begin kUaKeys rows further on.
+__device__ __forceinline__ uint64_t make_desc_mn_sw128(uint32_t smem_addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr & 0x3FFFF) >> 4);
+    d |= (uint64_t)((kUaKeys * 128) >> 4) << 16;                  // leading byte offset: between 64-column groups
+    d |= (uint64_t)(1024 >> 4) << 32;                             // stride byte offset: between groups of 8 keys
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+template <int DH>
+__global__ void __launch_bounds__(kUaRows, 2) moa_attention_umma_kernel(const __grid_constant__ AttnArgs P, const int groups) {
+    using S = UaShape<DH>;
+    constexpr int CH = DH / 8;
+    extern __shared__ unsigned char moa_ua_smem[];
+    __shared__ int seq_s[kUaRows], last_s[kUaRows];
+    __shared__ uint64_t bar[2];
+    __shared__ uint32_t tmem_s;
+    __shared__ volatile int abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t raw = ptx::smem_u32(moa_ua_smem), base = (raw + 1023u) & ~1023u;
+    unsigned char* const smem = moa_ua_smem + (base - raw);
+    const uint32_t sQ = base, sK = sQ + S::QB, sV = sK + 2 * S::KB;
+    const int j = (int)(blockIdx.x % P.n_head), tile = (int)(blockIdx.x / P.n_head);
+    const int span = groups * kShWarps * P.group_tpt;             // tokens of a tile
+    const int tg0 = tile * span, ng = min(P.T - tg0, span);
+    if (tid == 0) {
+        ptx::mbar_init(ptx::smem_u32(&bar[0]), 1);
+        ptx::mbar_init(ptx::smem_u32(&bar[1]), 1);
+        abort_flag = 0;
+        ptx::fence_barrier_init();
+    }
+    chain_wait();
+    if (warp == 0) {
+        ptx::tmem_alloc(ptx::smem_u32(&tmem_s), S::TMEM);
+        ptx::tmem_relinquish();
+    }
+    if (tid < ng) {
+        const int t = tg0 + tid;
+        const int sq = P.tok_seq ? P.tok_seq[t] : 0, last = P.pos[t];
+        if (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
+        seq_s[tid] = min(max(sq, 0), P.n_seq - 1);
+        last_s[tid] = min(max(last, 0), P.L - 1);
+    }
+    // this thread's row of the tile: grouped row (-1: none), token of the tile
+    const int tl = tid / P.W, slot = tid % P.W;
+    int r = -1;
+    if (tl < ng) {
+        r = P.token_rows[(size_t)(tg0 + tl) * P.W + slot];
+        if (r >= P.amax) r = -1;
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tmem = tmem_s;
+    bool mixed = false;
+    for (int i = lane; i < ng; i += 32) mixed = mixed || (seq_s[i] != seq_s[0] && seq_s[i] != seq_s[ng - 1]);
+    bool redo = __any_sync(0xffffffffu, mixed);                   // (the same for all warps)
+
+    if (!redo) {
+        // queries: a warp's 32 rows, DH / 8 pieces of 16 bytes each, in the swizzle's order; rows that are none are zeros
+        for (int i = lane; i < 32 * CH; i += 32) {
+            const int row = i / CH, ch = i % CH, rr = __shfl_sync(0xffffffffu, r, row), at = warp * 32 + row;
+            const __nv_bfloat16* q = P.qa + (size_t)max(rr, 0) * P.H + j * DH + ch * 8;
+            const uint32_t dst = sQ + (uint32_t)((ch >> 3) * kUaRows * 128 + at * 128 + (((ch & 7) ^ (at & 7)) << 4)), nbytes = rr >= 0 ? 16u : 0u;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(q), "r"(nbytes) : "memory");
+        }
+        const auto zeros = [&]() {                                // where a token did not select an expert
+            for (int t = tg0 + warp; t < tg0 + ng; t += kUaRows / 32) {
+                const uint64_t sel = P.mask[t];
+                for (int idx = lane; idx < P.E * CH; idx += 32) {
+                    const int e = idx / CH, ch = idx % CH;
+                    if (!((sel >> e) & 1ull))
+                        *reinterpret_cast<uint4*>(P.dense + ((size_t)t * P.E + e) * P.H + j * DH + ch * 8) = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
+        };
+        const float sl2 = P.scale * 1.4426950408889634f;
+        const int last = r >= 0 ? last_s[tl] : -1, sq_of = r >= 0 ? seq_s[tl] : -1;
+        float m = -INFINITY, l = 0.f, o[DH];
+#pragma unroll
+        for (int i = 0; i < DH; ++i) o[i] = 0.f;
+        uint32_t phase = 0;
+        bool alive = true;
+        const int passes = seq_s[0] == seq_s[ng - 1] ? 1 : 2;
+        for (int pass = 0; pass < passes && alive; ++pass) {
+            const int sq = pass == 0 ? seq_s[0] : seq_s[ng - 1];
+            int mine = -1;
+            for (int i = lane; i < ng; i += 32)
+                if (seq_s[i] == sq) mine = max(mine, last_s[i]);
+            const int last_key = __reduce_max_sync(0xffffffffu, mine);
+            const int elast = sq_of == sq ? last : -1;
+            const __nv_bfloat16* Kh = P.Kc + ((size_t)(sq * P.n_head + j) * P.L) * DH;
+            const __nv_bfloat16* Vh = P.Vc + ((size_t)(sq * P.n_head + j) * P.L) * DH;
+            const int nblocks = last_key / kUaKeys + 1;
+            const auto fetch = [&](int b) {
+                const int key0 = b * kUaKeys, nk = min(kUaKeys, last_key + 1 - key0);
+                const uint32_t kd = sK + (b & 1) * S::KB, vd = sV + (b & 1) * S::KB;
+#pragma unroll
+                for (int i = 0; i < kUaKeys * CH / kUaRows; ++i) {
+                    const int idx = tid + kUaRows * i, row = idx / CH, ch = idx % CH;
+                    // rows past the last visible key are filled with zeros
+                    const size_t src = (size_t)(key0 + (row < nk ? row : 0)) * DH + ch * 8;
+                    const uint32_t nbytes = row < nk ? 16u : 0u;
+                    const uint32_t dst = (uint32_t)((ch >> 3) * kUaKeys * 128 + row * 128 + (((ch & 7) ^ (row & 7)) << 4));
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(kd + dst), "l"(Kh + src), "r"(nbytes) : "memory");
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(vd + dst), "l"(Vh + src), "r"(nbytes) : "memory");
+                }
+                ptx::cp_async_commit();
+            };
+            fetch(0);
+            if (P.dense && pass == 0) zeros();                    // (while the copies are on their way)
+            for (int b = 0; b < nblocks; ++b) {
+                if (b + 1 < nblocks) {
+                    fetch(b + 1);
+                    ptx::cp_async_wait<1>();
+                } else {
+                    ptx::cp_async_wait<0>();
+                }
+                ptx::fence_proxy_async();
+                ptx::tc_fence_before();
+                __syncthreads();
+                if (warp == 0 && ptx::elect_one()) {
+                    ptx::tc_fence_after();
+                    const uint32_t k0 = sK + (b & 1) * S::KB, idesc = ptx::make_idesc_bf16(kUaRows, kUaKeys);
+#pragma unroll
+                    for (int k = 0; k < DH / 16; ++k)
+                        ptx::umma_bf16(tmem, ptx::make_desc_k_sw128(sQ + (k >> 2) * kUaRows * 128 + (k & 3) * 32),
+                                       ptx::make_desc_k_sw128(k0 + (k >> 2) * kUaKeys * 128 + (k & 3) * 32), idesc, (uint32_t)(k != 0));
+                    ptx::umma_commit(ptx::smem_u32(&bar[0]));
+                }
+                __syncwarp();
+                alive = ptx::mbar_wait(ptx::smem_u32(&bar[0]), phase, &abort_flag);
+                alive = __syncthreads_and(alive);
+                if (!alive) break;
+                ptx::tc_fence_after();
+                const uint32_t row0 = tmem + ((uint32_t)(warp * 32) << 16);
+                uint32_t v[2][32];
+                ptx::tmem_ld32(row0, v[0]);
+                ptx::tmem_ld32(row0 + 32, v[1]);
+                ptx::tmem_ld_wait();
+                const uint32_t sP = S::P_ON_K ? sK + (b & 1) * S::KB : sV + 2 * S::KB;
+                const int seen = elast - b * kUaKeys;             // keys 0 .. seen of the block are this row's
+                float bm = -INFINITY, alpha;
+                const auto weigh = [&](float scale) {             // v -> weights, in base 2, relative to the running maximum
+                    const float n = fmaxf(m, bm), z = n == -INFINITY ? 0.f : n;
+                    alpha = n == -INFINITY ? 1.f : ex2(m - n);
+                    m = n;
+                    l *= alpha;
+#pragma unroll
+                    for (int c = 0; c < kUaKeys / 8; ++c) {
+                        uint32_t pk[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int at = c * 8 + 2 * i;
+                            const float p0 = ex2(fmaf(__uint_as_float(v[at / 32][at % 32]), scale, -z));
+                            const float p1 = ex2(fmaf(__uint_as_float(v[at / 32][at % 32 + 1]), scale, -z));
+                            pk[i] = pack_bf16(p0, p1);
+                            l += bf16_lo(pk[i]) + bf16_hi(pk[i]);     // (what is multiplied is what is divided by)
+                        }
+                        *reinterpret_cast<uint4*>(smem + (sP - base) + tid * 128 + ((c ^ (tid & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    }
+                };
+                if (__all_sync(0xffffffffu, seen >= kUaKeys - 1) && sl2 > 0.f) {       // nothing to hide from this warp's rows
+#pragma unroll
+                    for (int i = 0; i < kUaKeys; ++i) bm = fmaxf(bm, __uint_as_float(v[i / 32][i % 32]));
+                    bm *= sl2;
+                    weigh(sl2);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kUaKeys; ++i) {
+                        const float x = i <= seen ? __uint_as_float(v[i / 32][i % 32]) * sl2 : -INFINITY;
+                        v[i / 32][i % 32] = __float_as_uint(x);
+                        bm = fmaxf(bm, x);
+                    }
+                    weigh(1.f);
+                }
+                ptx::fence_proxy_async();
+                ptx::tc_fence_before();
+                __syncthreads();
+                if (warp == 0 && ptx::elect_one()) {
+                    ptx::tc_fence_after();
+                    const uint32_t v0 = sV + (b & 1) * S::KB, idesc = ptx::make_idesc_bf16(kUaRows, DH) | (1u << 16);      // B is N-major
+#pragma unroll
+                    for (int k = 0; k < kUaKeys / 16; ++k)
+                        ptx::umma_bf16(tmem + kUaKeys, ptx::make_desc_k_sw128(sP + k * 32), make_desc_mn_sw128(v0 + k * 2048), idesc, (uint32_t)(k != 0));
+                    ptx::umma_commit(ptx::smem_u32(&bar[1]));
+                }
+                __syncwarp();
+                alive = ptx::mbar_wait(ptx::smem_u32(&bar[1]), phase, &abort_flag);
+                phase ^= 1u;
+                alive = __syncthreads_and(alive);
+                if (!alive) break;
+                ptx::tc_fence_after();
+#pragma unroll
+                for (int c = 0; c < DH / 32; ++c) {
+                    uint32_t w[32];
+                    ptx::tmem_ld32(row0 + kUaKeys + c * 32, w);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[c * 32 + i] = fmaf(o[c * 32 + i], alpha, __uint_as_float(w[i]));
+                }
+            }
+        }
+        ptx::cp_async_wait<0>();
+        if (!alive && tid == 0) report_status(P.dev_status, DSMOE_ERR_TIMEOUT);
+        // A key or value that is not finite reaches all rows of the tile here, also those that do not see it: such a tile is done again
+        // the other way, whose tiles are 16 rows.
+        float sum = l * 0.f;
+#pragma unroll
+        for (int i = 0; i < DH; ++i) sum = fmaf(o[i], 0.f, sum);
+        redo = __syncthreads_or(!(sum == 0.f)) != 0;
+        if (!redo) {
+            chain_next();
+            // normalise (and weigh); the rows go out through shared memory (the queries' place), whole rows per store
+            float inv = 1.f / l;
+            __nv_bfloat16* dst = r >= 0 ? P.qa + (size_t)r * P.H + j * DH : nullptr;
+            if (P.dense && r >= 0) {
+                const int e = expert_of_slot(P.mask[tg0 + tl], slot);
+                dst = e >= 0 ? P.dense + ((size_t)(tg0 + tl) * P.E + e) * P.H + j * DH : nullptr;
+                inv *= P.row_gate[r];
+            }
+            unsigned char* const st = smem + warp * 32 * (DH * 2 + 16);
+#pragma unroll
+            for (int c = 0; c < CH; ++c)
+                *reinterpret_cast<uint4*>(st + lane * (DH * 2 + 16) + c * 16) =
+                    make_uint4(pack_bf16(o[c * 8] * inv, o[c * 8 + 1] * inv), pack_bf16(o[c * 8 + 2] * inv, o[c * 8 + 3] * inv),
+                               pack_bf16(o[c * 8 + 4] * inv, o[c * 8 + 5] * inv), pack_bf16(o[c * 8 + 6] * inv, o[c * 8 + 7] * inv));
+            __syncwarp();
+            for (int i = lane; i < 32 * CH; i += 32) {
+                const int row = i / CH, ch = i % CH;
+                __nv_bfloat16* const to = reinterpret_cast<__nv_bfloat16*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), row));
+                if (to) *reinterpret_cast<uint4*>(to + ch * 8) = *reinterpret_cast<const uint4*>(st + row * (DH * 2 + 16) + ch * 16);
+            }
+        }
+    }
+    if (redo) {
+        for (int g = 0; g < groups; ++g) {
+            const int group = tile * groups + g;
+            if (group * kShWarps * P.group_tpt >= P.T) break;
+            __syncthreads();
+            attend_group<DH>(P, smem, seq_s, last_s, j, group);
+        }
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc(tmem, S::TMEM);
     }
 }
 
@@ -789,6 +1086,25 @@ AttnArgs attn_args(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q
     return AttnArgs{q, token_rows, W, (W + 15) / 16, tpt, shared_tile_tokens(W), (long long)amax_of(p), c.n_head, p.H, p.T,
                     static_cast<const __nv_bfloat16*>(c.Kc), static_cast<const __nv_bfloat16*>(c.Vc), c.tok_seq, c.pos,
                     c.n_seq, c.L, c.scale, dev_status, leaves_mixed(p, c), static_cast<__nv_bfloat16*>(c.dense), p.E, c.mask, c.row_gate};
+}
+
+template <int DH>
+dsmoe_status launch_umma_attention(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
+                                   int32_t* dev_status, cudaStream_t s) {
+    static bool attr[kMaxDeviceSlots] = {};
+    int dev = 0;
+    DeviceState* st = nullptr;
+    DSMOE_TRY(device_state(&st, &dev));
+    if (!attr[dev]) {
+        DSMOE_CUDA_TRY(cudaFuncSetAttribute(moa_attention_umma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UaShape<DH>::smem));
+        attr[dev] = true;
+    }
+    const int W = width_of(p), groups = umma_attention_groups(W);
+    const long long span = (long long)groups * kShWarps * shared_tile_tokens(W), ctas = (p.T + span - 1) / span * c.n_head;
+    if (ctas > 0x7fffffffll) return DSMOE_ERR_UNSUPPORTED;
+    DSMOE_CUDA_TRY(launch_chained(moa_attention_umma_kernel<DH>, (unsigned)ctas, kUaRows, UaShape<DH>::smem, s,
+        attn_args(p, c, q, token_rows, shared_tile_tokens(W), dev_status), groups));
+    return DSMOE_OK;
 }
 
 template <int DH>
@@ -849,7 +1165,8 @@ template <int DH>
 dsmoe_status launch_mma_attention(const dsmoe_layer_desc& p, const MoaCore& c, __nv_bfloat16* q, const int32_t* token_rows,
                                   int32_t* dev_status, cudaStream_t s) {
     if (moa_shares_keys(p, c)) {
-        DSMOE_TRY(launch_shared_attention<DH>(p, c, q, token_rows, dev_status, s));
+        DSMOE_TRY(umma_attention_fits(p, c) ? launch_umma_attention<DH>(p, c, q, token_rows, dev_status, s)
+                                                         : launch_shared_attention<DH>(p, c, q, token_rows, dev_status, s));
         return leaves_mixed(p, c) ? launch_mma_attention_nw<DH, 8, true>(p, c, q, token_rows, dev_status, s) : DSMOE_OK;
     }
     if (c.L <= kTileMaxKeys) return launch_mma_attention_nw<DH, 2>(p, c, q, token_rows, dev_status, s);
