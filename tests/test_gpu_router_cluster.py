@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import dsmoe_inputs as gi
+import test_gpu_grouped_layer
 import paper_2404_05567_b200 as dm
 from harness import TOL_BF16, Layer, desc_of, layer_parity, to_dev
 
@@ -42,3 +43,18 @@ def test_no_farther_from_64_bits_than_the_fma_kernel(shape):
     got = L.ws[:4 * T * E].view(torch.float32).view(T, E)        # the workspace begins with the layer's scores
     err = [float((v.double() - exact).norm() / exact.norm()) for v in (got, fma)]
     assert err[0] <= 1.05 * err[1], err
+
+
+PART = [(200, 2048, 64, 16, 3), (700, 1024, 64, 32, 4), (384, 1024, 64, 64, 2), (1000, 1024, 128, 8, 2)]
+
+
+@pytest.mark.parametrize("sms", [16, 72])
+def test_on_a_part_of_the_gpu(sms, monkeypatch):
+    """Clusters of eight on a stream that owns some of the SMs."""
+    monkeypatch.setattr(test_gpu_grouped_layer, "PART", PART)
+    test_gpu_grouped_layer.test_on_a_part_of_the_gpu(sms)
+
+
+@pytest.mark.parametrize("shape", PART, ids=lambda s: f"T{s[0]}-d{s[1]}-H{s[2]}-E{s[3]}")
+def test_two_streams_with_a_workspace_each(shape):
+    test_gpu_grouped_layer.test_two_streams_with_a_workspace_each(shape)
