@@ -635,16 +635,16 @@ def run_moa(name: str, steps: int, warmup: int, sampler_index=0):
         gbs = (weight_bytes + kv_bytes) / (float(durs.sum()) * 1e-3) / 1e9
         head = dict(bound="hbm", achieved=gbs, peak=P["hbm"], unit="GB/s", peak_source=P["source"] + " (copy bandwidth)",
                     frac=gbs / P["hbm"], frac_nominal=gbs / NOMINAL["hbm"])
-    roof = dict(head, kernel="umma_gemm_kernel (projections) + " + ("moa_attention_mma_kernel" if w["layout"] == "decode" else
-                                                                         "moa_attention_umma_kernel"), roofline_ms=max(t_flop, t_byte) * 1e3,
+    roof = dict(head, kernel="moa_decode_gemm_kernel (projections) + moa_decode_attention_kernel" if w["layout"] == "decode" else
+                "umma_gemm_kernel (projections) + moa_attention_umma_kernel", roofline_ms=max(t_flop, t_byte) * 1e3,
                 frac_of_roofline_time=max(t_flop, t_byte) / (float(durs.sum()) * 1e-3),
                 step_frac_of_roofline_time=max(t_flop, t_byte) / (ms * 1e-3), step_frac=max(t_flop, t_byte) / (ms * 1e-3),
                 algorithmic_per_launch=proj_flops / 2, attention_flops=att_flops, kv_bytes=kv_bytes, traffic=None,
                 kernel_ms_per_step=float(durs.sum()), ms_per_step_with_events=ms, launch_ms_each=[float(v) for v in durs],
                 launches_per_step=3)
-    # router, row indices, query projection, attention, output projection; few tokens also the sums of the projection's pieces and
-    # of a token's experts
-    return dict(workload=name, library_launches=7 if w["layout"] == "decode" else 5, value=T / (ms * 1e-3), unit="tokens/s", ms_per_step=ms, steps=steps, roofline=roof, clocks=clocks,
+    # router, row indices, query projection, attention, output projection; decoding: router and query projection, attention, output
+    # projection with the sum over a token's experts
+    return dict(workload=name, library_launches=3 if w["layout"] == "decode" else 5, value=T / (ms * 1e-3), unit="tokens/s", ms_per_step=ms, steps=steps, roofline=roof, clocks=clocks,
                 assignments=A, active_experts=E, config=dict(w))
 
 

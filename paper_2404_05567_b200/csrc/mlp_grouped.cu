@@ -495,7 +495,9 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
             alive = __all_sync(0xffffffffu, alive);
         }
         chain_next();
-        if (lane == 0) GT_PUT(7, gt_h);
+#ifdef DSMOE_TRACE
+        if (gt_h) GT_PUT(7, gt_h);           // (the elected lane's)
+#endif
         if (!alive) {
             // copies already issued still land in this CTA's shared memory: give them time
             const uint64_t t0 = ptx::globaltimer_ns();
@@ -555,6 +557,8 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
 #ifdef DSMOE_TRACE
         if (lane == 0) {
             GT_SET(2);
+        }
+        if (gt_up | gt_down | gt_acc) {      // (the elected lane's)
             GT_PUT(4, gt_up);
             GT_PUT(5, gt_down);
             GT_PUT(6, gt_acc);
