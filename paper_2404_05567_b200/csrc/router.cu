@@ -5,6 +5,8 @@
 // One warp owns one token from the logits onward: lane e holds expert e (and e+32 when E > 32), so
 // the softmax and every selection rule are warp shuffles and ballots, and the selected set of a
 // token is one 64-bit ballot word.
+#include <type_traits>
+
 #include "common.cuh"
 #include "router_device.cuh"
 
@@ -14,6 +16,9 @@ static SelParams sel_params(const dsmoe_layer_desc& p) {
     return SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr};
 }
 
+template <typename XT>
+using RouterZero = std::conditional_t<sizeof(XT) == 2, ZeroInts, NoZero>;
+
 // Small T (decode): a block per TT tokens (1, or 4 (2 beyond 32 experts) from 64 tokens on: the tokens of a block share its loads of Wr, which
 // every block reads in full out of L2), the reduction over d split across all 256 threads.  A token's sums are formed
 // in the same order whatever TT is.
@@ -21,10 +26,10 @@ template <typename XT, int EP, int TT>
 __global__ void __launch_bounds__(256) router_small_kernel(const XT* x, const float* Wr,
                                                            const float* br, float* __restrict__ scores,
                                                            uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
-                                                           int T, int d, SelParams q) {
+                                                           int T, int d, SelParams q, const RouterZero<XT> zero) {
     chain_next();
     chain_wait();
-    zero_ints(q.zero);
+    zero_ints(zero);
     __shared__ float red[TT][8][EP];
     const int t0 = blockIdx.x * TT, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int E = q.E;
@@ -148,9 +153,9 @@ template <typename XT, int EPL>
 __global__ void __launch_bounds__(kRtThreads, 1) router_tile_kernel(const XT* x, const float* Wr,
                                                                     const float* br, float* __restrict__ scores,
                                                                     uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
-                                                                    int T, int d, SelParams q) {
+                                                                    int T, int d, SelParams q, const RouterZero<XT> zero) {
     chain_wait();
-    zero_ints(q.zero);
+    zero_ints(zero);
     constexpr int TB = kRtTB, KC = kRtKC, EP = 8 * EPL, XS = kRtXS, NT = kRtThreads;
     constexpr int NW = KC * EP / NT, NX = TB * KC / 8 / NT, KQ = KC / kRtSplit;
     static_assert(NX == 1 && NW >= 1, "staging: one 8-element group of x per thread");
@@ -364,17 +369,18 @@ __global__ void __launch_bounds__(1024) finalize_kernel(int32_t* __restrict__ co
 template <typename XT>
 static dsmoe_status launch_router_t(const dsmoe_layer_desc& p, const XT* x, const float* Wr, const float* br,
                                     float* scores, uint64_t* mask, int32_t* k_t, cudaStream_t s, const ZeroInts& zero) {
-    SelParams q = sel_params(p);
-    q.zero = zero;
+    const SelParams q = sel_params(p);
+    RouterZero<XT> z{};
+    if constexpr (sizeof(XT) == 2) z = zero;
     if (p.T <= 256) {
 #define ROUTER_SMALL(EP, TT)                                                                                            \
     do {                                                                                                                \
         if (p.T >= 64)                                                                                                  \
             DSMOE_CUDA_TRY(launch_chained(router_small_kernel<XT, EP, TT>, ceil_div(p.T, TT), 256, 0, s,                \
-                x, Wr, br, scores, mask, k_t, p.T, p.d, q));                                                            \
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q, z));                                                         \
         else                                                                                                            \
             DSMOE_CUDA_TRY(launch_chained(router_small_kernel<XT, EP, 1>, p.T, 256, 0, s,                               \
-                x, Wr, br, scores, mask, k_t, p.T, p.d, q));                                                            \
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q, z));                                                         \
     } while (0)
         if (p.E <= 8) ROUTER_SMALL(8, 4);
         else if (p.E <= 16) ROUTER_SMALL(16, 4);
@@ -395,10 +401,10 @@ static dsmoe_status launch_router_t(const dsmoe_layer_desc& p, const XT* x, cons
         }
         if (p.E <= 32)
             DSMOE_CUDA_TRY(launch_chained(router_tile_kernel<XT, 4>, grid, kRtThreads, router_tile_smem<4>(), s,
-                x, Wr, br, scores, mask, k_t, p.T, p.d, q));
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q, z));
         else
             DSMOE_CUDA_TRY(launch_chained(router_tile_kernel<XT, 8>, grid, kRtThreads, router_tile_smem<8>(), s,
-                x, Wr, br, scores, mask, k_t, p.T, p.d, q));
+                x, Wr, br, scores, mask, k_t, p.T, p.d, q, z));
     }
     return DSMOE_OK;
 }

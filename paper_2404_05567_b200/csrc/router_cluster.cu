@@ -36,14 +36,14 @@ template <int EP, int PER_SM>        // experts, padded; CTAs that an SM is to h
 __global__ void __launch_bounds__(kRcThreads, PER_SM) router_cluster_kernel(const __nv_bfloat16* x, const float* Wr, const float* br,
                                                                     float* __restrict__ scores, uint64_t* __restrict__ mask,
                                                                     int32_t* __restrict__ k_t, int32_t* __restrict__ chunk_counts, int T, int d,
-                                                                    const SelParams q) {
+                                                                    const SelParams q, const ZeroInts zero) {
     constexpr int NT = EP / 8, LD = EP + 8;              // floats between two tokens' sums: no bank conflicts
     extern __shared__ __align__(16) float rc_part[];     // [warps][tokens][LD]
     __shared__ uint64_t mask_s[kRcTokens];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q4 = lane & 3, E = q.E;
     const int group = blockIdx.x / kRcCtas, rank = blockIdx.x % kRcCtas;
     chain_wait();
-    zero_ints(q.zero);
+    zero_ints(zero);
     const int t0 = group * kRcTokens, steps = d / kRcStep;
     float acc[2][NT][4];
 #pragma unroll
@@ -171,7 +171,7 @@ dsmoe_status launch_ep(const dsmoe_layer_desc& p, const void* x, const float* Wr
     }
     DSMOE_CUDA_TRY(launch_chained_clusters(router_cluster_kernel<EP, PER_SM>, (unsigned)(ceil_div(p.T, kRcTokens) * kRcCtas), kRcThreads,
         smem, s, kRcCtas, true, static_cast<const __nv_bfloat16*>(x), Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d,
-        SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr, zero}));
+        SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr}, zero));
     return DSMOE_OK;
 }
 

@@ -12,13 +12,14 @@ struct SelParams {
     float eps;
     int eps_normalized, K, min_k;
     const int* K_dev;    // when set, the K of the top-K rule is read from here (Threshold-TopK: K comes from the batch)
-    ZeroInts zero{};     // counters of a later launch of the call that the router sets to zero on its way
 };
 
-// (after chain_wait)
+struct NoZero {};        // fp32 layers have no such launch
+// Counters of a later launch of the call, which the router sets to zero on its way (after chain_wait)
 __device__ __forceinline__ void zero_ints(const ZeroInts& z) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < z.n; i += (long long)gridDim.x * blockDim.x) z.at[i] = 0;
 }
+__device__ __forceinline__ void zero_ints(const NoZero&) {}
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll

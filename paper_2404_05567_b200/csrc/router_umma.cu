@@ -64,7 +64,7 @@ template <int EP, int C>
 __global__ void __launch_bounds__(kRuThreads, 1)
 router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, const float* br,
                    float* __restrict__ scores, uint64_t* __restrict__ mask, int32_t* __restrict__ k_t,
-                   int32_t* __restrict__ chunk_counts, int T, int d, const SelParams q, int32_t* __restrict__ dev_status) {
+                   int32_t* __restrict__ chunk_counts, int T, int d, const SelParams q, int32_t* __restrict__ dev_status, const ZeroInts zero) {
     using G = RuGeo<EP>;
     extern __shared__ uint8_t ru_smem[];
     const uint32_t raw = ptx::smem_u32(ru_smem), base = (raw + 1023u) & ~1023u;
@@ -105,7 +105,7 @@ router_umma_kernel(const __grid_constant__ CUtensorMap tmX, const float* Wr, con
     ptx::tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
     chain_wait();
-    zero_ints(q.zero);
+    zero_ints(zero);
 
     if (warp == 0) {
         if (ptx::elect_one()) {
@@ -313,8 +313,8 @@ dsmoe_status launch_clusters(const dsmoe_layer_desc& p, const CUtensorMap& mX, c
         attr[dev] = true;
     }
     DSMOE_CUDA_TRY(launch_chained_clusters(router_umma_kernel<EP, C>, ceil_div(p.T, kRuM) * C, kRuThreads, router_umma_smem<EP>(), s, C, true,
-        mX, Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d, SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr, zero},
-        dev_status));
+        mX, Wr, br, scores, mask, k_t, chunk_counts, p.T, p.d, SelParams{p.E, p.mode, p.eps, p.eps_normalized, p.K, p.min_k, nullptr},
+        dev_status, zero));
     return DSMOE_OK;
 }
 
