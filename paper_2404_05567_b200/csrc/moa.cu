@@ -787,9 +787,9 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
 // One CTA per (head, tile of neighbouring tokens: 24 of 5 rows each); a thread owns a row.  Per 64 keys: S = Q.K^T into TMEM, each thread its
 // row's maximum, weights and sum without a word from its neighbours, P (bf16) into the 128-byte swizzle where the keys lay, P.V into TMEM,
 // and the running values in the thread's registers (fp32; nothing is rescaled in TMEM).  Keys and values lie as in memory; V is an N-major
-// operand.  A block of both is copied while the one before is worked on, two CTAs fill an SM (113 KB, 255 registers a thread).
-// 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 102 us with the warp-level path, 81 so (cold caches; the layer 470 -> 445, 482 -> 452 by another
-// day's clocks).  Bound by the instruction issue of the weights and of the copies' addresses (0.34 a cycle and scheduler with two warps each; the
+// operand.  A block of both is copied while the one before is worked on, two CTAs fill an SM (255 registers a thread, 97 KB each).
+// 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 102 us with the warp-level path, 81 so (cold caches; the layer 482 -> 452).
+// Bound by the instruction issue of the weights and of the copies' addresses (0.34 a cycle and scheduler with two warps each; the
 // tensor pipe 9 % busy).  Asking for the next block's S before this one's weights, and adding P.V a block later: 85 us (registers).
 // The sums are of the rounded weights, which P.V is made of: whole layers of 4 heads of 128 and of 96 and 2 of 64 are 1.970e-3, 2.017e-3 and
 // 2.030e-3 from 64 bits (1.988e-3, 2.031e-3, 2.041e-3 before; 1.995e-3, 2.040e-3, 2.044e-3 with sums of the unrounded ones).
