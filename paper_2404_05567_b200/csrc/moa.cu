@@ -167,6 +167,13 @@ __device__ __forceinline__ void group_tokens(const AttnArgs& P, int group, int& 
     t0 = (group * kShWarps / P.row_tiles) * P.group_tpt;
     t1 = min(P.T, ((group * kShWarps + kShWarps - 1) / P.row_tiles) * P.group_tpt + P.group_tpt);
 }
+// Whether token u makes tokens a .. b - 1 mixed.  Every kernel asks here: a group is attended by exactly one launch, which puts its outputs
+// where the queries were.
+template <typename Seq>
+__device__ __forceinline__ bool mixes(const Seq& seq, int a, int b, int u) {
+    const int sq = seq(u);
+    return sq != seq(a) && sq != seq(b - 1);
+}
 __device__ __forceinline__ int seq_of(const AttnArgs& P, int t) { return P.tok_seq ? min(max(P.tok_seq[t], 0), P.n_seq - 1) : 0; }
 
 template <int DH, int kMmaWarps, bool MIXED>      // long caches: 8 warps share out the keys; short ones: 2, and several CTAs fit an SM
@@ -201,13 +208,10 @@ moa_attention_mma_kernel(__nv_bfloat16* __restrict__ qa, const int32_t* token_ro
             bool mixed = false;
             if (mine < n_tiles) {
                 int a, b;
-                const int t = (int)(mine / ((long long)row_tiles * n_head)) * tpt;
-                group_tokens(P, (t / P.group_tpt * row_tiles + (int)(mine % row_tiles)) / kShWarps, a, b);
-                const int first = seq_of(P, a), last = seq_of(P, b - 1);
-                for (int u = a + 1; u + 1 < b; ++u) {
-                    const int sq = seq_of(P, u);
-                    mixed = mixed || (sq != first && sq != last);
-                }
+                const int tt = (int)(mine / ((long long)row_tiles * n_head)) * tpt;
+                group_tokens(P, (tt / P.group_tpt * row_tiles + (int)(mine % row_tiles)) / kShWarps, a, b);
+                const auto seq = [&](int t) { return seq_of(P, t); };
+                for (int u = a + 1; u + 1 < b; ++u) mixed = mixed || mixes(seq, a, b, u);
             }
             if (threadIdx.x == 0) found_s = INT_MAX;
             __syncthreads();
@@ -756,7 +760,8 @@ __device__ __forceinline__ void attend_group(const AttnArgs& P, unsigned char* c
     tile_rows(P, t0, rt, lane >> 2, r, tk);
     __syncthreads();
     bool mixed = false;
-    for (int i = lane; i < ng; i += 32) mixed = mixed || (seq_s[i] != seq_s[0] && seq_s[i] != seq_s[ng - 1]);
+    const auto seq = [&](int i) { return seq_s[i]; };
+    for (int i = lane; i < ng; i += 32) mixed = mixed || mixes(seq, 0, ng, i);
     mixed = __any_sync(0xffffffffu, mixed);
     if (P.dense && rt == 0) {
         for (int t = t0; t < min(P.T, t0 + P.tpt); ++t) {
@@ -793,7 +798,8 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
 // tensor pipe 9 % busy).  Asking for the next block's S before this one's weights, and adding P.V a block later: 85 us (registers).
 // The sums are of the rounded weights, which P.V is made of: whole layers of 4 heads of 128 and of 96 and 2 of 64 are 1.970e-3, 2.017e-3 and
 // 2.030e-3 from 64 bits (1.988e-3, 2.031e-3, 2.041e-3 before; 1.995e-3, 2.040e-3, 2.044e-3 with sums of the unrounded ones).
-// What it does not take -- tiles of tokens of three sequences and more, keys or values that are not finite -- it does in the other form.
+// What it does not take -- tiles of tokens of three sequences and more, tiles with a mixed group that is the key-splitting kernel's, keys
+// or values that are not finite -- it does in the other form.
 constexpr int kUaRows = 128, kUaKeys = 64;
 
 // Groups of four 16-row tiles that one 128-row tile takes (0: not this kernel's)
@@ -877,8 +883,14 @@ __global__ void __launch_bounds__(kUaRows, 2) moa_attention_umma_kernel(const __
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = tmem_s;
+    // a tile of three sequences and more, or with a group that is left to another launch, goes the other way, group by group
     bool mixed = false;
-    for (int i = lane; i < ng; i += 32) mixed = mixed || (seq_s[i] != seq_s[0] && seq_s[i] != seq_s[ng - 1]);
+    const auto seq = [&](int i) { return seq_s[i]; };
+    const int per_group = kShWarps * P.group_tpt;
+    for (int i = lane; i < ng; i += 32) {
+        const int a = i / per_group * per_group;
+        mixed = mixed || mixes(seq, 0, ng, i) || (P.leave_mixed && mixes(seq, a, min(a + per_group, ng), i));
+    }
     bool redo = __any_sync(0xffffffffu, mixed);                   // (the same for all warps)
 
     if (!redo) {

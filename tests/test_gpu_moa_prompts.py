@@ -1,6 +1,6 @@
 """Attention of prompts in tiles of up to 128 rows (csrc/moa.cu, moa_attention_umma_kernel) against the oracle: the head widths, 1 to 16 rows a
-token (tiles that 128 rows do and do not fill), caches that end inside a block of 64 keys, tiles of two sequences and of many, values
-that are not finite (GPU required)."""
+token (tiles that 128 rows do and do not fill), caches that end inside a block of 64 keys, tiles of two sequences, in order and not, and of
+many, values that are not finite (GPU required)."""
 import math
 
 import numpy as np
@@ -31,6 +31,40 @@ def test_prompts(case):
     T, d, E, nh, dh, n_seq, L, layout, mode, sel = case
     s, *rest = _moa_case(f"uprompt{T}x{dh}x{L}", T, d, E, nh, dh, n_seq, L, layout, mode, **sel)
     e, er = _run(s, *rest, nh, 1.0 / math.sqrt(dh), sample=60)
+    assert er <= TOL_BF16, (e, er)
+
+
+# Two sequences out of order with a cache beyond 512 positions: a group of four 16-row tiles with a token whose sequence is neither its
+# first's nor its last's is the key-splitting kernel's, also inside a tile of 128 rows that holds no third sequence.
+# T, d, E, n_head, d_head, mode, selection
+OUT_OF_ORDER = [
+    (1200, 128, 8, 4, 128, gi.MODE_THRESHOLD, dict(eps=0.1)),
+    (1000, 128, 8, 4, 128, gi.MODE_TOPK, dict(K=5)),
+    (1000, 128, 8, 4, 128, gi.MODE_TOPK, dict(K=5, fuse_combine=1)),
+    (1003, 128, 8, 4, 96, gi.MODE_TOPK, dict(K=5, fuse_combine=2)),
+    (1201, 128, 8, 4, 96, gi.MODE_THRESHOLD, dict(eps=0.15)),
+    (1250, 128, 16, 2, 64, gi.MODE_TOPK, dict(K=6)),
+    (1200, 128, 4, 4, 64, gi.MODE_ALL, dict()),
+    (1000, 128, 9, 4, 64, gi.MODE_TOPK, dict(K=9)),                             # three groups of four tokens a tile
+    # the dense output projection
+    (2369, 2048, 8, 4, 128, gi.MODE_TOPK, dict(K=5)),
+    (2433, 2048, 8, 4, 96, gi.MODE_TOPK, dict(K=5)),
+    (4700, 1024, 8, 2, 64, gi.MODE_TOPK, dict(K=4)),
+]
+
+
+@pytest.mark.parametrize("order", ["random", "one_inside_a_group"])
+@pytest.mark.parametrize("case", OUT_OF_ORDER, ids=lambda c: f"T{c[0]}-{c[3]}x{c[4]}-m{c[5]}" + "".join(f"-{k}{v}" for k, v in c[6].items()))
+def test_two_sequences_out_of_order_in_a_long_cache(case, order):
+    T, d, E, nh, dh, mode, sel = case
+    s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos = _moa_case(f"uorder{T}x{dh}", T, d, E, nh, dh, 2, 600, "mixed", mode, **sel)
+    if order == "one_inside_a_group":                      # A A B A ... | ... B, tile by tile
+        W = s.K if mode == gi.MODE_TOPK else E
+        group = 4 * (16 // W)
+        tile = group * (128 // (group * W))
+        at = np.arange(T) % tile
+        seq = ((at == 2) | (at >= group)).astype(np.int32)
+    e, er = _run(s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos, nh, 1.0 / math.sqrt(dh))
     assert er <= TOL_BF16, (e, er)
 
 
