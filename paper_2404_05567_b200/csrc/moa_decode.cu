@@ -419,6 +419,18 @@ struct DecodeAttnParams {
     int32_t* dev_status;
 };
 
+}  // namespace
+
+// Aligned runs over pairs of `units` units each: where CTA c's begins.  split: `per` CTAs to a pair, else `per` pairs to a CTA.
+// (units * r / per without the product, which a cache of 233 million positions takes out of an int's range)
+__host__ __device__ int decode_run_start(int c, int units, int per, int pairs, bool split) {
+    if (!split) return (c * per < pairs ? c * per : pairs) * units;
+    const int r = c % per;
+    return c / per * units + units / per * r + units % per * r / per;
+}
+
+namespace {
+
 template <int DH>
 __global__ void __launch_bounds__(32 * kDaWarps, 1) moa_decode_attention_kernel(const DecodeAttnParams P) {
     using G = DaGeo<DH>;
@@ -477,8 +489,7 @@ __global__ void __launch_bounds__(32 * kDaWarps, 1) moa_decode_attention_kernel(
     if ((int)blockIdx.x >= n_cta) return;
     const int share = total / n_cta, extra = total - share * n_cta;
     const auto run_start = [&](int c) {
-        if (!aligned) return c * share + min(c, extra);
-        return split ? c / per * units0 + units0 * (c % per) / per : min(c * per, pairs) * units0;
+        return aligned ? decode_run_start(c, units0, per, pairs, split) : c * share + min(c, extra);
     };
     const int u0 = run_start(blockIdx.x), u1 = run_start(blockIdx.x + 1);
 
