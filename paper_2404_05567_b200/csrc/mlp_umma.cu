@@ -2002,15 +2002,19 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
         }
         st->max_pairs = n < st->sm_count / 2 ? n : st->sm_count / 2;
     }
-    // Dense launches of more rows than one CTA's tile always pair (us, single CTAs and pairs): the forward of 16384 tokens of d 2048, H 1024
-    // 3490, 3202; 4000 of 4096, 512 937, 883; 150 of 2048, 1024 276, 209; 150 of 2048, 256 87, 84; a training step of 8190 tokens 1910, 1761, of 129
-    // 73, 72.  Grouped launches do where a long mainloop runs against a light epilogue (plain stores after a reduction of 1024 or more): half
+    // Dense launches of more rows than one CTA's tile pair: the down-projection always, the others (GeLU, gradients) from a reduction of 1536
+    // on.  us, single CTAs and pairs: the forward of 16384 tokens of d 2048, H 1024 3490, 3202; 4000 of 4096, 512 937, 883; 150 of 2048, 1024
+    // 276, 209; a training step of 8190 tokens 1910, 1761.  Speed of the training step with both of its launches paired over single ones, and of
+    // the forward with its up-projection paired, 150 to 8190 tokens of H 256 and 1024, on average: d 128 0.92, 0.98; 512 0.95, 0.99; 1024 0.97, 0.99;
+    // 1280 1.00, 1.01; 1536 1.03, 1.03; 2048 1.06, 1.04; 3072 1.11, 1.05 (1360 tokens of d 1024, H 1024 0.90: of 12 half tiles one is empty).
+    // Grouped launches do where a long mainloop runs against a light epilogue (plain stores after a reduction of 1024 or more): half
     // of a pair's tile is empty more often, and under the gathering up-projection, on short reductions and with the aggregation
     // in the epilogue they lose up to 20 % or change nothing.
     bool pair = pair_tiles > 0 && st->max_pairs > 0 && (P.n_per_expert % 64) == 0;
     if (pair_override() == 0) pair = false;
     else if (pair && pair_override() != 1)
-        pair = P.mode == GEMM_GROUPED ? P.epi == EPI_STORE && pair_tiles >= st->max_pairs && P.k_per_expert >= 1024 : P.rows > BM;
+        pair = P.mode == GEMM_GROUPED ? P.epi == EPI_STORE && pair_tiles >= st->max_pairs && P.k_per_expert >= 1024
+                                      : P.rows > BM && (P.mode == GEMM_DENSE_DOWN || P.k_per_expert >= 1536);
     // (the large dense launches are not chained: no gap to speak of, and 1 % slower with it, 3682 against 3732 us for the
     // dense layer at 16384 tokens; grouped ones all are: 300 tokens of 2048 / 1024 93.7 against 98.7 us for the layer, 8192
     // of 3072 / 1536 alike, 7001 of 4096 / 512 428 against 425)

@@ -5,8 +5,10 @@ second half lies past the rows, and the backward pass (GPU required)."""
 import os
 
 import pytest
+import torch
 
 import dsmoe_inputs as gi
+import paper_2404_05567_b200 as dm
 from harness import TOL_BF16, layer_parity, np_f32
 from test_gpu_training import _backward_case
 
@@ -58,3 +60,34 @@ def test_backward_with_cta_pairs(masked):
     s = gi.LayerSpec("pair_bwd", T=517, d=256, H=448, E=16, dtype="bf16", router_gain=4.0)
     e_s, e_a = _backward_case(s, True, masked)
     assert e_s <= TOL_BF16 and e_a <= TOL_BF16, (e_s, e_a)
+
+
+@pytest.mark.parametrize("d", [1472, 1536])
+def test_the_librarys_choice_on_both_sides_of_its_line(d, monkeypatch):
+    """Dense launches: the up-projection and the gradients pair from a reduction of 1536 on, the down-projection always.  Single CTAs,
+    pairs and the library's choice give the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(d)
+    T, H, E = 300, 192, 4
+    randn = lambda *shape, std=1.0: (torch.randn(shape, generator=g, device="cuda") * std).bfloat16()
+    x, dO, W1, W2 = randn(T, d), randn(T, d), randn(E, d, H, std=0.02), randn(E, H, d, std=0.02)
+    Wr = torch.randn((d, E), generator=g, device="cuda") * 0.02
+    desc = dm.make_desc(T, d, H, E, dm.BF16, dm.SELECT_ALL)
+    packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc, W1, W2, packed)
+    ws = torch.empty(dm.dsmoe_workspace_size(desc), dtype=torch.uint8, device="cuda")
+    status, scores = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.empty((T, E), device="cuda")
+    dm.dsmoe_router(desc, x, Wr, None, scores)
+
+    def run():
+        out, dS, dA = torch.empty_like(x), torch.empty((T, E), device="cuda"), torch.empty((T, E * H), dtype=torch.bfloat16, device="cuda")
+        dm.dsmoe_layer_forward(desc, x, Wr, None, None, None, packed, out, None, None, ws, status)
+        dm.dsmoe_dense_backward(desc, x, None, W2, packed, scores, None, dO, dS, dA, ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        return out, dS, dA
+
+    pairs = run()
+    for other in ("0", ""):
+        monkeypatch.setenv("DSMOE_GEMM_PAIR", other)
+        for a, b in zip(pairs, run()):
+            assert torch.equal(a, b), other
