@@ -14,7 +14,7 @@ struct SelParams {
     const int* K_dev;    // when set, the K of the top-K rule is read from here (Threshold-TopK: K comes from the batch)
 };
 
-struct NoZero {};        // fp32 layers have no such launch
+struct NoZero {};        // a call without such a launch
 // Counters of a later launch of the call, which the router sets to zero on its way (after chain_wait)
 __device__ __forceinline__ void zero_ints(const ZeroInts& z) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < z.n; i += (long long)gridDim.x * blockDim.x) z.at[i] = 0;
