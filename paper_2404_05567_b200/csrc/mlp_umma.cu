@@ -2002,11 +2002,13 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
         }
         st->max_pairs = n < st->sm_count / 2 ? n : st->sm_count / 2;
     }
-    // Dense launches of more rows than one CTA's tile pair: the down-projection always, the others (GeLU, gradients) from a reduction of 1536
-    // on.  us, single CTAs and pairs: the forward of 16384 tokens of d 2048, H 1024 3490, 3202; 4000 of 4096, 512 937, 883; 150 of 2048, 1024
-    // 276, 209; a training step of 8190 tokens 1910, 1761.  Speed of the training step with both of its launches paired over single ones, and of
-    // the forward with its up-projection paired, 150 to 8190 tokens of H 256 and 1024, on average: d 128 0.92, 0.98; 512 0.95, 0.99; 1024 0.97, 0.99;
-    // 1280 1.00, 1.01; 1536 1.03, 1.03; 2048 1.06, 1.04; 3072 1.11, 1.05 (1360 tokens of d 1024, H 1024 0.90: of 12 half tiles one is empty).
+    // Dense launches of more rows than one CTA's tile pair from a reduction of 1536 on (GeLU, gradients), or 1024 (down-projection; 8192 below d
+    // 1536, where it would be the call's only one on pairs).  us, single CTAs and pairs: the forward of 16384 tokens of d 2048, H 1024 3490, 3202; 4000
+    // of 4096, 512 937, 883; 150 of 2048, 1024 276, 209; a training step of 8190 tokens 1910, 1761.  Speed of the training step with both of its
+    // launches paired over single ones, and of the forward with its up-projection paired, 150 to 8190 tokens of H 256 and 1024, on average: d 128 0.92,
+    // 0.98; 512 0.95, 0.99; 1024 0.97, 0.99; 1280 1.00, 1.01; 1536 1.03, 1.03; 2048 1.06, 1.04; 3072 1.11, 1.05 (1360 tokens of d 1024, H 1024 0.90: of 12
+    // half tiles one is empty).  Of the forward with its down-projection paired, E * H of 512, 1024, 2048, 4096 and 8192: d 1024 0.93, 0.94, 0.95, 0.97,
+    // 1.04; d 2048 1.00, 1.01, 1.01, 1.04, 1.07.
     // Grouped launches do where a long mainloop runs against a light epilogue (plain stores after a reduction of 1024 or more): half
     // of a pair's tile is empty more often, and under the gathering up-projection, on short reductions and with the aggregation
     // in the epilogue they lose up to 20 % or change nothing.
@@ -2014,7 +2016,8 @@ dsmoe_status launch_gemm(const CUtensorMap& a, const BMaps& b, const GemmParams&
     if (pair_override() == 0) pair = false;
     else if (pair && pair_override() != 1)
         pair = P.mode == GEMM_GROUPED ? P.epi == EPI_STORE && pair_tiles >= st->max_pairs && P.k_per_expert >= 1024
-                                      : P.rows > BM && (P.mode == GEMM_DENSE_DOWN || P.k_per_expert >= 1536);
+                                      : P.rows > BM && (P.mode == GEMM_DENSE_DOWN ? P.E * P.k_per_expert >= (P.n_per_expert >= 1536 ? 1024 : 8192)
+                                                                                  : P.k_per_expert >= 1536);
     // (the large dense launches are not chained: no gap to speak of, and 1 % slower with it, 3682 against 3732 us for the
     // dense layer at 16384 tokens; grouped ones all are: 300 tokens of 2048 / 1024 93.7 against 98.7 us for the layer, 8192
     // of 3072 / 1536 alike, 7001 of 4096 / 512 428 against 425)

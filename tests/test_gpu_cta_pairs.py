@@ -62,12 +62,13 @@ def test_backward_with_cta_pairs(masked):
     assert e_s <= TOL_BF16 and e_a <= TOL_BF16, (e_s, e_a)
 
 
-@pytest.mark.parametrize("d", [1472, 1536])
-def test_the_librarys_choice_on_both_sides_of_its_line(d, monkeypatch):
-    """Dense launches: the up-projection and the gradients pair from a reduction of 1536 on, the down-projection always.  Single CTAs,
-    pairs and the library's choice give the same bits."""
+@pytest.mark.parametrize("d,E,H", [(1472, 4, 192), (1536, 5, 192), (1536, 4, 256), (256, 16, 448), (256, 16, 512)],
+                         ids=lambda v: str(v))
+def test_the_librarys_choice_on_both_sides_of_its_lines(d, E, H, monkeypatch):
+    """Dense launches: the up-projection and the gradients pair from a reduction of 1536 on, the down-projection from 1024 or 8192.  Single
+    CTAs, pairs and the library's choice give the same bits."""
     g = torch.Generator(device="cuda").manual_seed(d)
-    T, H, E = 300, 192, 4
+    T = 300
     randn = lambda *shape, std=1.0: (torch.randn(shape, generator=g, device="cuda") * std).bfloat16()
     x, dO, W1, W2 = randn(T, d), randn(T, d), randn(E, d, H, std=0.02), randn(E, H, d, std=0.02)
     Wr = torch.randn((d, E), generator=g, device="cuda") * 0.02
