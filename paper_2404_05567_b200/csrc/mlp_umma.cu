@@ -890,7 +890,7 @@ struct SmallParams {
     void* out;
     int out_f32;
     int* sync;               // 8 ints, zero at launch: barrier counters [0..2] and an abort flag [4]
-    int* group_done;         // zero at launch: the router's finished slices of each group of tokens
+    int* group_done;         // zero at launch, ceil(T / 2) ints: the router's finished slices of each group of tokens
     int spec;                // start streaming under "every expert selected" before the router has finished
     int32_t* dev_status;
 };
@@ -2249,9 +2249,10 @@ dsmoe_status launch_layer_small(const dsmoe_layer_desc& p, const void* x, const 
     // up-projection under that assumption while its router is still running; it starts over if the router disagrees.
     P.spec = p.T >= kSpecMinT ? 1 : 0;
     P.group_done = reinterpret_cast<int*>(ws + L.tile_done);
-    // (tile_done follows sync in the workspace)
+    // (tile_done, 64 ints and more, follows sync in the workspace; a group is two tokens or more: at most 64 counters)
+    static_assert((kSmallMaxT + 1) / 2 <= kMaxExperts, "a counter a group");
     const bool by_groups = small_groups(p, G);
-    DSMOE_CUDA_TRY(cudaMemsetAsync(P.sync, 0, by_groups ? L.tile_done - L.sync + (size_t)p.T * sizeof(int) : 32, s));
+    DSMOE_CUDA_TRY(cudaMemsetAsync(P.sync, 0, by_groups ? L.tile_done - L.sync + (size_t)ceil_div(p.T, 2) * sizeof(int) : 32, s));
     void* args[] = {&mX, &mW1, &mHg, &mW2, &P};
     int timed = -1;
     DSMOE_TRY(timing_begin(s, &timed));
