@@ -128,13 +128,14 @@ __global__ void __launch_bounds__(kLfThreads, 2) layer_f32_tile_kernel(const Til
         }
         commit_copies();
     }
-    // (the selection is not the up tiles' work: when a down tile starts, they have all seen the router's end)
+    // (the selection is not the up tiles' work: when a down tile starts, they have all seen the router's end, and its words lie in L2.  Nothing
+    // but its own wait tells a CTA what its SM's L1 may still hold of them from an earlier call: they are read past it)
     if (UP) {
         chain_wait();
         chain_next();
     }
     // the expert's tokens, in order
-    const uint64_t m = tid < T ? P.mask[tid] : 0;
+    const uint64_t m = tid < T ? __ldcg(reinterpret_cast<const unsigned long long*>(P.mask) + tid) : 0;
     mask_s[tid] = m;
     const bool mine = (m >> e) & 1ull;
     const unsigned hit = __ballot_sync(0xffffffffu, mine);

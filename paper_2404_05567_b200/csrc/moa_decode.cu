@@ -444,7 +444,8 @@ __global__ void __launch_bounds__(32 * kDaWarps, 1) moa_decode_attention_kernel(
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q4 = lane & 3;
     const int nh = P.n_head, T = P.T;
     if (tid < T) {
-        const int sq = P.tok_seq ? P.tok_seq[tid] : 0, last = P.pos[tid];
+        // (before the wait, as the keys are: past an L1 that may hold an earlier step's positions)
+        const int sq = P.tok_seq ? __ldcg(P.tok_seq + tid) : 0, last = __ldcg(P.pos + tid);
         if (blockIdx.x == 0 && (sq < 0 || sq >= P.n_seq || last < 0 || last >= P.L)) report_status(P.dev_status, DSMOE_ERR_INVALID_ARG);
         seq_s[tid] = min(max(sq, 0), P.n_seq - 1);
         last_s[tid] = min(max(last, 0), P.L - 1);

@@ -5,9 +5,11 @@ import math
 
 import numpy as np
 import pytest
+import torch
 
 import dsmoe_inputs as gi
-from harness import TOL_BF16
+import paper_2404_05567_b200 as dm
+from harness import TOL_BF16, to_dev
 from test_gpu_moa import _moa_case, _run
 
 pytestmark = pytest.mark.gpu
@@ -34,3 +36,41 @@ def test_moa_decode(case):
         seq = np.arange(T, dtype=np.int32)
     e, er = _run(s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos, nh, 1.0 / math.sqrt(dh))
     assert er <= TOL_BF16, (e, er)
+
+
+def test_steps_that_change_positions_and_cache_in_place():
+    """Steps without a wait in between, each behind kernels that move the positions on, hand tokens other sequences and write new keys and
+    values into the same buffers: the bits of the same steps on buffers of their own with a wait after each."""
+    T, d, E, nh, dh, L, steps = 24, 256, 8, 4, 128, 200, 10
+    s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos = _moa_case("in_place", T, d, E, nh, dh, T, L, "decode", gi.MODE_TOPK, K=5)
+    desc = dm.make_desc(T, d, nh * dh, E, dm.BF16, dm.SELECT_TOPK, K=5)
+    packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc, to_dev(Wq), to_dev(Wo), packed)
+    ws = torch.empty(dm.dsmoe_workspace_size_packed(desc), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    x_d, Wr_d, br_d, K_d, V_d = (to_dev(a) for a in (x, Wr, br, Kc, Vc))
+    seq_d, pos_d = to_dev(seq), torch.full((T,), 90, dtype=torch.int32, device="cuda") + torch.arange(T, device="cuda", dtype=torch.int32)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    new = torch.randn((steps, 2, T, nh, dh), generator=g, device="cuda").bfloat16()
+    every = torch.arange(T, device="cuda")
+
+    def run(wait):
+        K, V, q, p, outs = K_d.clone(), V_d.clone(), seq_d.clone(), pos_d.clone(), []
+        for i in range(steps):
+            q.copy_(q.roll(1))
+            p.add_(7)
+            K[every, :, p.long()], V[every, :, p.long()] = new[i, 0], new[i, 1]
+            out = torch.empty((T, d), dtype=torch.bfloat16, device="cuda")
+            args = [t.clone() for t in (K, V, q, p)] if wait else (K, V, q, p)
+            if wait:
+                torch.cuda.synchronize()
+            dm.dsmoe_moa_forward(desc, nh, 0.09, *args, x_d, Wr_d, br_d, packed, out, None, None, ws, status)
+            if wait:
+                torch.cuda.synchronize()
+            outs.append(out)
+        torch.cuda.synchronize()
+        return outs
+
+    for a, b in zip(run(True), run(False)):
+        assert torch.equal(a, b)
+    assert int(status.item()) == 0
