@@ -95,7 +95,9 @@ CALLS = {
     "layer_fused_sum": lambda: _layer(T=700, d=512, H=256, E=4, dtype="bf16", mode=gi.MODE_TOPK, K=2, fuse_combine=1),
     "layer_threshold_topk": lambda: _layer(T=513, d=256, H=128, E=16, dtype="bf16", mode=gi.MODE_THRESHOLD_TOPK, eps=0.03),
     "layer_dense": lambda: _layer(T=700, d=256, H=128, E=8, dtype="bf16", mode=gi.MODE_ALL),
-    # either side of the number of tokens beyond which the aggregation is launched the ordinary way
+    # either side of the number of tokens beyond which the aggregation is launched the ordinary way (d 256 to 128 tokens is layer_f32.cu's)
+    "layer_plain_wide_128": lambda: _layer(T=128, d=520, H=128, E=8, dtype="f32", mode=gi.MODE_TOPK, K=2),
+    "layer_plain_wide_129": lambda: _layer(T=129, d=520, H=128, E=8, dtype="f32", mode=gi.MODE_TOPK, K=2),
     "layer_plain_128": lambda: _layer(T=128, d=256, H=128, E=8, dtype="f32", mode=gi.MODE_TOPK, K=2),
     "layer_plain_129": lambda: _layer(T=129, d=256, H=128, E=8, dtype="f32", mode=gi.MODE_TOPK, K=2),
     "layer_grouped_129": lambda: _layer(T=129, d=512, H=256, E=32, dtype="bf16", mode=gi.MODE_TOPK, K=4, fuse_combine=0),

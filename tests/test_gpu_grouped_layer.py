@@ -230,3 +230,50 @@ def test_a_workspace_for_the_running_sums_alone_is_still_enough():
                 run(0, small)
         err = (run(0, full).float() - run(1, small).float()).norm() / run(1, small).float().norm()
         assert err <= 2 ** -8                                     # one rounding to bf16 of sums that differ by rounding in fp32
+
+
+def test_the_other_entry_points_take_that_workspace_too():
+    """dsmoe_moa_forward (sum inside, as with fuse_combine = 1), dsmoe_expert_mlp and dsmoe_dense_backward (nothing of theirs lies there):
+    the bits of a call with the full workspace, or of fuse_combine = 1; with one byte less the call is refused."""
+    T, d, E, K, H, nh, L = 2048, 128, 4, 2, 1024, 8, 64
+    g = torch.Generator(device="cuda").manual_seed(6)
+    randn = lambda *s, std=1.0: (torch.randn(s, generator=g, device="cuda") * std).bfloat16()
+    x, dO, W1, W2 = randn(T, d), randn(T, d), randn(E, d, H, std=0.05), randn(E, H, d, std=0.05)
+    Wr, Kc, Vc = torch.randn((d, E), generator=g, device="cuda") * 0.1, randn(2, nh, L, H // nh), randn(2, nh, L, H // nh)
+    tok = torch.arange(T, device="cuda", dtype=torch.int32)
+    seq, pos = tok // 1024, tok % L
+    desc = {f: dm.make_desc(T, d, H, E, dm.BF16, dm.SELECT_TOPK, K=K, fuse_combine=f) for f in (0, 1)}
+    packed = torch.empty(dm.dsmoe_packed_size(desc[0]), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc[0], W1, W2, packed)
+    small, full = dm.dsmoe_workspace_size_packed(desc[1]), dm.dsmoe_workspace_size_packed(desc[0])
+    assert small < full
+    status, scores = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.empty((T, E), device="cuda")
+    dm.dsmoe_router(desc[0], x, Wr, None, scores)
+    offsets = torch.arange(E + 1, device="cuda", dtype=torch.int32) * (T * K // E)
+    xp = randn(T * K, d)
+
+    def moa(f, n):
+        out = torch.empty((T, d), dtype=torch.bfloat16, device="cuda")
+        dm.dsmoe_moa_forward(desc[f], nh, 0.09, Kc, Vc, seq, pos, x, Wr, None, packed, out, None, None, ws[:n], status)
+        return [out]
+
+    def experts(f, n):
+        yp = torch.empty((T * K, d), dtype=torch.bfloat16, device="cuda")
+        dm.dsmoe_expert_mlp(desc[f], xp, None, None, packed, offsets, yp, ws[:n], status)
+        return [yp]
+
+    def backward(f, n):
+        dS, dA = torch.empty((T, E), device="cuda"), torch.empty((T, E * H), dtype=torch.bfloat16, device="cuda")
+        dm.dsmoe_dense_backward(desc[f], x, None, W2, packed, scores, None, dO, dS, dA, ws[:n], status)
+        return [dS, dA]
+
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+    for call, like in ((moa, (1, small)), (experts, (0, full)), (backward, (0, full))):
+        ws.fill_(0x5a)
+        got = call(0, small)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and (ws[small:] == 0x5a).all()
+        for a, b in zip(got, call(*like)):
+            assert torch.equal(a, b), call.__name__
+        with pytest.raises(dm.DsmoeError):
+            call(0, small - 1)

@@ -172,8 +172,10 @@ def test_moa_prompts(case):
     assert er <= TOL_BF16, (e, er)
 
 
-# One case per attention kernel: tiles that share their keys, the key-splitting and the tile-per-warp form, the plain kernel
-CLAMPED = [("clamp_prompt", 40, 64, 3, 65), ("clamp_split", 12, 64, 4, 600), ("clamp_tiles", 12, 64, 4, 90), ("clamp_plain", 20, 32, 3, 33)]
+# One case per attention kernel: tiles that share their keys, decoding tokens (long and short caches), the plain kernel; of more tokens than
+# the decoding one takes, the key-splitting and the tile-per-warp form; tiles of 128 rows with the key-splitting kernel behind them
+CLAMPED = [("clamp_prompt", 40, 64, 3, 65), ("clamp_split", 12, 64, 4, 600), ("clamp_tiles", 12, 64, 4, 90), ("clamp_plain", 20, 32, 3, 33),
+           ("clamp_split_80", 80, 64, 12, 600), ("clamp_tiles_80", 80, 64, 12, 90), ("clamp_tile_of_128", 3000, 64, 2, 600)]
 
 
 @pytest.mark.parametrize("case", CLAMPED, ids=[c[0] for c in CLAMPED])
