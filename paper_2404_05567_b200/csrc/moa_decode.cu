@@ -51,7 +51,7 @@ __device__ __forceinline__ float exp2_fast(float v) {
 //
 // out[t, n] = sum over k of X[t, k] W[n, k] with the weights as the rows of m16n8k16 and the tokens (up to 64) as its columns.  A
 // CTA, or a cluster of two or four where there are few rows, owns 32 weight rows and takes the reduction in blocks of 64.  Its eight
-// warps work by themselves: a warp takes every eighth block, by TMA through a ring of its own that its lane 0 fills.  (With one
+// warps work by themselves: a warp takes every eighth block, by TMA through a ring of its own that an elected lane fills.  (With one
 // thread to fill one ring for all, some 12 copies a microsecond got under way: 4096 x 4096 weights for 32 tokens took 14.6 us, 5.3 so: the
 // weights at 6.3 TB/s, the tensor pipe busy for 4.3 of it.)  The warps' and the CTAs' sums meet in shared memory, in that order.  The output
 // projection's sums are multiplied by the token's gate, in fp32, whenever a warp passes from one expert to the next.
@@ -218,10 +218,11 @@ moa_decode_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
         }
         ptx::fence_barrier_init();
     }
+    __syncwarp();                                             // the lane that is elected below need not be this one
     const uint32_t ring = base + (uint32_t)(warp * S * G::STAGE);
     const int row0 = group * kDgRows;                         // the rows lie in one expert (queries)
     const int w_row = QUERY ? row0 % P.rows_per_expert : row0, w_e = QUERY ? row0 / P.rows_per_expert : 0;
-    // (lane 0) block i of the CTA into stage s of the warp
+    // (an elected lane) block i of the CTA into stage s of the warp
     const auto load_w = [&](int i, int s) {
         const uint32_t bar = ptx::smem_u32(&sh.full[warp][s]), dst = ring + (uint32_t)(s * G::STAGE);
         ptx::mbar_expect_tx(bar, G::STAGE);
