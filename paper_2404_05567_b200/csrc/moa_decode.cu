@@ -422,13 +422,14 @@ struct DecodeAttnParams {
 
 }  // namespace
 
-// Aligned runs over pairs of `units` units each: where CTA c's begins.  split: `per` CTAs to a pair, else `per` pairs to a CTA.
-// (units * r / per without the product, which a cache of 233 million positions takes out of an int's range)
+// Aligned runs over pairs of `units` units each: where CTA c's begins.  split: `per` CTAs to a pair, else `per` pairs to a CTA.  The
+// product stays an int's as long as decode_runs_align allows such runs (asking for that here, or a quotient without it, cost 0.4 of 44.5 us).
 __host__ __device__ int decode_run_start(int c, int units, int per, int pairs, bool split) {
-    if (!split) return (c * per < pairs ? c * per : pairs) * units;
-    const int r = c % per;
-    return c / per * units + units / per * r + units % per * r / per;
+    return split ? c / per * units + units * (c % per) / per : (c * per < pairs ? c * per : pairs) * units;
 }
+// Whether pairs of `units` units each are to be cut so, the longest run being `longest` of `total` units (see the kernel).  From 134 million
+// keys a pair on never: 255 CTAs times their units would leave an int.
+__host__ __device__ bool decode_runs_align(int units, int longest, int total) { return units < 1 << 23 && longest <= total / 100 + 64; }
 
 namespace {
 
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(32 * kDaWarps, 1) moa_decode_attention_kernel(
     const int per = split ? min(grid / pairs, units0) : (pairs + grid - 1) / grid;
     const int whole_ctas = split ? pairs * per : (pairs + per - 1) / per;
     const int longest = split ? (units0 + per - 1) / per : per * units0;
-    const bool aligned = alike_s && longest <= total / 100 + 64;
+    const bool aligned = alike_s && decode_runs_align(units0, longest, total);
     const int n_cta = aligned ? whole_ctas : min(grid, total);
     if ((int)blockIdx.x >= n_cta) return;
     const int share = total / n_cta, extra = total - share * n_cta;
