@@ -19,8 +19,8 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 
 // One lane of a converged warp, the same one every time.  The roles that issue tensor copies or MMAs choose their thread this way and
 // not by its number: only so does the compiler know that one thread is active, and keeps the instructions' operands (which live in
-// the warp's uniform registers) without a loop over the lanes around each of them.  A thread got 10.8 instead of 6.1 copies a microsecond
-// under way (16 to 64 rows of 128 bytes out of L2), 39 instead of 46 clocks an MMA of 16 columns.
+// the warp's uniform registers) without a loop over the lanes around each of them.  A thread that also waits for its slots gets 7.5 instead of
+// 5.3 copies a microsecond under way (16 to 64 rows of 128 bytes out of L2: diagnostics/tma_copy_rate.cu).
 __device__ __forceinline__ bool elect_one() {
     uint32_t one;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));

@@ -12,6 +12,8 @@
 
 using namespace dsmoe;
 
+// ELECT: the issuing lane is elected, as everywhere in the library; otherwise chosen by its number
+template <bool ELECT>
 __global__ void __launch_bounds__(256, 1) stream_kernel(const __grid_constant__ CUtensorMap tm, int rows, int depth,
                                                        int copies_per_cta, int evict_first, long long rows_total,
                                                        long long span_rows, unsigned long long* gave_up) {
@@ -27,8 +29,7 @@ __global__ void __launch_bounds__(256, 1) stream_kernel(const __grid_constant__ 
     __syncthreads();
     // `issuers` warps (blockDim.x / 32) each run the same single-thread loop on their own slots and their own share
     // of the CTA's copies: does the copy rate depend on how many threads issue?
-    // (an elected lane: behind `lane == 0` a copy takes 165 ns to issue instead of 93)
-    if (!ptx::elect_one()) return;
+    if (!(ELECT ? ptx::elect_one() : (threadIdx.x & 31) == 0)) return;
     const int issuer = threadIdx.x >> 5, issuers = blockDim.x >> 5;
     uint64_t* full = full_all + issuer * depth;
     copies_per_cta /= issuers;
@@ -84,7 +85,8 @@ int main() {
     if (cudaMalloc(&buf, bytes) != cudaSuccess || cudaMalloc(&gave_up, 8) != cudaSuccess) return 1;
     cudaMemset(buf, 1, bytes);
     cudaMemset(gave_up, 0, 8);
-    cudaFuncSetAttribute(stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 170 * 1024);
+    cudaFuncSetAttribute(stream_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 170 * 1024);
+    cudaFuncSetAttribute(stream_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 170 * 1024);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -105,28 +107,30 @@ int main() {
         for (int depth = 1; depth <= 32; depth *= 2) {
             if ((long long)issuers * depth * rows * 128 > 160 * 1024 || issuers * depth > 64) continue;
             if (issuers > 1 && depth != 2 && depth != 4) continue;
-            float gbs[2];
-            for (int hint = 0; hint < 2; ++hint) {
-                if (from_l2 && hint) {       // evict-first makes no sense for data that is meant to stay
-                    gbs[1] = gbs[0];
-                    continue;
-                }
-                const long long per_cta = 4ll << 20;
-                const int copies = (int)(per_cta / (rows * 128));
+            const long long per_cta = 4ll << 20;
+            const int copies = (int)(per_cta / (rows * 128));
+            // elected without and with the evict-first hint (which makes no sense for data that is meant to stay); lane 0
+            float gbs[3] = {};
+            for (int form = 0; form < 3; ++form) {
+                if (from_l2 && form == 1) continue;
+                const int hint = from_l2 ? 0 : form != 0;
                 float best = 1e9f;
                 for (int rep = 0; rep < 3; ++rep) {
                     cudaEventRecord(e0);
-                    stream_kernel<<<sms, 32 * issuers, 170 * 1024>>>(tm, rows, depth, copies, hint, rows_total, span_rows, gave_up);
+                    auto* kernel = form < 2 ? stream_kernel<true> : stream_kernel<false>;
+                    kernel<<<sms, 32 * issuers, 170 * 1024>>>(tm, rows, depth, copies, hint, rows_total, span_rows, gave_up);
                     cudaEventRecord(e1);
                     cudaEventSynchronize(e1);
                     float ms;
                     cudaEventElapsedTime(&ms, e0, e1);
                     best = ms < best ? ms : best;
                 }
-                gbs[hint] = (float)((double)sms * per_cta / best / 1e6);
+                gbs[form] = (float)((double)sms * per_cta / best / 1e6);
             }
-            printf("copy %6d B  x %2d in flight x %d issuing warps = %7d B per SM : %7.1f / %7.1f GB/s   (%.2f copies per us and SM)\n",
-                   rows * 128, depth, issuers, issuers * depth * rows * 128, gbs[0], gbs[1], gbs[1] * 1e3 / sms / (rows * 128));
+            if (from_l2) gbs[1] = gbs[0];
+            const double per_us = 1e3 / sms / (rows * 128);
+            printf("copy %6d B  x %2d in flight x %d issuing warps = %7d B per SM : %7.1f / %7.1f GB/s   (copies per us and SM: %.2f, behind lane == 0 %.2f)\n",
+                   rows * 128, depth, issuers, issuers * depth * rows * 128, gbs[0], gbs[1], gbs[1] * per_us, gbs[2] * per_us);
         }
     }
     unsigned long long h = 0;
