@@ -793,7 +793,7 @@ __global__ void __launch_bounds__(32 * kShWarps, 3) moa_attention_shared_kernel(
 // row's maximum, weights and sum without a word from its neighbours, P (bf16) into the 128-byte swizzle where the keys lay, P.V into TMEM,
 // and the running values in the thread's registers (fp32; nothing is rescaled in TMEM).  Keys and values lie as in memory; V is an N-major
 // operand.  A block of both is copied while the one before is worked on, two CTAs fill an SM (255 registers a thread, 97 KB each).
-// 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 102 us with the warp-level path, 81 so (cold caches; the layer 482 -> 452).
+// 32 prompts of 256 tokens, 4 heads of 128, 8 experts top-5: 102 us with the warp-level path, 81 to 84 so (cold caches; the layer 482 -> 452).
 // Bound by the instruction issue of the weights and of the copies' addresses (0.34 a cycle and scheduler with two warps each; the
 // tensor pipe 9 % busy).  Asking for the next block's S before this one's weights, and adding P.V a block later: 85 us (registers).
 // The sums are of the rounded weights, which P.V is made of: whole layers of 4 heads of 128 and of 96 and 2 of 64 are 1.970e-3, 2.017e-3 and
@@ -809,6 +809,9 @@ int umma_attention_groups(int W) { return W <= 16 ? kUaRows / (W * kShWarps * sh
 // top-5, us a layer, that kernel and this one: 400 tokens, 68 CTAs, 83, 86; 1024, 172 CTAs, 119, 117; 8192 482, 452; one prompt of 2048
 // 243, 215; 16 of 2 heads of 64, top-6: 800 tokens, 100 CTAs, 63, 65; 2048, 256 CTAs, 101, 98), and with prompts long enough that few tiles walk two
 // (16 of 2 heads of 64: 30 prompts of 100 tokens 86, 88, of 128 159, 156; 8 of 4 heads of 128: 60 of 64 234, 237, 30 of 100 192, 181).
+// Tokens of several sequences in no order, which the host does not see, are slower here (8 of 4 heads of 128, that kernel alone and this one: 2500 tokens of
+// 5 sequences at random, 300 positions, 262, 302; 4096 of 16, 256 positions, 355, 397; 1250 of 2, 400 positions, 169, 183; in rounds of two 160, 140): their
+// groups take the other form with 8 warps an SM for its 12.  Left to a launch of their own they were no faster and prompts in order 2 to 9 % slower.
 bool umma_attention_fits(const dsmoe_layer_desc& p, const MoaCore& c) {
     const int W = width_of(p);
     const long long span = (long long)umma_attention_groups(W) * kShWarps * shared_tile_tokens(W), n_seq = c.tok_seq ? c.n_seq : 1;
