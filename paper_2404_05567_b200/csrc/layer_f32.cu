@@ -5,7 +5,7 @@
 //   down    rows gate * (h . W2[e]) by tiles likewise; of the CTAs of a column range the one that comes last adds up every token's
 //           rows, in ascending order of the experts
 //
-// A CTA finds its expert's tokens in the selection words itself, and a token's row for its i-th selected expert is row t * W + i of h and of
+// A CTA finds its expert's tokens in the selection words itself, and a token's row for its i-th selected expert (i < W) is row t * W + i of h and of
 // the outputs: no row indices, no launch that computes them.  A tile's weights (all of its reduction) are asked for before the CTA waits
 // for its predecessor: nothing that the call itself writes.  Bound by the chain of short steps (router 2.3 us; tokens found, rows fetched,
 // multiplied and stored 6 and, without the first, 5; the last CTA's sum 2; some 0.9 from a launch's end to the next one's start): 64 tokens of
@@ -135,7 +135,13 @@ __global__ void __launch_bounds__(kLfThreads, 2) layer_f32_tile_kernel(const Til
         chain_next();
     }
     // the expert's tokens, in order
-    const uint64_t m = tid < T ? __ldcg(reinterpret_cast<const unsigned long long*>(P.mask) + tid) : 0;
+    uint64_t m = tid < T ? __ldcg(reinterpret_cast<const unsigned long long*>(P.mask) + tid) : 0;
+    if (UP && n0 == 0 && P.counts_out) {
+        const int n = __syncthreads_count((m >> e) & 1ull);
+        if (tid == 0) P.counts_out[e] = n;
+    }
+    // a token has W rows: one whose scores are no numbers is selected by all experts under top-K, and keeps the first W
+    while (__popcll(m) > P.W) m ^= 1ull << (63 - __clzll((long long)m));
     mask_s[tid] = m;
     const bool mine = (m >> e) & 1ull;
     const unsigned hit = __ballot_sync(0xffffffffu, mine);
@@ -148,7 +154,6 @@ __global__ void __launch_bounds__(kLfThreads, 2) layer_f32_tile_kernel(const Til
         n_rows += count_s[w];
     }
     if (mine) list_s[before + __popc(hit & ((1u << lane) - 1u))] = tid;
-    if (UP && n0 == 0 && tid == 0 && P.counts_out) P.counts_out[e] = n_rows;
     if (!UP) {
         chain_wait();
         chain_next();
