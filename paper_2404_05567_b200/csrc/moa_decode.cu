@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(32 * kDaWarps, 1) moa_decode_attention_kernel(
     for (int at = u0; at < u1;) {
         const int units = units_s[seg.t], end = min(u1, at + units - seg.k), t = seg.t, j = seg.j, first_k = seg.k;
         const uint64_t sel = next_sel;
-        const int rows = min(__popcll(sel), 16);
+        const int rows = min(__popcll(sel), P.W);        // (under top-K more are set where a token's scores are no numbers: a part has W rows)
         // the queries of all experts: the selection comes with them, not before
         if (tid < P.E * CH) *reinterpret_cast<uint4*>(q_s + (tid / CH) * STRIDE + tid % CH * 16) = next_q;
         __syncthreads();

@@ -1,11 +1,15 @@
 """Tokens whose scores are not numbers under a top-K selection: every expert selects them (a score that is no number is beaten by none), more than
 the K rows that a token has.  They get NaN, or an error is reported; nothing is written past the workspace, and the other tokens' outputs
 are those of a call without them (GPU required)."""
+import math
+
 import pytest
 import torch
 
 import dsmoe_inputs as gi
-from harness import Layer
+import paper_2404_05567_b200 as dm
+from harness import Layer, to_dev
+from test_gpu_moa import _moa_case
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +39,31 @@ def test_fp32_layer(T, d, H, E, K):
     assert torch.equal(out[_others(T, bad)], clean[_others(T, bad)]) and out[bad].isnan().all()
     assert all(int(L.mask[t]) == 2 ** E - 1 for t in bad)
     assert L.counts[:E].tolist() == [int(((L.mask >> e) & 1).sum()) for e in range(E)]
+
+
+@pytest.mark.parametrize("ragged", [False, True], ids=["alike", "ragged"])
+@pytest.mark.parametrize("T,E,K,dh", [(8, 8, 3, 128), (20, 16, 1, 64), (33, 16, 6, 96)], ids=lambda v: str(v))
+def test_decoding_attention(T, E, K, dh, ragged):
+    """Few enough pairs of tokens and heads that several CTAs share each one's keys and leave parts of K rows."""
+    d, nh, L = 1024, 2, 400
+    s, x, Wr, br, Wq, Wo, Kc, Vc, seq, pos = _moa_case(f"nanmoa{T}", T, d, E, nh, dh, T, L, "decode", gi.MODE_TOPK, K=K)
+    if not ragged:
+        pos[:] = L - 1
+    desc = dm.make_desc(T, d, nh * dh, E, dm.BF16, dm.SELECT_TOPK, K=K, out_fp32=1)
+    packed = torch.empty(dm.dsmoe_packed_size(desc), dtype=torch.uint8, device="cuda")
+    dm.dsmoe_pack_weights(desc, to_dev(Wq), to_dev(Wo), packed)
+    nbytes, status = dm.dsmoe_workspace_size_packed(desc), torch.zeros(1, dtype=torch.int32, device="cuda")
+    args = [to_dev(a) for a in (Kc, Vc, seq, pos)]
+    Wr_d, br_d, x_d = to_dev(Wr), to_dev(br), to_dev(x)
+
+    def run(x_d):
+        buf, out = _guarded(nbytes), torch.empty((T, d), device="cuda")
+        dm.dsmoe_moa_forward(desc, nh, 1 / math.sqrt(dh), *args, x_d, Wr_d, br_d, packed, out, None, None, buf[:nbytes], status)
+        torch.cuda.synchronize()
+        assert (buf[nbytes:] == 0x5a).all()
+        return out
+
+    bad = [2, T - 1]
+    clean, out = run(x_d), run(_bad_tokens(x_d, bad))
+    assert int(status.item()) == 0
+    assert torch.equal(out[_others(T, bad)], clean[_others(T, bad)]) and out[bad].isnan().all()
