@@ -581,8 +581,11 @@ grouped_layer_kernel(const __grid_constant__ BMaps tmW1, const __grid_constant__
                 find_tokens<FOLD ? FOLD : 1>(bits, t.e, first + q * 32, first + t.rows_valid - 1, lane, tok);
                 if (valid) {
                     g = P.fold.scores[(size_t)tok[0] * P.E + t.e];
-                    if (t.n0 == 0)       // once a row: where the aggregation finds it
-                        P.fold.token_rows[(size_t)tok[0] * P.W + __popcll(P.fold.mask[tok[0]] & ((1ull << t.e) - 1ull))] = t.row0 + row;
+                    if (t.n0 == 0) {     // once a row: where the aggregation finds it
+                        const int slot = __popcll(P.fold.mask[tok[0]] & ((1ull << t.e) - 1ull));
+                        // (a token of top-K whose scores are no numbers is selected by all experts)
+                        if (slot < P.W) P.fold.token_rows[(size_t)tok[0] * P.W + slot] = t.row0 + row;
+                    }
                 }
             } else if (!t.up && valid) {
                 g = P.row_gate[t.row0 + row];

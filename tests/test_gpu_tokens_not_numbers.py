@@ -67,3 +67,24 @@ def test_decoding_attention(T, E, K, dh, ragged):
     clean, out = run(x_d), run(_bad_tokens(x_d, bad))
     assert int(status.item()) == 0
     assert torch.equal(out[_others(T, bad)], clean[_others(T, bad)]) and out[bad].isnan().all()
+
+
+@pytest.mark.parametrize("T,E,K", [(200, 8, 2), (300, 33, 3), (1500, 16, 1)], ids=lambda v: str(v))
+def test_rows_from_selection_words(T, E, K):
+    """Grouped by expert there are then more rows than T * K: the experts whose segments end beyond are reported and count as empty."""
+    L = Layer(gi.LayerSpec(f"nanfold{T}", T=T, d=128, H=64, E=E, dtype="bf16", mode=gi.MODE_TOPK, K=K, router_gain=4.0))
+    clean, mask, nbytes, x = L.forward().clone(), L.mask.clone(), L.ws.numel(), L.x_d
+    t = T // 2
+    buf = _guarded(nbytes)
+    L.ws, L.x_d = buf[:nbytes], _bad_tokens(x, [t])
+    with pytest.raises(AssertionError, match="device status 1"):
+        L.forward()
+    assert (buf[nbytes:] == 0x5a).all() and int(L.mask[t]) == 2 ** E - 1
+    ends = L.counts[:E].cumsum(0)
+    lost = sum(1 << e for e in range(E) if int(ends[e]) > T * K)
+    kept = [i for i in _others(T, [t]) if int(mask[i]) & lost == 0]
+    assert len(kept) > T // 2
+    assert torch.equal(L.out[kept], clean[kept])
+    L.dev_status.zero_()
+    L.x_d = x
+    assert torch.equal(L.forward(), clean)
